@@ -1,0 +1,536 @@
+"""Performance cases of the split-LoRA library: what a training program has it do, over the range of sizes,
+types and options that such programs use.
+
+Five kinds of case, each through the public entry points of `paper_2407_00952_b200.binding`:
+  round      one iteration of Algorithm 1 (client forward, server step, client backward, aggregation) on one
+             context, as one call (`round` / `round_host`) or as the separate calls (`calls`)
+  lora       forward and backward of the grouped LoRA linear layer (a program with a block of its own)
+  attention  causal attention on a fused qkv buffer, forward and backward
+  handoff    the cut-layer tensor to 8-bit codes and back (sender and receiver of a compressed link)
+  aggregate  the weighted average of the clients' adapters (the fed server's step by itself)
+
+All inputs are synthetic and made on the GPU from the seed: frozen weights and adapters N(0, 0.02) (adapters as
+in mid-training, B not zero), gains near one, small biases, token ids from a bounded Zipf law.
+"""
+from __future__ import annotations
+
+import math
+
+import torch
+
+from paper_2407_00952_b200 import binding as B
+
+SIZES = {  # width, heads, MLP width of the shapes this repository names, and generic narrower ones
+    "gpt2-medium": (1024, 16, 4096),
+    "gpt2-small": (768, 12, 3072),
+    "w512": (512, 8, 2048),
+    "w256": (256, 4, 1024),
+    "tiny": (128, 4, 512),
+    "llama2-7b": (4096, 32, 11008),
+    "llama-w1024": (1024, 8, 2816),
+}
+
+
+def _round(name, size, dtype="bf16", arch="gpt", layers=12, cut=3, K=4, b=8, T=512, r=4, targets="qv", vocab=50257,
+           optimizer="adamw", api="round", padded=False, cut_min=0, mixed_ranks=False, lr=2e-4):
+    c = {"kind": "round", "size": size, "dtype": dtype, "arch": arch, "layers": layers, "cut": cut, "K": K, "b": b, "T": T,
+         "r": r, "targets": targets, "vocab": vocab, "optimizer": optimizer, "api": api, "padded": padded,
+         "cut_min": cut_min, "mixed_ranks": mixed_ranks, "lr": lr}
+    return dict(c, name=name) if name else c
+
+
+def _lora(name, M, n_in, n_out, r, G, dtype="bf16"):
+    c = {"kind": "lora", "M": M, "n_in": n_in, "n_out": n_out, "r": r, "G": G, "dtype": dtype}
+    return dict(c, name=name) if name else c
+
+
+def _attention(name, nseq, T, heads, width, dtype="bf16"):
+    c = {"kind": "attention", "nseq": nseq, "T": T, "heads": heads, "width": width, "dtype": dtype}
+    return dict(c, name=name) if name else c
+
+
+def listed():
+    return [
+        # the paper-sized toy of the functional tests, fp32 throughout: 512 tokens, every launch is short
+        _round("round_tiny_fp32", "tiny", dtype="fp32", layers=2, cut=1, K=2, b=4, T=64, vocab=1024, lr=1e-3),
+        # a GPT-2-medium-shaped round with very few tokens (two clients, one short sequence each): the host and
+        # the length of the chain of launches count
+        _round("round_few_tokens", "gpt2-medium", layers=24, cut=6, K=2, b=1, T=256, api="host"),
+        # the GPT-2-small-shaped workload, tokens handed over from host memory
+        _round("round_gpt2_small", "gpt2-small", api="host"),
+        # the GPT-2-medium-shaped workload of the benchmark
+        _round("round_gpt2_medium", "gpt2-medium", layers=24, cut=6, K=8),
+        # the Llama-2-7B-shaped block at 4 of its 32 layers (width, heads, rank, batch and targets unchanged)
+        _round("round_llama", "llama2-7b", arch="llama", layers=4, cut=1, K=4, b=2, T=1024, r=16, targets="qkvo", vocab=32000),
+        # heterogeneous clients: own cut depths and ranks, a sequence length off the tile sizes, padded sequences,
+        # plain SGD, the steps called one by one as a program with real links does
+        _round("round_ragged_clients", "gpt2-small", K=4, b=8, T=288, cut=4, cut_min=2, mixed_ranks=True, optimizer="sgd",
+               api="calls", padded=True),
+        # the centralised baseline (one client) on a batch whose token count is a multiple of nothing
+        _round("round_ragged_single", "gpt2-small", K=1, b=5, T=333, padded=True),
+        # one adapted qkv projection of eight clients, and one of a single adapter at an odd size and rank
+        _lora("lora_linear_grouped", 16384, 1024, 3072, 4, 8),
+        _lora("lora_linear_odd", 1000, 768, 2304, 6, 1),
+        # attention of a batch of sequences of odd length
+        _attention("attention_ragged", 16, 777, 12, 64),
+        # the cut-layer tensor of the GPT-2-medium-shaped workload over a compressed link
+        {"kind": "handoff", "name": "handoff_codec", "M": 32768, "d": 1024, "dtype": "bf16"},
+        # averaging eight clients' adapter sets of 8 MiB
+        {"kind": "aggregate", "name": "aggregate_8_clients", "K": 8, "P": 1 << 21},
+    ]
+
+
+def _log(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    kind = rng.choice(["round", "round", "round", "llama", "tiny", "lora", "lora", "attention", "attention", "handoff", "aggregate"])
+    if kind == "round":
+        size = rng.choice(["gpt2-medium", "gpt2-small", "w512", "w256"])
+        layers = _log(rng, 2, 12)
+        cut = rng.randint(1, max(1, layers // 2))
+        K = rng.choice([1, 1, 2, 3, 4, 8])
+        T = _log(rng, 24, 1024)
+        if K == 1:        # one client: any length and batch
+            b = max(1, min(16, _log(rng, 64, 4096) // T, 2_000_000 // (T * T)))
+        else:             # several clients: whole 256-token tiles per client
+            T = max(32, T // 16 * 16 if rng.random() < 0.6 else T // 128 * 128)
+            rows = K * T * (256 // math.gcd(T, 256))
+            if rows > 16384 or (T % 64 and rows * T > 2_000_000):
+                T = max(128, T // 128 * 128)
+            unit = 256 // math.gcd(T, 256)
+            b = unit * max(1, min(4, _log(rng, 256, 8192) // (unit * T * K) if T % 64 == 0 else 1))
+        hetero = K > 1 and rng.random() < 0.3
+        cut = max(cut, 2) if hetero and layers > 2 else cut
+        return _round(None, size, layers=layers, cut=cut, K=K, b=b, T=T, r=rng.choice([1, 2, 4, 6, 8, 16, 32]),
+                      targets=rng.choice(["qv", "qv", "q", "qkv", "qvo"]), optimizer=rng.choice(["adamw", "adamw", "sgd"]),
+                      api=rng.choice(["round", "host", "calls"]), padded=rng.random() < 0.5, cut_min=1 if hetero else 0,
+                      mixed_ranks=hetero)
+    if kind == "llama":
+        size = rng.choice(["llama-w1024", "llama-w1024", "llama2-7b"])
+        K, T = rng.choice([1, 2, 4]), rng.choice([128, 256, 384, 512, 1024, 200 if K == 1 else 640])
+        unit = 256 // math.gcd(T, 256) if K > 1 else 1
+        b = unit * max(1, min(2, 2048 // (unit * T * K)))
+        return _round(None, size, arch="llama", layers=rng.randint(2, 4) if size != "llama2-7b" else 2, cut=1, K=K, b=b, T=T,
+                      r=rng.choice([4, 8, 16]), targets=rng.choice(["qkvo", "qv"]), vocab=32000)
+    if kind == "tiny":
+        K = rng.choice([1, 2, 4])
+        T = rng.choice([64, 128, 192]) if K > 1 else rng.randint(20, 256)
+        return _round(None, rng.choice(["tiny", "w256"]), dtype="fp32", layers=rng.randint(2, 4), cut=1, K=K, b=4, T=T,
+                      r=rng.choice([2, 4, 8]), vocab=rng.choice([1000, 1024, 5003]), optimizer=rng.choice(["adamw", "sgd"]), lr=1e-3)
+    if kind == "lora":
+        G = rng.choice([1, 1, 2, 4, 8, 16])
+        M = _log(rng, 100, 65536) if G == 1 else G * 128 * max(1, _log(rng, 256, 65536) // (G * 128))
+        n_in = rng.choice([256, 768, 1000, 1024, 4096])
+        n_out = rng.choice([256, 768, 1000, 2304, 3072, 4096])
+        if G == 1 and (M % 128 or n_in % 64):
+            M = min(M, 4096)
+        if n_in % 64 or n_out % 64:
+            M = min(M, 8192 // G // 128 * G * 128 if G > 1 else 4096)
+        return _lora(None, M, n_in, n_out, rng.choice([1, 2, 4, 6, 8, 16, 32, 64]), G)
+    if kind == "attention":
+        width = rng.choice([32, 64, 64, 64, 128, 128])
+        heads = rng.choice([4, 8, 12, 16])
+        T = _log(rng, 32, 2048) if rng.random() < 0.6 else 64 * _log(rng, 1, 32)
+        fast = width >= 64 and T % 64 == 0
+        nseq = max(1, min(64, _log(rng, 1024, 32768 if fast else 4096) // T))
+        return _attention(None, nseq, T, heads, width, dtype="bf16" if rng.random() < 0.85 or T > 600 else "fp32")
+    if kind == "handoff":
+        return {"kind": "handoff", "M": _log(rng, 100, 65536), "d": rng.choice([256, 768, 1024, 2048, 4096]) if rng.random() < 0.7 else 8 * rng.randint(10, 400),
+                "dtype": rng.choice(["bf16", "bf16", "fp32"])}
+    return {"kind": "aggregate", "K": rng.choice([1, 2, 3, 5, 8, 16, 32]), "P": 4 * _log(rng, 1024, 1 << 20)}
+
+
+# ---- inputs ---------------------------------------------------------------------------------------
+
+def _dt(case):
+    return torch.bfloat16 if case["dtype"] == "bf16" else torch.float32
+
+
+def _gen(seed):
+    return torch.Generator(device="cuda").manual_seed(seed)
+
+
+def _shape(case):
+    d, heads, ff = SIZES[case["size"]]
+    return d, heads, ff
+
+
+def _cuts(case):
+    """Per-client cut depths, from cut_min to cut (one depth for all unless cut_min is set)."""
+    K, lo, hi = case["K"], case["cut_min"] or case["cut"], case["cut"]
+    return [lo + (hi - lo) * i // max(1, K - 1) for i in range(K)]
+
+
+def _ranks(case):
+    return [max(1, case["r"] >> (i % 3)) if case["mixed_ranks"] else case["r"] for i in range(case["K"])]
+
+
+def _frozen(case, g):
+    """(name, tensor) of the frozen model, in the case's type."""
+    d, _, ff = _shape(case)
+    dt, V, T = _dt(case), case["vocab"], case["T"]
+    mat = lambda *s: torch.empty(*s, device="cuda", dtype=dt).normal_(0.0, 0.02, generator=g)  # noqa: E731
+    gain = lambda n: (1.0 + 0.1 * torch.randn(n, device="cuda", generator=g)).to(dt)  # noqa: E731
+    llama = case["arch"] == "llama"
+    out = [("wte", mat(V, d)), ("head.w", mat(V, d)) if llama else ("wpe", mat(T, d)), ("lnf.g", gain(d))]
+    if not llama:
+        out.append(("lnf.b", mat(d)))
+    for l in range(case["layers"]):
+        p = f"h.{l}."
+        out += [(p + "ln1.g", gain(d)), (p + "attn.qkv.w", mat(3 * d, d)), (p + "attn.proj.w", mat(d, d)), (p + "ln2.g", gain(d))]
+        if llama:
+            out += [(p + "mlp.gate_up.w", mat(2 * ff, d)), (p + "mlp.down.w", mat(d, ff))]
+        else:
+            out += [(p + "ln1.b", mat(d)), (p + "attn.qkv.b", mat(3 * d)), (p + "attn.proj.b", mat(d)), (p + "ln2.b", mat(d)),
+                    (p + "mlp.fc1.w", mat(ff, d)), (p + "mlp.fc1.b", mat(ff)), (p + "mlp.fc2.w", mat(d, ff)), (p + "mlp.fc2.b", mat(d))]
+    return out
+
+
+def _adapters(case, g):
+    """fp32 adapters of the clients [K, cut, targets, 2, r*d] and of the server [layers - first, targets, 2, r*d]:
+    A [r, d] and B [d, r] of each target in the order q, k, v, o."""
+    d = _shape(case)[0]
+    n, r, first = len(case["targets"]), case["r"], case["cut_min"] or case["cut"]
+    client = torch.empty(case["K"], case["cut"], n, 2, r * d, device="cuda").normal_(0.0, 0.02, generator=g)
+    server = torch.empty(case["layers"] - first, n, 2, r * d, device="cuda").normal_(0.0, 0.02, generator=g)
+    return client, server
+
+
+def _tokens(case, g):
+    """Token ids [K, b, T] and the next ids as labels; with `padded`, sequences end early and the rest is ignored."""
+    K, b, T, V = case["K"], case["b"], case["T"], case["vocab"]
+    p = torch.arange(1, V + 1, device="cuda", dtype=torch.float64) ** -1.1
+    order = torch.randperm(V, device="cuda", generator=g)
+    # inverse of the distribution function: one uniform number per token
+    cdf = torch.cumsum(p / p.sum(), 0)
+    u = torch.rand(K, b, T + 1, device="cuda", generator=g, dtype=torch.float64)
+    ids = order[torch.searchsorted(cdf, u).clamp_(max=V - 1)].int()
+    tokens, labels = ids[..., :T].contiguous(), ids[..., 1:].contiguous()
+    if case["padded"]:
+        length = torch.randint((T + 1) // 2, T + 1, (K, b, 1), device="cuda", generator=g)
+        labels = torch.where(torch.arange(T, device="cuda") < length, labels, torch.full_like(labels, -1)).contiguous()
+    counts = [200 + (37 * (i + 1) * (i + 5)) % 801 for i in range(K)]
+    return tokens, labels, counts
+
+
+def _prepare_round(case, seed):
+    g = _gen(seed)
+    d, heads, ff = _shape(case)
+    bits = 0
+    for t in case["targets"]:
+        bits |= B.TARGET_BITS[t]
+    cfg = B.Config(n_layer=case["layers"], cut=case["cut"], d_model=d, n_head=heads, d_ff=ff, vocab=case["vocab"], max_seq=case["T"],
+                   lora_r=case["r"], lora_alpha=8.0 * case["r"] if case["r"] <= 4 else 32.0, lora_targets=bits, n_clients=case["K"],
+                   batch_per_client=case["b"], seq=case["T"], dtype=B.DTYPE_BF16 if case["dtype"] == "bf16" else B.DTYPE_FP32,
+                   optimizer=B.OPT_ADAMW if case["optimizer"] == "adamw" else B.OPT_SGD, lr_client=case["lr"], lr_server=case["lr"],
+                   beta1=0.9, beta2=0.999, adam_eps=1e-8, weight_decay=0.01, agg_interval=1, norm_eps=1e-5, gelu_tanh=1,
+                   use_tensor_cores=1, arch=B.ARCH_LLAMA if case["arch"] == "llama" else B.ARCH_GPT, rope_theta=10000.0,
+                   cut_min=case["cut_min"])
+    eng = B.SplitLoRA(cfg)
+    for name, t in _frozen(case, g):
+        eng.bind_frozen(name, t)
+    cuts, first = _cuts(case), case["cut_min"] or case["cut"]
+    if case["cut_min"]:
+        eng.set_client_cuts(cuts)
+    client, server = _adapters(case, g)
+    r = case["r"]
+    for t, target in enumerate(case["targets"]):
+        bit = B.TARGET_BITS[target]
+        for i in range(case["K"]):
+            for l in range(cuts[i]):
+                eng.set_adapter(B.SIDE_CLIENT, i, l, bit, client[i, l, t, 0].view(r, d), client[i, l, t, 1].view(d, r))
+        for l in range(first, case["layers"]):
+            eng.set_adapter(B.SIDE_SERVER, 0, l, bit, server[l - first, t, 0].view(r, d), server[l - first, t, 1].view(d, r))
+    if case["mixed_ranks"]:
+        eng.set_client_ranks(_ranks(case))
+    tokens, labels, counts = _tokens(case, g)
+    s = {"case": case, "eng": eng, "tokens": tokens, "labels": labels, "counts": counts}
+    if case["api"] == "host":
+        s["tokens"], s["labels"] = tokens.cpu().pin_memory(), labels.cpu().pin_memory()
+    if case["api"] == "calls":
+        s["S"], s["dS"] = eng.new_activation_buffer(), eng.new_activation_buffer()
+    s["out"] = {"client": eng.adapter_buffer(B.SIDE_CLIENT, 0), "client_grad": eng.adapter_buffer(B.SIDE_CLIENT, 1)}
+    if case["layers"] > first:
+        s["out"]["server"], s["out"]["server_grad"] = eng.adapter_buffer(B.SIDE_SERVER, 0), eng.adapter_buffer(B.SIDE_SERVER, 1)
+    if case["api"] == "calls":
+        s["out"]["S"], s["out"]["dS"] = s["S"], s["dS"]
+    return s
+
+
+def _lora_inputs(case, seed):
+    g = _gen(seed)
+    M, i, o, r, G, dt = case["M"], case["n_in"], case["n_out"], case["r"], case["G"], _dt(case)
+    x = torch.randn(M, i, device="cuda", generator=g).to(dt)
+    W = (torch.randn(o, i, device="cuda", generator=g) * i ** -0.5).to(dt)
+    bias = (0.02 * torch.randn(o, device="cuda", generator=g)).to(dt)
+    A = torch.randn(G, r, i, device="cuda", generator=g) * i ** -0.5
+    Bm = torch.randn(G, o, r, device="cuda", generator=g) * r ** -0.5
+    dy = (torch.randn(M, o, device="cuda", generator=g) * o ** -0.5).to(dt)
+    return x, W, bias, A, Bm, dy
+
+
+def _attention_inputs(case, seed):
+    g = _gen(seed)
+    d = case["heads"] * case["width"]
+    rows = case["nseq"] * case["T"]
+    return (torch.randn(rows, 3 * d, device="cuda", generator=g).to(_dt(case)),
+            torch.randn(rows, d, device="cuda", generator=g).to(_dt(case)))
+
+
+def _handoff_input(case, seed):
+    g = _gen(seed)
+    rows = torch.exp(torch.randn(case["M"], 1, device="cuda", generator=g))
+    return (torch.randn(case["M"], case["d"], device="cuda", generator=g) * rows).to(_dt(case))
+
+
+def _aggregate_inputs(case, seed):
+    params = torch.randn(case["K"], case["P"], device="cuda", generator=_gen(seed)) * 0.02
+    counts = [200 + (37 * (i + 1) * (i + 5)) % 801 for i in range(case["K"])]
+    return params, [n / sum(counts) for n in counts]
+
+
+def prepare(case, seed):
+    kind = case["kind"]
+    if kind == "round":
+        return _prepare_round(case, seed)
+    s = {"case": case}
+    if kind == "lora":
+        x, W, bias, A, Bm, dy = _lora_inputs(case, seed)
+        M, i, o, r, G = case["M"], case["n_in"], case["n_out"], case["r"], case["G"]
+        s.update(x=x, W=W, Wt=B.transpose(W), bias=bias, A=A, B=Bm, dy=dy, y=torch.empty(M, o, device="cuda", dtype=x.dtype),
+                 ws=B.lora_linear_workspace(B.DTYPE_BF16 if case["dtype"] == "bf16" else B.DTYPE_FP32, M, i, o, r, G),
+                 out=(torch.empty(M, i, device="cuda", dtype=x.dtype), torch.empty(G, r, i, device="cuda"), torch.empty(G, o, r, device="cuda")))
+    elif kind == "attention":
+        s["qkv"], s["do"] = _attention_inputs(case, seed)
+    elif kind == "handoff":
+        x = _handoff_input(case, seed)
+        s.update(x=x, codes=torch.empty(x.shape, device="cuda", dtype=torch.uint8), scales=torch.empty(x.shape[0], device="cuda"),
+                 y=torch.empty_like(x))
+    else:
+        s["params"], s["weights"] = _aggregate_inputs(case, seed)
+    return s
+
+
+# ---- one pass -------------------------------------------------------------------------------------
+
+def run(s):
+    case = s["case"]
+    kind = case["kind"]
+    if kind == "round":
+        eng, api = s["eng"], case["api"]
+        if api == "host":       # the program reads every round's loss
+            loss = eng.round_host(s["tokens"], s["labels"], s["counts"])
+        elif api == "calls":
+            eng.client_fwd(s["tokens"], s["S"])
+            eng.server_step(s["S"], s["labels"], s["dS"], want_loss=False)
+            eng.client_bwd(s["dS"])
+            eng.aggregate(s["counts"])
+            loss = eng.loss_tensor()
+        else:
+            eng.round(s["tokens"], s["labels"], s["counts"], want_loss=False)
+            loss = eng.loss_tensor()
+        return dict(s["out"], loss=loss)
+    if kind == "lora":
+        y = B.lora_linear_fwd(s["x"], s["W"], s["bias"], s["A"], s["B"], 16.0, y=s["y"], workspace=s["ws"])
+        dx, dA, dB = B.lora_linear_bwd(s["x"], s["Wt"], s["dy"], s["A"], s["B"], 16.0, workspace=s["ws"], out=s["out"])
+        return {"y": y, "dx": dx, "dA": dA, "dB": dB}
+    if kind == "attention":
+        o, lse = B.attention_fwd(s["qkv"], case["nseq"], case["T"], case["heads"])
+        dqkv = B.attention_bwd(s["qkv"], o, lse, s["do"], case["nseq"], case["T"], case["heads"])
+        return {"o": o, "lse": lse, "dqkv": dqkv}
+    if kind == "handoff":
+        codes, scales = B.handoff_quantize(s["x"], s["codes"], s["scales"])
+        return {"codes": codes, "scales": scales, "y": B.handoff_dequantize(codes, scales, s["y"])}
+    B.aggregate_buffers(s["params"], s["weights"])
+    return s["params"]
+
+
+# ---- what a pass cannot do without ----------------------------------------------------------------
+
+def work(case):
+    kind = case["kind"]
+    es = 2 if case.get("dtype") == "bf16" else 4
+    if kind == "round":
+        d, _, ff = _shape(case)
+        L, T, M, V, r = case["layers"], case["T"], case["K"] * case["b"] * case["T"], case["vocab"], case["r"]
+        mats = 3 if case["arch"] == "llama" else 2
+        n, cuts, first = len(case["targets"]), _cuts(case), case["cut_min"] or case["cut"]
+        weights = L * (4 * d * d + mats * d * ff)
+        # forward and the gradient with respect to the input of every linear layer but the first block's qkv
+        # projection (nothing below it is trained); causal attention 2 T d forward, 2.5 times that backward;
+        # rank-r products: down and up, forward and backward, and the two adapter gradients
+        flops = M * (4.0 * weights - 2.0 * 3 * d * d) + 4.0 * M * d * V + L * M * 3.5 * 2.0 * T * d + 12.0 * M * L * n * r * d
+        params = 2 * n * r * d * (sum(cuts) + L - first)
+        state = 6 if case["optimizer"] == "adamw" else 2          # parameters (and both moments) read and written
+        rows = 4 * M * d * es if case["api"] == "calls" else 0     # S and dS, written and read
+        head = 2 if case["arch"] == "llama" else 1
+        return {"bytes": es * (weights + head * V * d) + 4.0 * params * (state + 1) + 8.0 * M + rows, "flops": flops}
+    if kind == "lora":
+        M, i, o, r, G = case["M"], case["n_in"], case["n_out"], case["r"], case["G"]
+        return {"bytes": es * (2.0 * M * i + 2.0 * M * o + i * o) + 4.0 * 2 * G * r * (i + o), "flops": 4.0 * M * i * o + 6.0 * M * r * (i + o)}
+    if kind == "attention":
+        n, T, d = case["nseq"], case["T"], case["heads"] * case["width"]
+        return {"bytes": es * n * T * 8.0 * d + 4.0 * n * T * case["heads"], "flops": 3.5 * 2.0 * n * T * T * d}
+    if kind == "handoff":
+        return {"bytes": case["M"] * (case["d"] * (2.0 * es + 1) + 4), "flops": 0}
+    return {"bytes": 8.0 * case["K"] * case["P"], "flops": 2.0 * case["K"] * case["P"]}
+
+
+def tolerance(case):
+    kind = case["kind"]
+    if kind == "handoff":
+        return "exact"          # codes, scales and restored values are fixed to the bit by the format
+    if kind == "aggregate":
+        return {"rel": 1e-6, "max": 1e-5}
+    if case["dtype"] == "fp32":
+        # AdamW's first step is lr * sign(g): a gradient within rounding of zero may move its weight either way
+        return {"rel": 1e-4, "max": 0.2} if kind == "round" else {"rel": 1e-5, "max": 1e-3}
+    return {"rel": 0.03, "max": 1.0 - 1e-9} if kind == "round" else {"rel": 0.01, "max": 0.1}
+
+
+# ---- the same in 64 bits --------------------------------------------------------------------------
+
+def _exact_round(case, seed):
+    g = _gen(seed)
+    d, heads, ff = _shape(case)
+    dh, T, b, r, L = d // heads, case["T"], case["b"], case["r"], case["layers"]
+    llama = case["arch"] == "llama"
+    p = {}
+    for name, t in _frozen(case, g):
+        p[name] = t.double()
+    client, server = (t.double() for t in _adapters(case, g))
+    tokens, labels, counts = _tokens(case, g)
+    cuts, first = _cuts(case), case["cut_min"] or case["cut"]
+    n, K = len(case["targets"]), case["K"]
+    # a client holds its own depth and its own rank only
+    keep = torch.zeros_like(client)
+    for i in range(K):
+        A = keep[i, :, :, 0].view(case["cut"], n, r, d)
+        Bm = keep[i, :, :, 1].view(case["cut"], n, d, r)
+        A[:cuts[i], :, :_ranks(case)[i]] = 1
+        Bm[:cuts[i], :, :, :_ranks(case)[i]] = 1
+    client = (client * keep).requires_grad_()
+    server = server.requires_grad_()
+    s = (8.0 * r if r <= 4 else 32.0) / r
+    eps = 1e-5
+    if llama:
+        half = dh // 2
+        ang = torch.arange(T, device="cuda", dtype=torch.float64)[:, None] * 10000.0 ** (-2.0 * torch.arange(half, device="cuda", dtype=torch.float64) / dh)
+        cos, sin = torch.cos(ang)[None, :, None], torch.sin(ang)[None, :, None]
+    causal = torch.ones(T, T, device="cuda", dtype=torch.bool).tril()
+
+    def norm(x, l):
+        if llama:
+            return x * torch.rsqrt((x * x).mean(-1, keepdim=True) + eps) * p[l + ".g"]
+        return torch.nn.functional.layer_norm(x, (d,), p[l + ".g"], p[l + ".b"], eps)
+
+    def lora(x, ad, t):
+        return s * (x @ ad[t, 0].view(r, d).T) @ ad[t, 1].view(d, r).T
+
+    def block(x, l, ad):
+        h, u = f"h.{l}.", norm(x, f"h.{l}.ln1")
+        qkv = list((u @ p[h + "attn.qkv.w"].T + (0 if llama else p[h + "attn.qkv.b"])).split(d, -1))
+        for t, target in enumerate(case["targets"]):
+            if target != "o":
+                j = "qkv".index(target)
+                qkv[j] = qkv[j] + lora(u, ad, t)
+        q, k, v = (z.view(-1, T, heads, dh) for z in qkv)
+        if llama:
+            rot = lambda z: torch.cat([z[..., :half] * cos - z[..., half:] * sin, z[..., :half] * sin + z[..., half:] * cos], -1)  # noqa: E731
+            q, k = rot(q), rot(k)
+        q, k, v = (z.transpose(1, 2) for z in (q, k, v))
+        a = torch.softmax((q @ k.transpose(-1, -2) * dh ** -0.5).masked_fill(~causal, -math.inf), -1) @ v
+        o = a.transpose(1, 2).reshape(-1, T, d)
+        y = o @ p[h + "attn.proj.w"].T + (0 if llama else p[h + "attn.proj.b"])
+        if "o" in case["targets"]:
+            y = y + lora(o, ad, case["targets"].index("o"))
+        x = x + y
+        u = norm(x, f"h.{l}.ln2")
+        if llama:
+            gate, up = (u @ p[h + "mlp.gate_up.w"].T).split(ff, -1)
+            return x + (torch.nn.functional.silu(gate) * up) @ p[h + "mlp.down.w"].T
+        z = u @ p[h + "mlp.fc1.w"].T + p[h + "mlp.fc1.b"]
+        return x + torch.nn.functional.gelu(z, approximate="tanh") @ p[h + "mlp.fc2.w"].T + p[h + "mlp.fc2.b"]
+
+    valid = int(((labels >= 0) & (labels < case["vocab"])).sum())
+    loss, S, dS = 0.0, [], []
+    step = max(1, min(b, 4096 // T))                      # sequences at a time: bounds what autograd keeps
+    for i in range(K):
+        for b0 in range(0, b, step):
+            tok, lab = tokens[i, b0:b0 + step].long(), labels[i, b0:b0 + step].long()
+            x = p["wte"][tok] + (0 if llama else p["wpe"][:T])
+            for l in range(cuts[i]):
+                x = block(x, l, client[i, l])
+            x.retain_grad()
+            cut = x
+            for l in range(cuts[i], L):
+                x = block(x, l, server[l - first])
+            logits = norm(x, "lnf") @ p["head.w" if llama else "wte"].T
+            part = torch.nn.functional.cross_entropy(logits.view(-1, logits.shape[-1]), lab.reshape(-1), ignore_index=-1, reduction="sum") / valid
+            part.backward()
+            loss += float(part)
+            S.append(cut.detach())
+            dS.append(cut.grad)
+            del logits, x, part, cut
+
+    def update(w, gr):
+        if case["optimizer"] == "sgd":
+            return w - case["lr"] * gr
+        return w * (1 - case["lr"] * 0.01) - case["lr"] * gr / (gr.abs() + 1e-8)   # first step: m / bc1 = g, v / bc2 = g^2
+
+    with torch.no_grad():
+        cg = client.grad
+        new = update(client, cg)
+        mean = new.clone()
+        for l in range(case["cut"]):
+            holders = [i for i in range(K) if cuts[i] > l]
+            if len(holders) > 1 or case["cut_min"] == 0:
+                total = sum(counts[i] for i in holders)
+                mean[holders, l] = sum(counts[i] / total * new[i, l] for i in holders)
+        out = {"client": (mean * keep).reshape(-1) if case["mixed_ranks"] else mean.reshape(-1), "client_grad": cg.reshape(-1)}
+        if L > first:
+            out["server"], out["server_grad"] = update(server, server.grad).reshape(-1), server.grad.reshape(-1)
+        if case["api"] == "calls":
+            out["S"] = torch.cat(S).view(K, b, T, d)
+            out["dS"] = torch.cat(dS).view(K, b, T, d)
+        out["loss"] = loss if case["api"] == "host" else torch.tensor([loss], dtype=torch.float64, device="cuda")
+    return out
+
+
+def exact(case, seed):
+    kind = case["kind"]
+    if kind == "round":
+        return _exact_round(case, seed)
+    if kind == "lora":
+        x, W, bias, A, Bm, dy = (t.double() for t in _lora_inputs(case, seed))
+        G, s = case["G"], 16.0 / case["r"]
+        xg, dyg = x.view(G, -1, x.shape[1]), dy.view(G, -1, dy.shape[1])
+        h, dh = xg @ A.transpose(1, 2), s * dyg @ Bm
+        return {"y": x @ W.T + bias + s * (h @ Bm.transpose(1, 2)).reshape(dy.shape), "dx": dy @ W + (dh @ A).reshape(x.shape),
+                "dA": dh.transpose(1, 2) @ xg, "dB": s * dyg.transpose(1, 2) @ h}
+    if kind == "attention":
+        qkv, do = (t.double() for t in _attention_inputs(case, seed))
+        n, T, H, w = case["nseq"], case["T"], case["heads"], case["width"]
+        causal = torch.ones(T, T, device="cuda", dtype=torch.bool).tril()
+        o, lse, grads = [], [], []
+        for rows, dy in zip(qkv.view(n, T, 3, H, w), do.view(n, T, H, w)):
+            q, k, v = (rows[:, j].transpose(0, 1).contiguous().requires_grad_() for j in range(3))
+            z = (q @ k.transpose(1, 2) * w ** -0.5).masked_fill(~causal, -math.inf)
+            y = torch.softmax(z, -1) @ v
+            y.backward(dy.transpose(0, 1))
+            o.append(y.detach().transpose(0, 1).reshape(T, H * w))
+            lse.append(torch.logsumexp(z.detach(), -1))
+            grads.append(torch.stack([t.grad.transpose(0, 1) for t in (q, k, v)], 1).reshape(T, 3 * H * w))
+        return {"o": torch.cat(o), "lse": torch.stack(lse), "dqkv": torch.cat(grads)}
+    if kind == "handoff":
+        # the codes are whole numbers: what they stand for is seen in the restored values
+        x = _handoff_input(case, seed)
+        peak = x.float().abs().amax(1, keepdim=True)
+        codes = torch.where(peak > 0, x.float() * (448.0 / peak), torch.zeros_like(x, dtype=torch.float32)).to(torch.float8_e4m3fn)
+        scales = peak.double() / 448.0
+        return {"codes": None, "scales": scales[:, 0], "y": codes.double() * scales}
+    params, weights = _aggregate_inputs(case, seed)
+    mean = sum(w * t for w, t in zip(weights, params.double()))
+    return mean.expand(case["K"], -1).contiguous()
