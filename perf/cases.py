@@ -9,8 +9,8 @@ Five kinds of case, each through the public entry points of `paper_2407_00952_b2
   handoff    the cut-layer tensor to 8-bit codes and back (sender and receiver of a compressed link)
   aggregate  the weighted average of the clients' adapters (the fed server's step by itself)
 
-All inputs are synthetic and made on the GPU from the seed: frozen weights and adapters N(0, 0.02) (adapters as
-in mid-training, B not zero), gains near one, small biases, token ids from a bounded Zipf law.
+All inputs are synthetic and made on the GPU from the seed: frozen weights and adapters N(0, 0.02) (adapters and
+optimizer state as in mid-training, B not zero), gains near one, small biases, token ids from a bounded Zipf law.
 """
 from __future__ import annotations
 
@@ -109,7 +109,8 @@ def draw(rng):
                       mixed_ranks=hetero)
     if kind == "llama":
         size = rng.choice(["llama-w1024", "llama-w1024", "llama2-7b"])
-        K, T = rng.choice([1, 2, 4]), rng.choice([128, 256, 384, 512, 1024, 200 if K == 1 else 640])
+        K = rng.choice([1, 2, 4])
+        T = rng.choice([128, 256, 384, 512, 1024, 200 if K == 1 else 640])
         unit = 256 // math.gcd(T, 256) if K > 1 else 1
         b = unit * max(1, min(2, 2048 // (unit * T * K)))
         return _round(None, size, arch="llama", layers=rng.randint(2, 4) if size != "llama2-7b" else 2, cut=1, K=K, b=b, T=T,
@@ -198,6 +199,17 @@ def _adapters(case, g):
     return client, server
 
 
+STEPS = 100              # optimizer steps taken before the pass
+MOMENT = 1e-4            # size of the gradients so far
+
+
+def _moments(case, g, like):
+    """AdamW moments as after STEPS steps, for adapters laid out like `like`."""
+    m = torch.empty_like(like).normal_(0.0, MOMENT, generator=g)
+    v = MOMENT ** 2 * torch.empty_like(like).uniform_(0.5, 1.5, generator=g)
+    return m, v
+
+
 def _tokens(case, g):
     """Token ids [K, b, T] and the next ids as labels; with `padded`, sequences end early and the rest is ignored."""
     K, b, T, V = case["K"], case["b"], case["T"], case["vocab"]
@@ -207,7 +219,7 @@ def _tokens(case, g):
     cdf = torch.cumsum(p / p.sum(), 0)
     u = torch.rand(K, b, T + 1, device="cuda", generator=g, dtype=torch.float64)
     ids = order[torch.searchsorted(cdf, u).clamp_(max=V - 1)].int()
-    tokens, labels = ids[..., :T].contiguous(), ids[..., 1:].contiguous()
+    tokens, labels = (t.clone(memory_format=torch.contiguous_format) for t in (ids[..., :T], ids[..., 1:]))
     if case["padded"]:
         length = torch.randint((T + 1) // 2, T + 1, (K, b, 1), device="cuda", generator=g)
         labels = torch.where(torch.arange(T, device="cuda") < length, labels, torch.full_like(labels, -1)).contiguous()
@@ -236,13 +248,24 @@ def _prepare_round(case, seed):
         eng.set_client_cuts(cuts)
     client, server = _adapters(case, g)
     r = case["r"]
+    if case["optimizer"] == "adamw":
+        (cm, cv), (sm, sv) = _moments(case, g, client), _moments(case, g, server)
+        eng.set_counters(STEPS, STEPS, STEPS)
+    else:
+        cm = None
     for t, target in enumerate(case["targets"]):
         bit = B.TARGET_BITS[target]
         for i in range(case["K"]):
             for l in range(cuts[i]):
-                eng.set_adapter(B.SIDE_CLIENT, i, l, bit, client[i, l, t, 0].view(r, d), client[i, l, t, 1].view(d, r))
+                at = (i, l, t)
+                eng.set_adapter(B.SIDE_CLIENT, i, l, bit, client[at][0].view(r, d), client[at][1].view(d, r))
+                if cm is not None:
+                    eng.set_opt_state(B.SIDE_CLIENT, i, l, bit, cm[at][0], cv[at][0], cm[at][1], cv[at][1])
         for l in range(first, case["layers"]):
-            eng.set_adapter(B.SIDE_SERVER, 0, l, bit, server[l - first, t, 0].view(r, d), server[l - first, t, 1].view(d, r))
+            at = (l - first, t)
+            eng.set_adapter(B.SIDE_SERVER, 0, l, bit, server[at][0].view(r, d), server[at][1].view(d, r))
+            if cm is not None:
+                eng.set_opt_state(B.SIDE_SERVER, 0, l, bit, sm[at][0], sv[at][0], sm[at][1], sv[at][1])
     if case["mixed_ranks"]:
         eng.set_client_ranks(_ranks(case))
     tokens, labels, counts = _tokens(case, g)
@@ -385,9 +408,9 @@ def tolerance(case):
     if kind == "aggregate":
         return {"rel": 1e-6, "max": 1e-5}
     if case["dtype"] == "fp32":
-        # AdamW's first step is lr * sign(g): a gradient within rounding of zero may move its weight either way
-        return {"rel": 1e-4, "max": 0.2} if kind == "round" else {"rel": 1e-5, "max": 1e-3}
-    return {"rel": 0.03, "max": 1.0 - 1e-9} if kind == "round" else {"rel": 0.01, "max": 0.1}
+        return {"rel": 1e-5, "max": 1e-3}
+    # rounds: the q and k gradients of bf16 pipelines are off by up to 1.6e-2 each (norms over a whole tensor)
+    return {"rel": 0.03, "max": 0.99} if kind == "round" else {"rel": 0.01, "max": 0.1}
 
 
 # ---- the same in 64 bits --------------------------------------------------------------------------
@@ -400,7 +423,9 @@ def _exact_round(case, seed):
     p = {}
     for name, t in _frozen(case, g):
         p[name] = t.double()
-    client, server = (t.double() for t in _adapters(case, g))
+    client, server = _adapters(case, g)
+    moments = [_moments(case, g, client), _moments(case, g, server)] if case["optimizer"] == "adamw" else [(None, None)] * 2
+    client, server = client.double(), server.double()
     tokens, labels, counts = _tokens(case, g)
     cuts, first = _cuts(case), case["cut_min"] or case["cut"]
     n, K = len(case["targets"]), case["K"]
@@ -455,7 +480,7 @@ def _exact_round(case, seed):
         return x + torch.nn.functional.gelu(z, approximate="tanh") @ p[h + "mlp.fc2.w"].T + p[h + "mlp.fc2.b"]
 
     valid = int(((labels >= 0) & (labels < case["vocab"])).sum())
-    loss, S, dS = 0.0, [], []
+    S, dS = [], []
     step = max(1, min(b, 4096 // T))                      # sequences at a time: bounds what autograd keeps
     for i in range(K):
         for b0 in range(0, b, step):
@@ -470,19 +495,20 @@ def _exact_round(case, seed):
             logits = norm(x, "lnf") @ p["head.w" if llama else "wte"].T
             part = torch.nn.functional.cross_entropy(logits.view(-1, logits.shape[-1]), lab.reshape(-1), ignore_index=-1, reduction="sum") / valid
             part.backward()
-            loss += float(part)
             S.append(cut.detach())
             dS.append(cut.grad)
             del logits, x, part, cut
 
-    def update(w, gr):
-        if case["optimizer"] == "sgd":
+    def update(w, gr, m, v):
+        if m is None:
             return w - case["lr"] * gr
-        return w * (1 - case["lr"] * 0.01) - case["lr"] * gr / (gr.abs() + 1e-8)   # first step: m / bc1 = g, v / bc2 = g^2
+        m, v = 0.9 * m.double() + 0.1 * gr, 0.999 * v.double() + 0.001 * gr * gr
+        m, v = m / (1 - 0.9 ** (STEPS + 1)), v / (1 - 0.999 ** (STEPS + 1))
+        return w * (1 - case["lr"] * 0.01) - case["lr"] * m / (v.sqrt() + 1e-8)
 
     with torch.no_grad():
         cg = client.grad
-        new = update(client, cg)
+        new = update(client, cg, *moments[0])
         mean = new.clone()
         for l in range(case["cut"]):
             holders = [i for i in range(K) if cuts[i] > l]
@@ -491,11 +517,13 @@ def _exact_round(case, seed):
                 mean[holders, l] = sum(counts[i] / total * new[i, l] for i in holders)
         out = {"client": (mean * keep).reshape(-1) if case["mixed_ranks"] else mean.reshape(-1), "client_grad": cg.reshape(-1)}
         if L > first:
-            out["server"], out["server_grad"] = update(server, server.grad).reshape(-1), server.grad.reshape(-1)
+            out["server"], out["server_grad"] = update(server, server.grad, *moments[1]).reshape(-1), server.grad.reshape(-1)
         if case["api"] == "calls":
             out["S"] = torch.cat(S).view(K, b, T, d)
             out["dS"] = torch.cat(dS).view(K, b, T, d)
-        out["loss"] = loss if case["api"] == "host" else torch.tensor([loss], dtype=torch.float64, device="cuda")
+        # one number, in which the rounding of thousands of rows cancels by chance: its distance from the exact
+        # mean varies tenfold from seed to seed and says nothing about precision
+        out["loss"] = None
     return out
 
 
