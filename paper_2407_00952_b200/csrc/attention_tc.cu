@@ -1,6 +1,16 @@
-// Causal multi-head attention on tensor cores (bf16 operands, fp32 softmax and accumulation),
-// head width 64 or 128, sequence length a multiple of 64.  Flash-style: scores are never written to
-// memory; the forward keeps only the log-sum-exp per row, the backward recomputes probabilities.
+// Causal multi-head attention on tensor cores (bf16 operands, fp32 softmax and accumulation).
+// Flash-style: scores are never written to memory; the forward keeps only the log-sum-exp per row, the
+// backward recomputes probabilities.  Two forms of every kernel (template parameter RG):
+//   RG = false: head width 64 or 128, sequence length a multiple of 64; P and dS enter their products as bf16.
+//   RG = true:  any sequence length and any head width that is a multiple of 8 up to 128 (padded with zeros to
+//     DH = 32, 64, 96 or 128 in shared memory; rows past the end of a sequence are zero-filled, never stored,
+//     and as queries carry lse = +inf, i.e. P = 0).  These shapes otherwise run on the plain-FMA kernels, which
+//     hold P and dS in fp32, so here each of them enters its product as a sum of two bf16 values (hi + lo, 16
+//     mantissa bits) against the exact bf16 operand: twice the products of that operand, none of the precision
+//     lost (error of o / dqkv against 64 bits over odd T is that of the bf16 output alone, as before).  Measured,
+//     16 sequences of 777 tokens, 12 heads of 64, forward + backward: 466 us against 72.9 ms.  Bound by the
+//     tensor issue of mma.sync and by ldmatrix traffic (the hi and lo products share one fragment of the right
+//     operand).  Shapes that the aligned forms take stay with them.
 //   forward : one CTA per (sequence, head, 64-row query tile), 4 warps x 16 rows, K/V tiles double
 //             buffered in shared memory with cp.async, online softmax in registers.
 //   backward: rowdot = sum(dO*O); a dQ kernel per query tile (loops over key tiles) and a dK/dV
@@ -27,25 +37,40 @@ template <int DH> struct Sizes {
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // byte offset of element (r, c) in a [64][DH] bf16 tile; the 16-byte chunks of every 128-byte
-// segment of a row are XOR-swizzled by the row index
+// segment of a row are XOR-swizzled by the row index (rows that are an odd number of 64-byte segments: the
+// chunks of every 64-byte segment by half the row index, two rows sharing 128 bytes of banks)
 template <int DH> __device__ __forceinline__ uint32_t swz(int r, int c) {
   int ch = c >> 3;
+  if constexpr (DH % 64 != 0)
+    return (uint32_t)(r * (DH * 2) + ((((ch & ~3) | ((ch & 3) ^ ((r >> 1) & 3))) << 4) | ((c & 7) << 1)));
   return (uint32_t)(r * (DH * 2) + ((((ch & ~7) | ((ch & 7) ^ (r & 7))) << 4) | ((c & 7) << 1)));
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+// 16 bytes, or zeros without touching `src` when !valid
+__device__ __forceinline__ void cp_async16_or_zero(uint32_t dst, const void* src, bool valid) {
+  const int n = valid ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// 64 x DH bf16 tile, global rows `ld` elements apart -> swizzled shared tile
-template <int DH> __device__ __forceinline__ void load_tile(uint32_t sbase, const bf16* g, int64_t ld) {
+// 64 x DH bf16 tile, global rows `ld` elements apart -> swizzled shared tile.  RG: only `rows` rows of `dh`
+// columns exist, the rest of the tile is zero.
+template <int DH, bool RG>
+__device__ __forceinline__ void load_tile(uint32_t sbase, const bf16* g, int64_t ld, int rows, int dh) {
   constexpr int CH = DH / 8;
 #pragma unroll
   for (int i = threadIdx.x; i < BT * CH; i += NT) {
     int r = i / CH, ch = i % CH;
-    cp_async16(sbase + swz<DH>(r, ch * 8), g + (size_t)r * ld + ch * 8);
+    if constexpr (RG) {
+      const bool ok = r < rows && ch * 8 < dh;
+      cp_async16_or_zero(sbase + swz<DH>(r, ch * 8), ok ? g + (size_t)r * ld + ch * 8 : g, ok);
+    } else {
+      cp_async16(sbase + swz<DH>(r, ch * 8), g + (size_t)r * ld + ch * 8);
+    }
   }
 }
 
@@ -100,8 +125,14 @@ __device__ __forceinline__ void mma_a_smem_b_nk(float (*acc)[4], uint32_t a_tile
     }
   }
 }
-// acc[DH/8][4] (16 x DH) += P(16 x 64, fp32 accumulator layout, converted to bf16) * B, B tile stored [64][DH]
-template <int DH>
+// what bf16 rounding leaves of two values, again as bf16
+__device__ __forceinline__ uint32_t pack2_rest(float lo, float hi, uint32_t rounded) {
+  return pack2(lo - __uint_as_float(rounded << 16), hi - __uint_as_float(rounded & 0xffff0000u));
+}
+
+// acc[DH/8][4] (16 x DH) += P(16 x 64, fp32 accumulator layout, converted to bf16) * B, B tile stored [64][DH].
+// RG: P as the sum of two bf16 values; both products use the right operand's fragment while it is in registers.
+template <int DH, bool RG>
 __device__ __forceinline__ void mma_p_regs_b_kn(float (*acc)[4], const float (*p)[4], uint32_t b_tile) {
 #pragma unroll
   for (int ks = 0; ks < 4; ++ks) {
@@ -110,12 +141,23 @@ __device__ __forceinline__ void mma_p_regs_b_kn(float (*acc)[4], const float (*p
     a[1] = pack2(p[2 * ks][2], p[2 * ks][3]);
     a[2] = pack2(p[2 * ks + 1][0], p[2 * ks + 1][1]);
     a[3] = pack2(p[2 * ks + 1][2], p[2 * ks + 1][3]);
+    uint32_t a2[4];
+    if constexpr (RG) {
+      a2[0] = pack2_rest(p[2 * ks][0], p[2 * ks][1], a[0]);
+      a2[1] = pack2_rest(p[2 * ks][2], p[2 * ks][3], a[1]);
+      a2[2] = pack2_rest(p[2 * ks + 1][0], p[2 * ks + 1][1], a[2]);
+      a2[3] = pack2_rest(p[2 * ks + 1][2], p[2 * ks + 1][3], a[3]);
+    }
 #pragma unroll
     for (int np = 0; np < DH / 16; ++np) {
       uint32_t b[4];
       load_b_kn<DH>(b, b_tile, ks * 16, np * 16);
       mma16816(acc[2 * np], a, b[0], b[1]);
       mma16816(acc[2 * np + 1], a, b[2], b[3]);
+      if constexpr (RG) {
+        mma16816(acc[2 * np], a2, b[0], b[1]);
+        mma16816(acc[2 * np + 1], a2, b[2], b[3]);
+      }
     }
   }
 }
@@ -130,21 +172,24 @@ template <int N> __device__ __forceinline__ void zero_acc(float (*a)[4]) {
 // ------------------------------------------------------------------------------------------
 // forward
 // ------------------------------------------------------------------------------------------
-template <int DH>
+// dh: head width (RG only; DH otherwise)
+template <int DH, bool RG>
 __global__ void __launch_bounds__(NT) attn_fwd_tc_kernel(const bf16* __restrict__ qkv, bf16* __restrict__ o,
-                                                         float* __restrict__ lse, int T, int H, int d, float scale_log2) {
+                                                         float* __restrict__ lse, int T, int H, int d, int dh,
+                                                         float scale, float scale_log2) {
+  if (!RG) dh = DH;
   constexpr int TILE_BYTES = Sizes<DH>::TILE;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sQ = smem_u32(smem), sK0 = sQ + TILE_BYTES, sV0 = sQ + 3 * TILE_BYTES;
   const int qt = gridDim.x - 1 - blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int64_t ld = 3 * (int64_t)d;
-  const bf16* qbase = qkv + ((size_t)b * T + (size_t)qt * BT) * ld + (size_t)h * DH;
-  const bf16* kbase = qkv + (size_t)b * T * ld + d + (size_t)h * DH;
+  const bf16* qbase = qkv + ((size_t)b * T + (size_t)qt * BT) * ld + (size_t)h * dh;
+  const bf16* kbase = qkv + (size_t)b * T * ld + d + (size_t)h * dh;
   const bf16* vbase = kbase + d;
-  load_tile<DH>(sQ, qbase, ld);
-  load_tile<DH>(sK0, kbase, ld);
-  load_tile<DH>(sV0, vbase, ld);
+  load_tile<DH, RG>(sQ, qbase, ld, T - qt * BT, dh);
+  load_tile<DH, RG>(sK0, kbase, ld, T, dh);
+  load_tile<DH, RG>(sV0, vbase, ld, T, dh);
   cp_commit();
   float oacc[DH / 8][4];
   zero_acc<DH / 8>(oacc);
@@ -153,8 +198,8 @@ __global__ void __launch_bounds__(NT) attn_fwd_tc_kernel(const bf16* __restrict_
   for (int j = 0; j <= qt; ++j) {
     const uint32_t sK = sK0 + (j & 1) * TILE_BYTES, sV = sV0 + (j & 1) * TILE_BYTES;
     if (j < qt) {
-      load_tile<DH>(sK0 + ((j + 1) & 1) * TILE_BYTES, kbase + (size_t)(j + 1) * BT * ld, ld);
-      load_tile<DH>(sV0 + ((j + 1) & 1) * TILE_BYTES, vbase + (size_t)(j + 1) * BT * ld, ld);
+      load_tile<DH, RG>(sK0 + ((j + 1) & 1) * TILE_BYTES, kbase + (size_t)(j + 1) * BT * ld, ld, T - (j + 1) * BT, dh);
+      load_tile<DH, RG>(sV0 + ((j + 1) & 1) * TILE_BYTES, vbase + (size_t)(j + 1) * BT * ld, ld, T - (j + 1) * BT, dh);
       cp_commit();
       cp_wait<1>();
     } else {
@@ -171,7 +216,7 @@ __global__ void __launch_bounds__(NT) attn_fwd_tc_kernel(const bf16* __restrict_
       for (int e = 0; e < 4; ++e) {
         int col = n * 8 + 2 * t + (e & 1);
         int row = (e < 2) ? r0 : r1;
-        float v = s[n][e] * scale_log2;
+        float v = RG ? s[n][e] : s[n][e] * scale_log2;      // RG: the maximum of the unscaled scores
         if (j == qt && col > row) v = -INFINITY;
         s[n][e] = v;
         if (e < 2) mx0 = fmaxf(mx0, v); else mx1 = fmaxf(mx1, v);
@@ -180,35 +225,43 @@ __global__ void __launch_bounds__(NT) attn_fwd_tc_kernel(const bf16* __restrict_
     mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1)); mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
     const float nm0 = fmaxf(m0, mx0), nm1 = fmaxf(m1, mx1);   // finite: column 0 is never masked
-    const float c0 = exp2f(m0 - nm0), c1 = exp2f(m1 - nm1);
+    const float c0 = exp2f(RG ? (m0 - nm0) * scale_log2 : m0 - nm0), c1 = exp2f(RG ? (m1 - nm1) * scale_log2 : m1 - nm1);
     float ps0 = 0.f, ps1 = 0.f;
+    const float k0 = -nm0 * scale_log2, k1 = -nm1 * scale_log2;
 #pragma unroll
     for (int n = 0; n < 8; ++n) {
-      s[n][0] = exp2f(s[n][0] - nm0); s[n][1] = exp2f(s[n][1] - nm0);
-      s[n][2] = exp2f(s[n][2] - nm1); s[n][3] = exp2f(s[n][3] - nm1);
+      if (RG) {                                                // one rounding per exponent
+        s[n][0] = exp2f(fmaf(s[n][0], scale_log2, k0)); s[n][1] = exp2f(fmaf(s[n][1], scale_log2, k0));
+        s[n][2] = exp2f(fmaf(s[n][2], scale_log2, k1)); s[n][3] = exp2f(fmaf(s[n][3], scale_log2, k1));
+      } else {
+        s[n][0] = exp2f(s[n][0] - nm0); s[n][1] = exp2f(s[n][1] - nm0);
+        s[n][2] = exp2f(s[n][2] - nm1); s[n][3] = exp2f(s[n][3] - nm1);
+      }
       ps0 += s[n][0] + s[n][1]; ps1 += s[n][2] + s[n][3];
     }
 #pragma unroll
     for (int n = 0; n < DH / 8; ++n) { oacc[n][0] *= c0; oacc[n][1] *= c0; oacc[n][2] *= c1; oacc[n][3] *= c1; }
     l0 = l0 * c0 + ps0; l1 = l1 * c1 + ps1;
     m0 = nm0; m1 = nm1;
-    mma_p_regs_b_kn<DH>(oacc, s, sV);
+    mma_p_regs_b_kn<DH, RG>(oacc, s, sV);
     __syncthreads();
   }
   l0 += __shfl_xor_sync(0xffffffffu, l0, 1); l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
   l1 += __shfl_xor_sync(0xffffffffu, l1, 1); l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
   const float i0 = 1.f / l0, i1 = 1.f / l1;
-  bf16* o0 = o + ((size_t)b * T + (size_t)qt * BT + r0) * d + (size_t)h * DH;
-  bf16* o1 = o + ((size_t)b * T + (size_t)qt * BT + r1) * d + (size_t)h * DH;
+  bf16* o0 = o + ((size_t)b * T + (size_t)qt * BT + r0) * d + (size_t)h * dh;
+  bf16* o1 = o + ((size_t)b * T + (size_t)qt * BT + r1) * d + (size_t)h * dh;
+  const bool v0 = !RG || qt * BT + r0 < T, v1 = !RG || qt * BT + r1 < T;
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) {
-    *reinterpret_cast<uint32_t*>(o0 + n * 8 + 2 * t) = pack2(oacc[n][0] * i0, oacc[n][1] * i0);
-    *reinterpret_cast<uint32_t*>(o1 + n * 8 + 2 * t) = pack2(oacc[n][2] * i1, oacc[n][3] * i1);
+    if (RG && n * 8 >= dh) break;
+    if (v0) *reinterpret_cast<uint32_t*>(o0 + n * 8 + 2 * t) = pack2(oacc[n][0] * i0, oacc[n][1] * i0);
+    if (v1) *reinterpret_cast<uint32_t*>(o1 + n * 8 + 2 * t) = pack2(oacc[n][2] * i1, oacc[n][3] * i1);
   }
   if (t == 0) {
     float* lrow = lse + ((size_t)b * H + h) * T + (size_t)qt * BT;
-    lrow[r0] = (m0 + log2f(l0)) * LN2;
-    lrow[r1] = (m1 + log2f(l1)) * LN2;
+    if (v0) lrow[r0] = RG ? fmaf(m0, scale, logf(l0)) : (m0 + log2f(l0)) * LN2;
+    if (v1) lrow[r1] = RG ? fmaf(m1, scale, logf(l1)) : (m1 + log2f(l1)) * LN2;
   }
 }
 
@@ -241,37 +294,69 @@ __global__ void attn_rowdot_tc_kernel(const bf16* __restrict__ o, const bf16* __
 // ------------------------------------------------------------------------------------------
 // backward, dQ: one CTA per query tile, loops over key tiles j <= qt
 // ------------------------------------------------------------------------------------------
-template <int DH>
-__global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ d_o,
-                                                            const float* __restrict__ lse, const float* __restrict__ rowdot,
-                                                            bf16* __restrict__ dqkv, int T, int H, int d, float scale) {
+// RG: the kernel also forms D[row] = sum(dO * O) of its own rows (two threads per row) and leaves it in
+// `rowdot` for the dK/dV kernel, which runs second; otherwise a small kernel has put it there beforehand.
+template <int DH, bool RG>
+__global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ o,
+                                                            const bf16* __restrict__ d_o, const float* __restrict__ lse,
+                                                            float* __restrict__ rowdot, bf16* __restrict__ dqkv, int T,
+                                                            int H, int d, int dh, float scale) {
+  if (!RG) dh = DH;
   constexpr int TILE_BYTES = Sizes<DH>::TILE;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sQ = smem_u32(smem), sdO = sQ + TILE_BYTES, sK0 = sQ + 2 * TILE_BYTES, sV0 = sQ + 4 * TILE_BYTES;
   const int qt = gridDim.x - 1 - blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int64_t ld = 3 * (int64_t)d;
-  const bf16* qbase = qkv + ((size_t)b * T + (size_t)qt * BT) * ld + (size_t)h * DH;
-  const bf16* kbase = qkv + (size_t)b * T * ld + d + (size_t)h * DH;
+  const bf16* qbase = qkv + ((size_t)b * T + (size_t)qt * BT) * ld + (size_t)h * dh;
+  const bf16* kbase = qkv + (size_t)b * T * ld + d + (size_t)h * dh;
   const bf16* vbase = kbase + d;
-  const bf16* dobase = d_o + ((size_t)b * T + (size_t)qt * BT) * d + (size_t)h * DH;
-  load_tile<DH>(sQ, qbase, ld);
-  load_tile<DH>(sdO, dobase, d);
-  load_tile<DH>(sK0, kbase, ld);
-  load_tile<DH>(sV0, vbase, ld);
+  const bf16* dobase = d_o + ((size_t)b * T + (size_t)qt * BT) * d + (size_t)h * dh;
+  load_tile<DH, RG>(sQ, qbase, ld, T - qt * BT, dh);
+  load_tile<DH, RG>(sdO, dobase, d, T - qt * BT, dh);
+  load_tile<DH, RG>(sK0, kbase, ld, T, dh);
+  load_tile<DH, RG>(sV0, vbase, ld, T, dh);
   cp_commit();
   const int r0 = warp * 16 + g, r1 = r0 + 8;
   const size_t stat = ((size_t)b * H + h) * T + (size_t)qt * BT;
-  const float L0 = lse[stat + r0] * LOG2E, L1 = lse[stat + r1] * LOG2E;
-  const float D0 = rowdot[stat + r0], D1 = rowdot[stat + r1];
+  const bool v0 = !RG || qt * BT + r0 < T, v1 = !RG || qt * BT + r1 < T;
+  const float L0 = v0 ? lse[stat + r0] * LOG2E : INFINITY, L1 = v1 ? lse[stat + r1] * LOG2E : INFINITY;
+  float D0, D1;
+  if constexpr (RG) {
+    __shared__ float sD[BT];
+    const int dr = threadIdx.x >> 1;
+    float acc = 0.f;
+    if (qt * BT + dr < T) {
+      const size_t off = ((size_t)b * T + (size_t)qt * BT + dr) * d + (size_t)h * dh;
+      for (int c = (threadIdx.x & 1) * 8; c < dh; c += 16) {
+        const uint4 ov = *reinterpret_cast<const uint4*>(o + off + c), gv = *reinterpret_cast<const uint4*>(d_o + off + c);
+        const uint32_t* ow = reinterpret_cast<const uint32_t*>(&ov);
+        const uint32_t* gw = reinterpret_cast<const uint32_t*>(&gv);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc = fmaf(__uint_as_float(ow[i] << 16), __uint_as_float(gw[i] << 16), acc);
+          acc = fmaf(__uint_as_float(ow[i] & 0xffff0000u), __uint_as_float(gw[i] & 0xffff0000u), acc);
+        }
+      }
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if ((threadIdx.x & 1) == 0) {
+      sD[dr] = acc;
+      if (qt * BT + dr < T) rowdot[stat + dr] = acc;
+    }
+    __syncthreads();
+    D0 = sD[r0]; D1 = sD[r1];
+  } else {
+    D0 = rowdot[stat + r0]; D1 = rowdot[stat + r1];
+  }
   const float scale_log2 = scale * LOG2E;
   float dq[DH / 8][4];
   zero_acc<DH / 8>(dq);
   for (int j = 0; j <= qt; ++j) {
     const uint32_t sK = sK0 + (j & 1) * TILE_BYTES, sV = sV0 + (j & 1) * TILE_BYTES;
     if (j < qt) {
-      load_tile<DH>(sK0 + ((j + 1) & 1) * TILE_BYTES, kbase + (size_t)(j + 1) * BT * ld, ld);
-      load_tile<DH>(sV0 + ((j + 1) & 1) * TILE_BYTES, vbase + (size_t)(j + 1) * BT * ld, ld);
+      load_tile<DH, RG>(sK0 + ((j + 1) & 1) * TILE_BYTES, kbase + (size_t)(j + 1) * BT * ld, ld, T - (j + 1) * BT, dh);
+      load_tile<DH, RG>(sV0 + ((j + 1) & 1) * TILE_BYTES, vbase + (size_t)(j + 1) * BT * ld, ld, T - (j + 1) * BT, dh);
       cp_commit();
       cp_wait<1>();
     } else {
@@ -294,15 +379,16 @@ __global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restri
         s[n][e] = p * (dp[n][e] - ((e < 2) ? D0 : D1));    // dS (without the 1/sqrt(dh) factor)
       }
     }
-    mma_p_regs_b_kn<DH>(dq, s, sK);                  // dQ += dS K
+    mma_p_regs_b_kn<DH, RG>(dq, s, sK);                  // dQ += dS K
     __syncthreads();
   }
-  bf16* q0 = dqkv + ((size_t)b * T + (size_t)qt * BT + r0) * ld + (size_t)h * DH;
-  bf16* q1 = dqkv + ((size_t)b * T + (size_t)qt * BT + r1) * ld + (size_t)h * DH;
+  bf16* q0 = dqkv + ((size_t)b * T + (size_t)qt * BT + r0) * ld + (size_t)h * dh;
+  bf16* q1 = dqkv + ((size_t)b * T + (size_t)qt * BT + r1) * ld + (size_t)h * dh;
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) {
-    *reinterpret_cast<uint32_t*>(q0 + n * 8 + 2 * t) = pack2(dq[n][0] * scale, dq[n][1] * scale);
-    *reinterpret_cast<uint32_t*>(q1 + n * 8 + 2 * t) = pack2(dq[n][2] * scale, dq[n][3] * scale);
+    if (RG && n * 8 >= dh) break;
+    if (v0) *reinterpret_cast<uint32_t*>(q0 + n * 8 + 2 * t) = pack2(dq[n][0] * scale, dq[n][1] * scale);
+    if (v1) *reinterpret_cast<uint32_t*>(q1 + n * 8 + 2 * t) = pack2(dq[n][2] * scale, dq[n][3] * scale);
   }
 }
 
@@ -311,32 +397,39 @@ __global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restri
 // Works on the transposed score tile S^T = K Q^T so that P^T and dS^T land in the register layout
 // the next product needs as its left operand.
 // ------------------------------------------------------------------------------------------
-template <int DH>
+template <int DH, bool RG>
 __global__ void __launch_bounds__(NT) attn_bwd_dkv_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ d_o,
                                                              const float* __restrict__ lse, const float* __restrict__ rowdot,
-                                                             bf16* __restrict__ dqkv, int T, int H, int d, float scale) {
+                                                             bf16* __restrict__ dqkv, int T, int H, int d, int dh,
+                                                             float scale) {
+  if (!RG) dh = DH;
   constexpr int TILE_BYTES = Sizes<DH>::TILE;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t sK = smem_u32(smem), sV = sK + TILE_BYTES, sQ0 = sK + 2 * TILE_BYTES, sdO0 = sK + 4 * TILE_BYTES;
   float* sL = reinterpret_cast<float*>(smem + 6 * TILE_BYTES);     // [2][64] lse * log2e
   float* sD = sL + 2 * BT;                                         // [2][64] rowdot
   const int kt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int nT = T / BT;
+  const int nT = RG ? (T + BT - 1) / BT : T / BT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int64_t ld = 3 * (int64_t)d;
-  const bf16* qhead = qkv + (size_t)b * T * ld + (size_t)h * DH;
+  const bf16* qhead = qkv + (size_t)b * T * ld + (size_t)h * dh;
   const bf16* kbase = qhead + (size_t)kt * BT * ld + d;
-  const bf16* dohead = d_o + (size_t)b * T * d + (size_t)h * DH;
+  const bf16* dohead = d_o + (size_t)b * T * d + (size_t)h * dh;
   const size_t stat = ((size_t)b * H + h) * T;
-  load_tile<DH>(sK, kbase, ld);
-  load_tile<DH>(sV, kbase + d, ld);
-  load_tile<DH>(sQ0 + (kt & 1) * TILE_BYTES, qhead + (size_t)kt * BT * ld, ld);
-  load_tile<DH>(sdO0 + (kt & 1) * TILE_BYTES, dohead + (size_t)kt * BT * d, d);
+  load_tile<DH, RG>(sK, kbase, ld, T - kt * BT, dh);
+  load_tile<DH, RG>(sV, kbase + d, ld, T - kt * BT, dh);
+  load_tile<DH, RG>(sQ0 + (kt & 1) * TILE_BYTES, qhead + (size_t)kt * BT * ld, ld, T - kt * BT, dh);
+  load_tile<DH, RG>(sdO0 + (kt & 1) * TILE_BYTES, dohead + (size_t)kt * BT * d, d, T - kt * BT, dh);
   cp_commit();
-  if (threadIdx.x < BT) {
-    sL[(kt & 1) * BT + threadIdx.x] = lse[stat + (size_t)kt * BT + threadIdx.x] * LOG2E;
-    sD[(kt & 1) * BT + threadIdx.x] = rowdot[stat + (size_t)kt * BT + threadIdx.x];
-  }
+  auto load_stats = [&](int i) {
+    if (threadIdx.x < BT) {
+      const int row = i * BT + threadIdx.x;
+      const bool ok = !RG || row < T;               // a query past the end of the sequence: P = exp(-inf) = 0
+      sL[(i & 1) * BT + threadIdx.x] = ok ? lse[stat + row] * LOG2E : INFINITY;
+      sD[(i & 1) * BT + threadIdx.x] = ok ? rowdot[stat + row] : 0.f;
+    }
+  };
+  load_stats(kt);
   const float scale_log2 = scale * LOG2E;
   const int r0 = warp * 16 + g, r1 = r0 + 8;       // key rows of this thread inside the tile
   float dk[DH / 8][4], dv[DH / 8][4];
@@ -346,13 +439,10 @@ __global__ void __launch_bounds__(NT) attn_bwd_dkv_tc_kernel(const bf16* __restr
     const float* Lq = sL + (i & 1) * BT;
     const float* Dq = sD + (i & 1) * BT;
     if (i + 1 < nT) {
-      load_tile<DH>(sQ0 + ((i + 1) & 1) * TILE_BYTES, qhead + (size_t)(i + 1) * BT * ld, ld);
-      load_tile<DH>(sdO0 + ((i + 1) & 1) * TILE_BYTES, dohead + (size_t)(i + 1) * BT * d, d);
+      load_tile<DH, RG>(sQ0 + ((i + 1) & 1) * TILE_BYTES, qhead + (size_t)(i + 1) * BT * ld, ld, T - (i + 1) * BT, dh);
+      load_tile<DH, RG>(sdO0 + ((i + 1) & 1) * TILE_BYTES, dohead + (size_t)(i + 1) * BT * d, d, T - (i + 1) * BT, dh);
       cp_commit();
-      if (threadIdx.x < BT) {
-        sL[((i + 1) & 1) * BT + threadIdx.x] = lse[stat + (size_t)(i + 1) * BT + threadIdx.x] * LOG2E;
-        sD[((i + 1) & 1) * BT + threadIdx.x] = rowdot[stat + (size_t)(i + 1) * BT + threadIdx.x];
-      }
+      load_stats(i + 1);
       cp_wait<1>();
     } else {
       cp_wait<0>();
@@ -371,61 +461,75 @@ __global__ void __launch_bounds__(NT) attn_bwd_dkv_tc_kernel(const bf16* __restr
         int krow = (e < 2) ? r0 : r1;
         float p = exp2f(st[n][e] * scale_log2 - Lq[qcol]);
         if (i == kt && qcol < krow) p = 0.f;        // causal: query must not precede key
+        float ds = p * (dpt[n][e] - Dq[qcol]);      // dS^T (without the 1/sqrt(dh) factor)
+        if (RG && i == nT - 1 && i * BT + qcol >= T) p = ds = 0.f;   // also where a key's own values are not finite
         st[n][e] = p;
-        dpt[n][e] = p * (dpt[n][e] - Dq[qcol]);     // dS^T (without the 1/sqrt(dh) factor)
+        dpt[n][e] = ds;
       }
     }
-    mma_p_regs_b_kn<DH>(dv, st, sdO);                 // dV += P^T dO
-    mma_p_regs_b_kn<DH>(dk, dpt, sQ);                 // dK += dS^T Q
+    mma_p_regs_b_kn<DH, RG>(dv, st, sdO);                 // dV += P^T dO
+    mma_p_regs_b_kn<DH, RG>(dk, dpt, sQ);                 // dK += dS^T Q
     __syncthreads();
   }
-  bf16* k0 = dqkv + ((size_t)b * T + (size_t)kt * BT + r0) * ld + d + (size_t)h * DH;
-  bf16* k1 = dqkv + ((size_t)b * T + (size_t)kt * BT + r1) * ld + d + (size_t)h * DH;
+  bf16* k0 = dqkv + ((size_t)b * T + (size_t)kt * BT + r0) * ld + d + (size_t)h * dh;
+  bf16* k1 = dqkv + ((size_t)b * T + (size_t)kt * BT + r1) * ld + d + (size_t)h * dh;
+  const bool v0 = !RG || kt * BT + r0 < T, v1 = !RG || kt * BT + r1 < T;
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) {
-    *reinterpret_cast<uint32_t*>(k0 + n * 8 + 2 * t) = pack2(dk[n][0] * scale, dk[n][1] * scale);
-    *reinterpret_cast<uint32_t*>(k1 + n * 8 + 2 * t) = pack2(dk[n][2] * scale, dk[n][3] * scale);
-    *reinterpret_cast<uint32_t*>(k0 + d + n * 8 + 2 * t) = pack2(dv[n][0], dv[n][1]);
-    *reinterpret_cast<uint32_t*>(k1 + d + n * 8 + 2 * t) = pack2(dv[n][2], dv[n][3]);
+    if (RG && n * 8 >= dh) break;
+    if (v0) {
+      *reinterpret_cast<uint32_t*>(k0 + n * 8 + 2 * t) = pack2(dk[n][0] * scale, dk[n][1] * scale);
+      *reinterpret_cast<uint32_t*>(k0 + d + n * 8 + 2 * t) = pack2(dv[n][0], dv[n][1]);
+    }
+    if (v1) {
+      *reinterpret_cast<uint32_t*>(k1 + n * 8 + 2 * t) = pack2(dk[n][2] * scale, dk[n][3] * scale);
+      *reinterpret_cast<uint32_t*>(k1 + d + n * 8 + 2 * t) = pack2(dv[n][2], dv[n][3]);
+    }
   }
 }
 
-template <int DH>
+template <int DH, bool RG>
 cudaError_t launch_fwd(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st) {
   static PerDeviceOnce once;                    // one per instantiation; attributes are per device
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(attn_fwd_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::FWD);
+    cudaError_t e = cudaFuncSetAttribute(attn_fwd_tc_kernel<DH, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::FWD);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
-  dim3 grid(T / BT, H, nseq);
-  attn_fwd_tc_kernel<DH><<<grid, NT, Sizes<DH>::FWD, st>>>((const bf16*)qkv, (bf16*)o, lse, T, H, d,
-                                                          LOG2E / sqrtf((float)DH));
+  const int dh = d / H;
+  dim3 grid((T + BT - 1) / BT, H, nseq);
+  attn_fwd_tc_kernel<DH, RG><<<grid, NT, Sizes<DH>::FWD, st>>>((const bf16*)qkv, (bf16*)o, lse, T, H, d, dh,
+                                                              1.0f / sqrtf((float)dh), LOG2E / sqrtf((float)dh));
   return cudaGetLastError();
 }
 
-template <int DH>
+template <int DH, bool RG>
 cudaError_t launch_bwd(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H, int d,
                        void* dqkv, float* rowdot, int* status, cudaStream_t st) {
   static PerDeviceOnce once;
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(attn_bwd_dq_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::DQ);
+    cudaError_t e = cudaFuncSetAttribute(attn_bwd_dq_tc_kernel<DH, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::DQ);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_bwd_dkv_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::DKV);
+    e = cudaFuncSetAttribute(attn_bwd_dkv_tc_kernel<DH, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::DKV);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
-  int64_t threads = (int64_t)nseq * T * H * (DH / 8);
-  attn_rowdot_tc_kernel<DH><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>((const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
-  dim3 grid(T / BT, H, nseq);
-  const float scale = 1.0f / sqrtf((float)DH);
-  if (DH == 128 && attention_bwd_t5_128_supported(DT_BF16, T, H, d))
-    // dQ, dK, dV on the tcgen05 kernels (they read D[row] from `rowdot`, written just above)
-    return attention_bwd_t5_128(qkv, lse, d_o, rowdot, nseq, T, H, d, dqkv, status, st);
-  attn_bwd_dq_tc_kernel<DH><<<grid, NT, Sizes<DH>::DQ, st>>>((const bf16*)qkv, (const bf16*)d_o, lse, rowdot, (bf16*)dqkv, T, H, d, scale);
-  attn_bwd_dkv_tc_kernel<DH><<<grid, NT, Sizes<DH>::DKV, st>>>((const bf16*)qkv, (const bf16*)d_o, lse, rowdot, (bf16*)dqkv, T, H, d, scale);
+  const int dh = d / H;
+  const float scale = 1.0f / sqrtf((float)dh);
+  if constexpr (!RG) {
+    int64_t threads = (int64_t)nseq * T * H * (DH / 8);
+    attn_rowdot_tc_kernel<DH><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>((const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
+    if (DH == 128 && attention_bwd_t5_128_supported(DT_BF16, T, H, d))
+      // dQ, dK, dV on the tcgen05 kernels (they read D[row] from `rowdot`, written just above)
+      return attention_bwd_t5_128(qkv, lse, d_o, rowdot, nseq, T, H, d, dqkv, status, st);
+  }
+  dim3 grid((T + BT - 1) / BT, H, nseq);
+  attn_bwd_dq_tc_kernel<DH, RG><<<grid, NT, Sizes<DH>::DQ, st>>>((const bf16*)qkv, (const bf16*)o, (const bf16*)d_o, lse, rowdot,
+                                                                (bf16*)dqkv, T, H, d, dh, scale);
+  attn_bwd_dkv_tc_kernel<DH, RG><<<grid, NT, Sizes<DH>::DKV, st>>>((const bf16*)qkv, (const bf16*)d_o, lse, rowdot, (bf16*)dqkv,
+                                                                  T, H, d, dh, scale);
   return cudaGetLastError();
 }
 
@@ -441,7 +545,8 @@ cudaError_t attention_fwd_tc(const void* qkv, int nseq, int T, int H, int d, voi
                              cudaStream_t st) {
   if (!attention_tc_supported(DT_BF16, T, H, d)) return cudaErrorInvalidValue;
   if (attention_fwd_t5_supported(DT_BF16, T, H, d)) return attention_fwd_t5(qkv, nseq, T, H, d, o, lse, status, st);
-  return d / H == 64 ? launch_fwd<64>(qkv, nseq, T, H, d, o, lse, st) : launch_fwd<128>(qkv, nseq, T, H, d, o, lse, st);
+  return d / H == 64 ? launch_fwd<64, false>(qkv, nseq, T, H, d, o, lse, st)
+                     : launch_fwd<128, false>(qkv, nseq, T, H, d, o, lse, st);
 }
 
 cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
@@ -449,8 +554,39 @@ cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, c
   if (!attention_tc_supported(DT_BF16, T, H, d)) return cudaErrorInvalidValue;
   if (attention_t5_supported(DT_BF16, T, H, d))
     return attention_bwd_t5(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
-  return d / H == 64 ? launch_bwd<64>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st)
-                     : launch_bwd<128>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
+  return d / H == 64 ? launch_bwd<64, false>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st)
+                     : launch_bwd<128, false>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
+}
+
+// The 16-byte copies need every head's first column of every row on a 16-byte boundary (d and the head width
+// multiples of 8, aligned bases); sequences and heads are grid dimensions y and z.
+bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const void* qkv, const void* o, const void* d_o,
+                                const void* dqkv) {
+  auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
+  if (dt != DT_BF16 || H < 1 || d % H != 0 || T < 1 || nseq < 1) return false;
+  const int dh = d / H;
+  return dh % 8 == 0 && dh <= 128 && H <= 65535 && nseq <= 65535 && al16(qkv) && al16(o) && al16(d_o) && al16(dqkv);
+}
+
+cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st) {
+  switch ((d / H + 31) / 32) {
+    case 1: return launch_fwd<32, true>(qkv, nseq, T, H, d, o, lse, st);
+    case 2: return launch_fwd<64, true>(qkv, nseq, T, H, d, o, lse, st);
+    case 3: return launch_fwd<96, true>(qkv, nseq, T, H, d, o, lse, st);
+    case 4: return launch_fwd<128, true>(qkv, nseq, T, H, d, o, lse, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
+                                 int d, void* dqkv, float* rowdot, cudaStream_t st) {
+  switch ((d / H + 31) / 32) {
+    case 1: return launch_bwd<32, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);
+    case 2: return launch_bwd<64, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);
+    case 3: return launch_bwd<96, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);
+    case 4: return launch_bwd<128, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace sl

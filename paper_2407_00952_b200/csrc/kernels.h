@@ -110,6 +110,14 @@ cudaError_t attention_fwd_tc(const void* qkv, int nseq, int T, int H, int d, voi
 cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq,
                              int T, int H, int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
 
+// mma.sync attention for the remaining bf16 shapes: any T, head widths that are multiples of 8; P and dS kept to
+// 16 mantissa bits (attention_tc.cu).  Pointers that a direction does not use may be null.
+bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const void* qkv, const void* o, const void* d_o,
+                                const void* dqkv);
+cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st);
+cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
+                                 int d, void* dqkv, float* rowdot, cudaStream_t st);
+
 // Adapter gradients: for nt targets of rank r (weight columns wcol0 + t*rp + jj of Wt),
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c],  c < C,
 // stored at out + g*out_group_stride + t*out_target_stride + jj*out_sj + c*out_sc.

@@ -223,6 +223,8 @@ int splitlora_attention_fwd(int dtype, int use_tc, const void* qkv, int nseq, in
   cudaError_t e;
   if (use_tc && attention_tc_supported(dtype, T, n_head, d_model))
     e = attention_fwd_tc(qkv, nseq, T, n_head, d_model, o, lse, nullptr, (cudaStream_t)stream);
+  else if (use_tc && attention_ragged_supported(dtype, nseq, T, n_head, d_model, qkv, o, nullptr, nullptr))
+    e = attention_fwd_ragged(qkv, nseq, T, n_head, d_model, o, lse, (cudaStream_t)stream);
   else
     e = attention_fwd_simt(dtype, qkv, nseq, T, n_head, d_model, o, lse, (cudaStream_t)stream);
   return e == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;
@@ -236,6 +238,8 @@ int splitlora_attention_bwd(int dtype, int use_tc, const void* qkv, const void* 
   cudaError_t e;
   if (use_tc && attention_tc_supported(dtype, T, n_head, d_model))
     e = attention_bwd_tc(qkv, o, lse, d_o, nseq, T, n_head, d_model, dqkv, rowdot, nullptr, (cudaStream_t)stream);
+  else if (use_tc && attention_ragged_supported(dtype, nseq, T, n_head, d_model, qkv, o, d_o, dqkv))
+    e = attention_bwd_ragged(qkv, o, lse, d_o, nseq, T, n_head, d_model, dqkv, rowdot, (cudaStream_t)stream);
   else
     e = attention_bwd_simt(dtype, qkv, o, lse, d_o, nseq, T, n_head, d_model, dqkv, rowdot, (cudaStream_t)stream);
   return e == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;

@@ -417,6 +417,8 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
   { Scope s(c, "attention_fwd", 1);
     if (c->tc && attention_tc_supported(c->dt, T, H, d))
       e = attention_fwd_tc(qkv, M / T, T, H, d, o, lse, c->status, c->st);
+    else if (c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, nullptr, nullptr))
+      e = attention_fwd_ragged(qkv, M / T, T, H, d, o, lse, c->st);
     else
       e = attention_fwd_simt(c->dt, qkv, M / T, T, H, d, o, lse, c->st);
     if (e) return e; }
@@ -511,9 +513,13 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
       a.we_grouped = grouped;
     }
     if ((e = linear(c, c->has_o ? "lora_linear_bwd" : "linear_bwd", a))) return e; }
-  { Scope s(c, "attention_bwd", c->tc && attention_t5_supported(c->dt, T, H, d) ? 2 : 3);
-    if (c->tc && attention_tc_supported(c->dt, T, H, d))
+  { const bool aligned_form = c->tc && attention_tc_supported(c->dt, T, H, d);
+    const bool ragged_form = !aligned_form && c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, c->g_do, c->g_dqkv);
+    Scope s(c, "attention_bwd", ragged_form || (c->tc && attention_t5_supported(c->dt, T, H, d)) ? 2 : 3);
+    if (aligned_form)
       e = attention_bwd_tc(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->status, c->st);
+    else if (ragged_form)
+      e = attention_bwd_ragged(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->st);
     else
       e = attention_bwd_simt(c->dt, qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->st);
     if (e) return e; }
