@@ -437,9 +437,9 @@ int pick_bn(const GemmArgs& a) {
 
 bool pair_ok(const GemmArgs& a) {
   if (max_pairs() < 1 || a.k_gap_len > 0) return false;
-  if (a.M % (2 * BM) != 0 || a.N < 256) return false;
-  if (a.rows_per_group > 0 && a.rows_per_group % (2 * BM) != 0) return false;
-  return true;
+  if (a.M <= BM || a.N < 256) return false;
+  if (a.rows_per_group > 0 && a.rows_per_group % (2 * BM) != 0) return false;   // 0 when there is one group
+  return a.rows_per_group > 0 || a.M % (2 * BM) == 0 || a.M % BM != 0;
 }
 
 // Fills the parameters both kernels share and encodes the tensor maps; box rows of the W maps differ.
@@ -449,7 +449,7 @@ bool prepare(const GemmArgs& a, int* status, int w_box_rows, CUtensorMap* mX, CU
   const int w_rows = a.w_rows > 0 ? a.w_rows : a.N;
   if (!make_map(mX, a.X, a.M, a.K + a.k_gap_len, a.ldx, BM)) return false;
   if (!make_map(mW, a.W, a.w_grouped ? (uint64_t)G * a.N : (uint64_t)w_rows, a.K + a.k_gap_len, a.ldw, w_box_rows)) return false;
-  p->M = a.M; p->N = a.N; p->K = a.K; p->num_kb = a.K / BK;
+  p->M = a.M; p->N = a.N; p->K = a.K; p->num_kb = (a.K + BK - 1) / BK;      // the tail of the last block is zero-filled by the copies
   p->gap_kb = a.k_gap_len / BK;
   p->gap_kb_begin = a.k_gap_len > 0 ? a.k_gap_begin / BK : p->num_kb;
   if (a.Ke > 0) {
@@ -469,6 +469,9 @@ bool prepare(const GemmArgs& a, int* status, int w_box_rows, CUtensorMap* mX, CU
   p->w_group_rows = a.w_grouped ? a.N : 0;
   p->we_group_rows = a.we_grouped ? a.N : 0;
   p->epi = a.epi; p->gelu_tanh = a.gelu_tanh;
+  // Off the tile sizes these layers are otherwise computed with tanhf (gemm_simt.cu): they keep that accuracy here
+  // (two special-function instructions per element instead of one).
+  p->gelu_exact = a.gelu_tanh && (a.M % BM != 0 || a.K % BK != 0);
   p->bias = (const bf16*)a.bias; p->R = (const bf16*)a.R; p->ldr = a.ldr;
   p->Y = (bf16*)a.Y; p->ldy = a.ldy; p->Z = (bf16*)a.Z; p->ldz = a.ldz;
   p->status = status;
@@ -479,7 +482,7 @@ template <int BN, bool DEEP = false>
 cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
   using C = Cfg<BN, DEEP>;
   const int sms = num_sms();
-  if (BN == 64 && !DEEP && (a.M / BM) * ((a.N + BN - 1) / BN) <= sms) return launch<64, true>(a, status, st);
+  if (BN == 64 && !DEEP && ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN) <= sms) return launch<64, true>(a, status, st);
   static PerDeviceOnce once;                    // one per instantiation; attributes are per device
   const int dev = current_device();
   if (once.needed(dev)) {
@@ -490,7 +493,7 @@ cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
   CUtensorMap mX, mW, mXe, mWe, mY, mZ;
   TcParams p;
   if (!prepare(a, status, BN, &mX, &mW, &mXe, &mWe, &mY, &mZ, &p)) return cudaErrorInvalidValue;
-  p.tiles_m = a.M / BM; p.tiles_n = (a.N + BN - 1) / BN;
+  p.tiles_m = (a.M + BM - 1) / BM; p.tiles_n = (a.N + BN - 1) / BN;
   const int tiles = p.tiles_m * p.tiles_n;
   const int slots = sms * C::CTAS_PER_SM;
   const int grid = tiles < slots ? tiles : slots;
@@ -503,7 +506,7 @@ cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
   CUtensorMap mX, mW, mXe, mWe, mY, mZ, mR;
   TcParams p;
   if (!prepare(a, status, BN / 2, &mX, &mW, &mXe, &mWe, &mY, &mZ, &p)) return cudaErrorInvalidValue;
-  p.tiles_m = a.M / (2 * BM); p.tiles_n = (a.N + BN - 1) / BN;
+  p.tiles_m = (a.M + 2 * BM - 1) / (2 * BM); p.tiles_n = (a.N + BN - 1) / BN;
   const int tiles = p.tiles_m * p.tiles_n;
   const int pairs = tiles < max_pairs() ? tiles : max_pairs();
   const bool need_r = a.epi == EPI_BIAS_RESID || a.epi == EPI_MUL_GELUGRAD;
@@ -546,8 +549,12 @@ int gemm_tc_init() {
 bool gemm_tc_supported(const GemmArgs& a) {
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   if (!tensor_map_encoder() || a.dtype != DT_BF16) return false;
-  if (a.M < BM || a.M % BM != 0 || a.K < BK || a.K % BK != 0 || a.N < 8 || a.N % 8 != 0) return false;
-  if (a.rows_per_group > 0 && (a.rows_per_group % BM != 0 || a.M % a.rows_per_group != 0)) return false;
+  // M and K may be anything the copies' 16-byte rule allows: rows past M and columns past K are zero-filled on the
+  // way in, rows past M clipped on the way out (on the plain-FMA kernel instead, a GPT-2-small-shaped round of
+  // 5 x 333 tokens takes 22 times as long).  Groups must not share a tile.
+  if (a.M < 1 || a.K < 8 || a.K % 8 != 0 || a.N < 8 || a.N % 8 != 0) return false;
+  if (a.rows_per_group > 0 && a.rows_per_group < a.M && (a.rows_per_group % BM != 0 || a.M % a.rows_per_group != 0)) return false;
+  if (a.k_gap_len > 0 && a.K % BK != 0) return false;
   if (a.ldx % 8 || a.ldw % 8 || a.ldy % 8) return false;
   if (a.k_gap_len < 0 || a.k_gap_begin < 0 || a.k_gap_len % BK || a.k_gap_begin % BK || a.k_gap_begin > a.K) return false;
   if (!al16(a.X) || !al16(a.W) || !al16(a.Y)) return false;
@@ -561,8 +568,10 @@ bool gemm_tc_supported(const GemmArgs& a) {
   return true;
 }
 
-cudaError_t gemm_tc(const GemmArgs& a, int* status, cudaStream_t st) {
-  if (!gemm_tc_supported(a)) return cudaErrorInvalidValue;
+cudaError_t gemm_tc(const GemmArgs& args, int* status, cudaStream_t st) {
+  if (!gemm_tc_supported(args)) return cudaErrorInvalidValue;
+  GemmArgs a = args;
+  if (a.rows_per_group >= a.M) a.rows_per_group = 0;      // one group
   if (pair_ok(a)) return launch_pair(a, status, st);
   switch (pick_bn(a)) {
     case 256: return launch<256>(a, status, st);

@@ -49,8 +49,8 @@ struct GemmArgs {
 
 // Plain-FMA tiled kernel, any shape, fp32 or bf16 storage with fp32 accumulation.
 cudaError_t gemm_simt(const GemmArgs& a, cudaStream_t st);
-// tcgen05 / TMEM / TMA kernel (bf16 only).  Shape rules: M % 128 == 0, K % 64 == 0, N % 8 == 0,
-// rows_per_group % 128 == 0, leading dimensions multiples of 8 elements, 16-byte aligned bases.
+// tcgen05 / TMEM / TMA kernel (bf16 only).  Shape rules: any M with one group, else rows_per_group % 128 == 0;
+// K % 8 == 0, N % 8 == 0, leading dimensions multiples of 8 elements, 16-byte aligned bases.
 // status: device word that receives a non-zero code if a bounded wait expires.
 bool gemm_tc_supported(const GemmArgs& a);
 cudaError_t gemm_tc(const GemmArgs& a, int* status, cudaStream_t st);
@@ -121,7 +121,7 @@ cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* ls
 // Adapter gradients: for nt targets of rank r (weight columns wcol0 + t*rp + jj of Wt),
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c],  c < C,
 // stored at out + g*out_group_stride + t*out_target_stride + jj*out_sj + c*out_sc.
-// rows_per_group (0: one group) must be a multiple of 128.  partial: scratch of at least
+// rows_per_group must be a multiple of 128 unless there is one group (0, or >= M).  partial: scratch of at least
 // lora_grad_scratch_floats(M, nt*r, C) floats.
 size_t lora_grad_scratch_floats(int M, int R, int C);
 cudaError_t lora_grad(int dt, const void* Z, int64_t ldz, int zcol0, int C, const void* Wt, int64_t ldwt,

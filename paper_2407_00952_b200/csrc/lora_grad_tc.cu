@@ -192,7 +192,8 @@ bool al16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 bool lora_grad_tc_supported(int dt, const void* Z, int64_t ldz, int zcol0, int C, const void* Wt, int64_t ldwt,
                             int wcol0, int r, int rp, int nt, int M, int rows_per_group) {
   if (dt != DT_BF16 || !(rp == 16 || rp == 32 || rp == 64) || r < 1 || r > rp || nt < 1) return false;
-  if (M % 128 != 0 || (rows_per_group > 0 && (rows_per_group % 128 != 0 || M % rows_per_group != 0))) return false;
+  // one group: any M (rows past the last are zero-filled by the copies); several: whole 128-row blocks each
+  if (rows_per_group > 0 && rows_per_group < M && (rows_per_group % 128 != 0 || M % rows_per_group != 0)) return false;
   if (C % 8 != 0 || ldz % 8 != 0 || zcol0 % 8 != 0 || ldwt % 64 != 0 || !al16(Z) || !al16(Wt)) return false;
   const int wsel0 = wcol0 % LT_N;
   if (wsel0 + (nt - 1) * rp + r > LT_N || wcol0 - wsel0 + LT_N > ldwt) return false;
@@ -223,8 +224,9 @@ cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M
   if (!init_device()) return cudaErrorNotSupported;
   if (!status) status = library_status_word();
   if (!status) return cudaErrorNotSupported;
-  const int rpg = rows_per_group > 0 ? rows_per_group : M;
-  const int groups = M / rpg;
+  const bool one = rows_per_group <= 0 || rows_per_group >= M;
+  const int rpg = one ? (M + 127) / 128 * 128 : rows_per_group;
+  const int groups = one ? 1 : M / rpg;
   const int C = jobs[0].C;
   const int ctiles = (C + LT_C - 1) / LT_C;
   const int s = pick_chunks(ctiles * groups * njobs, rpg);

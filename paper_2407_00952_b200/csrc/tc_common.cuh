@@ -30,6 +30,7 @@ struct TcParams {
   int we_group_rows;              // rows between groups in We
   int tiles_m, tiles_n;
   int epi, gelu_tanh;
+  int gelu_exact;                 // tanh to fp32 accuracy instead of tanh.approx (see gemm_tc.cu, prepare)
   const bf16* bias;
   const bf16* R; long long ldr;
   bf16* Y; long long ldy;
@@ -256,6 +257,18 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 __device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t w) {
   return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
+// tanh as 1 - 2 / (1 + e^2x): two special-function instructions, absolute error of a few 2^-24 (tanh.approx: 2^-11)
+__device__ __forceinline__ float tanh_exact(float x) { return 1.0f - __fdividef(2.0f, 1.0f + __expf(2.0f * x)); }
+__device__ __forceinline__ float gelu_tanh_exact(float z) {
+  const float hz = 0.5f * z;
+  return fmaf(hz, tanh_exact(z * fmaf(0.7978845608028654f * 0.044715f, z * z, 0.7978845608028654f)), hz);
+}
+__device__ __forceinline__ float gelu_grad_tanh_exact(float z) {
+  const float z2 = z * z;
+  const float t = tanh_exact(z * fmaf(0.7978845608028654f * 0.044715f, z2, 0.7978845608028654f));
+  const float du = fmaf(0.7978845608028654f * 0.134145f, z2, 0.7978845608028654f);
+  return fmaf(0.5f * z * du, fmaf(-t, t, 1.0f), fmaf(0.5f, t, 0.5f));
+}
 __device__ __forceinline__ void gelu_tanh_pair(float& a, float& b) {
   const uint64_t c1 = pack2(0.7978845608028654f, 0.7978845608028654f);
   const uint64_t c2 = pack2(0.7978845608028654f * 0.044715f, 0.7978845608028654f * 0.044715f);
@@ -362,13 +375,13 @@ __device__ __forceinline__ void epilogue_drain(int lane) {
   __syncwarp();
 }
 
-// The second epilogue operand (residual, or the saved pre-activation) of columns [n, n+32) of row m.
-// Issued one chunk ahead of its use so that its latency overlaps the previous chunk's work.
+// The second epilogue operand (residual, or the saved pre-activation) of columns [n, n+32) of row m (zero past
+// the last row).  Issued one chunk ahead of its use so that its latency overlaps the previous chunk's work.
 __device__ __forceinline__ void load_r_chunk(const TcParams& p, int m, int n, uint4* r) {
   const bf16* rrow = p.R + (size_t)m * p.ldr + n;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    if (n + 8 * j < p.N) r[j] = *reinterpret_cast<const uint4*>(rrow + 8 * j);
+    if (n + 8 * j < p.N && m < p.M) r[j] = *reinterpret_cast<const uint4*>(rrow + 8 * j);
     else r[j] = make_uint4(0u, 0u, 0u, 0u);
   }
 }
@@ -423,7 +436,10 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
       zr[2 * i + 1] = __high2float(z2);
     }
     epi_yield();
-    if (tanh_form) {
+    if (p.gelu_exact) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = gelu_tanh_exact(zr[i]);
+    } else if (tanh_form) {
 #pragma unroll
       for (int i = 0; i < 32; i += 2) {
         v[i] = zr[i]; v[i + 1] = zr[i + 1]; gelu_tanh_pair(v[i], v[i + 1]);
@@ -433,7 +449,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = gelu_f(zr[i], false);
     }
-    stage_and_store(stage + (uint32_t)buf * 2048u, mapZ, packed, lane, n, m_warp0);
+    if (m_warp0 < p.M) stage_and_store(stage + (uint32_t)buf * 2048u, mapZ, packed, lane, n, m_warp0);
     buf ^= 1;
   } else if (p.epi == EPI_BIAS_RESID) {
 #pragma unroll
@@ -444,7 +460,14 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
       if (j & 1) epi_yield();
     }
   } else if (p.epi == EPI_MUL_GELUGRAD) {
-    if (tanh_form) {
+    if (p.gelu_exact) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bf16* rp = reinterpret_cast<const bf16*>(&rpre[j]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[8 * j + i] *= gelu_grad_tanh_exact(__bfloat162float(rp[i]));
+      }
+    } else if (tanh_form) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const uint32_t* rw = reinterpret_cast<const uint32_t*>(&rpre[j]);
@@ -469,7 +492,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
     packed[i] = *reinterpret_cast<uint32_t*>(&y2);
   }
   epi_yield();
-  stage_and_store(stage + (uint32_t)buf * 2048u, mapY, packed, lane, n, m_warp0);
+  if (m_warp0 < p.M) stage_and_store(stage + (uint32_t)buf * 2048u, mapY, packed, lane, n, m_warp0);   // clipped at row M
   buf ^= 1;
 }
 

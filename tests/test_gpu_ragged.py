@@ -60,3 +60,57 @@ def test_attention_ragged_writes_inside_its_rows_only():
     B.attention_bwd_static(qkv, o, lse, do, nseq, T, H, dqkv=inner)
     assert bool((buf[:guard] == 7).all()) and bool((buf[guard + nseq * T:] == 7).all())
     assert torch.equal(inner, B.attention_bwd(qkv, o, lse, do, nseq, T, H))
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (5, 72, 264), (127, 64, 72), (129, 200, 256), (255, 768, 1000), (257, 128, 520),
+                                   (1000, 136, 256), (300, 1000, 8)])
+@pytest.mark.parametrize("epilogue", [B.EPI_BIAS, B.EPI_BIAS_GELU, B.EPI_BIAS_RESID, B.EPI_MUL_GELUGRAD])
+def test_linear_any_row_count_and_depth(M, K, N, epilogue):
+    """Against 64 bits: no further off than the plain-FMA kernel (the products of bf16 values are exact in both and
+    both round to bf16 once, so the errors agree to a few per mille); rows past M stay untouched."""
+    g = torch.Generator(device="cuda").manual_seed(M + K + N)
+    mk = lambda *s, sc=1.0: (torch.randn(*s, device="cuda", generator=g) * sc).bfloat16()  # noqa: E731
+    x, W, bias, r = mk(M, K), mk(N, K, sc=K ** -0.5), mk(N), mk(M, N, sc=2.0)
+    acc = x.double() @ W.double().T
+    z = (acc + bias.double())
+    gelu = lambda t: torch.nn.functional.gelu(t, approximate="tanh")  # noqa: E731
+    if epilogue == B.EPI_MUL_GELUGRAD:
+        t = r.double().requires_grad_()
+        gelu(t).sum().backward()
+        ref = acc * t.grad
+    else:
+        ref = {B.EPI_BIAS: z, B.EPI_BIAS_GELU: gelu(z), B.EPI_BIAS_RESID: z + r.double()}[epilogue]
+    errs = []
+    for tc in (True, False):
+        buf = torch.full((M + 160, N), 7.0, device="cuda", dtype=torch.bfloat16)
+        zbuf = torch.full((M + 160, N), 7.0, device="cuda", dtype=torch.bfloat16)
+        B.linear(x, W, None if epilogue == B.EPI_MUL_GELUGRAD else bias, epilogue, r=r, y=buf[:M], z=zbuf[:M], use_tensor_cores=tc)
+        assert bool((buf[M:] == 7).all()) and bool((zbuf[M:] == 7).all())
+        errs.append([_norm_err(buf[:M], ref)] + ([_norm_err(zbuf[:M], z)] if epilogue == B.EPI_BIAS_GELU else []))
+    for got, plain in zip(*errs):
+        assert got <= 1.02 * plain + 2e-5, errs
+
+
+@pytest.mark.parametrize("M,n_in,n_out,r,G", [(1, 64, 72, 4, 1), (77, 200, 136, 6, 1), (129, 768, 256, 1, 1), (300, 136, 768, 40, 1),
+                                              (512, 200, 1000, 8, 2), (640, 72, 72, 64, 5)])
+def test_lora_linear_any_size(M, n_in, n_out, r, G):
+    """Forward and backward against 64 bits, next to the plain-FMA kernels' errors."""
+    g = torch.Generator(device="cuda").manual_seed(M + n_in)
+    x = torch.randn(M, n_in, device="cuda", generator=g).bfloat16()
+    W = (torch.randn(n_out, n_in, device="cuda", generator=g) * n_in ** -0.5).bfloat16()
+    dy = (torch.randn(M, n_out, device="cuda", generator=g) * n_out ** -0.5).bfloat16()
+    A = torch.randn(G, r, n_in, device="cuda", generator=g) * n_in ** -0.5
+    Bm = torch.randn(G, n_out, r, device="cuda", generator=g) * r ** -0.5
+    s = 16.0 / r
+    xg, dyg, A64, B64 = x.double().view(G, -1, n_in), dy.double().view(G, -1, n_out), A.double(), Bm.double()
+    h, dh = xg @ A64.transpose(1, 2), s * dyg @ B64
+    ref = ((x.double() @ W.double().T + s * (h @ B64.transpose(1, 2)).reshape(M, n_out)), (dy.double() @ W.double() + (dh @ A64).reshape(M, n_in)),
+           dh.transpose(1, 2) @ xg, s * dyg.transpose(1, 2) @ h)
+    errs = []
+    for tc in (True, False):
+        y = B.lora_linear_fwd(x, W, None, A, Bm, 16.0, use_tensor_cores=tc)
+        got = (y,) + B.lora_linear_bwd(x, B.transpose(W), dy, A, Bm, 16.0, use_tensor_cores=tc)
+        errs.append([_norm_err(a, b) for a, b in zip(got, ref)])
+    assert B.library_status() == 0
+    for got, plain in zip(*errs):
+        assert got <= 1.02 * plain + 2e-5, errs
