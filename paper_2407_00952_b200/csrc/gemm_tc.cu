@@ -21,6 +21,12 @@
 // Warp roles (320 threads): warp 0 = TMA producer, warp 1 = tensor-memory owner + MMA issuer,
 // warps 2..9 = epilogue (a warp reads the 32 accumulator lanes its warp id modulo 4 selects; the
 // two warps of a lane quarter take one half of the tile's columns each).
+// The producer and issuer loops run as whole converged warps and one elected lane issues: in a loop that only one lane
+// enters, the operands of every product go to uniform registers one by one, and a 64-deep block cost the issuing
+// lane 500 cycles (330 in this form, next to 512 that the pair's four products take); the slack goes to the
+// epilogue warps.  Isolated launches at M 32768, before -> after: output projection (bias + residual) 65.4 ->
+// 60.2 us, fc1 (GELU) 240 -> 229.5, fc2 212 -> 204, fc2 backward (x GELU') 244 -> 230, QKV + LoRA 151 -> 137,
+// plain backward products 193 -> 191 and 54.6 -> 53.1.
 // Every wait on an mbarrier is bounded: when it expires the kernel records a code in `status`,
 // stops issuing work, waits briefly for copies in flight, frees its tensor memory and returns.
 #include "host_common.h"
@@ -96,19 +102,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      int stage = 0; uint32_t phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        int tm, tn; tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
-        const int m0 = tm * BM, n0 = tn * BN;
-        const int g = p.rows_per_group > 0 ? m0 / p.rows_per_group : 0;
-        const int w_row = g * p.w_group_rows + n0;
-        const int we_row = g * p.we_group_rows + n0;
-        for (int kb = 0; kb < kb_total; ++kb) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 1)) { ok = false; break; }
+    const bool leader = elect_one();
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      int tm, tn; tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
+      const int m0 = tm * BM, n0 = tn * BN;
+      const int g = p.rows_per_group > 0 ? m0 / p.rows_per_group : 0;
+      const int w_row = g * p.w_group_rows + n0;
+      const int we_row = g * p.we_group_rows + n0;
+      for (int kb = 0; kb < kb_total; ++kb) {
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 1)) { ok = false; break; }
+        const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+        if (leader) {
           mbar_expect_tx(full_bar(stage), C::STAGE_BYTES);
-          const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
           if (kb < p.num_kb) {
             const int kc = (kb < p.gap_kb_begin ? kb : kb + p.gap_kb) * BK;
             tma_load_2d(sa, &mapX, full_bar(stage), kc, m0);
@@ -118,49 +125,56 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
             tma_load_2d(sa, &mapXe, full_bar(stage), e * BK, m0);
             tma_load_2d(sb, &mapWe, full_bar(stage), e * BK, we_row);
           }
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int stage = 0; uint32_t phase = 0;
-      int as = 0; uint32_t aphase = 0;
-      bool ok = true;
-      const uint32_t a_lo0 = desc_lo(base);
-      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        if (!mbar_wait(tempty_bar(as), aphase ^ 1u, abort_flag, p.status, 2)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(as * BN);
-        // main contraction: four products per block, issued back to back (advancing 16 elements
-        // along K inside the swizzled row = +32 bytes = +2 in descriptor units)
-        for (int kb = 0; kb < p.num_kb; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status, 3)) { ok = false; break; }
-          const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
-          const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
+    const bool leader = elect_one();
+    int stage = 0; uint32_t phase = 0;
+    int as = 0; uint32_t aphase = 0;
+    bool ok = true;
+    const uint32_t a_lo0 = desc_lo(base);
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      if (!mbar_wait_warp(tempty_bar(as), aphase ^ 1u, abort_flag, p.status, 2)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(as * BN);
+      // main contraction: four products per block, issued back to back (advancing 16 elements
+      // along K inside the swizzled row = +32 bytes = +2 in descriptor units)
+      for (int kb = 0; kb < p.num_kb; ++kb) {
+        if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status, 3)) { ok = false; break; }
+        const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
+        const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
+        if (leader) {
           tc_mma_lo(d_tmem, alo, blo, C::IDESC, (uint32_t)kb);
           tc_mma_lo_acc(d_tmem, alo + 2, blo + 2, C::IDESC);
           tc_mma_lo_acc(d_tmem, alo + 4, blo + 4, C::IDESC);
           tc_mma_lo_acc(d_tmem, alo + 6, blo + 6, C::IDESC);
           tc_commit(empty_bar(stage));          // frees the stage once these products have read it
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
-        // rank-r extension: the last block may hold fewer than four products
-        for (int kb = p.num_kb; kb < kb_total && ok; ++kb) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status, 3)) { ok = false; break; }
-          const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
-          const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
-          const int nmma = kb == kb_total - 1 ? p.ext_last_mmas : BK / UMMA_K;
+        __syncwarp();
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+      }
+      // rank-r extension: the last block may hold fewer than four products
+      for (int kb = p.num_kb; kb < kb_total && ok; ++kb) {
+        if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status, 3)) { ok = false; break; }
+        const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
+        const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
+        const int nmma = kb == kb_total - 1 ? p.ext_last_mmas : BK / UMMA_K;
+        if (leader) {
 #pragma unroll 1
           for (int k = 0; k < nmma; ++k) tc_mma_lo_acc(d_tmem, alo + 2 * k, blo + 2 * k, C::IDESC);
           tc_commit(empty_bar(stage));
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        tc_commit(tfull_bar(as));               // accumulator complete
-        if (++as == 2) { as = 0; aphase ^= 1u; }
+        __syncwarp();
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       }
+      if (!ok) break;
+      if (leader) tc_commit(tfull_bar(as));     // accumulator complete
+      __syncwarp();
+      if (++as == 2) { as = 0; aphase ^= 1u; }
     }
   } else {
     // ---------------- epilogue ----------------
@@ -279,38 +293,43 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
-      int stage = 0; uint32_t phase = 0;
-      int tcount = 0;                              // tiles this CTA has started
-      bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-        int tm, tn; tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
-        const int m0 = tm * 2 * BM + (int)rank * BM, n0 = tn * BN + (int)rank * (BN / 2);
-        const int g = p.rows_per_group > 0 ? m0 / p.rows_per_group : 0;
-        const int w_row = g * p.w_group_rows + n0;
-        const int we_row = g * p.we_group_rows + n0;
-        // R block of this tile: issued as soon as the epilogue has released the buffer (checked
-        // between operand blocks so that the operand ring never waits for it)
-        bool r_pending = NEED_R;
-        auto issue_r = [&](bool blocking) -> bool {
-          if (!r_pending) return true;
-          const uint32_t par = ((uint32_t)tcount & 1u) ^ 1u;
-          if (blocking) { if (!mbar_wait(rempty_bar, par, abort_flag, p.status, 15)) return false; }
-          else if (!mbar_try(rempty_bar, par)) return true;
+    const bool leader = elect_one();
+    int stage = 0; uint32_t phase = 0;
+    int tcount = 0;                                // tiles this CTA has started
+    bool ok = true;
+    for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
+      int tm, tn; tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
+      const int m0 = tm * 2 * BM + (int)rank * BM, n0 = tn * BN + (int)rank * (BN / 2);
+      const int g = p.rows_per_group > 0 ? m0 / p.rows_per_group : 0;
+      const int w_row = g * p.w_group_rows + n0;
+      const int we_row = g * p.we_group_rows + n0;
+      // R block of this tile: issued as soon as the epilogue has released the buffer (checked between operand
+      // blocks so that the operand ring never waits for it; test_wait: a try_wait here suspends the warp, which
+      // cost the tiles with a second operand 20 %)
+      bool r_pending = NEED_R;
+      auto issue_r = [&](bool blocking) -> bool {
+        if (!r_pending) return true;
+        const uint32_t par = ((uint32_t)tcount & 1u) ^ 1u;
+        if (blocking) { if (!mbar_wait_warp(rempty_bar, par, abort_flag, p.status, 15)) return false; }
+        else if (!__all_sync(0xffffffffu, mbar_test(rempty_bar, par))) return true;
+        if (leader) {
           mbar_expect_tx(rfull_bar, C::R_BYTES);
 #pragma unroll
           for (int j = 0; j < BN / BK; ++j)
             tma_load_2d(r_base + j * (BM * BK * 2), &mapR, rfull_bar, tn * BN + j * BK, m0);
-          r_pending = false;
-          return true;
-        };
-        for (int kb = 0; kb < kb_total; ++kb) {
-          issue_r(false);
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 11)) { ok = false; break; }
-          // the leader's barrier collects the bytes of both CTAs' copies
+        }
+        __syncwarp();
+        r_pending = false;
+        return true;
+      };
+      for (int kb = 0; kb < kb_total; ++kb) {
+        issue_r(false);
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 11)) { ok = false; break; }
+        const uint32_t leader_full = map_to_cta(full_bar(stage), 0);
+        const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+        if (leader) {
+          // the first CTA's barrier collects the bytes of both CTAs' copies
           if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * C::STAGE_BYTES);
-          const uint32_t leader_full = map_to_cta(full_bar(stage), 0);
-          const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
           if (kb < p.num_kb) {
             tma_load_2d_pair(sa, &mapX, leader_full, kb * BK, m0);
             tma_load_2d_pair(sb, &mapW, leader_full, kb * BK, w_row);
@@ -319,46 +338,55 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
             tma_load_2d_pair(sa, &mapXe, leader_full, e * BK, m0);
             tma_load_2d_pair(sb, &mapWe, leader_full, e * BK, we_row);
           }
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok && !issue_r(true)) ok = false;
-        ++tcount;
+        __syncwarp();
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       }
+      if (ok && !issue_r(true)) ok = false;
+      ++tcount;
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer (leader only) ----------------
-    if (lane == 0 && rank == 0) {
+    // ---------------- MMA issuer (first CTA of the pair only) ----------------
+    if (rank == 0) {
+      const bool leader = elect_one();
       int stage = 0; uint32_t phase = 0;
       int as = 0; uint32_t aphase = 0;
       bool ok = true;
       const uint32_t a_lo0 = desc_lo(base);
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-        if (!mbar_wait(tempty_bar(as), aphase ^ 1u, abort_flag, p.status, 12)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty_bar(as), aphase ^ 1u, abort_flag, p.status, 12)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * BN);
         for (int kb = 0; kb < p.num_kb; ++kb) {    // four products per block, issued back to back
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status, 13)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status, 13)) { ok = false; break; }
           const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
           const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
-          tc_mma_pair_lo(d_tmem, alo, blo, C::IDESC, (uint32_t)kb);
-          tc_mma_pair_lo_acc(d_tmem, alo + 2, blo + 2, C::IDESC);
-          tc_mma_pair_lo_acc(d_tmem, alo + 4, blo + 4, C::IDESC);
-          tc_mma_pair_lo_acc(d_tmem, alo + 6, blo + 6, C::IDESC);
-          tc_commit_pair(empty_bar(stage), 3);     // frees the stage in both CTAs
+          if (leader) {
+            tc_mma_pair_lo(d_tmem, alo, blo, C::IDESC, (uint32_t)kb);
+            tc_mma_pair_lo_acc(d_tmem, alo + 2, blo + 2, C::IDESC);
+            tc_mma_pair_lo_acc(d_tmem, alo + 4, blo + 4, C::IDESC);
+            tc_mma_pair_lo_acc(d_tmem, alo + 6, blo + 6, C::IDESC);
+            tc_commit_pair(empty_bar(stage), 3);   // frees the stage in both CTAs
+          }
+          __syncwarp();
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
         for (int kb = p.num_kb; kb < kb_total && ok; ++kb) {   // rank-r extension
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status, 13)) { ok = false; break; }
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status, 13)) { ok = false; break; }
           const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
           const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
           const int nmma = kb == kb_total - 1 ? p.ext_last_mmas : BK / UMMA_K;
+          if (leader) {
 #pragma unroll 1
-          for (int k = 0; k < nmma; ++k) tc_mma_pair_lo_acc(d_tmem, alo + 2 * k, blo + 2 * k, C::IDESC);
-          tc_commit_pair(empty_bar(stage), 3);
+            for (int k = 0; k < nmma; ++k) tc_mma_pair_lo_acc(d_tmem, alo + 2 * k, blo + 2 * k, C::IDESC);
+            tc_commit_pair(empty_bar(stage), 3);
+          }
+          __syncwarp();
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        tc_commit_pair(tfull_bar(as), 3);          // accumulator halves complete in both CTAs
+        if (leader) tc_commit_pair(tfull_bar(as), 3);          // accumulator halves complete in both CTAs
+        __syncwarp();
         if (++as == 2) { as = 0; aphase ^= 1u; }
       }
     }

@@ -101,35 +101,39 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0) {
-    if (lane == 0) {
-      for (int kb = 0; kb < kblocks; ++kb) {
-        const int s = kb % LT_STAGES;
-        if (!mbar_wait(EMPTY(s), (((uint32_t)(kb / LT_STAGES)) & 1u) ^ 1u, abort_flag, p.status, 40)) break;
+  if (warp == 0) {                       // producer and issuer as converged warps (see gemm_tc.cu)
+    const bool leader = elect_one();
+    for (int kb = 0; kb < kblocks; ++kb) {
+      const int s = kb % LT_STAGES;
+      if (!mbar_wait_warp(EMPTY(s), (((uint32_t)(kb / LT_STAGES)) & 1u) ^ 1u, abort_flag, p.status, 40)) break;
+      const uint32_t dst = base + s * LT_STAGE;
+      const int row = row0 + kb * LT_K;
+      if (leader) {
         mbar_expect_tx(FULL(s), LT_STAGE);
-        const uint32_t dst = base + s * LT_STAGE;
-        const int row = row0 + kb * LT_K;
         tma_load_2d(dst, &mapZ, FULL(s), c0, row);
         tma_load_2d(dst + LT_ZBOX, &mapZ, FULL(s), c0 + 64, row);      // past the last column: zero fill
         tma_load_2d(dst + 2 * LT_ZBOX, &mapW, FULL(s), wx0, row);
       }
+      __syncwarp();
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      bool ok = true;
-      for (int kb = 0; kb < kblocks && ok; ++kb) {
-        const int s = kb % LT_STAGES;
-        if (!mbar_wait(FULL(s), ((uint32_t)(kb / LT_STAGES)) & 1u, abort_flag, p.status, 41)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t a = base + s * LT_STAGE, b = a + 2 * LT_ZBOX;
+    const bool leader = elect_one();
+    bool ok = true;
+    for (int kb = 0; kb < kblocks && ok; ++kb) {
+      const int s = kb % LT_STAGES;
+      if (!mbar_wait_warp(FULL(s), ((uint32_t)(kb / LT_STAGES)) & 1u, abort_flag, p.status, 41)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t a = base + s * LT_STAGE, b = a + 2 * LT_ZBOX;
+      if (leader) {
 #pragma unroll
         for (int k = 0; k < LT_K / UMMA_K; ++k)     // 16 tokens = two 8-row groups = 2048 bytes
           tc_mma_bf16(tmem_base, desc_mn(a + k * 2048, LT_ZBOX), desc_mn(b + k * 2048, 16), LT_IDESC,
                       (kb | k) != 0 ? 1u : 0u);
         tc_commit(EMPTY(s));
       }
-      if (ok) tc_commit(ACC);
+      __syncwarp();
     }
+    if (ok && leader) tc_commit(ACC);
   } else {
     // accumulator read-back: lane group (warp % 4) of tensor memory, one feature column per thread
     const int q = warp & 3;
