@@ -9,7 +9,7 @@
 // through a second pair of tensor maps whose rows are selected by the row group (client) of the
 // tile, so K clients with their own adapters share one pass over the frozen W.
 //
-// Two kernels:
+// Three kernels (pick_kernel chooses):
 //   gemm_tc_pair_kernel   CTA pairs (cluster of 2, tcgen05 cta_group::2): a pair owns a 256 x 256
 //                         tile; each CTA stages its 128 rows of X and one half (128 rows) of the W
 //                         tile, the leader issues 256 x 256 x 16 products that read both CTAs'
@@ -17,6 +17,8 @@
 //                         64-deep block (131 FLOP per byte from L2), 6 stages.
 //   gemm_tc_kernel<BN>    one CTA per tile of 128 x BN (BN 256 / 128 / 64): narrow outputs (the
 //                         rank-r down projections) and shapes the pair kernel does not take.
+//   gemm_tc_split_kernel  few tiles: one 128 x 64 or 128 x 128 tile per cluster of 1-8 CTAs that share the
+//                         contraction.
 //
 // Warp roles (320 threads): warp 0 = TMA producer, warp 1 = tensor-memory owner + MMA issuer,
 // warps 2..9 = epilogue (a warp reads the 32 accumulator lanes its warp id modulo 4 selects; the
@@ -42,27 +44,25 @@ constexpr int NUM_THREADS = 320;
 // ------------------------------------------------------------------------------------------
 // one CTA per tile
 // ------------------------------------------------------------------------------------------
-template <int BN, bool DEEP = false> struct Cfg {
+template <int BN> struct Cfg {
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int B_BYTES = BN * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  // BN 64 is the HBM-bound rank-r down projection: two CTAs per SM (three stages each) keep every
-  // SM streaming when the tiles do not fill whole waves of one CTA per SM.  DEEP is for the case
-  // with fewer tiles than SMs (few tokens, wide rows): then a CTA has an SM to itself and what
-  // limits it is the bytes it keeps in flight, so it takes an eight-stage ring.
-  static constexpr int CTAS_PER_SM = (BN == 64 && !DEEP) ? 2 : 1;
-  static constexpr int STAGES = BN == 64 ? (DEEP ? 8 : 3) : ((196608 / STAGE_BYTES) > 8 ? 8 : (196608 / STAGE_BYTES));
+  // BN 64 is the HBM-bound rank-r down projection with more tiles than SMs (fewer: gemm_tc_split_kernel): two
+  // CTAs per SM (three stages each) keep every SM streaming when the tiles do not fill whole waves of one CTA per SM.
+  static constexpr int CTAS_PER_SM = BN == 64 ? 2 : 1;
+  static constexpr int STAGES = BN == 64 ? 3 : ((196608 / STAGE_BYTES) > 8 ? 8 : (196608 / STAGE_BYTES));
   static constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
   static constexpr uint32_t IDESC = make_idesc(BM, BN);
 };
 
-template <int BN, bool DEEP = false>
-__global__ void __launch_bounds__(NUM_THREADS, Cfg<BN, DEEP>::CTAS_PER_SM)
+template <int BN>
+__global__ void __launch_bounds__(NUM_THREADS, Cfg<BN>::CTAS_PER_SM)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                const __grid_constant__ CUtensorMap mapXe, const __grid_constant__ CUtensorMap mapWe,
                const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapZ, TcParams p) {
-  using C = Cfg<BN, DEEP>;
+  using C = Cfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -435,6 +435,227 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// few tiles: one tile per cluster, the contraction split over its CTAs
+// ------------------------------------------------------------------------------------------
+// S CTAs (a cluster) share one 128 x BN tile: each contracts its range of 64-deep blocks into its own tensor
+// memory, then every 32 x 32 piece of the tile is added up by one of them (piece u by CTA u % S), which the
+// others have sent their fp32 partial sums to through distributed shared memory, and leaves through that CTA's
+// epilogue.  The sums are added in rank order: results do not depend on scheduling.
+// What bounds it: the few tiles of a layer over few tokens are a chain (launch, set-up, first loads, blocks one by
+// one, epilogue) rather than traffic, so the chain of blocks is cut into S.
+template <int BN, int S, int STAGES_> struct SplitCfg {
+  static constexpr int A_BYTES = BM * BK * 2;
+  static constexpr int B_BYTES = BN * BK * 2;
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int STAGES = STAGES_;
+  static constexpr int PIECES = BN / 64;                             // pieces per epilogue warp
+  static constexpr int RECV_BYTES = (8 * PIECES / S) * (S - 1) * 4096;
+  // the output staging of the epilogue takes the operand ring, which is idle once the accumulator is complete
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + RECV_BYTES + 1024 + 256;
+  static constexpr uint32_t IDESC = make_idesc(BM, BN);
+  static_assert(STAGES * STAGE_BYTES >= EPI_STAGE_BYTES && (8 * PIECES) % S == 0, "");
+};
+
+template <int BN, int S, int STAGES_>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
+gemm_tc_split_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
+                     const __grid_constant__ CUtensorMap mapXe, const __grid_constant__ CUtensorMap mapWe,
+                     const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapZ, TcParams p) {
+  using C = SplitCfg<BN, S, STAGES_>;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* base_ptr = smem_raw + (base - raw);
+  const uint32_t recv_base = base + C::STAGES * C::STAGE_BYTES;
+  const uint32_t bar_base = recv_base + C::RECV_BYTES;
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (C::STAGES + s); };
+  const uint32_t tfull_bar = bar_base + 8u * (2 * C::STAGES);
+  uint8_t* tail = base_ptr + C::STAGES * C::STAGE_BYTES + C::RECV_BYTES + 8 * (2 * C::STAGES + 1);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(tail);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tail + 8);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = S > 1 ? (int)cluster_ctarank() : 0;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+    mbar_init(tfull_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32((const void*)tmem_slot)), "r"((uint32_t)BN) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (S > 1) cluster_arrive();                       // awaited before the first store to another CTA
+  const uint32_t tmem_base = *tmem_slot;
+
+  const int kb_total = p.num_kb + p.ext_blocks;
+  const int kb0 = (int)((long long)kb_total * rank / S), kb1 = (int)((long long)kb_total * (rank + 1) / S);
+  int tm, tn;
+  tile_coords((int)blockIdx.x / S, p.tiles_m, p.tiles_n, tm, tn);
+  const int m0 = tm * BM, n0 = tn * BN;
+
+  if (warp == 0) {
+    // ---------------- TMA producer ----------------
+    const bool leader = elect_one();
+    const int g = p.rows_per_group > 0 ? m0 / p.rows_per_group : 0;
+    const int w_row = g * p.w_group_rows + n0;
+    const int we_row = g * p.we_group_rows + n0;
+    int stage = 0; uint32_t phase = 0;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 51)) break;
+      const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+      if (leader) {
+        mbar_expect_tx(full_bar(stage), C::STAGE_BYTES);
+        if (kb < p.num_kb) {
+          const int kc = (kb < p.gap_kb_begin ? kb : kb + p.gap_kb) * BK;
+          tma_load_2d(sb, &mapW, full_bar(stage), kc, w_row);
+          tma_load_2d(sa, &mapX, full_bar(stage), kc, m0);
+        } else {
+          const int e = kb - p.num_kb;
+          tma_load_2d(sb, &mapWe, full_bar(stage), e * BK, we_row);
+          tma_load_2d(sa, &mapXe, full_bar(stage), e * BK, m0);
+        }
+      }
+      __syncwarp();
+      if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    const bool leader = elect_one();
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    const uint32_t a_lo0 = desc_lo(base);
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status, 53)) { ok = false; break; }
+      const uint32_t alo = a_lo0 + (uint32_t)stage * (uint32_t)(C::STAGE_BYTES >> 4);
+      const uint32_t blo = alo + (uint32_t)(C::A_BYTES >> 4);
+      const int nmma = kb == kb_total - 1 && p.ext_blocks > 0 ? p.ext_last_mmas : BK / UMMA_K;
+      if (leader) {
+        tc_mma_lo(tmem_base, alo, blo, C::IDESC, (uint32_t)(kb - kb0));
+        if (nmma == 4) {
+          tc_mma_lo_acc(tmem_base, alo + 2, blo + 2, C::IDESC);
+          tc_mma_lo_acc(tmem_base, alo + 4, blo + 4, C::IDESC);
+          tc_mma_lo_acc(tmem_base, alo + 6, blo + 6, C::IDESC);
+        } else {
+          for (int k = 1; k < nmma; ++k) tc_mma_lo_acc(tmem_base, alo + 2 * k, blo + 2 * k, C::IDESC);
+        }
+        tc_commit(empty_bar(stage));
+      }
+      __syncwarp();
+      if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+    }
+    if (ok && leader) tc_commit(tfull_bar);
+  }
+  __syncwarp();
+
+  // ---------------- epilogue ----------------
+  const int ew = warp - 2;                           // epilogue warp 0..7
+  const int q = warp & 3, half = ew >> 2;
+  const int m_warp0 = m0 + q * 32;
+  const bool need_r = p.epi == EPI_BIAS_RESID || p.epi == EPI_MUL_GELUGRAD;
+  const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16);
+  uint4 bcur[C::PIECES][4], rcur[C::PIECES][4];
+  bool ok = false;
+  // piece j of a warp: columns n0 + half * BN/2 + 32 j; pieces are numbered u = PIECES * (4 half + q) + j
+  auto piece = [&](int j) { return C::PIECES * (half * 4 + q) + j; };
+  auto column = [&](int j) { return half * (BN / 2) + 32 * j; };
+  if (warp >= 2) {
+#pragma unroll
+    for (int j = 0; j < C::PIECES; ++j) {            // in flight while the accumulator is awaited
+      if (S > 1 && piece(j) % S != rank) continue;
+      load_bias_chunk(p, n0 + column(j), bcur[j]);
+      if (need_r) load_r_chunk(p, m_warp0 + lane, n0 + column(j), rcur[j]);
+    }
+    ok = mbar_wait(tfull_bar, 0u, abort_flag, p.status, 54);
+    tc_fence_after();
+  }
+  if constexpr (S > 1) {
+    cluster_wait();                                  // every CTA of the cluster runs: its shared memory exists
+    if (warp >= 2 && ok) {
+#pragma unroll
+      for (int j = 0; j < C::PIECES; ++j) {
+        const int u = piece(j), owner = u % S;
+        if (owner == rank || n0 + column(j) >= p.N || m_warp0 >= p.M) continue;
+        float v[32];
+        tc_ld32(t_row + (uint32_t)column(j), v);
+        tc_wait_ld();
+        // slot: the owner's (u / S)-th piece, sender number (this rank among the others)
+        const int sender = rank < owner ? rank : rank - 1;
+        const uint32_t dst = map_to_cta(recv_base + (uint32_t)(((u / S) * (S - 1) + sender) * 4096 + lane * 16), (uint32_t)owner);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(i * 512)), "f"(v[4 * i]),
+                       "f"(v[4 * i + 1]), "f"(v[4 * i + 2]), "f"(v[4 * i + 3]) : "memory");
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();
+  }
+  if (warp >= 2) {
+    if (ok) {
+      const bool tanh_form = p.gelu_tanh != 0;
+      const uint32_t stage = base + (uint32_t)ew * 4096u;   // this warp's two staging buffers, in the idle operand ring
+      int buf = 0;
+#pragma unroll
+      for (int j = 0; j < C::PIECES; ++j) {
+        const int u = piece(j), n = n0 + column(j);
+        if ((S > 1 && u % S != rank) || n >= p.N) continue;
+        float v[32];
+        tc_ld32(t_row + (uint32_t)column(j), v);
+        tc_wait_ld();
+        if constexpr (S > 1) {
+          // partial sums in rank order: the contribution of rank 0 first
+          float acc[32];
+#pragma unroll
+          for (int r = 0; r < S; ++r) {
+            if (r == rank) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) acc[i] = r == 0 ? v[i] : acc[i] + v[i];
+            } else {
+              const int sender = r < rank ? r : r - 1;
+              const uint32_t src = recv_base + (uint32_t)(((u / S) * (S - 1) + sender) * 4096 + lane * 16);
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                float x0, x1, x2, x3;
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x0), "=f"(x1), "=f"(x2), "=f"(x3) : "r"(src + (uint32_t)(i * 512)) : "memory");
+                acc[4 * i] = r == 0 ? x0 : acc[4 * i] + x0;
+                acc[4 * i + 1] = r == 0 ? x1 : acc[4 * i + 1] + x1;
+                acc[4 * i + 2] = r == 0 ? x2 : acc[4 * i + 2] + x2;
+                acc[4 * i + 3] = r == 0 ? x3 : acc[4 * i + 3] + x3;
+              }
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = acc[i];
+        }
+        epilogue_chunk(p, v, bcur[j], rcur[j], n, tanh_form, stage, buf, &mapY, &mapZ, m_warp0, lane);
+      }
+    }
+    epilogue_drain(lane);
+  }
+
+  // ---------------- teardown ----------------
+  __syncwarp();
+  if (*abort_flag) {
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)BN) : "memory");
+  }
+}
+
 // ---- host side -----------------------------------------------------------------------------
 // CTA pairs that can be resident at once, per device (0: pair kernel unavailable there)
 int g_max_pairs[MAX_DEVICES] = {};
@@ -468,6 +689,41 @@ bool pair_ok(const GemmArgs& a) {
   if (a.M <= BM || a.N < 256) return false;
   if (a.rows_per_group > 0 && a.rows_per_group % (2 * BM) != 0) return false;   // 0 when there is one group
   return a.rows_per_group > 0 || a.M % (2 * BM) == 0 || a.M % BM != 0;
+}
+
+// Which kernel takes a layer: the one with the least estimated time, from the number of rounds its CTAs need on the
+// chip, the 64-deep blocks per CTA and each kernel's measured constants (ns; CUDA graph replays over operands that
+// exceed L2, M 128-8192, K 768-4096, N 64-4096): a fixed part (launch, set-up, first loads, epilogue of the last
+// tile), the time of a block, and for the kernels that are not persistent what every further round starts with.
+// The persistent kernels fill the chip from about 60 tiles of 256 x 256 on; below that they leave SMs idle and a
+// block takes a lone CTA pair 275 ns whatever the tile.  Measured at M 512 (pair kernel -> this choice): 1024 -> 1024
+// 10.9 -> 7.0 us, 1024 -> 3072 11.3 -> 8.4, 4096 -> 1024 24.4 -> 11.8, rank-r projections from 1024 8.6 -> 6.4 and
+// (8192 tokens) from 4096 21.5 -> 16.0; 4096 tokens and more of the wide layers stay with the pair kernel
+// (1024 -> 1024: 11.6 against 17.4).
+enum Kernel { KERNEL_SINGLE, KERNEL_PAIR, KERNEL_SPLIT64_1, KERNEL_SPLIT64_2, KERNEL_SPLIT64_4, KERNEL_SPLIT64_8, KERNEL_SPLIT128_1 };
+Kernel pick_kernel(const GemmArgs& a) {
+  const int64_t sms = num_sms();
+  const int64_t kb = (a.K + BK - 1) / BK + (a.Ke + BK - 1) / BK;
+  auto cdiv = [](int64_t x, int64_t y) { return (x + y - 1) / y; };
+  Kernel best = KERNEL_SINGLE;
+  int64_t best_ns = INT64_MAX;
+  auto offer = [&](Kernel k, int64_t ns) { if (ns < best_ns) { best_ns = ns; best = k; } };
+  if (pair_ok(a)) {
+    offer(KERNEL_PAIR, 5500 + cdiv(cdiv(a.M, 2 * BM) * cdiv(a.N, 256), max_pairs()) * kb * 275);
+  } else {
+    const int bn = pick_bn(a);
+    offer(KERNEL_SINGLE, 5500 + cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), bn == 64 ? 2 * sms : sms) * kb * (bn == 64 ? 200 : 300));
+  }
+  auto split = [&](Kernel k, int bn, int s, int64_t fixed) {
+    const int64_t rounds = cdiv(cdiv(a.M, BM) * cdiv(a.N, bn) * s, sms);
+    if (s == 1 || kb >= 2 * s) offer(k, fixed + rounds * cdiv(kb, s) * 190 + (rounds - 1) * 3000);
+  };
+  split(KERNEL_SPLIT64_1, 64, 1, 3600);
+  split(KERNEL_SPLIT64_2, 64, 2, 4700);
+  split(KERNEL_SPLIT64_4, 64, 4, 5000);
+  split(KERNEL_SPLIT64_8, 64, 8, 5500);
+  split(KERNEL_SPLIT128_1, 128, 1, 4400);
+  return best;
 }
 
 // Fills the parameters both kernels share and encodes the tensor maps; box rows of the W maps differ.
@@ -506,15 +762,14 @@ bool prepare(const GemmArgs& a, int* status, int w_box_rows, CUtensorMap* mX, CU
   return true;
 }
 
-template <int BN, bool DEEP = false>
+template <int BN>
 cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
-  using C = Cfg<BN, DEEP>;
+  using C = Cfg<BN>;
   const int sms = num_sms();
-  if (BN == 64 && !DEEP && ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN) <= sms) return launch<64, true>(a, status, st);
   static PerDeviceOnce once;                    // one per instantiation; attributes are per device
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
@@ -525,8 +780,32 @@ cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
   const int tiles = p.tiles_m * p.tiles_n;
   const int slots = sms * C::CTAS_PER_SM;
   const int grid = tiles < slots ? tiles : slots;
-  gemm_tc_kernel<BN, DEEP><<<grid, NUM_THREADS, C::SMEM_BYTES, st>>>(mX, mW, mXe, mWe, mY, mZ, p);
+  gemm_tc_kernel<BN><<<grid, NUM_THREADS, C::SMEM_BYTES, st>>>(mX, mW, mXe, mWe, mY, mZ, p);
   return cudaGetLastError();
+}
+
+template <int BN, int S, int STAGES>
+cudaError_t launch_split(const GemmArgs& a, int* status, cudaStream_t st) {
+  using C = SplitCfg<BN, S, STAGES>;
+  static PerDeviceOnce once;
+  const int dev = current_device();
+  if (once.needed(dev)) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_split_kernel<BN, S, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    once.done(dev);
+  }
+  CUtensorMap mX, mW, mXe, mWe, mY, mZ;
+  TcParams p;
+  if (!prepare(a, status, BN, &mX, &mW, &mXe, &mWe, &mY, &mZ, &p)) return cudaErrorInvalidValue;
+  p.tiles_m = (a.M + BM - 1) / BM; p.tiles_n = (a.N + BN - 1) / BN;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(p.tiles_m * p.tiles_n * S)); cfg.blockDim = dim3(NUM_THREADS);
+  cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, gemm_tc_split_kernel<BN, S, STAGES>, mX, mW, mXe, mWe, mY, mZ, p);
 }
 
 cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
@@ -600,7 +879,15 @@ cudaError_t gemm_tc(const GemmArgs& args, int* status, cudaStream_t st) {
   if (!gemm_tc_supported(args)) return cudaErrorInvalidValue;
   GemmArgs a = args;
   if (a.rows_per_group >= a.M) a.rows_per_group = 0;      // one group
-  if (pair_ok(a)) return launch_pair(a, status, st);
+  switch (pick_kernel(a)) {
+    case KERNEL_SPLIT64_1: return launch_split<64, 1, 8>(a, status, st);
+    case KERNEL_SPLIT64_2: return launch_split<64, 2, 8>(a, status, st);
+    case KERNEL_SPLIT64_4: return launch_split<64, 4, 8>(a, status, st);
+    case KERNEL_SPLIT64_8: return launch_split<64, 8, 8>(a, status, st);
+    case KERNEL_SPLIT128_1: return launch_split<128, 1, 6>(a, status, st);
+    case KERNEL_PAIR: return launch_pair(a, status, st);
+    default: break;
+  }
   switch (pick_bn(a)) {
     case 256: return launch<256>(a, status, st);
     case 128: return launch<128>(a, status, st);

@@ -63,7 +63,10 @@ def test_attention_ragged_writes_inside_its_rows_only():
 
 
 @pytest.mark.parametrize("M,K,N", [(1, 8, 8), (5, 72, 264), (127, 64, 72), (129, 200, 256), (255, 768, 1000), (257, 128, 520),
-                                   (1000, 136, 256), (300, 1000, 8)])
+                                   (1000, 136, 256), (300, 1000, 8),
+                                   # few tiles: every split of the contraction, both tile widths, tails of each
+                                   (128, 4096, 64), (512, 1024, 64), (256, 512, 64), (512, 4096, 1024), (300, 584, 1000),
+                                   (1024, 1024, 1024), (512, 1024, 3072), (2000, 1032, 1000)])
 @pytest.mark.parametrize("epilogue", [B.EPI_BIAS, B.EPI_BIAS_GELU, B.EPI_BIAS_RESID, B.EPI_MUL_GELUGRAD])
 def test_linear_any_row_count_and_depth(M, K, N, epilogue):
     """Against 64 bits: no further off than the plain-FMA kernel (the products of bf16 values are exact in both and
@@ -92,7 +95,8 @@ def test_linear_any_row_count_and_depth(M, K, N, epilogue):
 
 
 @pytest.mark.parametrize("M,n_in,n_out,r,G", [(1, 64, 72, 4, 1), (77, 200, 136, 6, 1), (129, 768, 256, 1, 1), (300, 136, 768, 40, 1),
-                                              (512, 200, 1000, 8, 2), (640, 72, 72, 64, 5)])
+                                              (512, 200, 1000, 8, 2), (640, 72, 72, 64, 5),
+                                              (512, 1024, 1024, 4, 2), (256, 4096, 512, 16, 1), (1024, 1024, 1024, 40, 4)])
 def test_lora_linear_any_size(M, n_in, n_out, r, G):
     """Forward and backward against 64 bits, next to the plain-FMA kernels' errors."""
     g = torch.Generator(device="cuda").manual_seed(M + n_in)
