@@ -4,6 +4,7 @@
 // accumulations are one feature per lane with the probability broadcast by shuffle.
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 namespace {
@@ -22,6 +23,7 @@ __device__ __forceinline__ float dot_row(const float* __restrict__ a_s, const T*
 template <typename T>
 __global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restrict__ qkv, int nseq, int Tn, int H,
                                                               int d, T* __restrict__ o, float* __restrict__ lse) {
+  overlap_sync();
   __shared__ float q_s[WARPS][MAX_DH];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t w = (int64_t)blockIdx.x * WARPS + wib;
@@ -71,6 +73,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restric
 template <typename T>
 __global__ void attn_rowdot_kernel(const T* __restrict__ o, const T* __restrict__ d_o, int nseq, int Tn, int H,
                                    int d, float* __restrict__ rowdot) {
+  overlap_sync();
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= (int64_t)nseq * H * Tn) return;
@@ -88,6 +91,7 @@ template <typename T>
 __global__ void __launch_bounds__(WARPS * 32) attn_bwd_dq_kernel(const T* __restrict__ qkv, const float* __restrict__ lse,
                                                                  const T* __restrict__ d_o, const float* __restrict__ rowdot,
                                                                  int nseq, int Tn, int H, int d, T* __restrict__ dqkv) {
+  overlap_sync();
   __shared__ float q_s[WARPS][MAX_DH], do_s[WARPS][MAX_DH];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t w = (int64_t)blockIdx.x * WARPS + wib;
@@ -139,6 +143,7 @@ template <typename T>
 __global__ void __launch_bounds__(WARPS * 32) attn_bwd_dkv_kernel(const T* __restrict__ qkv, const float* __restrict__ lse,
                                                                   const T* __restrict__ d_o, const float* __restrict__ rowdot,
                                                                   int nseq, int Tn, int H, int d, T* __restrict__ dqkv) {
+  overlap_sync();
   __shared__ float k_s[WARPS][MAX_DH], v_s[WARPS][MAX_DH];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t w = (int64_t)blockIdx.x * WARPS + wib;
@@ -194,8 +199,8 @@ cudaError_t attention_fwd_simt(int dt, const void* qkv, int nseq, int T, int H, 
   if (d % H != 0 || d / H > MAX_DH) return cudaErrorInvalidValue;
   int64_t warps = (int64_t)nseq * H * T;
   unsigned blocks = (unsigned)((warps + WARPS - 1) / WARPS);
-  if (dt == DT_BF16) attn_fwd_kernel<bf16><<<blocks, WARPS * 32, 0, st>>>((const bf16*)qkv, nseq, T, H, d, (bf16*)o, lse);
-  else attn_fwd_kernel<float><<<blocks, WARPS * 32, 0, st>>>((const float*)qkv, nseq, T, H, d, (float*)o, lse);
+  if (dt == DT_BF16) launch_in_order(attn_fwd_kernel<bf16>, blocks, WARPS * 32, 0, st, (const bf16*)qkv, nseq, T, H, d, (bf16*)o, lse);
+  else launch_in_order(attn_fwd_kernel<float>, blocks, WARPS * 32, 0, st, (const float*)qkv, nseq, T, H, d, (float*)o, lse);
   return cudaGetLastError();
 }
 
@@ -206,13 +211,13 @@ cudaError_t attention_bwd_simt(int dt, const void* qkv, const void* o, const flo
   unsigned blocks = (unsigned)((warps + WARPS - 1) / WARPS);
   unsigned rb = (unsigned)((warps * 32 + 255) / 256);
   if (dt == DT_BF16) {
-    attn_rowdot_kernel<bf16><<<rb, 256, 0, st>>>((const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
-    attn_bwd_dq_kernel<bf16><<<blocks, WARPS * 32, 0, st>>>((const bf16*)qkv, lse, (const bf16*)d_o, rowdot, nseq, T, H, d, (bf16*)dqkv);
-    attn_bwd_dkv_kernel<bf16><<<blocks, WARPS * 32, 0, st>>>((const bf16*)qkv, lse, (const bf16*)d_o, rowdot, nseq, T, H, d, (bf16*)dqkv);
+    launch_in_order(attn_rowdot_kernel<bf16>, rb, 256, 0, st, (const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
+    launch_in_order(attn_bwd_dq_kernel<bf16>, blocks, WARPS * 32, 0, st, (const bf16*)qkv, lse, (const bf16*)d_o, rowdot, nseq, T, H, d, (bf16*)dqkv);
+    launch_in_order(attn_bwd_dkv_kernel<bf16>, blocks, WARPS * 32, 0, st, (const bf16*)qkv, lse, (const bf16*)d_o, rowdot, nseq, T, H, d, (bf16*)dqkv);
   } else {
-    attn_rowdot_kernel<float><<<rb, 256, 0, st>>>((const float*)o, (const float*)d_o, nseq, T, H, d, rowdot);
-    attn_bwd_dq_kernel<float><<<blocks, WARPS * 32, 0, st>>>((const float*)qkv, lse, (const float*)d_o, rowdot, nseq, T, H, d, (float*)dqkv);
-    attn_bwd_dkv_kernel<float><<<blocks, WARPS * 32, 0, st>>>((const float*)qkv, lse, (const float*)d_o, rowdot, nseq, T, H, d, (float*)dqkv);
+    launch_in_order(attn_rowdot_kernel<float>, rb, 256, 0, st, (const float*)o, (const float*)d_o, nseq, T, H, d, rowdot);
+    launch_in_order(attn_bwd_dq_kernel<float>, blocks, WARPS * 32, 0, st, (const float*)qkv, lse, (const float*)d_o, rowdot, nseq, T, H, d, (float*)dqkv);
+    launch_in_order(attn_bwd_dkv_kernel<float>, blocks, WARPS * 32, 0, st, (const float*)qkv, lse, (const float*)d_o, rowdot, nseq, T, H, d, (float*)dqkv);
   }
   return cudaGetLastError();
 }

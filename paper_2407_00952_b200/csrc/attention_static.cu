@@ -9,6 +9,7 @@
 
 #include "../../include/splitlora.h"
 #include "kernels.h"
+#include "launch.cuh"
 
 using namespace sl;
 
@@ -42,6 +43,7 @@ int scratch_address(float** out) {
 extern "C" int splitlora_attention_bwd_static(int dtype, int use_tc, const void* qkv, const void* o, const float* lse,
                                               const void* d_o, int nseq, int T, int n_head, int d_model, void* dqkv,
                                               void* stream) {
+  LaunchChain chain;
   if (!qkv || !o || !lse || !d_o || !dqkv || nseq < 1 || T < 1 || n_head < 1 || d_model % n_head != 0 ||
       d_model / n_head > 128 || (dtype != DT_F32 && dtype != DT_BF16))
     return SPLITLORA_ERR_ARG;

@@ -20,6 +20,7 @@
 // 2..5 the first half of the score and output columns, warps 6..9 the second).
 // All mbarrier waits are bounded (see tc_common.cuh); on expiry a code is left in `status`.
 #include "host_common.h"
+#include "launch.cuh"
 #include "tc_common.cuh"
 
 namespace sl {
@@ -119,6 +120,7 @@ attn_fwd_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  overlap_sync();
   const uint32_t tS = tmem_base, tO = tmem_base + 128u, tP = tmem_base + 128u + (uint32_t)DH;
 
   if (warp == 0) {
@@ -425,7 +427,7 @@ cudaError_t attention_fwd_t5(const void* qkv, int nseq, int T, int H, int d, voi
   p.status = status;
   p.nitems = nseq * H;
   const int cap = FwdCfg<128>::CTAS_PER_SM * sms;                                  // persistent CTAs
-  attn_fwd_t5_kernel<128><<<p.nitems < cap ? p.nitems : cap, T5_THREADS, FwdCfg<128>::SMEM, st>>>(mQKV, mO, p);
+  launch_overlapped(attn_fwd_t5_kernel<128>, p.nitems < cap ? p.nitems : cap, T5_THREADS, FwdCfg<128>::SMEM, st, mQKV, mO, p);
   return cudaGetLastError();
 }
 

@@ -27,6 +27,7 @@
 // contraction step ("augmented contraction" below), so the element-wise threads never read them.
 // All mbarrier waits are bounded (tc_common.cuh); on expiry a code is left in `status`.
 #include "host_common.h"
+#include "launch.cuh"
 #include "tc_common.cuh"
 
 namespace sl {
@@ -294,6 +295,7 @@ attn_bwd_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
   }
+  overlap_sync();
   const int nq = p.T / BT;
   // persistent: the work units are (item, tile) pairs, item = (sequence, head).  The grid is a multiple of
   // nq CTAs; in round t the CTAs nq*s .. nq*s + nq-1 take the nq tiles of one item (the s-th of the round's
@@ -659,6 +661,7 @@ attn_bwd_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_c
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
   }
+  overlap_sync();
   const int nq = p.T / BT;
   // persistent: the work units are (item, tile) pairs, item = (sequence, head).  The grid is a multiple of
   // nq CTAs; in round t the CTAs nq*s .. nq*s + nq-1 take the nq tiles of one item (the s-th of the round's
@@ -1022,8 +1025,8 @@ cudaError_t attention_bwd_t5(const void* qkv, const void* o, const float* lse, c
   const int nq = T / BT, units = p.nitems * nq;
   dim3 grid((unsigned)(((units < sms ? units : sms) / nq) * nq));   // one persistent CTA per SM, whole items per round
   // dQ first: it leaves D[row] = sum(dO * O) in `rowdot` for the dK/dV kernel
-  attn_bwd_dq_t5_kernel<64><<<grid, Roles<64>::NTHREADS_DQ, dq::Cfg<64>::SMEM, st>>>(mQKV, mDO, mO, mDQKV, p);
-  attn_bwd_dkv_t5_kernel<64><<<grid, Roles<64>::NTHREADS_DKV, dkv::Cfg<64>::SMEM, st>>>(mQKV, mDO, mDQKV, p);
+  launch_overlapped(attn_bwd_dq_t5_kernel<64>, grid, Roles<64>::NTHREADS_DQ, dq::Cfg<64>::SMEM, st, mQKV, mDO, mO, mDQKV, p);
+  launch_overlapped(attn_bwd_dkv_t5_kernel<64>, grid, Roles<64>::NTHREADS_DKV, dkv::Cfg<64>::SMEM, st, mQKV, mDO, mDQKV, p);
   return cudaGetLastError();
 }
 
@@ -1050,8 +1053,8 @@ cudaError_t attention_bwd_t5_128(const void* qkv, const float* lse, const void* 
   p.nitems = nseq * H;
   const int nq = T / BT, units = p.nitems * nq;
   dim3 grid((unsigned)(((units < sms ? units : sms) / nq) * nq));
-  attn_bwd_dq_t5_kernel<128><<<grid, Roles<128>::NTHREADS_DQ, dq::Cfg<128>::SMEM, st>>>(mQKV, mDO, mDO /* unused */, mDQKV, p);
-  attn_bwd_dkv_t5_kernel<128><<<grid, Roles<128>::NTHREADS_DKV, dkv::Cfg<128>::SMEM, st>>>(mQKV, mDO, mDQKV, p);
+  launch_overlapped(attn_bwd_dq_t5_kernel<128>, grid, Roles<128>::NTHREADS_DQ, dq::Cfg<128>::SMEM, st, mQKV, mDO, mDO /* unused */, mDQKV, p);
+  launch_overlapped(attn_bwd_dkv_t5_kernel<128>, grid, Roles<128>::NTHREADS_DKV, dkv::Cfg<128>::SMEM, st, mQKV, mDO, mDQKV, p);
   return cudaGetLastError();
 }
 

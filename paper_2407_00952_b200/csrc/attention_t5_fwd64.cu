@@ -19,6 +19,7 @@
 // softmax (warp w owns accumulator lanes 32*(w%4)..+31).
 // All mbarrier waits are bounded (see tc_common.cuh); on expiry a code is left in `status`.
 #include "host_common.h"
+#include "launch.cuh"
 #include "tc_common.cuh"
 
 namespace sl {
@@ -115,6 +116,7 @@ attn_fwd_t5_h64_kernel(const __grid_constant__ CUtensorMap mapQKV, F64Params p) 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  overlap_sync();
   const uint32_t tS = tmem_base, tO = tmem_base + 128u, tP = tmem_base + 192u;
 
   if (warp == 0) {
@@ -376,7 +378,7 @@ cudaError_t attention_fwd_t5_h64(const void* qkv, int nseq, int T, int H, int d,
   const int nq = T / BQ, units = p.nitems * nq, cap = 2 * sms;
   const int grid = ((units < cap ? units : cap) / nq) * nq;          // a multiple of nq: whole items per round
   if (grid < nq) return cudaErrorInvalidValue;
-  attn_fwd_t5_h64_kernel<<<grid, THREADS, SMEM, st>>>(mQKV, p);
+  launch_overlapped(attn_fwd_t5_h64_kernel, grid, THREADS, SMEM, st, mQKV, p);
   return cudaGetLastError();
 }
 

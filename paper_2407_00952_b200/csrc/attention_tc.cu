@@ -20,6 +20,7 @@
 #include "common.cuh"
 #include "host_common.h"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 namespace {
@@ -177,6 +178,7 @@ template <int DH, bool RG>
 __global__ void __launch_bounds__(NT) attn_fwd_tc_kernel(const bf16* __restrict__ qkv, bf16* __restrict__ o,
                                                          float* __restrict__ lse, int T, int H, int d, int dh,
                                                          float scale, float scale_log2) {
+  overlap_sync();
   if (!RG) dh = DH;
   constexpr int TILE_BYTES = Sizes<DH>::TILE;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -269,6 +271,7 @@ __global__ void __launch_bounds__(NT) attn_fwd_tc_kernel(const bf16* __restrict_
 template <int DH>
 __global__ void attn_rowdot_tc_kernel(const bf16* __restrict__ o, const bf16* __restrict__ d_o, int nseq, int T, int H,
                                       int d, float* __restrict__ rowdot) {
+  overlap_sync();
   constexpr int LPR = DH / 8;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t rowhead = idx / LPR;
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restri
                                                             const bf16* __restrict__ d_o, const float* __restrict__ lse,
                                                             float* __restrict__ rowdot, bf16* __restrict__ dqkv, int T,
                                                             int H, int d, int dh, float scale) {
+  overlap_sync();
   if (!RG) dh = DH;
   constexpr int TILE_BYTES = Sizes<DH>::TILE;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -402,6 +406,7 @@ __global__ void __launch_bounds__(NT) attn_bwd_dkv_tc_kernel(const bf16* __restr
                                                              const float* __restrict__ lse, const float* __restrict__ rowdot,
                                                              bf16* __restrict__ dqkv, int T, int H, int d, int dh,
                                                              float scale) {
+  overlap_sync();
   if (!RG) dh = DH;
   constexpr int TILE_BYTES = Sizes<DH>::TILE;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -499,7 +504,7 @@ cudaError_t launch_fwd(const void* qkv, int nseq, int T, int H, int d, void* o, 
   }
   const int dh = d / H;
   dim3 grid((T + BT - 1) / BT, H, nseq);
-  attn_fwd_tc_kernel<DH, RG><<<grid, NT, Sizes<DH>::FWD, st>>>((const bf16*)qkv, (bf16*)o, lse, T, H, d, dh,
+  launch_overlapped(attn_fwd_tc_kernel<DH, RG>, grid, NT, Sizes<DH>::FWD, st, (const bf16*)qkv, (bf16*)o, lse, T, H, d, dh,
                                                               1.0f / sqrtf((float)dh), LOG2E / sqrtf((float)dh));
   return cudaGetLastError();
 }
@@ -520,15 +525,15 @@ cudaError_t launch_bwd(const void* qkv, const void* o, const float* lse, const v
   const float scale = 1.0f / sqrtf((float)dh);
   if constexpr (!RG) {
     int64_t threads = (int64_t)nseq * T * H * (DH / 8);
-    attn_rowdot_tc_kernel<DH><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>((const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
+    launch_overlapped(attn_rowdot_tc_kernel<DH>, (unsigned)((threads + 255) / 256), 256, 0, st, (const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
     if (DH == 128 && attention_bwd_t5_128_supported(DT_BF16, T, H, d))
       // dQ, dK, dV on the tcgen05 kernels (they read D[row] from `rowdot`, written just above)
       return attention_bwd_t5_128(qkv, lse, d_o, rowdot, nseq, T, H, d, dqkv, status, st);
   }
   dim3 grid((T + BT - 1) / BT, H, nseq);
-  attn_bwd_dq_tc_kernel<DH, RG><<<grid, NT, Sizes<DH>::DQ, st>>>((const bf16*)qkv, (const bf16*)o, (const bf16*)d_o, lse, rowdot,
+  launch_overlapped(attn_bwd_dq_tc_kernel<DH, RG>, grid, NT, Sizes<DH>::DQ, st, (const bf16*)qkv, (const bf16*)o, (const bf16*)d_o, lse, rowdot,
                                                                 (bf16*)dqkv, T, H, d, dh, scale);
-  attn_bwd_dkv_tc_kernel<DH, RG><<<grid, NT, Sizes<DH>::DKV, st>>>((const bf16*)qkv, (const bf16*)d_o, lse, rowdot, (bf16*)dqkv,
+  launch_overlapped(attn_bwd_dkv_tc_kernel<DH, RG>, grid, NT, Sizes<DH>::DKV, st, (const bf16*)qkv, (const bf16*)d_o, lse, rowdot, (bf16*)dqkv,
                                                                   T, H, d, dh, scale);
   return cudaGetLastError();
 }

@@ -4,6 +4,7 @@
 // All global accesses are 16-byte vectors where the layout allows; reductions use warp shuffles.
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 
@@ -13,6 +14,7 @@ namespace sl {
 template <typename T>
 __global__ void embed_kernel(const int32_t* __restrict__ tok, const T* __restrict__ wte,
                              const T* __restrict__ wpe, T* __restrict__ out, int M, int Tseq, int d, int vocab) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   const int vec_per_row = d / N;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -39,9 +41,9 @@ cudaError_t embed(int dt, const int32_t* tokens, const void* wte, const void* wp
   int64_t total = (int64_t)M * (d / n);
   int blocks = (int)((total + 255) / 256);
   if (dt == DT_BF16)
-    embed_kernel<bf16><<<blocks, 256, 0, st>>>(tokens, (const bf16*)wte, (const bf16*)wpe, (bf16*)out, M, T, d, vocab);
+    launch_overlapped(embed_kernel<bf16>, blocks, 256, 0, st, tokens, (const bf16*)wte, (const bf16*)wpe, (bf16*)out, M, T, d, vocab);
   else
-    embed_kernel<float><<<blocks, 256, 0, st>>>(tokens, (const float*)wte, (const float*)wpe, (float*)out, M, T, d, vocab);
+    launch_overlapped(embed_kernel<float>, blocks, 256, 0, st, tokens, (const float*)wte, (const float*)wpe, (float*)out, M, T, d, vocab);
   return cudaGetLastError();
 }
 
@@ -52,6 +54,7 @@ template <typename T>
 __global__ void ln_fwd_kernel(const T* __restrict__ x, const T* __restrict__ g, const T* __restrict__ b,
                               T* __restrict__ y, float* __restrict__ mean, float* __restrict__ rstd, int M,
                               int d, float eps) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int row = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
@@ -86,6 +89,7 @@ template <typename T>
 __global__ void ln_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ x, const T* __restrict__ g,
                               const float* __restrict__ mean, const float* __restrict__ rstd,
                               const T* __restrict__ resid, T* __restrict__ dx, int M, int d) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int row = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
@@ -128,6 +132,7 @@ __global__ void __launch_bounds__(256) ln_fwd_reg_kernel(const T* __restrict__ x
                                                          const T* __restrict__ b, T* __restrict__ y,
                                                          float* __restrict__ mean, float* __restrict__ rstd, int M,
                                                          int d, float eps) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int row = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
@@ -166,6 +171,7 @@ __global__ void __launch_bounds__(256) ln_bwd_reg_kernel(const T* __restrict__ d
                                                          const T* __restrict__ g, const float* __restrict__ mean,
                                                          const float* __restrict__ rstd, const T* __restrict__ resid,
                                                          T* __restrict__ dx, int M, int d) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int row = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
@@ -211,17 +217,17 @@ cudaError_t layernorm_fwd(int dt, const void* x, const void* g, const void* b, v
                           int M, int d, float eps, cudaStream_t st) {
   int blocks = (M + 7) / 8;
   if (dt == DT_BF16 && d == 1024) {
-    ln_fwd_reg_kernel<bf16, 4><<<blocks, 256, 0, st>>>((const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)y, mean, rstd, M, d, eps);
+    launch_overlapped(ln_fwd_reg_kernel<bf16, 4>, blocks, 256, 0, st, (const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)y, mean, rstd, M, d, eps);
     return cudaGetLastError();
   }
   if (dt == DT_BF16 && d == 768) {
-    ln_fwd_reg_kernel<bf16, 3><<<blocks, 256, 0, st>>>((const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)y, mean, rstd, M, d, eps);
+    launch_overlapped(ln_fwd_reg_kernel<bf16, 3>, blocks, 256, 0, st, (const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)y, mean, rstd, M, d, eps);
     return cudaGetLastError();
   }
   if (dt == DT_BF16)
-    ln_fwd_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)y, mean, rstd, M, d, eps);
+    launch_overlapped(ln_fwd_kernel<bf16>, blocks, 256, 0, st, (const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)y, mean, rstd, M, d, eps);
   else
-    ln_fwd_kernel<float><<<blocks, 256, 0, st>>>((const float*)x, (const float*)g, (const float*)b, (float*)y, mean, rstd, M, d, eps);
+    launch_overlapped(ln_fwd_kernel<float>, blocks, 256, 0, st, (const float*)x, (const float*)g, (const float*)b, (float*)y, mean, rstd, M, d, eps);
   return cudaGetLastError();
 }
 
@@ -229,17 +235,17 @@ cudaError_t layernorm_bwd(int dt, const void* dy, const void* x, const void* g, 
                           const float* rstd, const void* resid, void* dx, int M, int d, cudaStream_t st) {
   int blocks = (M + 7) / 8;
   if (dt == DT_BF16 && d == 1024) {
-    ln_bwd_reg_kernel<bf16, 4><<<blocks, 256, 0, st>>>((const bf16*)dy, (const bf16*)x, (const bf16*)g, mean, rstd, (const bf16*)resid, (bf16*)dx, M, d);
+    launch_overlapped(ln_bwd_reg_kernel<bf16, 4>, blocks, 256, 0, st, (const bf16*)dy, (const bf16*)x, (const bf16*)g, mean, rstd, (const bf16*)resid, (bf16*)dx, M, d);
     return cudaGetLastError();
   }
   if (dt == DT_BF16 && d == 768) {
-    ln_bwd_reg_kernel<bf16, 3><<<blocks, 256, 0, st>>>((const bf16*)dy, (const bf16*)x, (const bf16*)g, mean, rstd, (const bf16*)resid, (bf16*)dx, M, d);
+    launch_overlapped(ln_bwd_reg_kernel<bf16, 3>, blocks, 256, 0, st, (const bf16*)dy, (const bf16*)x, (const bf16*)g, mean, rstd, (const bf16*)resid, (bf16*)dx, M, d);
     return cudaGetLastError();
   }
   if (dt == DT_BF16)
-    ln_bwd_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)dy, (const bf16*)x, (const bf16*)g, mean, rstd, (const bf16*)resid, (bf16*)dx, M, d);
+    launch_overlapped(ln_bwd_kernel<bf16>, blocks, 256, 0, st, (const bf16*)dy, (const bf16*)x, (const bf16*)g, mean, rstd, (const bf16*)resid, (bf16*)dx, M, d);
   else
-    ln_bwd_kernel<float><<<blocks, 256, 0, st>>>((const float*)dy, (const float*)x, (const float*)g, mean, rstd, (const float*)resid, (float*)dx, M, d);
+    launch_overlapped(ln_bwd_kernel<float>, blocks, 256, 0, st, (const float*)dy, (const float*)x, (const float*)g, mean, rstd, (const float*)resid, (float*)dx, M, d);
   return cudaGetLastError();
 }
 
@@ -249,6 +255,7 @@ cudaError_t layernorm_bwd(int dt, const void* dy, const void* x, const void* g, 
 // ------------------------------------------------------------------------------------------
 __global__ void count_valid_kernel(const int32_t* __restrict__ labels, int M, int V, int* __restrict__ n_valid,
                                    int normalizer_override) {
+  overlap_sync();
   if (normalizer_override > 0) {       // the batch is one shard of a larger one: use the global count
     if (threadIdx.x == 0) *n_valid = normalizer_override;
     return;
@@ -269,6 +276,7 @@ __global__ void count_valid_kernel(const int32_t* __restrict__ labels, int M, in
 template <typename T>
 __global__ void ce_kernel(T* __restrict__ logits, int64_t ld, const int32_t* __restrict__ labels, int V,
                           float* __restrict__ row_loss, const int* __restrict__ n_valid) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   __shared__ float sh_m[32], sh_s[32];
   __shared__ float sh_lse;
@@ -357,6 +365,7 @@ __device__ __forceinline__ float ce_ex2(float x) {
 __global__ void __launch_bounds__(256)
 ce_bf16_kernel(bf16* __restrict__ logits, int64_t ld, const int32_t* __restrict__ labels, int V,
                float* __restrict__ row_loss, const int* __restrict__ n_valid) {
+  overlap_sync();
   __shared__ float sh_m[32], sh_s[32];
   __shared__ float sh_lse, sh_zy;
   const float L = 1.4426950408889634f;
@@ -443,6 +452,7 @@ ce_bf16_kernel(bf16* __restrict__ logits, int64_t ld, const int32_t* __restrict_
 
 __global__ void loss_reduce_kernel(const float* __restrict__ row_loss, int M, const int* __restrict__ n_valid,
                                    float* __restrict__ loss) {
+  overlap_sync();
   __shared__ double sh[32];
   double s = 0.0;
   for (int i = threadIdx.x; i < M; i += blockDim.x) s += (double)row_loss[i];
@@ -459,12 +469,12 @@ __global__ void loss_reduce_kernel(const float* __restrict__ row_loss, int M, co
 
 cudaError_t cross_entropy(int dt, void* logits, int64_t ld, const int32_t* labels, int M, int V, float* row_loss,
                           int* n_valid, float* loss, int normalizer_override, cudaStream_t st) {
-  count_valid_kernel<<<1, 1024, 0, st>>>(labels, M, V, n_valid, normalizer_override);
+  launch_overlapped(count_valid_kernel, 1, 1024, 0, st, labels, M, V, n_valid, normalizer_override);
   if (dt == DT_BF16 && ld % 8 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0)
-    ce_bf16_kernel<<<M, 256, 0, st>>>((bf16*)logits, ld, labels, V, row_loss, n_valid);
-  else if (dt == DT_BF16) ce_kernel<bf16><<<M, 256, 0, st>>>((bf16*)logits, ld, labels, V, row_loss, n_valid);
-  else ce_kernel<float><<<M, 256, 0, st>>>((float*)logits, ld, labels, V, row_loss, n_valid);
-  loss_reduce_kernel<<<1, 1024, 0, st>>>(row_loss, M, n_valid, loss);
+    launch_overlapped(ce_bf16_kernel, M, 256, 0, st, (bf16*)logits, ld, labels, V, row_loss, n_valid);
+  else if (dt == DT_BF16) launch_overlapped(ce_kernel<bf16>, M, 256, 0, st, (bf16*)logits, ld, labels, V, row_loss, n_valid);
+  else launch_overlapped(ce_kernel<float>, M, 256, 0, st, (float*)logits, ld, labels, V, row_loss, n_valid);
+  launch_overlapped(loss_reduce_kernel, 1, 1024, 0, st, row_loss, M, n_valid, loss);
   return cudaGetLastError();
 }
 
@@ -473,6 +483,7 @@ cudaError_t cross_entropy(int dt, void* logits, int64_t ld, const int32_t* label
 // ------------------------------------------------------------------------------------------
 __global__ void optimizer_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                                  float* __restrict__ v, int64_t n4, OptArgs o) {
+  overlap_sync();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n4) return;
   float4 pv = reinterpret_cast<float4*>(p)[i];
@@ -506,7 +517,7 @@ cudaError_t optimizer_step(float* p, const float* g, float* m, float* v, int64_t
   if (n % 4 != 0) return cudaErrorInvalidValue;
   if (n == 0) return cudaSuccess;     // a side without adapters (all blocks on the clients)
   int64_t n4 = n / 4;
-  optimizer_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(p, g, m, v, n4, o);
+  launch_overlapped(optimizer_kernel, (unsigned)((n4 + 255) / 256), 256, 0, st, p, g, m, v, n4, o);
   return cudaGetLastError();
 }
 
@@ -518,6 +529,7 @@ struct AggWeights { float w[AGG_MAX_CLIENTS]; };
 
 __global__ void __launch_bounds__(256) aggregate_kernel(float* __restrict__ params, int K, int64_t P4, int64_t S4,
                                                         AggWeights w) {
+  overlap_sync();
   // P4: float4s averaged per client, S4: float4s between two clients' rows (S4 >= P4)
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P4; i += stride) {
@@ -538,6 +550,7 @@ __global__ void __launch_bounds__(256) aggregate_kernel(float* __restrict__ para
 // afterwards written to every local client's row (the downlink of step b3).
 __global__ void __launch_bounds__(256) weighted_sum_kernel(const float* __restrict__ params, int K, int64_t P4,
                                                            AggWeights w, float* __restrict__ sum) {
+  overlap_sync();
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P4; i += stride) {
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -553,6 +566,7 @@ __global__ void __launch_bounds__(256) weighted_sum_kernel(const float* __restri
 }
 __global__ void __launch_bounds__(256) broadcast_rows_kernel(const float* __restrict__ sum, int K, int64_t P4,
                                                              float* __restrict__ params) {
+  overlap_sync();
   int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P4; i += stride) {
     const float4 v = reinterpret_cast<const float4*>(sum)[i];
@@ -566,6 +580,7 @@ __global__ void __launch_bounds__(256) broadcast_rows_kernel(const float* __rest
 // (rows of A, columns of B), e.g. after the average of Eq. 8-9 has been written back to everyone.
 struct ClientRanks { int r[AGG_MAX_CLIENTS]; };
 __global__ void rank_mask_kernel(float* __restrict__ p, int64_t n, int64_t P, int r, int d, ClientRanks ranks) {
+  overlap_sync();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n) return;
   const int client = (int)(e / P);
@@ -579,7 +594,7 @@ cudaError_t rank_mask(float* params, int K, int64_t P, int r, int d, const int* 
   ClientRanks ranks;
   for (int k = 0; k < AGG_MAX_CLIENTS; ++k) ranks.r[k] = k < K ? ranks_host[k] : r;
   const int64_t n = (int64_t)K * P;
-  rank_mask_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(params, n, P, r, d, ranks);
+  launch_overlapped(rank_mask_kernel, (unsigned)((n + 255) / 256), 256, 0, st, params, n, P, r, d, ranks);
   return cudaGetLastError();
 }
 
@@ -593,7 +608,7 @@ cudaError_t aggregate(float* params, int K, int64_t P, const float* w_host, cuda
   const int64_t cap = 148 * 8;      // a few resident blocks per SM, grid-stride beyond that
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  aggregate_kernel<<<(unsigned)blocks, 256, 0, st>>>(params, K, P4, row_stride / 4, w);
+  launch_overlapped(aggregate_kernel, (unsigned)blocks, 256, 0, st, params, K, P4, row_stride / 4, w);
   return cudaGetLastError();
 }
 
@@ -608,13 +623,13 @@ cudaError_t aggregate_local_sum(const float* params, int K, int64_t P, const flo
   if (K < 1 || K > AGG_MAX_CLIENTS || P % 4 != 0) return cudaErrorInvalidValue;
   AggWeights w;
   for (int k = 0; k < AGG_MAX_CLIENTS; ++k) w.w[k] = k < K ? w_host[k] : 0.f;
-  weighted_sum_kernel<<<agg_blocks(P / 4), 256, 0, st>>>(params, K, P / 4, w, sum);
+  launch_overlapped(weighted_sum_kernel, agg_blocks(P / 4), 256, 0, st, params, K, P / 4, w, sum);
   return cudaGetLastError();
 }
 
 cudaError_t aggregate_broadcast(const float* sum, int K, int64_t P, float* params, cudaStream_t st) {
   if (K < 1 || K > AGG_MAX_CLIENTS || P % 4 != 0) return cudaErrorInvalidValue;
-  broadcast_rows_kernel<<<agg_blocks(P / 4), 256, 0, st>>>(sum, K, P / 4, params);
+  launch_overlapped(broadcast_rows_kernel, agg_blocks(P / 4), 256, 0, st, sum, K, P / 4, params);
   return cudaGetLastError();
 }
 
@@ -623,6 +638,7 @@ cudaError_t aggregate_broadcast(const float* sum, int K, int64_t P, float* param
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void adapter_copy_kernel(AdapterCopyArgs a) {
+  overlap_sync();
   const int64_t nA = (int64_t)a.r * a.d_in, nB = (int64_t)a.r * a.d_out;
   const int64_t per_t = nA + nB;
   const int64_t total = (int64_t)a.G * a.n_targets * per_t;
@@ -656,8 +672,8 @@ cudaError_t refresh_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st) {
   int64_t total = (int64_t)a.G * a.n_targets * a.r * ((int64_t)a.d_in + a.d_out);
   if (total == 0) return cudaSuccess;
   unsigned blocks = (unsigned)((total + 255) / 256);
-  if (a.dtype == DT_BF16) adapter_copy_kernel<bf16><<<blocks, 256, 0, st>>>(a);
-  else adapter_copy_kernel<float><<<blocks, 256, 0, st>>>(a);
+  if (a.dtype == DT_BF16) launch_overlapped(adapter_copy_kernel<bf16>, blocks, 256, 0, st, a);
+  else launch_overlapped(adapter_copy_kernel<float>, blocks, 256, 0, st, a);
   return cudaGetLastError();
 }
 
@@ -666,6 +682,7 @@ cudaError_t refresh_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st) {
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void transpose_kernel(const T* __restrict__ in, int rows, int cols, T* __restrict__ out, int64_t ldo) {
+  overlap_sync();
   __shared__ T tile[32][33];
   int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -681,8 +698,8 @@ __global__ void transpose_kernel(const T* __restrict__ in, int rows, int cols, T
 
 cudaError_t transpose(int dt, const void* in, int rows, int cols, void* out, int64_t ldo, cudaStream_t st) {
   dim3 grid((cols + 31) / 32, (rows + 31) / 32), block(32, 8);
-  if (dt == DT_BF16) transpose_kernel<bf16><<<grid, block, 0, st>>>((const bf16*)in, rows, cols, (bf16*)out, ldo);
-  else transpose_kernel<float><<<grid, block, 0, st>>>((const float*)in, rows, cols, (float*)out, ldo);
+  if (dt == DT_BF16) launch_overlapped(transpose_kernel<bf16>, grid, block, 0, st, (const bf16*)in, rows, cols, (bf16*)out, ldo);
+  else launch_overlapped(transpose_kernel<float>, grid, block, 0, st, (const float*)in, rows, cols, (float*)out, ldo);
   return cudaGetLastError();
 }
 

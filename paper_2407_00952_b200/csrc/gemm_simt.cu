@@ -2,6 +2,7 @@
 // It is the arithmetic of the fp32 configuration and a second opinion for the tensor-core kernel.
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 
@@ -10,6 +11,7 @@ constexpr int BM = 64, BN = 64, BK = 16;
 
 template <typename T>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs a) {
+  overlap_sync();
   __shared__ float As[BK][BM + 4];
   __shared__ float Bs[BK][BN + 4];
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -93,8 +95,8 @@ cudaError_t gemm_simt(const GemmArgs& a, cudaStream_t st) {
   if (a.rows_per_group > 0 && (a.rows_per_group % BM) != 0 && (a.w_grouped || a.we_grouped))
     return cudaErrorInvalidValue;
   dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM);
-  if (a.dtype == DT_BF16) gemm_simt_kernel<bf16><<<grid, 256, 0, st>>>(a);
-  else gemm_simt_kernel<float><<<grid, 256, 0, st>>>(a);
+  if (a.dtype == DT_BF16) launch_in_order(gemm_simt_kernel<bf16>, grid, 256, 0, st, a);
+  else launch_in_order(gemm_simt_kernel<float>, grid, 256, 0, st, a);
   return cudaGetLastError();
 }
 

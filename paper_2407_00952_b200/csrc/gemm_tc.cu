@@ -32,6 +32,7 @@
 // Every wait on an mbarrier is bounded: when it expires the kernel records a code in `status`,
 // stops issuing work, waits briefly for copies in flight, frees its tensor memory and returns.
 #include "host_common.h"
+#include "launch.cuh"
 #include "tc_common.cuh"
 
 namespace sl {
@@ -96,6 +97,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  overlap_sync();
 
   const int num_tiles = p.tiles_m * p.tiles_n;
   const int kb_total = p.num_kb + p.ext_blocks;
@@ -287,6 +289,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
   cluster_sync_all();                                // the partner's barriers are initialised too
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  overlap_sync();
 
   const int num_tiles = p.tiles_m * p.tiles_n;       // tiles of 256 x 256
   const int kb_total = p.num_kb + p.ext_blocks;
@@ -496,6 +499,7 @@ gemm_tc_split_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
   tc_fence_after();
   if (S > 1) cluster_arrive();                       // awaited before the first store to another CTA
   const uint32_t tmem_base = *tmem_slot;
+  overlap_sync();
 
   const int kb_total = p.num_kb + p.ext_blocks;
   const int kb0 = (int)((long long)kb_total * rank / S), kb1 = (int)((long long)kb_total * (rank + 1) / S);
@@ -780,7 +784,7 @@ cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
   const int tiles = p.tiles_m * p.tiles_n;
   const int slots = sms * C::CTAS_PER_SM;
   const int grid = tiles < slots ? tiles : slots;
-  gemm_tc_kernel<BN><<<grid, NUM_THREADS, C::SMEM_BYTES, st>>>(mX, mW, mXe, mWe, mY, mZ, p);
+  launch_overlapped(gemm_tc_kernel<BN>, grid, NUM_THREADS, C::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, p);
   return cudaGetLastError();
 }
 
@@ -801,10 +805,10 @@ cudaError_t launch_split(const GemmArgs& a, int* status, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.tiles_m * p.tiles_n * S)); cfg.blockDim = dim3(NUM_THREADS);
   cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  cfg.attrs = at; cfg.numAttrs = chain_attribute(at, 1);
   return cudaLaunchKernelEx(&cfg, gemm_tc_split_kernel<BN, S, STAGES>, mX, mW, mXe, mWe, mY, mZ, p);
 }
 
@@ -819,10 +823,10 @@ cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
   const bool need_r = a.epi == EPI_BIAS_RESID || a.epi == EPI_MUL_GELUGRAD;
   if (need_r) {
     if (!make_map(&mR, a.R, a.M, a.N, a.ldr, BM)) return cudaErrorInvalidValue;
-    gemm_tc_pair_kernel<true><<<2 * pairs, NUM_THREADS, PairCfg<true>::SMEM_BYTES, st>>>(mX, mW, mXe, mWe, mY, mZ, mR, p);
+    launch_overlapped(gemm_tc_pair_kernel<true>, 2 * pairs, NUM_THREADS, PairCfg<true>::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
   } else {
     mR = mY;
-    gemm_tc_pair_kernel<false><<<2 * pairs, NUM_THREADS, PairCfg<false>::SMEM_BYTES, st>>>(mX, mW, mXe, mWe, mY, mZ, mR, p);
+    launch_overlapped(gemm_tc_pair_kernel<false>, 2 * pairs, NUM_THREADS, PairCfg<false>::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
   }
   return cudaGetLastError();
 }

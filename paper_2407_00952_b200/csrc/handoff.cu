@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 namespace {
@@ -33,6 +34,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 handoff_quantize_kernel(const T* __restrict__ x, int64_t M, int d, uint8_t* __restrict__ codes,
                         float* __restrict__ scales) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -64,6 +66,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 handoff_dequantize_kernel(const uint8_t* __restrict__ codes, const float* __restrict__ scales, int64_t M, int d,
                           T* __restrict__ y) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -90,16 +93,16 @@ handoff_dequantize_kernel(const uint8_t* __restrict__ codes, const float* __rest
 
 cudaError_t handoff_quantize(int dt, const void* x, int64_t M, int d, uint8_t* codes, float* scales, cudaStream_t st) {
   const unsigned blocks = (unsigned)((M + 7) / 8);
-  if (dt == DT_BF16) handoff_quantize_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)x, M, d, codes, scales);
-  else handoff_quantize_kernel<float><<<blocks, 256, 0, st>>>((const float*)x, M, d, codes, scales);
+  if (dt == DT_BF16) launch_overlapped(handoff_quantize_kernel<bf16>, blocks, 256, 0, st, (const bf16*)x, M, d, codes, scales);
+  else launch_overlapped(handoff_quantize_kernel<float>, blocks, 256, 0, st, (const float*)x, M, d, codes, scales);
   return cudaGetLastError();
 }
 
 cudaError_t handoff_dequantize(int dt, const uint8_t* codes, const float* scales, int64_t M, int d, void* y,
                                cudaStream_t st) {
   const unsigned blocks = (unsigned)((M + 7) / 8);
-  if (dt == DT_BF16) handoff_dequantize_kernel<bf16><<<blocks, 256, 0, st>>>(codes, scales, M, d, (bf16*)y);
-  else handoff_dequantize_kernel<float><<<blocks, 256, 0, st>>>(codes, scales, M, d, (float*)y);
+  if (dt == DT_BF16) launch_overlapped(handoff_dequantize_kernel<bf16>, blocks, 256, 0, st, codes, scales, M, d, (bf16*)y);
+  else launch_overlapped(handoff_dequantize_kernel<float>, blocks, 256, 0, st, codes, scales, M, d, (float*)y);
   return cudaGetLastError();
 }
 

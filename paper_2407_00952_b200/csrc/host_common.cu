@@ -1,11 +1,14 @@
 // Host-side state shared by the launchers (see host_common.h).
 #include "host_common.h"
+#include "launch.cuh"
 
 #include <cstring>
 #include <mutex>
 #include <unordered_map>
 
 namespace sl {
+
+thread_local bool t_in_chain = false;
 
 namespace {
 

@@ -5,6 +5,7 @@
 // t * theta^(-2j/dh); act = silu(gate) * up.
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 namespace {
@@ -26,6 +27,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(NORM_THREADS) rms_fwd_kernel(const T* __restrict__ x, const T* __restrict__ g,
                                                                T* __restrict__ y, float* __restrict__ rstd, int d,
                                                                float eps) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   __shared__ float sh[4];
   const size_t off = (size_t)blockIdx.x * d;
@@ -78,6 +80,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(NORM_THREADS) rms_bwd_kernel(const T* __restrict__ dy, const T* __restrict__ x,
                                                                const T* __restrict__ g, const float* __restrict__ rstd,
                                                                const T* __restrict__ resid, T* __restrict__ dx, int d) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   __shared__ float sh[4];
   const size_t off = (size_t)blockIdx.x * d;
@@ -146,10 +149,10 @@ template <typename T>
 cudaError_t rms_fwd_t(const void* x, const void* g, void* y, float* rstd, int M, int d, float eps, cudaStream_t st) {
   const int need = (d / Vec16<T>::N + NORM_THREADS - 1) / NORM_THREADS;
   const T *xp = (const T*)x, *gp = (const T*)g; T* yp = (T*)y;
-  if (need <= 1) rms_fwd_kernel<T, 1><<<M, NORM_THREADS, 0, st>>>(xp, gp, yp, rstd, d, eps);
-  else if (need <= 2) rms_fwd_kernel<T, 2><<<M, NORM_THREADS, 0, st>>>(xp, gp, yp, rstd, d, eps);
-  else if (need <= 4) rms_fwd_kernel<T, 4><<<M, NORM_THREADS, 0, st>>>(xp, gp, yp, rstd, d, eps);
-  else rms_fwd_kernel<T, 0><<<M, NORM_THREADS, 0, st>>>(xp, gp, yp, rstd, d, eps);
+  if (need <= 1) launch_overlapped(rms_fwd_kernel<T, 1>, M, NORM_THREADS, 0, st, xp, gp, yp, rstd, d, eps);
+  else if (need <= 2) launch_overlapped(rms_fwd_kernel<T, 2>, M, NORM_THREADS, 0, st, xp, gp, yp, rstd, d, eps);
+  else if (need <= 4) launch_overlapped(rms_fwd_kernel<T, 4>, M, NORM_THREADS, 0, st, xp, gp, yp, rstd, d, eps);
+  else launch_overlapped(rms_fwd_kernel<T, 0>, M, NORM_THREADS, 0, st, xp, gp, yp, rstd, d, eps);
   return cudaGetLastError();
 }
 
@@ -158,10 +161,10 @@ cudaError_t rms_bwd_t(const void* dy, const void* x, const void* g, const float*
                       int M, int d, cudaStream_t st) {
   const int need = (d / Vec16<T>::N + NORM_THREADS - 1) / NORM_THREADS;
   const T *dyp = (const T*)dy, *xp = (const T*)x, *gp = (const T*)g, *rp = (const T*)resid; T* dxp = (T*)dx;
-  if (need <= 1) rms_bwd_kernel<T, 1><<<M, NORM_THREADS, 0, st>>>(dyp, xp, gp, rstd, rp, dxp, d);
-  else if (need <= 2) rms_bwd_kernel<T, 2><<<M, NORM_THREADS, 0, st>>>(dyp, xp, gp, rstd, rp, dxp, d);
-  else if (need <= 4) rms_bwd_kernel<T, 4><<<M, NORM_THREADS, 0, st>>>(dyp, xp, gp, rstd, rp, dxp, d);
-  else rms_bwd_kernel<T, 0><<<M, NORM_THREADS, 0, st>>>(dyp, xp, gp, rstd, rp, dxp, d);
+  if (need <= 1) launch_overlapped(rms_bwd_kernel<T, 1>, M, NORM_THREADS, 0, st, dyp, xp, gp, rstd, rp, dxp, d);
+  else if (need <= 2) launch_overlapped(rms_bwd_kernel<T, 2>, M, NORM_THREADS, 0, st, dyp, xp, gp, rstd, rp, dxp, d);
+  else if (need <= 4) launch_overlapped(rms_bwd_kernel<T, 4>, M, NORM_THREADS, 0, st, dyp, xp, gp, rstd, rp, dxp, d);
+  else launch_overlapped(rms_bwd_kernel<T, 0>, M, NORM_THREADS, 0, st, dyp, xp, gp, rstd, rp, dxp, d);
   return cudaGetLastError();
 }
 
@@ -174,6 +177,7 @@ cudaError_t rms_bwd_t(const void* dy, const void* x, const void* g, const float*
 template <typename T>
 __global__ void rope_kernel(T* __restrict__ qkv, const float2* __restrict__ table, int64_t total, int Tseq, int H,
                             int d, int half, float sign) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -203,6 +207,7 @@ __device__ __forceinline__ float sigmoid_f(float z) { return 1.0f / (1.0f + __ex
 // z [M, 2F]: columns [0, F) gate, [F, 2F) up.  act [M, F] = silu(gate) * up
 template <typename T>
 __global__ void swiglu_fwd_kernel(const T* __restrict__ z, T* __restrict__ act, int64_t total, int F) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -220,6 +225,7 @@ __global__ void swiglu_fwd_kernel(const T* __restrict__ z, T* __restrict__ act, 
 template <typename T>
 __global__ void swiglu_bwd_kernel(const T* __restrict__ dact, const T* __restrict__ z, T* __restrict__ dz,
                                   int64_t total, int F) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= total) return;
@@ -257,9 +263,9 @@ cudaError_t rope_inplace(int dt, void* qkv, const float* table, int M, int T, in
   const int64_t total = (int64_t)M * 2 * H * (half / n);
   const unsigned blocks = (unsigned)((total + 255) / 256);
   if (dt == DT_BF16)
-    rope_kernel<bf16><<<blocks, 256, 0, st>>>((bf16*)qkv, (const float2*)table, total, T, H, d, half, sign);
+    launch_overlapped(rope_kernel<bf16>, blocks, 256, 0, st, (bf16*)qkv, (const float2*)table, total, T, H, d, half, sign);
   else
-    rope_kernel<float><<<blocks, 256, 0, st>>>((float*)qkv, (const float2*)table, total, T, H, d, half, sign);
+    launch_overlapped(rope_kernel<float>, blocks, 256, 0, st, (float*)qkv, (const float2*)table, total, T, H, d, half, sign);
   return cudaGetLastError();
 }
 
@@ -267,8 +273,8 @@ cudaError_t swiglu_fwd(int dt, const void* z, void* act, int M, int F, cudaStrea
   const int n = dt == DT_BF16 ? 8 : 4;
   const int64_t total = (int64_t)M * (F / n);
   const unsigned blocks = (unsigned)((total + 255) / 256);
-  if (dt == DT_BF16) swiglu_fwd_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)z, (bf16*)act, total, F);
-  else swiglu_fwd_kernel<float><<<blocks, 256, 0, st>>>((const float*)z, (float*)act, total, F);
+  if (dt == DT_BF16) launch_overlapped(swiglu_fwd_kernel<bf16>, blocks, 256, 0, st, (const bf16*)z, (bf16*)act, total, F);
+  else launch_overlapped(swiglu_fwd_kernel<float>, blocks, 256, 0, st, (const float*)z, (float*)act, total, F);
   return cudaGetLastError();
 }
 
@@ -276,8 +282,8 @@ cudaError_t swiglu_bwd(int dt, const void* dact, const void* z, void* dz, int M,
   const int n = dt == DT_BF16 ? 8 : 4;
   const int64_t total = (int64_t)M * (F / n);
   const unsigned blocks = (unsigned)((total + 255) / 256);
-  if (dt == DT_BF16) swiglu_bwd_kernel<bf16><<<blocks, 256, 0, st>>>((const bf16*)dact, (const bf16*)z, (bf16*)dz, total, F);
-  else swiglu_bwd_kernel<float><<<blocks, 256, 0, st>>>((const float*)dact, (const float*)z, (float*)dz, total, F);
+  if (dt == DT_BF16) launch_overlapped(swiglu_bwd_kernel<bf16>, blocks, 256, 0, st, (const bf16*)dact, (const bf16*)z, (bf16*)dz, total, F);
+  else launch_overlapped(swiglu_bwd_kernel<float>, blocks, 256, 0, st, (const float*)dact, (const float*)z, (float*)dz, total, F);
   return cudaGetLastError();
 }
 

@@ -7,6 +7,7 @@
 // them in chunk order (no float atomics, so the result does not depend on scheduling).
 #include "common.cuh"
 #include "kernels.h"
+#include "launch.cuh"
 
 namespace sl {
 namespace {
@@ -33,6 +34,7 @@ template <typename T, bool VEC4>
 __global__ void __launch_bounds__(LG_CT * LG_RL, 4)
 lora_grad_partial_kernel(const T* __restrict__ Z, int64_t ldz, int zcol0, int C, const T* __restrict__ Wt,
                          int64_t ldwt, int wcol0, int r, int rp, int R, int M, float* __restrict__ partial) {
+  overlap_sync();
   constexpr int N = Vec16<T>::N;
   __shared__ float red[RJ * N][LG_CT];
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(RED_THREADS)
 lora_grad_reduce_kernel(const float* __restrict__ partial, int r, int R, int C, int chunks_per_group, float scale,
                         float* __restrict__ out, int64_t out_group_stride, int64_t out_target_stride,
                         int64_t out_sj, int64_t out_sc) {
+  overlap_sync();
   const int idx = blockIdx.x * RED_THREADS + threadIdx.x;   // over R*C
   const int g = blockIdx.y;
   if (idx >= R * C) return;
@@ -130,6 +133,7 @@ __global__ void __launch_bounds__(32 * RED_LANES)
 lora_grad_reduce_lanes_kernel(const float* __restrict__ partial, int r, int R, int C, int chunks_per_group, float scale,
                         float* __restrict__ out, int64_t out_group_stride, int64_t out_target_stride,
                         int64_t out_sj, int64_t out_sc) {
+  overlap_sync();
   __shared__ float red[RED_LANES][32];
   const int idx = blockIdx.x * 32 + threadIdx.x;   // over R*C
   const int g = blockIdx.y;
@@ -156,6 +160,7 @@ struct RedJob { const float* partial; float* out; int r, R; float scale; int64_t
 struct RedBatch { RedJob j[4]; };
 __global__ void __launch_bounds__(RED_THREADS)
 lora_grad_reduce_batch_kernel(RedBatch b, int C, int chunks_per_group) {
+  overlap_sync();
   const RedJob& jb = b.j[blockIdx.z];
   const int idx = blockIdx.x * RED_THREADS + threadIdx.x;   // over R*C
   const int g = blockIdx.y;
@@ -174,10 +179,10 @@ void launch_reduce(const float* partial, int r, int R, int C, int cpg, int group
                    int64_t out_group_stride, int64_t out_target_stride, int64_t out_sj, int64_t out_sc, cudaStream_t st) {
   if ((int64_t)R * C >= 32768) {
     dim3 g2((R * C + RED_THREADS - 1) / RED_THREADS, groups), b2(RED_THREADS);
-    lora_grad_reduce_kernel<<<g2, b2, 0, st>>>(partial, r, R, C, cpg, scale, out, out_group_stride, out_target_stride, out_sj, out_sc);
+    launch_overlapped(lora_grad_reduce_kernel, g2, b2, 0, st, partial, r, R, C, cpg, scale, out, out_group_stride, out_target_stride, out_sj, out_sc);
   } else {
     dim3 g2((R * C + 31) / 32, groups), b2(32, RED_LANES);
-    lora_grad_reduce_lanes_kernel<<<g2, b2, 0, st>>>(partial, r, R, C, cpg, scale, out, out_group_stride, out_target_stride, out_sj, out_sc);
+    launch_overlapped(lora_grad_reduce_lanes_kernel, g2, b2, 0, st, partial, r, R, C, cpg, scale, out, out_group_stride, out_target_stride, out_sj, out_sc);
   }
 }
 
@@ -186,9 +191,9 @@ void launch_partial(dim3 grid, cudaStream_t st, bool vec4, const void* Z, int64_
                     int64_t ldwt, int wcol0, int r, int rp, int R, int M, float* partial) {
   dim3 block(LG_CT, LG_RL);
   if (vec4)
-    lora_grad_partial_kernel<T, true><<<grid, block, 0, st>>>((const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+    launch_in_order(lora_grad_partial_kernel<T, true>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
   else
-    lora_grad_partial_kernel<T, false><<<grid, block, 0, st>>>((const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+    launch_in_order(lora_grad_partial_kernel<T, false>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
 }
 
 }  // namespace
@@ -268,7 +273,7 @@ cudaError_t lora_grad_batch(int dt, const LoraGradJob* jobs, int njobs, int M, i
         if (j < njobs && jb.nt * jb.r * jb.C > maxRC) maxRC = jb.nt * jb.r * jb.C;
       }
       dim3 g2((maxRC + RED_THREADS - 1) / RED_THREADS, groups, njobs);
-      lora_grad_reduce_batch_kernel<<<g2, RED_THREADS, 0, st>>>(rb, jobs[0].C, cpg);
+      launch_overlapped(lora_grad_reduce_batch_kernel, g2, RED_THREADS, 0, st, rb, jobs[0].C, cpg);
       return cudaGetLastError();
     }
     if (e != cudaErrorInvalidValue) return e;      // invalid value: the scratch does not hold the batch, go one by one

@@ -13,6 +13,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "host_common.h"
+#include "launch.cuh"
 #include "tc_common.cuh"
 
 namespace sl {
@@ -100,6 +101,7 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  overlap_sync();
 
   if (warp == 0) {                       // producer and issuer as converged warps (see gemm_tc.cu)
     const bool leader = elect_one();
@@ -251,7 +253,7 @@ cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M
   if (off > partial_floats) return cudaErrorInvalidValue;
   for (int j = njobs; j < LT_MAX_JOBS; ++j) { bt.mapZ[j] = bt.mapZ[0]; bt.mapW[j] = bt.mapW[0]; bt.p[j] = bt.p[0]; bt.wx0[j] = bt.wx0[0]; }
   dim3 grid(ctiles, groups * s, njobs);
-  lora_grad_tc_kernel<<<grid, LT_THREADS, LT_SMEM, st>>>(bt);
+  launch_overlapped(lora_grad_tc_kernel, grid, LT_THREADS, LT_SMEM, st, bt);
   *chunks_per_group = s;
   return cudaGetLastError();
 }

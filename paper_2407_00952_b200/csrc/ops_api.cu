@@ -6,6 +6,7 @@
 #include "../../include/splitlora.h"
 #include "host_common.h"
 #include "kernels.h"
+#include "launch.cuh"
 
 using namespace sl;
 
@@ -83,12 +84,14 @@ static int make_copies(int dtype, const LinearPlan& p, const float* A, const flo
     if (cudaMemsetAsync(ws + p.off_bextT, 0, (size_t)G * n_out * p.ext * es, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   }
   if (cudaMemsetAsync(ws + p.off_status, 0, 256, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
+  break_chain();
   return refresh_adapter_copies(a, st) == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;
 }
 
 int splitlora_lora_linear_fwd(int dtype, int use_tc, const void* x, const void* W, const void* bias, const float* A,
                               const float* B, float alpha, int M, int n_in, int n_out, int r, int G, void* y,
                               void* workspace, size_t workspace_bytes, void* stream) {
+  LaunchChain chain;
   return splitlora_lora_linear_fwd_parts(dtype, use_tc, x, W, bias, A, B, alpha, M, n_in, n_out, r, G, y, workspace,
                                          workspace_bytes, stream, 3);
 }
@@ -96,6 +99,7 @@ int splitlora_lora_linear_fwd(int dtype, int use_tc, const void* x, const void* 
 int splitlora_lora_linear_fwd_parts(int dtype, int use_tc, const void* x, const void* W, const void* bias, const float* A,
                                     const float* B, float alpha, int M, int n_in, int n_out, int r, int G, void* y,
                                     void* workspace, size_t workspace_bytes, void* stream, int parts) {
+  LaunchChain chain;
   int rc = check_linear(dtype, M, n_in, n_out, r, G);
   if (rc) return rc;
   if (parts < 1 || parts > 3) return SPLITLORA_ERR_ARG;
@@ -127,6 +131,7 @@ int splitlora_lora_linear_fwd_parts(int dtype, int use_tc, const void* x, const 
 int splitlora_lora_linear_bwd(int dtype, int use_tc, const void* x, const void* Wt, const void* dy, const float* A,
                               const float* B, float alpha, int M, int n_in, int n_out, int r, int G, void* dx,
                               float* dA, float* dB, void* workspace, size_t workspace_bytes, void* stream) {
+  LaunchChain chain;
   return splitlora_lora_linear_bwd_parts(dtype, use_tc, x, Wt, dy, A, B, alpha, M, n_in, n_out, r, G, dx, dA, dB, workspace,
                                          workspace_bytes, stream, 7);
 }
@@ -134,6 +139,7 @@ int splitlora_lora_linear_bwd(int dtype, int use_tc, const void* x, const void* 
 int splitlora_lora_linear_bwd_parts(int dtype, int use_tc, const void* x, const void* Wt, const void* dy, const float* A,
                                     const float* B, float alpha, int M, int n_in, int n_out, int r, int G, void* dx,
                                     float* dA, float* dB, void* workspace, size_t workspace_bytes, void* stream, int parts) {
+  LaunchChain chain;
   int rc = check_linear(dtype, M, n_in, n_out, r, G);
   if (rc) return rc;
   if (parts < 1 || parts > 7) return SPLITLORA_ERR_ARG;
@@ -188,11 +194,13 @@ int splitlora_library_status(int32_t* code) {
 }
 
 int splitlora_transpose(int dtype, const void* in, int rows, int cols, void* out, void* stream) {
+  LaunchChain chain;
   if (!in || !out || rows < 1 || cols < 1 || (dtype != DT_F32 && dtype != DT_BF16)) return SPLITLORA_ERR_ARG;
   return transpose(dtype, in, rows, cols, out, rows, (cudaStream_t)stream) == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;
 }
 
 int splitlora_handoff_quantize(int dtype, const void* x, int64_t M, int d, uint8_t* codes, float* scales, void* stream) {
+  LaunchChain chain;
   const int n = dtype == DT_BF16 ? 8 : 4;
   if (!x || !codes || !scales || M < 1 || d < n || d % n != 0 || (dtype != DT_F32 && dtype != DT_BF16)) return SPLITLORA_ERR_ARG;
   if (!aligned16(x) || !aligned16(codes)) return SPLITLORA_ERR_ALIGN;
@@ -201,6 +209,7 @@ int splitlora_handoff_quantize(int dtype, const void* x, int64_t M, int d, uint8
 
 int splitlora_handoff_dequantize(int dtype, const uint8_t* codes, const float* scales, int64_t M, int d, void* y,
                                  void* stream) {
+  LaunchChain chain;
   const int n = dtype == DT_BF16 ? 8 : 4;
   if (!y || !codes || !scales || M < 1 || d < n || d % n != 0 || (dtype != DT_F32 && dtype != DT_BF16)) return SPLITLORA_ERR_ARG;
   if (!aligned16(y) || !aligned16(codes)) return SPLITLORA_ERR_ALIGN;
@@ -208,6 +217,7 @@ int splitlora_handoff_dequantize(int dtype, const uint8_t* codes, const float* s
 }
 
 int splitlora_aggregate_buffers(float* params, int K, int64_t P, const double* weights, void* stream) {
+  LaunchChain chain;
   if (!params || !weights || K < 1 || K > AGG_MAX_CLIENTS || P < 4 || P % 4 != 0) return SPLITLORA_ERR_ARG;
   if (!aligned16(params)) return SPLITLORA_ERR_ALIGN;
   float w[AGG_MAX_CLIENTS];
@@ -217,6 +227,7 @@ int splitlora_aggregate_buffers(float* params, int K, int64_t P, const double* w
 
 int splitlora_attention_fwd(int dtype, int use_tc, const void* qkv, int nseq, int T, int n_head, int d_model, void* o,
                             float* lse, void* stream) {
+  LaunchChain chain;
   if (!qkv || !o || !lse || nseq < 1 || T < 1 || n_head < 1 || d_model % n_head != 0 || d_model / n_head > 128 ||
       (dtype != DT_F32 && dtype != DT_BF16))
     return SPLITLORA_ERR_ARG;
@@ -232,6 +243,7 @@ int splitlora_attention_fwd(int dtype, int use_tc, const void* qkv, int nseq, in
 
 int splitlora_attention_bwd(int dtype, int use_tc, const void* qkv, const void* o, const float* lse, const void* d_o,
                             int nseq, int T, int n_head, int d_model, void* dqkv, float* rowdot, void* stream) {
+  LaunchChain chain;
   if (!qkv || !o || !lse || !d_o || !dqkv || !rowdot || nseq < 1 || T < 1 || n_head < 1 || d_model % n_head != 0 ||
       d_model / n_head > 128 || (dtype != DT_F32 && dtype != DT_BF16))
     return SPLITLORA_ERR_ARG;
@@ -251,6 +263,7 @@ int splitlora_attention_bwd(int dtype, int use_tc, const void* qkv, const void* 
 extern "C" int splitlora_linear(int dtype, int use_tc, const void* x, const void* W, const void* bias, int epilogue,
                                 const void* r, void* z, int gelu_tanh, int M, int n_in, int n_out, void* y,
                                 int* status_word, void* stream) {
+  LaunchChain chain;
   if (!x || !W || !y || M < 1 || n_in < 8 || n_out < 8 || n_in % 8 || n_out % 8 || (dtype != DT_F32 && dtype != DT_BF16))
     return SPLITLORA_ERR_ARG;
   if (epilogue < EPI_BIAS || epilogue > EPI_MUL_GELUGRAD) return SPLITLORA_ERR_ARG;

@@ -12,6 +12,7 @@
 
 #include "../../include/splitlora.h"
 #include "kernels.h"
+#include "launch.cuh"
 
 using namespace sl;
 
@@ -374,6 +375,7 @@ cudaError_t copy_client_rows(splitlora_ctx* c, const void* src, void* dst, int c
   if (client_b <= client_a) return cudaSuccess;
   const size_t off = (size_t)client_a * c->rows_per_client * c->d * c->es;
   const size_t n = (size_t)(client_b - client_a) * c->rows_per_client * c->d * c->es;
+  break_chain();
   return cudaMemcpyAsync((char*)dst + off, (const char*)src + off, n, cudaMemcpyDeviceToDevice, c->st);
 }
 
@@ -653,6 +655,7 @@ int splitlora_workspace_bytes(const splitlora_config* cfg, size_t* bytes) {
 }
 
 int splitlora_bind_workspace(splitlora_ctx* c, void* dev, size_t bytes) {
+  LaunchChain chain;
   if (!c || !dev) return SPLITLORA_ERR_ARG;
   if (reinterpret_cast<uintptr_t>(dev) & 255u) return fail(c, SPLITLORA_ERR_ALIGN, "workspace must be 256-byte aligned");
   size_t need = plan(c, nullptr);
@@ -699,6 +702,7 @@ int splitlora_bind_workspace(splitlora_ctx* c, void* dev, size_t bytes) {
 }
 
 int splitlora_bind_frozen(splitlora_ctx* c, const char* name, const void* dev, size_t bytes) {
+  LaunchChain chain;
   if (!c || !name || !dev) return SPLITLORA_ERR_ARG;
   if (!c->ws) return fail(c, SPLITLORA_ERR_WORKSPACE, "bind the workspace first");
   if (!aligned16(dev)) return fail(c, SPLITLORA_ERR_ALIGN, std::string(name) + " is not 16-byte aligned");
@@ -754,6 +758,7 @@ int splitlora_bind_frozen(splitlora_ctx* c, const char* name, const void* dev, s
 
 int splitlora_set_adapter(splitlora_ctx* c, int side, int client, int layer, uint32_t target, const float* A,
                           const float* B) {
+  LaunchChain chain;
   if (!c) return SPLITLORA_ERR_ARG;
   if (!c->ws) return fail(c, SPLITLORA_ERR_WORKSPACE, "no workspace bound");
   int rc;
@@ -793,6 +798,7 @@ int splitlora_get_opt_state(splitlora_ctx* c, int side, int client, int layer, u
 }
 int splitlora_set_opt_state(splitlora_ctx* c, int side, int client, int layer, uint32_t target, const float* mA,
                             const float* vA, const float* mB, const float* vB) {
+  LaunchChain chain;
   if (!c) return SPLITLORA_ERR_ARG;
   if (!c->ws) return fail(c, SPLITLORA_ERR_WORKSPACE, "no workspace bound");
   int rc;
@@ -822,6 +828,7 @@ int splitlora_set_counters(splitlora_ctx* c, int64_t round_index, int64_t server
 // ---- Algorithm 1 ---------------------------------------------------------------------------
 
 int splitlora_client_fwd(splitlora_ctx* c, const int32_t* tokens, void* act_out) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   if (!tokens || !act_out) return fail(c, SPLITLORA_ERR_ARG, "null pointer");
@@ -846,6 +853,7 @@ int splitlora_client_fwd(splitlora_ctx* c, const int32_t* tokens, void* act_out)
 
 int splitlora_server_step(splitlora_ctx* c, const void* act_in, const int32_t* labels, void* act_grad_out,
                           float* loss_out) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   if (!act_in || !labels || !act_grad_out) return fail(c, SPLITLORA_ERR_ARG, "null pointer");
@@ -907,6 +915,7 @@ int splitlora_server_step(splitlora_ctx* c, const void* act_in, const int32_t* l
 }
 
 int splitlora_client_bwd(splitlora_ctx* c, const void* act_grad_in) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   if (!act_grad_in) return fail(c, SPLITLORA_ERR_ARG, "null pointer");
@@ -951,6 +960,7 @@ static int aggregation_weights(splitlora_ctx* c, const int64_t* counts, double t
 }
 
 int splitlora_set_client_ranks(splitlora_ctx* c, const int32_t* ranks) {
+  LaunchChain chain;
   if (!c) return SPLITLORA_ERR_ARG;
   if (!c->ws) return fail(c, SPLITLORA_ERR_WORKSPACE, "no workspace bound");
   if (!ranks) { c->client_rank.clear(); return SPLITLORA_OK; }
@@ -967,6 +977,7 @@ int splitlora_set_client_ranks(splitlora_ctx* c, const int32_t* ranks) {
 }
 
 int splitlora_aggregate(splitlora_ctx* c, const int64_t* counts) {
+  LaunchChain chain;
   float w[AGG_MAX_CLIENTS];
   int rc = aggregation_weights(c, counts, 0.0, w);
   if (rc) return rc;
@@ -1016,6 +1027,7 @@ int splitlora_set_client_cuts(splitlora_ctx* c, const int32_t* cuts) {
 
 int splitlora_aggregate_local_sum(splitlora_ctx* c, const int64_t* counts, int64_t total_count, float** sum_dev,
                                   int64_t* count) {
+  LaunchChain chain;
   if (!c || !sum_dev || !count) return SPLITLORA_ERR_ARG;
   if (total_count <= 0) return fail(c, SPLITLORA_ERR_COUNTS, "total_count must be positive");
   if (!uniform_cut(c)) return fail(c, SPLITLORA_ERR_UNSUPPORTED, "clients cut at different depths cannot be spread over devices");
@@ -1029,6 +1041,7 @@ int splitlora_aggregate_local_sum(splitlora_ctx* c, const int64_t* counts, int64
 }
 
 int splitlora_aggregate_broadcast(splitlora_ctx* c) {
+  LaunchChain chain;
   if (!c) return SPLITLORA_ERR_ARG;
   if (!c->ws) return fail(c, SPLITLORA_ERR_WORKSPACE, "no workspace bound");
   { Scope s(c, "aggregate", c->client_rank.empty() ? 1 : 2);
@@ -1052,6 +1065,7 @@ int splitlora_set_deferred_server_update(splitlora_ctx* c, int on) {
 }
 
 int splitlora_server_update(splitlora_ctx* c) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   CK(c, run_optimizer(c, false));
@@ -1070,6 +1084,7 @@ int splitlora_adapter_buffer(splitlora_ctx* c, int side, int kind, float** dev, 
 }
 
 int splitlora_adapters_changed(splitlora_ctx* c, int side) {
+  LaunchChain chain;
   if (!c) return SPLITLORA_ERR_ARG;
   if (side == SPLITLORA_SIDE_CLIENT) c->client_copies_dirty = true;
   else if (side == SPLITLORA_SIDE_SERVER) c->server_copies_dirty = true;
@@ -1079,6 +1094,7 @@ int splitlora_adapters_changed(splitlora_ctx* c, int side) {
 
 int splitlora_round(splitlora_ctx* c, const int32_t* tokens, const int32_t* labels, const int64_t* counts,
                     float* loss_out) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   if (!counts) return fail(c, SPLITLORA_ERR_ARG, "null counts");
@@ -1100,6 +1116,7 @@ int splitlora_round(splitlora_ctx* c, const int32_t* tokens, const int32_t* labe
 
 int splitlora_round_compressed(splitlora_ctx* c, const int32_t* tokens, const int32_t* labels, const int64_t* counts,
                                uint8_t* codes, float* scales, float* loss_out) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   if (!counts || !codes || !scales) return fail(c, SPLITLORA_ERR_ARG, "null pointer");
@@ -1134,6 +1151,7 @@ int splitlora_round_compressed(splitlora_ctx* c, const int32_t* tokens, const in
 
 int splitlora_round_host(splitlora_ctx* c, const int32_t* tokens_host, const int32_t* labels_host,
                          const int64_t* counts, float* loss_out) {
+  LaunchChain chain;
   int rc = check_ready(c);
   if (rc) return rc;
   if (!tokens_host || !labels_host) return fail(c, SPLITLORA_ERR_ARG, "null pointer");

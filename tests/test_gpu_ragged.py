@@ -103,8 +103,8 @@ def test_lora_linear_any_size(M, n_in, n_out, r, G):
     x = torch.randn(M, n_in, device="cuda", generator=g).bfloat16()
     W = (torch.randn(n_out, n_in, device="cuda", generator=g) * n_in ** -0.5).bfloat16()
     dy = (torch.randn(M, n_out, device="cuda", generator=g) * n_out ** -0.5).bfloat16()
-    A = torch.randn(G, r, n_in, device="cuda", generator=g) * n_in ** -0.5
-    Bm = torch.randn(G, n_out, r, device="cuda", generator=g) * r ** -0.5
+    A = torch.randn(G, r, n_in, device="cuda", generator=g, dtype=torch.float32) * n_in ** -0.5
+    Bm = torch.randn(G, n_out, r, device="cuda", generator=g, dtype=torch.float32) * r ** -0.5
     s = 16.0 / r
     xg, dyg, A64, B64 = x.double().view(G, -1, n_in), dy.double().view(G, -1, n_out), A.double(), Bm.double()
     h, dh = xg @ A64.transpose(1, 2), s * dyg @ B64
