@@ -184,7 +184,10 @@ struct AdapterCopyArgs {
   int slice_off[4];
   float scale;
   void *Acat, *AcatT, *Bext, *BextT;   // any of them may be null (skipped)
+  int* status = nullptr;               // write_adapter_copies: a word to clear
 };
+// The same for one target (n_targets 1, slice_off 0, n_out = d_out) into uninitialised copies: padding included.
+cudaError_t write_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st);
 cudaError_t refresh_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st);
 
 cudaError_t transpose(int dt, const void* in, int rows, int cols, void* out, int64_t ldo, cudaStream_t st);

@@ -156,14 +156,15 @@ lora_grad_reduce_lanes_kernel(const float* __restrict__ partial, int r, int R, i
 }
 
 // The second kernel for a batch of jobs (blockIdx.z): one output per thread, chunks added in order.
-struct RedJob { const float* partial; float* out; int r, R; float scale; int64_t ogs, ots, osj, osc; };
+struct RedJob { const float* partial; float* out; int r, R, C; float scale; int64_t ogs, ots, osj, osc; };
 struct RedBatch { RedJob j[4]; };
 __global__ void __launch_bounds__(RED_THREADS)
-lora_grad_reduce_batch_kernel(RedBatch b, int C, int chunks_per_group) {
+lora_grad_reduce_batch_kernel(RedBatch b, int chunks_per_group) {
   overlap_sync();
   const RedJob& jb = b.j[blockIdx.z];
   const int idx = blockIdx.x * RED_THREADS + threadIdx.x;   // over R*C
   const int g = blockIdx.y;
+  const int C = jb.C;
   if (idx >= jb.R * C) return;
   const size_t rc = (size_t)jb.R * C;
   const float* p = jb.partial + (size_t)g * chunks_per_group * rc + idx;
@@ -255,7 +256,7 @@ cudaError_t lora_grad_batch(int dt, const LoraGradJob* jobs, int njobs, int M, i
   bool batched = use_tc && status && dt == DT_BF16 && njobs >= 1 && njobs <= 4;
   for (int j = 0; j < njobs && batched; ++j) {
     const LoraGradJob& jb = jobs[j];
-    batched = jb.C == jobs[0].C && (jb.rp == 16 || jb.rp == 32 || jb.rp == 64) &&
+    batched = (jb.rp == 16 || jb.rp == 32 || jb.rp == 64) &&
               lora_grad_tc_supported(dt, jb.Z, jb.ldz, jb.zcol0, jb.C, jb.Wt, jb.ldwt, jb.wcol0, jb.r, jb.rp, jb.nt, M, rows_per_group);
   }
   if (batched) {
@@ -268,12 +269,12 @@ cudaError_t lora_grad_batch(int dt, const LoraGradJob* jobs, int njobs, int M, i
       int maxRC = 0;
       for (int j = 0; j < 4; ++j) {
         const LoraGradJob& jb = jobs[j < njobs ? j : 0];
-        rb.j[j] = {partial + offs[j < njobs ? j : 0], jb.out, jb.r, jb.nt * jb.r, jb.scale, jb.out_group_stride,
+        rb.j[j] = {partial + offs[j < njobs ? j : 0], jb.out, jb.r, jb.nt * jb.r, jb.C, jb.scale, jb.out_group_stride,
                    jb.out_target_stride, jb.out_sj, jb.out_sc};
         if (j < njobs && jb.nt * jb.r * jb.C > maxRC) maxRC = jb.nt * jb.r * jb.C;
       }
       dim3 g2((maxRC + RED_THREADS - 1) / RED_THREADS, groups, njobs);
-      launch_overlapped(lora_grad_reduce_batch_kernel, g2, RED_THREADS, 0, st, rb, jobs[0].C, cpg);
+      launch_overlapped(lora_grad_reduce_batch_kernel, g2, RED_THREADS, 0, st, rb, cpg);
       return cudaGetLastError();
     }
     if (e != cudaErrorInvalidValue) return e;      // invalid value: the scratch does not hold the batch, go one by one

@@ -70,6 +70,7 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
   const CUtensorMap& mapW = bt.mapW[blockIdx.z];
   const LgParams& p = bt.p[blockIdx.z];
   const int wx0 = bt.wx0[blockIdx.z];
+  if ((int)blockIdx.x * LT_C >= p.C) return;             // the grid is as wide as the widest job
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -206,12 +207,12 @@ bool lora_grad_tc_supported(int dt, const void* Z, int64_t ldz, int zcol0, int C
   return true;
 }
 
-// Chunks per group for a grid of `ctas_per_chunk_set` CTAs per chunk: the choice that minimises
+// Chunks per group (at most max_chunks) for a grid of `ctas_per_chunk_set` CTAs per chunk: the choice that minimises
 // (waves of 296 resident CTAs) x (rows per chunk), every chunk a whole number of 128-row blocks.
-static int pick_chunks(int ctas_per_chunk_set, int rpg) {
+static int pick_chunks(int ctas_per_chunk_set, int rpg, int64_t max_chunks) {
   int best = 1;
   double best_cost = 1e300;
-  for (int s = 1; s <= rpg / 128; ++s) {
+  for (int s = 1; s <= rpg / 128 && s <= max_chunks; ++s) {
     if (rpg % (s * 128) != 0) continue;
     const int ctas = ctas_per_chunk_set * s;
     const double cost = (double)((ctas + 295) / 296) * ((double)rpg / s + 256.0);   // + a chunk's start-up, in rows
@@ -222,7 +223,7 @@ static int pick_chunks(int ctas_per_chunk_set, int rpg) {
 
 // Chunk partials of job j go to partial + offset_j as [chunk][R_j][C] (R_j = nt*r); *chunks_per_group
 // receives the number of chunks per group (the same for every job) so that the caller's second kernel
-// can add them, offsets[j] the start of job j's partials (floats).  All jobs share M, rows_per_group and C.
+// can add them, offsets[j] the start of job j's partials (floats).  All jobs share M and rows_per_group.
 cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M, int rows_per_group, float* partial,
                                        size_t partial_floats, int* status, int* chunks_per_group, size_t* offsets,
                                        cudaStream_t st) {
@@ -233,24 +234,30 @@ cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M
   const bool one = rows_per_group <= 0 || rows_per_group >= M;
   const int rpg = one ? (M + 127) / 128 * 128 : rows_per_group;
   const int groups = one ? 1 : M / rpg;
-  const int C = jobs[0].C;
-  const int ctiles = (C + LT_C - 1) / LT_C;
-  const int s = pick_chunks(ctiles * groups * njobs, rpg);
+  int ctiles = 0, ctiles_sum = 0;
+  size_t set_floats = 0;                       // partials of one chunk per group, all jobs
+  for (int j = 0; j < njobs; ++j) {
+    const int t = (jobs[j].C + LT_C - 1) / LT_C;
+    ctiles = t > ctiles ? t : ctiles;
+    ctiles_sum += t;
+    set_floats += (size_t)groups * jobs[j].nt * jobs[j].r * jobs[j].C;
+  }
+  if (set_floats > partial_floats) return cudaErrorInvalidValue;
+  // the scratch bounds the number of chunks (few tokens: it holds one chunk of every job, not two)
+  const int s = pick_chunks(ctiles_sum * groups, rpg, (int64_t)(partial_floats / set_floats));
   LgBatch bt;
   size_t off = 0;
   for (int j = 0; j < njobs; ++j) {
     const LoraGradJob& jb = jobs[j];
-    if (jb.C != C) return cudaErrorInvalidValue;
-    if (!make_map(&bt.mapZ[j], (const bf16*)jb.Z + jb.zcol0, (uint64_t)M, (uint64_t)C, (uint64_t)jb.ldz)) return cudaErrorInvalidValue;
+    if (!make_map(&bt.mapZ[j], (const bf16*)jb.Z + jb.zcol0, (uint64_t)M, (uint64_t)jb.C, (uint64_t)jb.ldz)) return cudaErrorInvalidValue;
     if (!make_map(&bt.mapW[j], jb.Wt, (uint64_t)M, (uint64_t)jb.ldwt, (uint64_t)jb.ldwt)) return cudaErrorInvalidValue;
     LgParams& p = bt.p[j];
-    p.C = C; p.rows_per_chunk = rpg / s; p.R = jb.nt * jb.r; p.r = jb.r; p.rp = jb.rp; p.wsel0 = jb.wcol0 % LT_N;
+    p.C = jb.C; p.rows_per_chunk = rpg / s; p.R = jb.nt * jb.r; p.r = jb.r; p.rp = jb.rp; p.wsel0 = jb.wcol0 % LT_N;
     p.partial = partial + off; p.status = status;
     bt.wx0[j] = jb.wcol0 - p.wsel0;
     offsets[j] = off;
-    off += (size_t)groups * s * p.R * C;
+    off += (size_t)groups * s * p.R * jb.C;
   }
-  if (off > partial_floats) return cudaErrorInvalidValue;
   for (int j = njobs; j < LT_MAX_JOBS; ++j) { bt.mapZ[j] = bt.mapZ[0]; bt.mapW[j] = bt.mapW[0]; bt.p[j] = bt.p[0]; bt.wx0[j] = bt.wx0[0]; }
   dim3 grid(ctiles, groups * s, njobs);
   launch_overlapped(lora_grad_tc_kernel, grid, LT_THREADS, LT_SMEM, st, bt);

@@ -16,7 +16,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 struct LinearPlan {
   int rp, ext;
-  size_t off_acat, off_acatT, off_bext, off_bextT, off_h, off_dh, off_scratch, off_status, total;
+  size_t off_acat, off_acatT, off_bext, off_bextT, off_h, off_dh, off_scratch, off_status, total, scratch_floats;
 };
 
 LinearPlan plan_linear(int dtype, int M, int n_in, int n_out, int r, int G) {
@@ -33,7 +33,9 @@ LinearPlan plan_linear(int dtype, int M, int n_in, int n_out, int r, int G) {
   p.off_bextT = take((size_t)G * p.ext * n_out * es);
   p.off_h = take((size_t)M * p.ext * es);
   p.off_dh = take((size_t)M * p.ext * es);
-  size_t sc = lora_grad_scratch_floats(M, r, n_in > n_out ? n_in : n_out);
+  // at least two chunks per group of the wider reduction: dA and dB as one batch
+  size_t sc = lora_grad_scratch_floats(M > 256 * G ? M : 256 * G, r, n_in > n_out ? n_in : n_out);
+  p.scratch_floats = sc;
   p.off_scratch = take(sc * 4);
   p.total = align_up(off, 256);
   return p;
@@ -75,17 +77,8 @@ static int make_copies(int dtype, const LinearPlan& p, const float* A, const flo
   a.scale = alpha / (float)r;
   a.Acat = ws + p.off_acat; a.AcatT = fwd ? nullptr : ws + p.off_acatT;
   a.Bext = fwd ? ws + p.off_bext : nullptr; a.BextT = fwd ? nullptr : ws + p.off_bextT;
-  // the padding of the copies must be zero: clear the ones this call uses
-  if (cudaMemsetAsync(ws + p.off_acat, 0, (size_t)G * p.ext * n_in * es, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
-  if (fwd) {
-    if (cudaMemsetAsync(ws + p.off_bext, 0, (size_t)G * n_out * p.ext * es, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
-  } else {
-    if (cudaMemsetAsync(ws + p.off_acatT, 0, (size_t)G * p.ext * n_in * es, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
-    if (cudaMemsetAsync(ws + p.off_bextT, 0, (size_t)G * n_out * p.ext * es, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
-  }
-  if (cudaMemsetAsync(ws + p.off_status, 0, 256, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
-  break_chain();
-  return refresh_adapter_copies(a, st) == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;
+  a.status = (int*)(ws + p.off_status);
+  return write_adapter_copies(a, st) == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;
 }
 
 int splitlora_lora_linear_fwd(int dtype, int use_tc, const void* x, const void* W, const void* bias, const float* A,
@@ -176,11 +169,16 @@ int splitlora_lora_linear_bwd_parts(int dtype, int use_tc, const void* x, const 
     if (run_gemm(use_tc, a, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   }
   if (!(parts & 4)) return SPLITLORA_OK;
-  float* scratch = (float*)(ws + p.off_scratch);
-  if (lora_grad(dtype, x, n_in, 0, n_in, ws + p.off_dh, p.ext, 0, r, p.rp, 1, M, rpg, 1.0f, dA, (int64_t)r * n_in, 0, n_in, 1,
-                scratch, st, status, use_tc != 0) != cudaSuccess) return SPLITLORA_ERR_CUDA;
-  if (lora_grad(dtype, dy, n_out, 0, n_out, ws + p.off_h, p.ext, 0, r, p.rp, 1, M, rpg, s, dB, (int64_t)n_out * r, 0, 1, r,
-                scratch, st, status, use_tc != 0) != cudaSuccess) return SPLITLORA_ERR_CUDA;
+  // dA = dh^T x and dB = s dy^T h: one pair of launches where the tensor-core path applies
+  LoraGradJob jobs[2];
+  LoraGradJob &ja = jobs[0], &jb = jobs[1];
+  ja.Z = x; ja.ldz = n_in; ja.C = n_in; ja.Wt = ws + p.off_dh; ja.scale = 1.0f; ja.out = dA; ja.out_group_stride = (int64_t)r * n_in;
+  ja.out_sj = n_in; ja.out_sc = 1;
+  jb.Z = dy; jb.ldz = n_out; jb.C = n_out; jb.Wt = ws + p.off_h; jb.scale = s; jb.out = dB; jb.out_group_stride = (int64_t)n_out * r;
+  jb.out_sj = 1; jb.out_sc = r;
+  for (LoraGradJob& j : jobs) { j.ldwt = p.ext; j.r = r; j.rp = p.rp; j.nt = 1; }
+  if (lora_grad_batch(dtype, jobs, 2, M, rpg, (float*)(ws + p.off_scratch), p.scratch_floats, st, status, use_tc != 0) != cudaSuccess)
+    return SPLITLORA_ERR_CUDA;
   return SPLITLORA_OK;
 }
 

@@ -246,7 +246,7 @@ size_t plan(splitlora_ctx* c, char* ws) {
   c->xf = a.take(M * d * es); c->logits = a.take(M * (size_t)c->Vpad * es);
   c->meanf = (float*)a.take(M * 4); c->rstdf = (float*)a.take(M * 4); c->row_loss = (float*)a.take(M * 4);
   c->rowdot = (float*)a.take((size_t)c->nseq * c->cfg.n_head * c->cfg.seq * 4);
-  c->grad_scratch_floats = lora_grad_scratch_floats(c->M, c->nq * c->r, c->d);
+  c->grad_scratch_floats = lora_grad_scratch_floats(c->M > 256 ? c->M : 256, c->nq * c->r, c->d);   // room for a layer's jobs as one batch
   c->grad_scratch = (float*)a.take(c->grad_scratch_floats * 4);
   if (c->has_o) c->g_dhcat_o = a.take(M * ext_o * es);
   c->g_a = a.take(M * d * es); c->g_b = a.take(M * d * es); c->g_dz = a.take(M * Fz * es);
