@@ -118,3 +118,20 @@ def test_lora_linear_any_size(M, n_in, n_out, r, G):
     assert B.library_status() == 0
     for got, plain in zip(*errs):
         assert got <= 1.02 * plain + 2e-5, errs
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (33, 72, 40), (65, 136, 200), (512, 1024, 128), (31, 64, 1000), (700, 200, 1000),
+                                   (1600, 40, 1608)])
+def test_linear_fp32_any_size(M, K, N):
+    """Both tile sizes and the unaligned form: every element within the bound of a K-term fp32 sum in any order,
+    (K + 2) 2^-24 sum |x w|; rows past M stay untouched."""
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    x, W = (torch.randn(*s, device="cuda", generator=g, dtype=torch.float32) for s in ((M, K), (N, K)))
+    bias, r = (torch.randn(*s, device="cuda", generator=g, dtype=torch.float32) for s in ((N,), (M, N)))
+    ref = x.double() @ W.double().T + bias.double() + r.double()
+    bound = (K + 2) * 2.0 ** -24 * (x.double().abs() @ W.double().abs().T + bias.double().abs() + r.double().abs())
+    shifted = torch.empty(M * K + 1, device="cuda", dtype=torch.float32)[1:].view(M, K).copy_(x)
+    for xin in (x, shifted):
+        buf = torch.full((M + 64, N), 7.0, device="cuda", dtype=torch.float32)
+        B.linear(xin, W, bias, B.EPI_BIAS_RESID, r=r, y=buf[:M])
+        assert bool((buf[M:] == 7).all()) and bool(((buf[:M].double() - ref).abs() <= bound).all())
