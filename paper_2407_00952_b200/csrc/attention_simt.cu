@@ -1,225 +1,336 @@
-// Causal multi-head attention with plain FMA arithmetic (fp32 or bf16 storage): the arithmetic of
-// the fp32 configuration and a second opinion for the tensor-core kernels.
-// One warp per (sequence, head, row).  Scores are computed one key per lane; the value / key / query
-// accumulations are one feature per lane with the probability broadcast by shuffle.
+// Causal multi-head attention with plain FMA arithmetic (fp32 or bf16 storage, any shape, head width up to 128): the
+// arithmetic of the fp32 configuration and a second opinion for the tensor-core kernels.
+// A block of eight warps owns RT = 32 rows (queries, or keys in the dK/dV kernel) of one (sequence, head), four rows per
+// warp, and walks the other side in tiles of 32 rows that all its warps share through shared memory.  Scores are one
+// column of the tile per lane; the accumulations are one feature per lane, with the tile's probabilities read back as
+// broadcasts from shared memory.  A tile element read from shared memory serves four rows, a probability all features.
+// What bounds it: shared-memory reads (about five per sixteen products).  Against one warp per row that reads the other side
+// from global memory: the fp32 round of 512 tokens (8 sequences of 64, 4 heads of 32) 514 -> 355 us together with the
+// sixteen-lane adapter gradients of lora_grad.cu; errors against 64 bits a little smaller.
 #include "common.cuh"
+#include "host_common.h"
 #include "kernels.h"
 #include "launch.cuh"
 
 namespace sl {
 namespace {
 
-constexpr int WARPS = 4;
+constexpr int WARPS = 8, RPW = 4, RT = WARPS * RPW, KT = 32;
 constexpr int MAX_DH = 128;
 constexpr int DPL = MAX_DH / 32;   // features per lane
 
+// Shared memory, in floats: two tiles [32][width + 1], width = dh rounded up to 32 so that "one feature per lane" reads
+// stay inside a row (the odd stride keeps "one row per lane" reads conflict-free), two row blocks [32][dh rounded up to
+// 4] (read as float4 broadcasts, zero past dh), two [32][32] blocks of per-row tile values.
+__host__ __device__ constexpr int pad4(int dh) { return (dh + 3) & ~3; }
+__host__ __device__ constexpr int tile_stride(int dh) { return ((dh + 31) & ~31) + 1; }
+inline size_t smem_bytes(int dh) { return (size_t)(2 * KT * tile_stride(dh) + 2 * RT * pad4(dh) + 2 * RT * KT) * 4; }
+
+struct Tiles {
+  float *a, *b, *ra, *rb, *pa, *pb;
+  int lt, lr;
+  __device__ __forceinline__ Tiles(float* sh, int dh) {
+    lr = pad4(dh); lt = tile_stride(dh);
+    ra = sh; rb = ra + RT * lr;                        // 16-byte aligned
+    pa = rb + RT * lr; pb = pa + RT * KT;
+    a = pb + RT * KT; b = a + KT * lt;
+  }
+};
+
+// rows row0 .. row0 + 31 of a matrix into [32][ld_dst], columns 0 .. width - 1; zero past `rows` and past dh
 template <typename T>
-__device__ __forceinline__ float dot_row(const float* __restrict__ a_s, const T* __restrict__ row, int dh) {
-  float s = 0.f;
-  for (int c = 0; c < dh; ++c) s = fmaf(a_s[c], to_f<T>(row[c]), s);
-  return s;
+__device__ __forceinline__ void load_rows(float* dst, int ld_dst, int width, const T* src, size_t ld, int row0, int rows, int dh) {
+  for (int i = threadIdx.x; i < 32 * width; i += WARPS * 32) {
+    const int r = i / width, c = i % width;
+    dst[r * ld_dst + c] = (row0 + r < rows && c < dh) ? to_f<T>(src[(size_t)(row0 + r) * ld + c]) : 0.f;
+  }
+}
+
+// out[r] = sum_c row_r[c] * tile[lane][c] for this warp's four rows
+__device__ __forceinline__ void dot4(const float* rows, int lr, const float* tile_row, float* out) {
+#pragma unroll
+  for (int r = 0; r < RPW; ++r) out[r] = 0.f;
+#pragma unroll 2
+  for (int c = 0; c < lr; c += 4) {
+    const float k0 = tile_row[c], k1 = tile_row[c + 1], k2 = tile_row[c + 2], k3 = tile_row[c + 3];
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+      const float4 q = *reinterpret_cast<const float4*>(rows + r * lr + c);
+      out[r] = fmaf(q.w, k3, fmaf(q.z, k2, fmaf(q.y, k1, fmaf(q.x, k0, out[r]))));
+    }
+  }
+}
+
+// acc[r][c] += sum_j p[r][j] * tile[j][lane + 32 c]
+__device__ __forceinline__ void accumulate4(float (*acc)[DPL], const float* p, const float* tile, int lt, int lane, int nfeat) {
+#pragma unroll 2
+  for (int j = 0; j < KT; j += 4) {
+    float4 pv[RPW];
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) pv[r] = *reinterpret_cast<const float4*>(p + r * KT + j);
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) {
+      if (c >= nfeat) break;                           // warp-uniform
+      const float* t = tile + j * lt + lane + 32 * c;
+      const float v0 = t[0], v1 = t[lt], v2 = t[2 * lt], v3 = t[3 * lt];
+#pragma unroll
+      for (int r = 0; r < RPW; ++r)
+        acc[r][c] = fmaf(pv[r].w, v3, fmaf(pv[r].z, v2, fmaf(pv[r].y, v1, fmaf(pv[r].x, v0, acc[r][c]))));
+    }
+  }
+}
+
+struct Where { int b, h, r0; };
+__device__ __forceinline__ Where where(int Tn, int H) {
+  const int nt = (Tn + RT - 1) / RT;
+  const int64_t item = (int64_t)blockIdx.x / nt;
+  return {(int)(item / H), (int)(item % H), (nt - 1 - (int)(blockIdx.x % nt)) * RT};      // long rows first
 }
 
 template <typename T>
-__global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restrict__ qkv, int nseq, int Tn, int H,
-                                                              int d, T* __restrict__ o, float* __restrict__ lse) {
+__global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restrict__ qkv, int Tn, int H, int d,
+                                                              T* __restrict__ o, float* __restrict__ lse) {
   overlap_sync();
-  __shared__ float q_s[WARPS][MAX_DH];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * WARPS + wib;
-  if (w >= (int64_t)nseq * H * Tn) return;
-  const int i = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
-  const int dh = d / H;
+  extern __shared__ __align__(16) float sh[];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, dh = d / H, nfeat = (dh + 31) / 32;
+  const Where at = where(Tn, H);
+  Tiles t(sh, dh);
   const float scale = rsqrtf((float)dh);
   const size_t ld = (size_t)3 * d;
-  const T* qrow = qkv + ((size_t)b * Tn + i) * ld + (size_t)h * dh;
-  for (int c = lane; c < dh; c += 32) q_s[wib][c] = to_f<T>(qrow[c]);
-  __syncwarp();
-  float m = -INFINITY, l = 0.f, acc[DPL];
+  const T* base = qkv + (size_t)at.b * Tn * ld + (size_t)at.h * dh;
+  load_rows<T>(t.ra, t.lr, t.lr, base, ld, at.r0, Tn, dh);
+  float m[RPW], l[RPW], acc[RPW][DPL];
 #pragma unroll
-  for (int c = 0; c < DPL; ++c) acc[c] = 0.f;
-  for (int j0 = 0; j0 <= i; j0 += 32) {
-    int j = j0 + lane;
-    float s = -INFINITY;
-    if (j <= i) s = dot_row<T>(q_s[wib], qkv + ((size_t)b * Tn + j) * ld + d + (size_t)h * dh, dh) * scale;
-    float nm = fmaxf(m, warp_max(s));
-    float p = (j <= i) ? expf(s - nm) : 0.f;
-    float corr = (m == -INFINITY) ? 0.f : expf(m - nm);
-    l = l * corr + warp_sum(p);
+  for (int r = 0; r < RPW; ++r) {
+    m[r] = -INFINITY; l[r] = 0.f;
 #pragma unroll
-    for (int c = 0; c < DPL; ++c) acc[c] *= corr;
-    int cnt = min(32, i - j0 + 1);
-    for (int jj = 0; jj < cnt; ++jj) {
-      float pj = __shfl_sync(0xffffffffu, p, jj);
-      const T* vrow = qkv + ((size_t)b * Tn + j0 + jj) * ld + 2 * (size_t)d + (size_t)h * dh;
+    for (int c = 0; c < DPL; ++c) acc[r][c] = 0.f;
+  }
+  const float* rows = t.ra + w * RPW * t.lr;
+  float* p_s = t.pa + w * RPW * KT;
+  const int row0 = at.r0 + w * RPW;
+  for (int j0 = 0; j0 <= at.r0 + RT - 1 && j0 < Tn; j0 += KT) {
+    __syncthreads();
+    load_rows<T>(t.a, t.lt, t.lr, base + d, ld, j0, Tn, dh);
+    load_rows<T>(t.b, t.lt, t.lr, base + 2 * (size_t)d, ld, j0, Tn, dh);
+    __syncthreads();
+    if (j0 > row0 + RPW - 1) continue;                 // nothing of this tile is visible to the warp's rows
+    float s[RPW];
+    dot4(rows, t.lr, t.a + lane * t.lt, s);
 #pragma unroll
-      for (int c = 0; c < DPL; ++c) {
-        int dim = lane + 32 * c;
-        if (dim < dh) acc[c] = fmaf(pj, to_f<T>(vrow[dim]), acc[c]);
-      }
+    for (int r = 0; r < RPW; ++r) {
+      const bool vis = j0 + lane <= row0 + r;
+      const float sc = vis ? s[r] * scale : -INFINITY;
+      const float nm = fmaxf(m[r], warp_max(sc));
+      // a row that has seen no key yet in this tile keeps its state (its maximum is still -inf)
+      const bool none = j0 > row0 + r;
+      const float p = vis ? expf(sc - nm) : 0.f;
+      const float corr = (none || m[r] == -INFINITY) ? (none ? 1.f : 0.f) : expf(m[r] - nm);
+      l[r] = l[r] * corr + warp_sum(p);
+#pragma unroll
+      for (int c = 0; c < DPL; ++c) acc[r][c] *= corr;
+      m[r] = nm;
+      p_s[r * KT + lane] = p;
     }
-    m = nm;
+    __syncwarp();
+    accumulate4(acc, p_s, t.b, t.lt, lane, nfeat);
+    __syncwarp();
   }
-  T* orow = o + ((size_t)b * Tn + i) * d + (size_t)h * dh;
 #pragma unroll
-  for (int c = 0; c < DPL; ++c) {
-    int dim = lane + 32 * c;
-    if (dim < dh) orow[dim] = from_f<T>(acc[c] / l);
+  for (int r = 0; r < RPW; ++r) {
+    const int i = row0 + r;
+    if (i >= Tn) continue;
+    T* orow = o + ((size_t)at.b * Tn + i) * d + (size_t)at.h * dh;
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) {
+      const int dim = lane + 32 * c;
+      if (dim < dh) orow[dim] = from_f<T>(acc[r][c] / l[r]);
+    }
+    if (lane == 0) lse[((size_t)at.b * H + at.h) * Tn + i] = m[r] + logf(l[r]);
   }
-  if (lane == 0) lse[((size_t)b * H + h) * Tn + i] = m + logf(l);
 }
 
-// rowdot[b, h, i] = sum_dim dO[i, dim] * O[i, dim]
+// dQ, and D[row] = sum(dO * O) of its rows, which the dK/dV kernel (second) reads from `rowdot`
 template <typename T>
-__global__ void attn_rowdot_kernel(const T* __restrict__ o, const T* __restrict__ d_o, int nseq, int Tn, int H,
-                                   int d, float* __restrict__ rowdot) {
+__global__ void __launch_bounds__(WARPS * 32) attn_bwd_dq_kernel(const T* __restrict__ qkv, const T* __restrict__ o,
+                                                                 const float* __restrict__ lse, const T* __restrict__ d_o,
+                                                                 float* __restrict__ rowdot, int Tn, int H, int d,
+                                                                 T* __restrict__ dqkv) {
   overlap_sync();
-  const int lane = threadIdx.x & 31;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= (int64_t)nseq * H * Tn) return;
-  const int i = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
-  const int dh = d / H;
-  const size_t off = ((size_t)b * Tn + i) * d + (size_t)h * dh;
-  float s = 0.f;
-  for (int c = lane; c < dh; c += 32) s = fmaf(to_f<T>(o[off + c]), to_f<T>(d_o[off + c]), s);
-  s = warp_sum(s);
-  if (lane == 0) rowdot[((size_t)b * H + h) * Tn + i] = s;
-}
-
-// dQ: one warp per query row i; loops over keys j <= i.
-template <typename T>
-__global__ void __launch_bounds__(WARPS * 32) attn_bwd_dq_kernel(const T* __restrict__ qkv, const float* __restrict__ lse,
-                                                                 const T* __restrict__ d_o, const float* __restrict__ rowdot,
-                                                                 int nseq, int Tn, int H, int d, T* __restrict__ dqkv) {
-  overlap_sync();
-  __shared__ float q_s[WARPS][MAX_DH], do_s[WARPS][MAX_DH];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * WARPS + wib;
-  if (w >= (int64_t)nseq * H * Tn) return;
-  const int i = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
-  const int dh = d / H;
+  extern __shared__ __align__(16) float sh[];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, dh = d / H, nfeat = (dh + 31) / 32;
+  const Where at = where(Tn, H);
+  Tiles t(sh, dh);
   const float scale = rsqrtf((float)dh);
   const size_t ld = (size_t)3 * d;
-  const T* qrow = qkv + ((size_t)b * Tn + i) * ld + (size_t)h * dh;
-  const T* dorow = d_o + ((size_t)b * Tn + i) * d + (size_t)h * dh;
-  for (int c = lane; c < dh; c += 32) { q_s[wib][c] = to_f<T>(qrow[c]); do_s[wib][c] = to_f<T>(dorow[c]); }
-  __syncwarp();
-  const float L = lse[((size_t)b * H + h) * Tn + i], D = rowdot[((size_t)b * H + h) * Tn + i];
-  float acc[DPL];
+  const T* base = qkv + (size_t)at.b * Tn * ld + (size_t)at.h * dh;
+  const T* dobase = d_o + (size_t)at.b * Tn * d + (size_t)at.h * dh;
+  const T* obase = o + (size_t)at.b * Tn * d + (size_t)at.h * dh;
+  load_rows<T>(t.ra, t.lr, t.lr, base, ld, at.r0, Tn, dh);
+  load_rows<T>(t.rb, t.lr, t.lr, dobase, (size_t)d, at.r0, Tn, dh);
+  const int row0 = at.r0 + w * RPW;
+  const size_t stat = ((size_t)at.b * H + at.h) * Tn;
+  float L[RPW], D[RPW], acc[RPW][DPL];
 #pragma unroll
-  for (int c = 0; c < DPL; ++c) acc[c] = 0.f;
-  for (int j0 = 0; j0 <= i; j0 += 32) {
-    int j = j0 + lane;
-    float ds = 0.f;
-    if (j <= i) {
-      const T* krow = qkv + ((size_t)b * Tn + j) * ld + d + (size_t)h * dh;
-      const T* vrow = krow + d;
-      float s = dot_row<T>(q_s[wib], krow, dh) * scale;
-      float p = expf(s - L);
-      float dp = dot_row<T>(do_s[wib], vrow, dh);
-      ds = p * (dp - D) * scale;
-    }
-    int cnt = min(32, i - j0 + 1);
-    for (int jj = 0; jj < cnt; ++jj) {
-      float dsj = __shfl_sync(0xffffffffu, ds, jj);
-      const T* krow = qkv + ((size_t)b * Tn + j0 + jj) * ld + d + (size_t)h * dh;
+  for (int r = 0; r < RPW; ++r) {
+    const int i = row0 + r;
+    float s = 0.f;
+    if (i < Tn)
+      for (int c = lane; c < dh; c += 32) s = fmaf(to_f<T>(obase[(size_t)i * d + c]), to_f<T>(dobase[(size_t)i * d + c]), s);
+    D[r] = warp_sum(s);
+    L[r] = i < Tn ? lse[stat + i] : 0.f;
+    if (lane == 0 && i < Tn) rowdot[stat + i] = D[r];
 #pragma unroll
-      for (int c = 0; c < DPL; ++c) {
-        int dim = lane + 32 * c;
-        if (dim < dh) acc[c] = fmaf(dsj, to_f<T>(krow[dim]), acc[c]);
-      }
-    }
+    for (int c = 0; c < DPL; ++c) acc[r][c] = 0.f;
   }
-  T* out = dqkv + ((size_t)b * Tn + i) * ld + (size_t)h * dh;
+  const float* qrows = t.ra + w * RPW * t.lr;
+  const float* dorows = t.rb + w * RPW * t.lr;
+  float* ds_s = t.pa + w * RPW * KT;
+  for (int j0 = 0; j0 <= at.r0 + RT - 1 && j0 < Tn; j0 += KT) {
+    __syncthreads();
+    load_rows<T>(t.a, t.lt, t.lr, base + d, ld, j0, Tn, dh);
+    load_rows<T>(t.b, t.lt, t.lr, base + 2 * (size_t)d, ld, j0, Tn, dh);
+    __syncthreads();
+    if (j0 > row0 + RPW - 1) continue;
+    float s[RPW], dp[RPW];
+    dot4(qrows, t.lr, t.a + lane * t.lt, s);
+    dot4(dorows, t.lr, t.b + lane * t.lt, dp);
 #pragma unroll
-  for (int c = 0; c < DPL; ++c) {
-    int dim = lane + 32 * c;
-    if (dim < dh) out[dim] = from_f<T>(acc[c]);
+    for (int r = 0; r < RPW; ++r) {
+      const bool vis = j0 + lane <= row0 + r && row0 + r < Tn;
+      const float p = vis ? expf(s[r] * scale - L[r]) : 0.f;
+      ds_s[r * KT + lane] = vis ? p * (dp[r] - D[r]) * scale : 0.f;
+    }
+    __syncwarp();
+    accumulate4(acc, ds_s, t.a, t.lt, lane, nfeat);
+    __syncwarp();
+  }
+#pragma unroll
+  for (int r = 0; r < RPW; ++r) {
+    if (row0 + r >= Tn) continue;
+    T* out = dqkv + ((size_t)at.b * Tn + row0 + r) * ld + (size_t)at.h * dh;
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) {
+      const int dim = lane + 32 * c;
+      if (dim < dh) out[dim] = from_f<T>(acc[r][c]);
+    }
   }
 }
 
-// dK, dV: one warp per key row j; loops over queries i >= j.
+// dK, dV: rows are keys, tiles are queries
 template <typename T>
 __global__ void __launch_bounds__(WARPS * 32) attn_bwd_dkv_kernel(const T* __restrict__ qkv, const float* __restrict__ lse,
                                                                   const T* __restrict__ d_o, const float* __restrict__ rowdot,
-                                                                  int nseq, int Tn, int H, int d, T* __restrict__ dqkv) {
+                                                                  int Tn, int H, int d, T* __restrict__ dqkv) {
   overlap_sync();
-  __shared__ float k_s[WARPS][MAX_DH], v_s[WARPS][MAX_DH];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * WARPS + wib;
-  if (w >= (int64_t)nseq * H * Tn) return;
-  const int j = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
-  const int dh = d / H;
+  extern __shared__ __align__(16) float sh[];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, dh = d / H, nfeat = (dh + 31) / 32;
+  const Where at = where(Tn, H);
+  Tiles t(sh, dh);
   const float scale = rsqrtf((float)dh);
   const size_t ld = (size_t)3 * d;
-  const T* krow = qkv + ((size_t)b * Tn + j) * ld + d + (size_t)h * dh;
-  for (int c = lane; c < dh; c += 32) { k_s[wib][c] = to_f<T>(krow[c]); v_s[wib][c] = to_f<T>(krow[d + c]); }
-  __syncwarp();
-  float dk[DPL], dv[DPL];
+  const T* base = qkv + (size_t)at.b * Tn * ld + (size_t)at.h * dh;
+  const T* dobase = d_o + (size_t)at.b * Tn * d + (size_t)at.h * dh;
+  load_rows<T>(t.ra, t.lr, t.lr, base + d, ld, at.r0, Tn, dh);
+  load_rows<T>(t.rb, t.lr, t.lr, base + 2 * (size_t)d, ld, at.r0, Tn, dh);
+  const int row0 = at.r0 + w * RPW;
+  const size_t stat = ((size_t)at.b * H + at.h) * Tn;
+  float dk[RPW][DPL], dv[RPW][DPL];
 #pragma unroll
-  for (int c = 0; c < DPL; ++c) { dk[c] = 0.f; dv[c] = 0.f; }
-  for (int i0 = j; i0 < Tn; i0 += 32) {
-    int i = i0 + lane;
-    float p = 0.f, ds = 0.f;
-    if (i < Tn) {
-      const T* qrow = qkv + ((size_t)b * Tn + i) * ld + (size_t)h * dh;
-      const T* dorow = d_o + ((size_t)b * Tn + i) * d + (size_t)h * dh;
-      float s = dot_row<T>(k_s[wib], qrow, dh) * scale;
-      p = expf(s - lse[((size_t)b * H + h) * Tn + i]);
-      float dp = dot_row<T>(v_s[wib], dorow, dh);
-      ds = p * (dp - rowdot[((size_t)b * H + h) * Tn + i]) * scale;
+  for (int r = 0; r < RPW; ++r)
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) { dk[r][c] = 0.f; dv[r][c] = 0.f; }
+  const float* krows = t.ra + w * RPW * t.lr;
+  const float* vrows = t.rb + w * RPW * t.lr;
+  float* p_s = t.pa + w * RPW * KT;
+  float* ds_s = t.pb + w * RPW * KT;
+  for (int i0 = at.r0; i0 < Tn; i0 += KT) {
+    __syncthreads();
+    load_rows<T>(t.a, t.lt, t.lr, base, ld, i0, Tn, dh);
+    load_rows<T>(t.b, t.lt, t.lr, dobase, (size_t)d, i0, Tn, dh);
+    __syncthreads();
+    const int i = i0 + lane;
+    const float L = i < Tn ? lse[stat + i] : 0.f, D = i < Tn ? rowdot[stat + i] : 0.f;
+    float s[RPW], dp[RPW];
+    dot4(krows, t.lr, t.a + lane * t.lt, s);
+    dot4(vrows, t.lr, t.b + lane * t.lt, dp);
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+      const bool vis = i >= row0 + r && i < Tn;
+      const float p = vis ? expf(s[r] * scale - L) : 0.f;
+      p_s[r * KT + lane] = p;
+      ds_s[r * KT + lane] = vis ? p * (dp[r] - D) * scale : 0.f;
     }
-    int cnt = min(32, Tn - i0);
-    for (int ii = 0; ii < cnt; ++ii) {
-      float pi = __shfl_sync(0xffffffffu, p, ii), dsi = __shfl_sync(0xffffffffu, ds, ii);
-      const T* qrow = qkv + ((size_t)b * Tn + i0 + ii) * ld + (size_t)h * dh;
-      const T* dorow = d_o + ((size_t)b * Tn + i0 + ii) * d + (size_t)h * dh;
+    __syncwarp();
+    accumulate4(dv, p_s, t.b, t.lt, lane, nfeat);
+    accumulate4(dk, ds_s, t.a, t.lt, lane, nfeat);
+    __syncwarp();
+  }
 #pragma unroll
-      for (int c = 0; c < DPL; ++c) {
-        int dim = lane + 32 * c;
-        if (dim < dh) {
-          dv[c] = fmaf(pi, to_f<T>(dorow[dim]), dv[c]);
-          dk[c] = fmaf(dsi, to_f<T>(qrow[dim]), dk[c]);
-        }
-      }
+  for (int r = 0; r < RPW; ++r) {
+    if (row0 + r >= Tn) continue;
+    T* out = dqkv + ((size_t)at.b * Tn + row0 + r) * ld + (size_t)at.h * dh;
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) {
+      const int dim = lane + 32 * c;
+      if (dim < dh) { out[d + dim] = from_f<T>(dk[r][c]); out[2 * (size_t)d + dim] = from_f<T>(dv[r][c]); }
     }
   }
-  T* out = dqkv + ((size_t)b * Tn + j) * ld + (size_t)h * dh;
-#pragma unroll
-  for (int c = 0; c < DPL; ++c) {
-    int dim = lane + 32 * c;
-    if (dim < dh) { out[d + dim] = from_f<T>(dk[c]); out[2 * (size_t)d + dim] = from_f<T>(dv[c]); }
-  }
+}
+
+// room for the widest head, once per device and kernel
+template <typename K> cudaError_t allow_smem(K kernel, PerDeviceOnce& once) {
+  const int dev = current_device();
+  if (!once.needed(dev)) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(MAX_DH));
+  if (e == cudaSuccess) once.done(dev);
+  return e;
+}
+
+template <typename T>
+cudaError_t fwd(const void* qkv, unsigned blocks, int T_, int H, int d, void* o, float* lse, cudaStream_t st) {
+  static PerDeviceOnce once;
+  cudaError_t e = allow_smem(attn_fwd_kernel<T>, once);
+  if (e != cudaSuccess) return e;
+  return launch_in_order(attn_fwd_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, T_, H, d, (T*)o, lse);
+}
+
+template <typename T>
+cudaError_t bwd(const void* qkv, const void* o, const float* lse, const void* d_o, unsigned blocks, int T_, int H, int d,
+                void* dqkv, float* rowdot, cudaStream_t st) {
+  static PerDeviceOnce once_q, once_kv;
+  cudaError_t e = allow_smem(attn_bwd_dq_kernel<T>, once_q);
+  if (e == cudaSuccess) e = allow_smem(attn_bwd_dkv_kernel<T>, once_kv);
+  if (e != cudaSuccess) return e;
+  e = launch_in_order(attn_bwd_dq_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, (const T*)o, lse,
+                      (const T*)d_o, rowdot, T_, H, d, (T*)dqkv);
+  if (e != cudaSuccess) return e;
+  return launch_in_order(attn_bwd_dkv_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, lse, (const T*)d_o,
+                         rowdot, T_, H, d, (T*)dqkv);
+}
+
+bool grid_of(int nseq, int T, int H, int d, unsigned* blocks) {
+  if (d % H != 0 || d / H > MAX_DH) return false;
+  const int64_t n = (int64_t)nseq * H * ((T + RT - 1) / RT);
+  *blocks = (unsigned)n;
+  return n <= 0x7fffffff;
 }
 
 }  // namespace
 
 cudaError_t attention_fwd_simt(int dt, const void* qkv, int nseq, int T, int H, int d, void* o, float* lse,
                                cudaStream_t st) {
-  if (d % H != 0 || d / H > MAX_DH) return cudaErrorInvalidValue;
-  int64_t warps = (int64_t)nseq * H * T;
-  unsigned blocks = (unsigned)((warps + WARPS - 1) / WARPS);
-  if (dt == DT_BF16) launch_in_order(attn_fwd_kernel<bf16>, blocks, WARPS * 32, 0, st, (const bf16*)qkv, nseq, T, H, d, (bf16*)o, lse);
-  else launch_in_order(attn_fwd_kernel<float>, blocks, WARPS * 32, 0, st, (const float*)qkv, nseq, T, H, d, (float*)o, lse);
-  return cudaGetLastError();
+  unsigned blocks;
+  if (!grid_of(nseq, T, H, d, &blocks)) return cudaErrorInvalidValue;
+  return dt == DT_BF16 ? fwd<bf16>(qkv, blocks, T, H, d, o, lse, st) : fwd<float>(qkv, blocks, T, H, d, o, lse, st);
 }
 
 cudaError_t attention_bwd_simt(int dt, const void* qkv, const void* o, const float* lse, const void* d_o,
                                int nseq, int T, int H, int d, void* dqkv, float* rowdot, cudaStream_t st) {
-  if (d % H != 0 || d / H > MAX_DH) return cudaErrorInvalidValue;
-  int64_t warps = (int64_t)nseq * H * T;
-  unsigned blocks = (unsigned)((warps + WARPS - 1) / WARPS);
-  unsigned rb = (unsigned)((warps * 32 + 255) / 256);
-  if (dt == DT_BF16) {
-    launch_in_order(attn_rowdot_kernel<bf16>, rb, 256, 0, st, (const bf16*)o, (const bf16*)d_o, nseq, T, H, d, rowdot);
-    launch_in_order(attn_bwd_dq_kernel<bf16>, blocks, WARPS * 32, 0, st, (const bf16*)qkv, lse, (const bf16*)d_o, rowdot, nseq, T, H, d, (bf16*)dqkv);
-    launch_in_order(attn_bwd_dkv_kernel<bf16>, blocks, WARPS * 32, 0, st, (const bf16*)qkv, lse, (const bf16*)d_o, rowdot, nseq, T, H, d, (bf16*)dqkv);
-  } else {
-    launch_in_order(attn_rowdot_kernel<float>, rb, 256, 0, st, (const float*)o, (const float*)d_o, nseq, T, H, d, rowdot);
-    launch_in_order(attn_bwd_dq_kernel<float>, blocks, WARPS * 32, 0, st, (const float*)qkv, lse, (const float*)d_o, rowdot, nseq, T, H, d, (float*)dqkv);
-    launch_in_order(attn_bwd_dkv_kernel<float>, blocks, WARPS * 32, 0, st, (const float*)qkv, lse, (const float*)d_o, rowdot, nseq, T, H, d, (float*)dqkv);
-  }
-  return cudaGetLastError();
+  unsigned blocks;
+  if (!grid_of(nseq, T, H, d, &blocks)) return cudaErrorInvalidValue;
+  return dt == DT_BF16 ? bwd<bf16>(qkv, o, lse, d_o, blocks, T, H, d, dqkv, rowdot, st)
+                       : bwd<float>(qkv, o, lse, d_o, blocks, T, H, d, dqkv, rowdot, st);
 }
 
 }  // namespace sl

@@ -1,11 +1,12 @@
 // Adapter gradients G_A, G_B (Eq. 4-7): skinny reductions over the tokens of each group,
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c]
 // for nt targets of rank r (R = nt*r weight columns) and C feature columns.  HBM-bound: Z is read
-// once per 4 weight columns.  A block is 64 column threads (one 16-byte vector each) x 4 row lanes
+// once per 4 weight columns.  A block is 64 column threads (one 16-byte vector each) x 4 or 16 row lanes
 // over a chunk of LG_ROWS rows, four blocks per SM so that enough loads are in flight; the row
 // lanes are summed through shared memory, chunk partials go to scratch and a second kernel adds
 // them in chunk order (no float atomics, so the result does not depend on scheduling).
 #include "common.cuh"
+#include "host_common.h"
 #include "kernels.h"
 #include "launch.cuh"
 
@@ -14,7 +15,6 @@ namespace {
 
 constexpr int LG_ROWS = 128;   // rows per chunk; group sizes must be multiples of it
 constexpr int LG_CT = 64;      // column threads per block
-constexpr int LG_RL = 4;       // row lanes per block
 constexpr int RJ = 4;          // weight columns per block
 
 // four consecutive weights of one row
@@ -30,13 +30,15 @@ template <> __device__ __forceinline__ void load4<bf16>(const bf16* p, float* w)
   for (int i = 0; i < 4; ++i) w[i] = __bfloat162float(b[i]);
 }
 
-template <typename T, bool VEC4>
-__global__ void __launch_bounds__(LG_CT * LG_RL, 4)
+// LG_RL: row lanes per block.  Four and four blocks per SM where the chunks fill the chip; sixteen where there are few
+// (fp32, 512 tokens: 8 blocks, whose 32 rows per lane one after another took 17 us).
+template <typename T, bool VEC4, int LG_RL>
+__global__ void __launch_bounds__(LG_CT * LG_RL, LG_RL == 4 ? 4 : 1)
 lora_grad_partial_kernel(const T* __restrict__ Z, int64_t ldz, int zcol0, int C, const T* __restrict__ Wt,
                          int64_t ldwt, int wcol0, int r, int rp, int R, int M, float* __restrict__ partial) {
   overlap_sync();
   constexpr int N = Vec16<T>::N;
-  __shared__ float red[RJ * N][LG_CT];
+  __shared__ float red[LG_RL / 2][RJ * N][LG_CT];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int c = (blockIdx.x * LG_CT + tx) * N;
   const int chunk = blockIdx.y;
@@ -74,20 +76,21 @@ lora_grad_partial_kernel(const T* __restrict__ Z, int64_t ldz, int zcol0, int C,
       }
     }
   }
-  // add row lanes 1..3 into lane 0, one lane at a time (fixed order)
-  for (int lane = 1; lane < LG_RL; ++lane) {
-    if (ty == lane) {
+  // add the row lanes pairwise, upper half onto lower half (a fixed order)
+#pragma unroll
+  for (int half = LG_RL / 2; half > 0; half >>= 1) {
+    if (ty >= half && ty < 2 * half) {
 #pragma unroll
       for (int j = 0; j < RJ; ++j)
 #pragma unroll
-        for (int i = 0; i < N; ++i) red[j * N + i][tx] = acc[j][i];
+        for (int i = 0; i < N; ++i) red[ty - half][j * N + i][tx] = acc[j][i];
     }
     __syncthreads();
-    if (ty == 0) {
+    if (ty < half) {
 #pragma unroll
       for (int j = 0; j < RJ; ++j)
 #pragma unroll
-        for (int i = 0; i < N; ++i) acc[j][i] += red[j * N + i][tx];
+        for (int i = 0; i < N; ++i) acc[j][i] += red[ty][j * N + i][tx];
     }
     __syncthreads();
   }
@@ -187,14 +190,23 @@ void launch_reduce(const float* partial, int r, int R, int C, int cpg, int group
   }
 }
 
+template <typename T, int RL>
+void launch_partial_lanes(dim3 grid, cudaStream_t st, bool vec4, const void* Z, int64_t ldz, int zcol0, int C, const void* Wt,
+                          int64_t ldwt, int wcol0, int r, int rp, int R, int M, float* partial) {
+  dim3 block(LG_CT, RL);
+  if (vec4)
+    launch_in_order(lora_grad_partial_kernel<T, true, RL>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+  else
+    launch_in_order(lora_grad_partial_kernel<T, false, RL>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+}
 template <typename T>
 void launch_partial(dim3 grid, cudaStream_t st, bool vec4, const void* Z, int64_t ldz, int zcol0, int C, const void* Wt,
                     int64_t ldwt, int wcol0, int r, int rp, int R, int M, float* partial) {
-  dim3 block(LG_CT, LG_RL);
-  if (vec4)
-    launch_in_order(lora_grad_partial_kernel<T, true>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
-  else
-    launch_in_order(lora_grad_partial_kernel<T, false>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+  if constexpr (sizeof(T) == 4) {                      // (16 lanes of bf16 vectors do not fit shared memory)
+    if ((int64_t)grid.x * grid.y * grid.z <= num_sms())
+      return launch_partial_lanes<T, 16>(grid, st, vec4, Z, ldz, zcol0, C, Wt, ldwt, wcol0, r, rp, R, M, partial);
+  }
+  launch_partial_lanes<T, 4>(grid, st, vec4, Z, ldz, zcol0, C, Wt, ldwt, wcol0, r, rp, R, M, partial);
 }
 
 }  // namespace

@@ -517,7 +517,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
     if ((e = linear(c, c->has_o ? "lora_linear_bwd" : "linear_bwd", a))) return e; }
   { const bool aligned_form = c->tc && attention_tc_supported(c->dt, T, H, d);
     const bool ragged_form = !aligned_form && c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, c->g_do, c->g_dqkv);
-    Scope s(c, "attention_bwd", ragged_form || (c->tc && attention_t5_supported(c->dt, T, H, d)) ? 2 : 3);
+    Scope s(c, "attention_bwd", aligned_form && !attention_t5_supported(c->dt, T, H, d) ? 3 : 2);
     if (aligned_form)
       e = attention_bwd_tc(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->status, c->st);
     else if (ragged_form)
