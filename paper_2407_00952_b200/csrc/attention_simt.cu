@@ -292,7 +292,7 @@ cudaError_t fwd(const void* qkv, unsigned blocks, int T_, int H, int d, void* o,
   static PerDeviceOnce once;
   cudaError_t e = allow_smem(attn_fwd_kernel<T>, once);
   if (e != cudaSuccess) return e;
-  return launch_in_order(attn_fwd_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, T_, H, d, (T*)o, lse);
+  return launch_overlapped(attn_fwd_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, T_, H, d, (T*)o, lse);
 }
 
 template <typename T>
@@ -302,10 +302,10 @@ cudaError_t bwd(const void* qkv, const void* o, const float* lse, const void* d_
   cudaError_t e = allow_smem(attn_bwd_dq_kernel<T>, once_q);
   if (e == cudaSuccess) e = allow_smem(attn_bwd_dkv_kernel<T>, once_kv);
   if (e != cudaSuccess) return e;
-  e = launch_in_order(attn_bwd_dq_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, (const T*)o, lse,
+  e = launch_overlapped(attn_bwd_dq_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, (const T*)o, lse,
                       (const T*)d_o, rowdot, T_, H, d, (T*)dqkv);
   if (e != cudaSuccess) return e;
-  return launch_in_order(attn_bwd_dkv_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, lse, (const T*)d_o,
+  return launch_overlapped(attn_bwd_dkv_kernel<T>, blocks, WARPS * 32, smem_bytes(d / H), st, (const T*)qkv, lse, (const T*)d_o,
                          rowdot, T_, H, d, (T*)dqkv);
 }
 

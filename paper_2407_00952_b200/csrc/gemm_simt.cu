@@ -232,7 +232,7 @@ cudaError_t launch_f32(const GemmArgs& a, cudaStream_t st) {
     once.done(dev);
   }
   dim3 grid((a.N + C::TN - 1) / C::TN, (a.M + C::TM - 1) / C::TM);
-  return launch_in_order(gemm_f32_kernel<C>, grid, C::THREADS, C::SMEM, st, a);
+  return launch_overlapped(gemm_f32_kernel<C>, grid, C::THREADS, C::SMEM, st, a);
 }
 
 bool f32_vector_ok(const GemmArgs& a) {
@@ -253,8 +253,8 @@ cudaError_t gemm_simt(const GemmArgs& a, cudaStream_t st) {
     return tiles >= num_sms() ? launch_f32<F32Cfg<64, 64, 1, 32>>(a, st) : launch_f32<F32Cfg<32, 32, 4, 64>>(a, st);
   }
   dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM);
-  if (a.dtype == DT_BF16) launch_in_order(gemm_simt_kernel<bf16>, grid, 256, 0, st, a);
-  else launch_in_order(gemm_simt_kernel<float>, grid, 256, 0, st, a);
+  if (a.dtype == DT_BF16) launch_overlapped(gemm_simt_kernel<bf16>, grid, 256, 0, st, a);
+  else launch_overlapped(gemm_simt_kernel<float>, grid, 256, 0, st, a);
   return cudaGetLastError();
 }
 

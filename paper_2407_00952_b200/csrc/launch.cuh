@@ -48,15 +48,4 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// The same launch without the early start, for the plain-FMA kernels: their few long blocks are placed where the kernel
-// before left room, two to an SM, instead of one per SM (the fp32 round of 512 tokens: 980 us, 1,040 us with the early
-// start).
-template <typename... Params, typename... Args>
-inline cudaError_t launch_in_order(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  t_in_chain = true;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 }  // namespace sl

@@ -195,9 +195,9 @@ void launch_partial_lanes(dim3 grid, cudaStream_t st, bool vec4, const void* Z, 
                           int64_t ldwt, int wcol0, int r, int rp, int R, int M, float* partial) {
   dim3 block(LG_CT, RL);
   if (vec4)
-    launch_in_order(lora_grad_partial_kernel<T, true, RL>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+    launch_overlapped(lora_grad_partial_kernel<T, true, RL>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
   else
-    launch_in_order(lora_grad_partial_kernel<T, false, RL>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
+    launch_overlapped(lora_grad_partial_kernel<T, false, RL>, grid, block, 0, st, (const T*)Z, ldz, zcol0, C, (const T*)Wt, ldwt, wcol0, r, rp, R, M, partial);
 }
 template <typename T>
 void launch_partial(dim3 grid, cudaStream_t st, bool vec4, const void* Z, int64_t ldz, int zcol0, int C, const void* Wt,
