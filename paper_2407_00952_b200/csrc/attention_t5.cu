@@ -19,6 +19,9 @@
 // warps 2..9 softmax: two threads per query row (warp w owns accumulator lanes 32*(w%4)..+31, warps
 // 2..5 the first half of the score and output columns, warps 6..9 the second).
 // All mbarrier waits are bounded (see tc_common.cuh); on expiry a code is left in `status`.
+// The producer and issuer roles run as converged warps with one elected lane issuing (see gemm_tc.cu); at head width 128
+// the issue of the products was what a step waited for: 8 sequences of 1024, 32 heads, 172 -> 157 us (backward 327 -> 304;
+// head width 64, 64 sequences of 512, 16 heads: 94 -> 91.6 and 209 -> 202).
 #include "host_common.h"
 #include "launch.cuh"
 #include "tc_common.cuh"
@@ -125,66 +128,68 @@ attn_fwd_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_cons
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int it = 0;                                   // running step index of the K loads issued
       auto load_K = [&](int step, int j, int h, int seq_row0) -> bool {
         const int s = step & 1;
-        if (!mbar_wait(B(K_EMPTY + s), (((uint32_t)(step >> 1)) & 1u) ^ 1u, abort_flag, p.status, 21)) return false;
-        mbar_expect_tx(B(K_FULL + s), NB * TILE);
+        if (!mbar_wait_warp(B(K_EMPTY + s), (((uint32_t)(step >> 1)) & 1u) ^ 1u, abort_flag, p.status, 21)) return false;
+        if (leader) mbar_expect_tx(B(K_FULL + s), NB * TILE);
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
-          tma_load_2d(base + OFF_K + (s * NB + nb) * TILE, &mapQKV, B(K_FULL + s), p.d + h * DH + 64 * nb, seq_row0 + j * BKV);
+          if (leader) tma_load_2d(base + OFF_K + (s * NB + nb) * TILE, &mapQKV, B(K_FULL + s), p.d + h * DH + 64 * nb, seq_row0 + j * BKV);
         return true;
       };
       for (int tq = 0; tq < my_tiles && ok; ++tq) {
         const int qt = qt_of(tq);
         const int h = head_of(tq), seq_row0 = row0_of(tq);
         // Q of this query tile (the buffer is free once the previous tile's last S product is done)
-        if (!mbar_wait(B(Q_EMPTY), ((uint32_t)tq & 1u) ^ 1u, abort_flag, p.status, 20)) { ok = false; break; }
-        mbar_expect_tx(B(Q_FULL), NB * TILE);
+        if (!mbar_wait_warp(B(Q_EMPTY), ((uint32_t)tq & 1u) ^ 1u, abort_flag, p.status, 20)) { ok = false; break; }
+        if (leader) mbar_expect_tx(B(Q_FULL), NB * TILE);
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
-          tma_load_2d(base + OFF_Q + nb * TILE, &mapQKV, B(Q_FULL), h * DH + 64 * nb, seq_row0 + qt * BQ);
+          if (leader) tma_load_2d(base + OFF_Q + nb * TILE, &mapQKV, B(Q_FULL), h * DH + 64 * nb, seq_row0 + qt * BQ);
         if (tq == 0) ok = load_K(0, 0, h, seq_row0);   // K runs one step ahead of V
         for (int j = 0; j <= qt && ok; ++j, ++it) {
           // next step's K: the next key tile, or key tile 0 of the next query tile (maybe of the next item)
           if (j < qt) ok = load_K(it + 1, j + 1, h, seq_row0);
           else if (tq + 1 < my_tiles) ok = load_K(it + 1, 0, head_of(tq + 1), row0_of(tq + 1));
           if (!ok) break;
-          if (!mbar_wait(B(V_EMPTY), ((uint32_t)it & 1u) ^ 1u, abort_flag, p.status, 22)) { ok = false; break; }
-          mbar_expect_tx(B(V_FULL), NB * TILE);
+          if (!mbar_wait_warp(B(V_EMPTY), ((uint32_t)it & 1u) ^ 1u, abort_flag, p.status, 22)) { ok = false; break; }
+          if (leader) mbar_expect_tx(B(V_FULL), NB * TILE);
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb)
-            tma_load_2d(base + OFF_V + nb * TILE, &mapQKV, B(V_FULL), 2 * p.d + h * DH + 64 * nb, seq_row0 + j * BKV);
+            if (leader) tma_load_2d(base + OFF_V + nb * TILE, &mapQKV, B(V_FULL), 2 * p.d + h * DH + 64 * nb, seq_row0 + j * BKV);
         }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       const uint32_t lo_q = desc_lo(base + OFF_Q), lo_k0 = desc_lo(base + OFF_K), lo_v = desc_lo(base + OFF_V);
       constexpr uint32_t TILE16 = TILE >> 4;
       // S of step `step`; first_of_q: wait for the query tile iq; last_of_q: release the Q buffer
       auto issue_S = [&](int step, int tq, bool first_of_q, bool last_of_q) -> bool {
         const int s = step & 1;
-        if (first_of_q && !mbar_wait(B(Q_FULL), (uint32_t)tq & 1u, abort_flag, p.status, 25)) return false;
-        if (!mbar_wait(B(K_FULL + s), (uint32_t)(step >> 1) & 1u, abort_flag, p.status, 23)) return false;
-        if (!mbar_wait(B(S_FREE), ((uint32_t)step & 1u) ^ 1u, abort_flag, p.status, 24)) return false;
+        if (first_of_q && !mbar_wait_warp(B(Q_FULL), (uint32_t)tq & 1u, abort_flag, p.status, 25)) return false;
+        if (!mbar_wait_warp(B(K_FULL + s), (uint32_t)(step >> 1) & 1u, abort_flag, p.status, 23)) return false;
+        if (!mbar_wait_warp(B(S_FREE), ((uint32_t)step & 1u) ^ 1u, abort_flag, p.status, 24)) return false;
         tc_fence_after();
         const uint32_t lo_k = lo_k0 + (uint32_t)(s * NB) * TILE16;
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {                    // 64 features per block; 16 elements = +32 bytes = +2 units
           const uint32_t a = lo_q + (uint32_t)nb * TILE16, bq = lo_k + (uint32_t)nb * TILE16;
-          tc_mma_lo(tS, a, bq, IDESC_S, nb != 0 ? 1u : 0u);
-          tc_mma_lo_acc(tS, a + 2, bq + 2, IDESC_S);
-          tc_mma_lo_acc(tS, a + 4, bq + 4, IDESC_S);
-          tc_mma_lo_acc(tS, a + 6, bq + 6, IDESC_S);
+          if (leader) tc_mma_lo(tS, a, bq, IDESC_S, nb != 0 ? 1u : 0u);
+          if (leader) tc_mma_lo_acc(tS, a + 2, bq + 2, IDESC_S);
+          if (leader) tc_mma_lo_acc(tS, a + 4, bq + 4, IDESC_S);
+          if (leader) tc_mma_lo_acc(tS, a + 6, bq + 6, IDESC_S);
         }
-        tc_commit(B(K_EMPTY + s));
-        if (last_of_q) tc_commit(B(Q_EMPTY));
-        tc_commit(B(S_FULL));
+        if (leader) tc_commit(B(K_EMPTY + s));
+        if (last_of_q) if (leader) tc_commit(B(Q_EMPTY));
+        if (leader) tc_commit(B(S_FULL));
         return true;
       };
       int it = 0;
@@ -196,10 +201,10 @@ attn_fwd_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_cons
           if (j < qt) ok = issue_S(it + 1, tq, false, j + 1 == qt);
           else if (tq + 1 < my_tiles) ok = issue_S(it + 1, tq + 1, true, qt_of(tq + 1) == 0);
           if (!ok) break;
-          if (!mbar_wait(B(P_READY), (uint32_t)it & 1u, abort_flag, p.status, 26)) { ok = false; break; }
-          if (!mbar_wait(B(V_FULL), (uint32_t)it & 1u, abort_flag, p.status, 27)) { ok = false; break; }
+          if (!mbar_wait_warp(B(P_READY), (uint32_t)it & 1u, abort_flag, p.status, 26)) { ok = false; break; }
+          if (!mbar_wait_warp(B(V_FULL), (uint32_t)it & 1u, abort_flag, p.status, 27)) { ok = false; break; }
           // the first product of a query tile overwrites O: the previous tile's O must have been read
-          if (j == 0 && !mbar_wait(B(O_FREE), ((uint32_t)tq & 1u) ^ 1u, abort_flag, p.status, 28)) { ok = false; break; }
+          if (j == 0 && !mbar_wait_warp(B(O_FREE), ((uint32_t)tq & 1u) ^ 1u, abort_flag, p.status, 28)) { ok = false; break; }
           tc_fence_after();
           // P is read from tensor memory (16 keys = 8 columns per product);
           // V advances 16 key rows = 2048 bytes = 128 units per product
@@ -207,10 +212,10 @@ attn_fwd_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_cons
           for (int nb = 0; nb < NB; ++nb)                    // one 64-column block of O per block of V
 #pragma unroll
             for (int k = 0; k < BKV / UMMA_K; ++k)
-              tc_mma_ts_lo(tO + (uint32_t)(64 * nb), tP + (uint32_t)(8 * k), lo_v + (uint32_t)nb * TILE16 + (uint32_t)(128 * k),
+              if (leader) tc_mma_ts_lo(tO + (uint32_t)(64 * nb), tP + (uint32_t)(8 * k), lo_v + (uint32_t)nb * TILE16 + (uint32_t)(128 * k),
                            IDESC_PV, (j | k) != 0 ? 1u : 0u);
-          tc_commit(B(V_EMPTY));      // V (and P) reusable
-          tc_commit(B(O_FULL));       // this step's contribution is in O
+          if (leader) tc_commit(B(V_EMPTY));      // V (and P) reusable
+          if (leader) tc_commit(B(O_FULL));       // this step's contribution is in O
         }
       }
     }

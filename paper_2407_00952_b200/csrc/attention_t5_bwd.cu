@@ -310,7 +310,8 @@ attn_bwd_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_
   const uint32_t tPT = ALIAS ? tS : tmem_base + 384u, tDST = ALIAS ? tDP : tmem_base + 448u;
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int s = 0, n = 0;                            // ring stage and how often it has been used
       for (int tk = 0; tk < my_tiles && ok; ++tk) {
@@ -320,25 +321,25 @@ attn_bwd_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_
         const size_t stat0 = ((size_t)b * p.H + h) * p.T;
         (void)seq_row0; (void)stat0;
         const int kb = tk % KVB;
-        if (!mbar_wait(B(KV_EMPTY + kb), freed(tk / KVB), abort_flag, p.status, 41)) { ok = false; break; }
-        mbar_expect_tx(B(KV_FULL + kb), 2 * NB * TILE);
+        if (!mbar_wait_warp(B(KV_EMPTY + kb), freed(tk / KVB), abort_flag, p.status, 41)) { ok = false; break; }
+        if (leader) mbar_expect_tx(B(KV_FULL + kb), 2 * NB * TILE);
         const uint32_t kv = base + OFF_KV + kb * 2 * NB * TILE;
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
-          tma_load_2d(kv + nb * TILE, &mapQKV, B(KV_FULL + kb), p.d + h * DHT + 64 * nb, seq_row0 + kt * BT);
-          tma_load_2d(kv + (NB + nb) * TILE, &mapQKV, B(KV_FULL + kb), 2 * p.d + h * DHT + 64 * nb, seq_row0 + kt * BT);
+          if (leader) tma_load_2d(kv + nb * TILE, &mapQKV, B(KV_FULL + kb), p.d + h * DHT + 64 * nb, seq_row0 + kt * BT);
+          if (leader) tma_load_2d(kv + (NB + nb) * TILE, &mapQKV, B(KV_FULL + kb), 2 * p.d + h * DHT + 64 * nb, seq_row0 + kt * BT);
         }
         for (int i = kt; i < nq; ++i) {
-          if (!mbar_wait(B(QD_EMPTY + s), freed(n), abort_flag, p.status, 42)) { ok = false; break; }
-          mbar_expect_tx(B(QD_FULL + s), 2 * NB * TILE + 1024);
+          if (!mbar_wait_warp(B(QD_EMPTY + s), freed(n), abort_flag, p.status, 42)) { ok = false; break; }
+          if (leader) mbar_expect_tx(B(QD_FULL + s), 2 * NB * TILE + 1024);
           const uint32_t qd = base + OFF_QD + s * 2 * NB * TILE;
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb) {
-            tma_load_2d(qd + nb * TILE, &mapQKV, B(QD_FULL + s), h * DHT + 64 * nb, seq_row0 + i * BT);
-            tma_load_2d(qd + (NB + nb) * TILE, &mapDO, B(QD_FULL + s), h * DHT + 64 * nb, seq_row0 + i * BT);
+            if (leader) tma_load_2d(qd + nb * TILE, &mapQKV, B(QD_FULL + s), h * DHT + 64 * nb, seq_row0 + i * BT);
+            if (leader) tma_load_2d(qd + (NB + nb) * TILE, &mapDO, B(QD_FULL + s), h * DHT + 64 * nb, seq_row0 + i * BT);
           }
-          bulk_load(base + OFF_STAT + s * 1024, p.lse + stat0 + (size_t)i * BT, 512, B(QD_FULL + s));
-          bulk_load(base + OFF_STAT + s * 1024 + 512, p.rowdot + stat0 + (size_t)i * BT, 512, B(QD_FULL + s));
+          if (leader) bulk_load(base + OFF_STAT + s * 1024, p.lse + stat0 + (size_t)i * BT, 512, B(QD_FULL + s));
+          if (leader) bulk_load(base + OFF_STAT + s * 1024 + 512, p.rowdot + stat0 + (size_t)i * BT, 512, B(QD_FULL + s));
           if (++s == RINGN) { s = 0; ++n; }
         }
       }
@@ -350,7 +351,8 @@ attn_bwd_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_
     // computed while the element-wise warps still work on this step's second.  The accumulating
     // products are issued by another thread (warp ACC_WARP): one thread cannot issue 32 products of
     // 48 cycles each per step next to the busy element-wise warps.
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int it = 0, s = 0, n = 0;
       const uint32_t lo_kv = desc_lo(base + OFF_KV), lo_qd = desc_lo(base + OFF_QD), lo_aug = desc_lo_aug(base + OFF_AUG);
@@ -363,38 +365,39 @@ attn_bwd_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_
         (void)seq_row0; (void)stat0;
         const int kb = tk % KVB;
         const uint32_t lo_k = lo_kv + (uint32_t)(kb * 2 * NB) * TILE16, lo_v = lo_k + (uint32_t)NB * TILE16;
-        if (!mbar_wait(B(KV_FULL + kb), done(tk / KVB), abort_flag, p.status, 45)) { ok = false; break; }
+        if (!mbar_wait_warp(B(KV_FULL + kb), done(tk / KVB), abort_flag, p.status, 45)) { ok = false; break; }
         for (int i = kt; i < nq && ok; ++i, ++it) {
           const uint32_t lo_q = lo_qd + (uint32_t)(s * 2 * NB) * TILE16, lo_do = lo_q + (uint32_t)NB * TILE16;
-          if (!mbar_wait(B(QD_FULL + s), done(n), abort_flag, p.status, 43)) { ok = false; break; }
-          if (AUG && !mbar_wait(B(AUG_READY + s), done(n), abort_flag, p.status, 52)) { ok = false; break; }
+          if (!mbar_wait_warp(B(QD_FULL + s), done(n), abort_flag, p.status, 43)) { ok = false; break; }
+          if (AUG && !mbar_wait_warp(B(AUG_READY + s), done(n), abort_flag, p.status, 52)) { ok = false; break; }
           const uint32_t lo_aq = lo_aug + (uint32_t)((2 + s) * AUG_TILE >> 4);      // this stage's -lse/scale, -D rows
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
             // the half's columns are free once read (own P^T columns) or, where P^T and dS^T lie on
             // top of them, once the accumulating products of the previous step have used those
-            if (!mbar_wait(B((ALIAS ? P_FREE : S_FREE) + hh), freed(it), abort_flag, p.status, 44)) { ok = false; break; }
+            if (!mbar_wait_warp(B((ALIAS ? P_FREE : S_FREE) + hh), freed(it), abort_flag, p.status, 44)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)           // contraction over the head's features, 64 per block
-              mma_score_half(tS + 64u * hh, lo_k + (uint32_t)nb * TILE16, lo_q + (uint32_t)nb * TILE16, hh, nb == 0);
+              if (leader) mma_score_half(tS + 64u * hh, lo_k + (uint32_t)nb * TILE16, lo_q + (uint32_t)nb * TILE16, hh, nb == 0);
             // one more step: ones x (-lse/scale) of the half's 64 queries (8 row groups = 2048 bytes per half)
-            if (AUG) tc_mma_aug(tS + 64u * hh, lo_aug, lo_aq + (uint32_t)(128 * hh), IDESC_64KK);
+            if (AUG) if (leader) tc_mma_aug(tS + 64u * hh, lo_aug, lo_aq + (uint32_t)(128 * hh), IDESC_64KK);
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)
-              mma_score_half(tDP + 64u * hh, lo_v + (uint32_t)nb * TILE16, lo_do + (uint32_t)nb * TILE16, hh, nb == 0);
-            if (AUG) tc_mma_aug(tDP + 64u * hh, lo_aug + (uint32_t)(AUG_TILE >> 4), lo_aq + (uint32_t)(128 * hh), IDESC_64KK);
-            tc_commit(B(S_FULL + hh));
+              if (leader) mma_score_half(tDP + 64u * hh, lo_v + (uint32_t)nb * TILE16, lo_do + (uint32_t)nb * TILE16, hh, nb == 0);
+            if (AUG) if (leader) tc_mma_aug(tDP + 64u * hh, lo_aug + (uint32_t)(AUG_TILE >> 4), lo_aq + (uint32_t)(128 * hh), IDESC_64KK);
+            if (leader) tc_commit(B(S_FULL + hh));
           }
-          if (ok) tc_commit(B(QD_EMPTY + s));        // second arrival comes from the accumulating thread
+          if (ok) if (leader) tc_commit(B(QD_EMPTY + s));        // second arrival comes from the accumulating thread
           if (++s == RINGN) { s = 0; ++n; }
         }
-        if (ok) tc_commit(B(KV_EMPTY + kb));         // K, V are read by these products only
+        if (ok) if (leader) tc_commit(B(KV_EMPTY + kb));         // K, V are read by these products only
       }
     }
   } else if (warp == ACC_WARP) {
     // ---------------- accumulating products: dV += P^T dO, dK += dS^T Q ----------------
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int it = 0, s = 0, n = 0;
       const uint32_t lo_qd = desc_lo(base + OFF_QD);
@@ -406,26 +409,26 @@ attn_bwd_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_
         const size_t stat0 = ((size_t)b * p.H + h) * p.T;
         (void)seq_row0; (void)stat0;
         // the accumulators of the previous key tile must have been read
-        if (!mbar_wait(B(ACC_FREE), freed(tk), abort_flag, p.status, 46)) { ok = false; break; }
+        if (!mbar_wait_warp(B(ACC_FREE), freed(tk), abort_flag, p.status, 46)) { ok = false; break; }
         for (int i = kt; i < nq && ok; ++i, ++it) {
           const uint32_t lo_q = lo_qd + (uint32_t)(s * 2 * NB) * TILE16, lo_do = lo_q + (uint32_t)NB * TILE16;
-          if (!mbar_wait(B(QD_FULL + s), done(n), abort_flag, p.status, 43)) { ok = false; break; }
+          if (!mbar_wait_warp(B(QD_FULL + s), done(n), abort_flag, p.status, 43)) { ok = false; break; }
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            if (!mbar_wait(B(P_READY + hh), done(it), abort_flag, p.status, 47)) { ok = false; break; }
+            if (!mbar_wait_warp(B(P_READY + hh), done(it), abort_flag, p.status, 47)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)           // one 64-column block of dV per block of dO
-              mma_acc_half<ALIAS>(tDV + 64u * nb, tPT, lo_do + (uint32_t)nb * TILE16, hh, i == kt && hh == 0);
+              if (leader) mma_acc_half<ALIAS>(tDV + 64u * nb, tPT, lo_do + (uint32_t)nb * TILE16, hh, i == kt && hh == 0);
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)
-              mma_acc_half<ALIAS>(tDK + 64u * nb, tDST, lo_q + (uint32_t)nb * TILE16, hh, i == kt && hh == 0);
-            tc_commit(B(P_FREE + hh));
+              if (leader) mma_acc_half<ALIAS>(tDK + 64u * nb, tDST, lo_q + (uint32_t)nb * TILE16, hh, i == kt && hh == 0);
+            if (leader) tc_commit(B(P_FREE + hh));
           }
-          if (ok) tc_commit(B(QD_EMPTY + s));
+          if (ok) if (leader) tc_commit(B(QD_EMPTY + s));
           if (++s == RINGN) { s = 0; ++n; }
         }
-        if (ok) tc_commit(B(ACC_FULL));
+        if (ok) if (leader) tc_commit(B(ACC_FULL));
       }
     }
   } else if (warp < ACC_WARP) {
@@ -676,7 +679,8 @@ attn_bwd_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_c
 
   // query tiles are walked from the last (most key tiles) to the first
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int s = 0, n = 0;
       for (int tq = 0; tq < my_tiles && ok; ++tq) {
@@ -686,23 +690,23 @@ attn_bwd_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_c
         const size_t stat0 = ((size_t)b * p.H + h) * p.T;
         (void)seq_row0; (void)stat0;
         const int i = nq - 1 - qi, qb = tq % QOB;
-        if (!mbar_wait(B(QO_EMPTY + qb), freed(tq / QOB), abort_flag, p.status, 61)) { ok = false; break; }
-        mbar_expect_tx(B(QO_FULL + qb), QO_TILES * TILE);
+        if (!mbar_wait_warp(B(QO_EMPTY + qb), freed(tq / QOB), abort_flag, p.status, 61)) { ok = false; break; }
+        if (leader) mbar_expect_tx(B(QO_FULL + qb), QO_TILES * TILE);
         const uint32_t qo = base + OFF_QO + qb * QO_TILES * TILE;
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
-          tma_load_2d(qo + nb * TILE, &mapQKV, B(QO_FULL + qb), h * DHT + 64 * nb, seq_row0 + i * BT);
-          tma_load_2d(qo + (NB + nb) * TILE, &mapDO, B(QO_FULL + qb), h * DHT + 64 * nb, seq_row0 + i * BT);
-          if (HAS_O) tma_load_2d(qo + (2 * NB + nb) * TILE, &mapO, B(QO_FULL + qb), h * DHT + 64 * nb, seq_row0 + i * BT);
+          if (leader) tma_load_2d(qo + nb * TILE, &mapQKV, B(QO_FULL + qb), h * DHT + 64 * nb, seq_row0 + i * BT);
+          if (leader) tma_load_2d(qo + (NB + nb) * TILE, &mapDO, B(QO_FULL + qb), h * DHT + 64 * nb, seq_row0 + i * BT);
+          if (HAS_O) if (leader) tma_load_2d(qo + (2 * NB + nb) * TILE, &mapO, B(QO_FULL + qb), h * DHT + 64 * nb, seq_row0 + i * BT);
         }
         for (int j = 0; j <= i; ++j) {
-          if (!mbar_wait(B(KV_EMPTY + s), freed(n), abort_flag, p.status, 62)) { ok = false; break; }
-          mbar_expect_tx(B(KV_FULL + s), 2 * NB * TILE);
+          if (!mbar_wait_warp(B(KV_EMPTY + s), freed(n), abort_flag, p.status, 62)) { ok = false; break; }
+          if (leader) mbar_expect_tx(B(KV_FULL + s), 2 * NB * TILE);
           const uint32_t kv = base + OFF_KV + s * 2 * NB * TILE;
 #pragma unroll
           for (int nb = 0; nb < NB; ++nb) {
-            tma_load_2d(kv + nb * TILE, &mapQKV, B(KV_FULL + s), p.d + h * DHT + 64 * nb, seq_row0 + j * BT);
-            tma_load_2d(kv + (NB + nb) * TILE, &mapQKV, B(KV_FULL + s), 2 * p.d + h * DHT + 64 * nb, seq_row0 + j * BT);
+            if (leader) tma_load_2d(kv + nb * TILE, &mapQKV, B(KV_FULL + s), p.d + h * DHT + 64 * nb, seq_row0 + j * BT);
+            if (leader) tma_load_2d(kv + (NB + nb) * TILE, &mapQKV, B(KV_FULL + s), 2 * p.d + h * DHT + 64 * nb, seq_row0 + j * BT);
           }
           if (++s == RINGN) { s = 0; ++n; }
         }
@@ -710,7 +714,8 @@ attn_bwd_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_c
     }
   } else if (warp == 1) {
     // ---------------- score products: S = Q K^T, dP = dO V^T, in halves of 64 key columns ----------------
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int it = 0, s = 0, n = 0;
       const uint32_t lo_qo = desc_lo(base + OFF_QO), lo_kv = desc_lo(base + OFF_KV), lo_aug = desc_lo_aug(base + OFF_AUG);
@@ -724,50 +729,51 @@ attn_bwd_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_c
         const int steps = nq - qi;               // key tiles 0 .. i, i = nq-1-qi
         const int qb = tq % QOB;
         const uint32_t lo_q = lo_qo + (uint32_t)(qb * QO_TILES) * TILE16, lo_do = lo_q + (uint32_t)NB * TILE16;
-        if (!mbar_wait(B(QO_FULL + qb), done(tq / QOB), abort_flag, p.status, 65)) { ok = false; break; }
+        if (!mbar_wait_warp(B(QO_FULL + qb), done(tq / QOB), abort_flag, p.status, 65)) { ok = false; break; }
         const uint32_t lo_aq = lo_aug + (uint32_t)((1 + qb) * AUG_TILE >> 4);       // this tile's -lse/scale, -D rows
         for (int st = 0; st < steps && ok; ++st, ++it) {
           const uint32_t lo_k = lo_kv + (uint32_t)(s * 2 * NB) * TILE16;
-          if (!mbar_wait(B(KV_FULL + s), done(n), abort_flag, p.status, 63)) { ok = false; break; }
+          if (!mbar_wait_warp(B(KV_FULL + s), done(n), abort_flag, p.status, 63)) { ok = false; break; }
           // The rows with -lse/scale and -D are written by the statistics warp once Q, dO and O have arrived.
           // In a tile's first step both halves' products over the features are issued before that is waited
           // for, so the statistics are computed while the tensor pipe already works on the tile.
           const bool late_aug = AUG && st == 0;
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            if (!mbar_wait(B(S_FREE + hh), freed(it), abort_flag, p.status, 64)) { ok = false; break; }
+            if (!mbar_wait_warp(B(S_FREE + hh), freed(it), abort_flag, p.status, 64)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)           // contraction over the head's features, 64 per block
-              mma_score_half(tS + 64u * hh, lo_q + (uint32_t)nb * TILE16, lo_k + (uint32_t)nb * TILE16, hh, nb == 0);
+              if (leader) mma_score_half(tS + 64u * hh, lo_q + (uint32_t)nb * TILE16, lo_k + (uint32_t)nb * TILE16, hh, nb == 0);
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)
-              mma_score_half(tDP + 64u * hh, lo_do + (uint32_t)nb * TILE16, lo_k + (uint32_t)(NB + nb) * TILE16, hh, nb == 0);
+              if (leader) mma_score_half(tDP + 64u * hh, lo_do + (uint32_t)nb * TILE16, lo_k + (uint32_t)(NB + nb) * TILE16, hh, nb == 0);
             if (AUG && !late_aug) {
               // one more step: (-lse/scale of the queries) x ones, then (-D) x ones
-              tc_mma_aug(tS + 64u * hh, lo_aq, lo_aug, IDESC_64KK);
-              tc_mma_aug(tDP + 64u * hh, lo_aq, lo_aug + (uint32_t)(AUG_TILE / 2 >> 4), IDESC_64KK);
+              if (leader) tc_mma_aug(tS + 64u * hh, lo_aq, lo_aug, IDESC_64KK);
+              if (leader) tc_mma_aug(tDP + 64u * hh, lo_aq, lo_aug + (uint32_t)(AUG_TILE / 2 >> 4), IDESC_64KK);
             }
-            if (!late_aug) tc_commit(B(S_FULL + hh));
+            if (!late_aug) if (leader) tc_commit(B(S_FULL + hh));
           }
           if (ok && late_aug) {
-            if (!mbar_wait(B(AUG_READY + qb), done(tq / QOB), abort_flag, p.status, 72)) { ok = false; break; }
+            if (!mbar_wait_warp(B(AUG_READY + qb), done(tq / QOB), abort_flag, p.status, 72)) { ok = false; break; }
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-              tc_mma_aug(tS + 64u * hh, lo_aq, lo_aug, IDESC_64KK);
-              tc_mma_aug(tDP + 64u * hh, lo_aq, lo_aug + (uint32_t)(AUG_TILE / 2 >> 4), IDESC_64KK);
-              tc_commit(B(S_FULL + hh));
+              if (leader) tc_mma_aug(tS + 64u * hh, lo_aq, lo_aug, IDESC_64KK);
+              if (leader) tc_mma_aug(tDP + 64u * hh, lo_aq, lo_aug + (uint32_t)(AUG_TILE / 2 >> 4), IDESC_64KK);
+              if (leader) tc_commit(B(S_FULL + hh));
             }
           }
-          if (ok) tc_commit(B(KV_EMPTY + s));        // second arrival comes from the accumulating thread
+          if (ok) if (leader) tc_commit(B(KV_EMPTY + s));        // second arrival comes from the accumulating thread
           if (++s == RINGN) { s = 0; ++n; }
         }
-        if (ok) tc_commit(B(QO_EMPTY + qb));         // Q, dO are read by these products only
+        if (ok) if (leader) tc_commit(B(QO_EMPTY + qb));         // Q, dO are read by these products only
       }
     }
   } else if (warp == ACC_WARP) {
     // ---------------- accumulating products: dQ += dS K ----------------
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int it = 0, s = 0, n = 0;
       const uint32_t lo_kv = desc_lo(base + OFF_KV);
@@ -779,23 +785,23 @@ attn_bwd_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_c
         const size_t stat0 = ((size_t)b * p.H + h) * p.T;
         (void)seq_row0; (void)stat0;
         const int steps = nq - qi;
-        if (!mbar_wait(B(ACC_FREE), freed(tq), abort_flag, p.status, 66)) { ok = false; break; }
+        if (!mbar_wait_warp(B(ACC_FREE), freed(tq), abort_flag, p.status, 66)) { ok = false; break; }
         for (int st = 0; st < steps && ok; ++st, ++it) {
           const uint32_t lo_k = lo_kv + (uint32_t)(s * 2 * NB) * TILE16;
-          if (!mbar_wait(B(KV_FULL + s), done(n), abort_flag, p.status, 63)) { ok = false; break; }
+          if (!mbar_wait_warp(B(KV_FULL + s), done(n), abort_flag, p.status, 63)) { ok = false; break; }
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            if (!mbar_wait(B(P_READY + hh), done(it), abort_flag, p.status, 67)) { ok = false; break; }
+            if (!mbar_wait_warp(B(P_READY + hh), done(it), abort_flag, p.status, 67)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)           // one 64-column block of dQ per block of K
-              mma_acc_half(tDQ + 64u * nb, tDS, lo_k + (uint32_t)nb * TILE16, hh, st == 0 && hh == 0);
-            tc_commit(B(P_FREE + hh));
+              if (leader) mma_acc_half(tDQ + 64u * nb, tDS, lo_k + (uint32_t)nb * TILE16, hh, st == 0 && hh == 0);
+            if (leader) tc_commit(B(P_FREE + hh));
           }
-          if (ok) tc_commit(B(KV_EMPTY + s));
+          if (ok) if (leader) tc_commit(B(KV_EMPTY + s));
           if (++s == RINGN) { s = 0; ++n; }
         }
-        if (ok) tc_commit(B(ACC_FULL));
+        if (ok) if (leader) tc_commit(B(ACC_FULL));
       }
     }
   } else if (warp < ACC_WARP) {

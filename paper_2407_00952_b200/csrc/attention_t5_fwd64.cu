@@ -121,24 +121,25 @@ attn_fwd_t5_h64_kernel(const __grid_constant__ CUtensorMap mapQKV, F64Params p) 
 
   if (warp == 0) {
     // ---------------- TMA producer: Q per query tile (two buffers), K and V per 128 keys (two stages) ----------------
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       int ks = 0;                                   // 128-key steps issued so far
       for (int tq = 0; tq < my_tiles && ok; ++tq) {
         const int qt = qt_of(tq), h = head_of(tq), seq_row0 = row0_of(tq);
         const int qs = tq & 1;
-        if (!mbar_wait(B(Q_EMPTY + qs), (((uint32_t)(tq >> 1)) & 1u) ^ 1u, abort_flag, p.status, 20)) { ok = false; break; }
-        mbar_expect_tx(B(Q_FULL + qs), TILE);
-        tma_load_2d(base + OFF_Q + qs * TILE, &mapQKV, B(Q_FULL + qs), h * DH, seq_row0 + qt * BQ);
+        if (!mbar_wait_warp(B(Q_EMPTY + qs), (((uint32_t)(tq >> 1)) & 1u) ^ 1u, abort_flag, p.status, 20)) { ok = false; break; }
+        if (leader) mbar_expect_tx(B(Q_FULL + qs), TILE);
+        if (leader) tma_load_2d(base + OFF_Q + qs * TILE, &mapQKV, B(Q_FULL + qs), h * DH, seq_row0 + qt * BQ);
         for (int j = 0; j <= qt && ok; ++j, ++ks) {
           const int s = ks & 1;
           const uint32_t par = (((uint32_t)(ks >> 1)) & 1u) ^ 1u;
-          if (!mbar_wait(B(K_EMPTY + s), par, abort_flag, p.status, 21)) { ok = false; break; }
-          mbar_expect_tx(B(K_FULL + s), TILE);
-          tma_load_2d(base + OFF_K + s * TILE, &mapQKV, B(K_FULL + s), p.d + h * DH, seq_row0 + j * BKV);
-          if (!mbar_wait(B(V_EMPTY + s), par, abort_flag, p.status, 22)) { ok = false; break; }
-          mbar_expect_tx(B(V_FULL + s), TILE);
-          tma_load_2d(base + OFF_V + s * TILE, &mapQKV, B(V_FULL + s), 2 * p.d + h * DH, seq_row0 + j * BKV);
+          if (!mbar_wait_warp(B(K_EMPTY + s), par, abort_flag, p.status, 21)) { ok = false; break; }
+          if (leader) mbar_expect_tx(B(K_FULL + s), TILE);
+          if (leader) tma_load_2d(base + OFF_K + s * TILE, &mapQKV, B(K_FULL + s), p.d + h * DH, seq_row0 + j * BKV);
+          if (!mbar_wait_warp(B(V_EMPTY + s), par, abort_flag, p.status, 22)) { ok = false; break; }
+          if (leader) mbar_expect_tx(B(V_FULL + s), TILE);
+          if (leader) tma_load_2d(base + OFF_V + s * TILE, &mapQKV, B(V_FULL + s), 2 * p.d + h * DH, seq_row0 + j * BKV);
         }
       }
     }
@@ -146,7 +147,8 @@ attn_fwd_t5_h64_kernel(const __grid_constant__ CUtensorMap mapQKV, F64Params p) 
     // ---------------- MMA issuer ----------------
     // Half-steps are numbered `it` over the CTA's whole work; S(it) goes to score buffer it & 1, P(it)
     // comes from P buffer it & 1.  Issue order: S(0), S(1), then PV(it), S(it + 2) for it = 0, 1, ...
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       bool ok = true;
       const uint32_t lo_q0 = desc_lo(base + OFF_Q), lo_k0 = desc_lo(base + OFF_K), lo_v0 = desc_lo(base + OFF_V);
       constexpr uint32_t TILE16 = TILE >> 4;
@@ -156,20 +158,20 @@ attn_fwd_t5_h64_kernel(const __grid_constant__ CUtensorMap mapQKV, F64Params p) 
         if (s_tq >= my_tiles) return true;
         const int qt = qt_of(s_tq), nhs = 2 * (qt + 1);
         const int half = s_hs & 1, st = s_ks & 1, sb = s_it & 1, qs = s_tq & 1;
-        if (s_hs == 0 && !mbar_wait(B(Q_FULL + qs), (uint32_t)(s_tq >> 1) & 1u, abort_flag, p.status, 25)) return false;
-        if (half == 0 && !mbar_wait(B(K_FULL + st), (uint32_t)(s_ks >> 1) & 1u, abort_flag, p.status, 23)) return false;
-        if (!mbar_wait(B(S_FREE + sb), (((uint32_t)(s_it >> 1)) & 1u) ^ 1u, abort_flag, p.status, 24)) return false;
+        if (s_hs == 0 && !mbar_wait_warp(B(Q_FULL + qs), (uint32_t)(s_tq >> 1) & 1u, abort_flag, p.status, 25)) return false;
+        if (half == 0 && !mbar_wait_warp(B(K_FULL + st), (uint32_t)(s_ks >> 1) & 1u, abort_flag, p.status, 23)) return false;
+        if (!mbar_wait_warp(B(S_FREE + sb), (((uint32_t)(s_it >> 1)) & 1u) ^ 1u, abort_flag, p.status, 24)) return false;
         tc_fence_after();
         const uint32_t a = lo_q0 + (uint32_t)qs * TILE16;
         const uint32_t b = lo_k0 + (uint32_t)st * TILE16 + (uint32_t)half * 512u;     // 64 key rows = 8192 bytes
         const uint32_t d = tS + (uint32_t)(sb * HK);
-        tc_mma_lo(d, a, b, IDESC_S, 0u);
-        tc_mma_lo_acc(d, a + 2, b + 2, IDESC_S);
-        tc_mma_lo_acc(d, a + 4, b + 4, IDESC_S);
-        tc_mma_lo_acc(d, a + 6, b + 6, IDESC_S);
-        if (half == 1) tc_commit(B(K_EMPTY + st));
-        if (s_hs == nhs - 1) tc_commit(B(Q_EMPTY + qs));
-        tc_commit(B(S_FULL + sb));
+        if (leader) tc_mma_lo(d, a, b, IDESC_S, 0u);
+        if (leader) tc_mma_lo_acc(d, a + 2, b + 2, IDESC_S);
+        if (leader) tc_mma_lo_acc(d, a + 4, b + 4, IDESC_S);
+        if (leader) tc_mma_lo_acc(d, a + 6, b + 6, IDESC_S);
+        if (half == 1) if (leader) tc_commit(B(K_EMPTY + st));
+        if (s_hs == nhs - 1) if (leader) tc_commit(B(Q_EMPTY + qs));
+        if (leader) tc_commit(B(S_FULL + sb));
         ++s_it;
         if (half == 1) ++s_ks;
         if (++s_hs == nhs) { s_hs = 0; ++s_tq; }
@@ -181,18 +183,18 @@ attn_fwd_t5_h64_kernel(const __grid_constant__ CUtensorMap mapQKV, F64Params p) 
         const int nhs = 2 * (qt_of(tq) + 1);
         for (int hs = 0; hs < nhs && ok; ++hs, ++it) {
           const int half = hs & 1, st = ks & 1, pb = it & 1;
-          if (!mbar_wait(B(P_READY + pb), (uint32_t)(it >> 1) & 1u, abort_flag, p.status, 26)) { ok = false; break; }
-          if (half == 0 && !mbar_wait(B(V_FULL + st), (uint32_t)(ks >> 1) & 1u, abort_flag, p.status, 27)) { ok = false; break; }
+          if (!mbar_wait_warp(B(P_READY + pb), (uint32_t)(it >> 1) & 1u, abort_flag, p.status, 26)) { ok = false; break; }
+          if (half == 0 && !mbar_wait_warp(B(V_FULL + st), (uint32_t)(ks >> 1) & 1u, abort_flag, p.status, 27)) { ok = false; break; }
           // the first product of a query tile overwrites O: the previous tile's O must have been read
-          if (hs == 0 && !mbar_wait(B(O_FREE), ((uint32_t)tq & 1u) ^ 1u, abort_flag, p.status, 28)) { ok = false; break; }
+          if (hs == 0 && !mbar_wait_warp(B(O_FREE), ((uint32_t)tq & 1u) ^ 1u, abort_flag, p.status, 28)) { ok = false; break; }
           tc_fence_after();
           const uint32_t v = lo_v0 + (uint32_t)st * TILE16 + (uint32_t)half * 512u;   // 64 key rows = 8192 bytes
           const uint32_t a = tP + (uint32_t)(pb * 32);
 #pragma unroll
           for (int k = 0; k < HK / UMMA_K; ++k)       // 16 keys = 8 columns of P = 2048 bytes of V per product
-            tc_mma_ts_lo(tO, a + (uint32_t)(8 * k), v + (uint32_t)(128 * k), IDESC_PV, (hs | k) != 0 ? 1u : 0u);
-          tc_commit(B(P_FREE + pb));                  // also says: O holds the products up to this half-step
-          if (half == 1) { tc_commit(B(V_EMPTY + st)); ++ks; }
+            if (leader) tc_mma_ts_lo(tO, a + (uint32_t)(8 * k), v + (uint32_t)(128 * k), IDESC_PV, (hs | k) != 0 ? 1u : 0u);
+          if (leader) tc_commit(B(P_FREE + pb));                  // also says: O holds the products up to this half-step
+          if (half == 1) { if (leader) tc_commit(B(V_EMPTY + st)); ++ks; }
           ok = issue_S();                             // the score product two half-steps ahead
         }
       }
