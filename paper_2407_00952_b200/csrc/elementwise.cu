@@ -3,6 +3,7 @@
 // client-side aggregation of Eq. 8-9, adapter compute copies and transposes.
 // All global accesses are 16-byte vectors where the layout allows; reductions use warp shuffles.
 #include "common.cuh"
+#include "host_common.h"
 #include "kernels.h"
 #include "launch.cuh"
 
@@ -362,7 +363,10 @@ __device__ __forceinline__ float ce_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__global__ void __launch_bounds__(256)
+// The second pass is the last reader of the logits and its output goes to a product far larger than L2: both bypass
+// it, so that rows still to be read again stay.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 2048 / THREADS)
 ce_bf16_kernel(bf16* __restrict__ logits, int64_t ld, const int32_t* __restrict__ labels, int V,
                float* __restrict__ row_loss, const int* __restrict__ n_valid) {
   overlap_sync();
@@ -430,7 +434,7 @@ ce_bf16_kernel(bf16* __restrict__ logits, int64_t ld, const int32_t* __restrict_
   const float inv = (valid && nv > 0) ? 1.0f / (float)nv : 0.f;
   const float nl = -lse * L;
   for (int i = threadIdx.x; i < nfull; i += blockDim.x) {
-    const uint4 raw = zv[i];
+    const uint4 raw = __ldcs(zv + i);
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&raw);
     uint4 out;
     uint32_t* o = reinterpret_cast<uint32_t*>(&out);
@@ -441,7 +445,7 @@ ce_bf16_kernel(bf16* __restrict__ logits, int64_t ld, const int32_t* __restrict_
       __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
       o[k] = *reinterpret_cast<uint32_t*>(&pb);
     }
-    zv[i] = out;
+    __stcs(zv + i, out);
   }
   for (int c = 8 * nfull + threadIdx.x; c < 8 * nvec; c += blockDim.x)    // last valid columns, then the pad
     z[c] = __float2bfloat16_rn(c < V ? __expf(__bfloat162float(z[c]) - lse) * inv : 0.f);
@@ -470,8 +474,18 @@ __global__ void loss_reduce_kernel(const float* __restrict__ row_loss, int M, co
 cudaError_t cross_entropy(int dt, void* logits, int64_t ld, const int32_t* labels, int M, int V, float* row_loss,
                           int* n_valid, float* loss, int normalizer_override, cudaStream_t st) {
   launch_overlapped(count_valid_kernel, 1, 1024, 0, st, labels, M, V, n_valid, normalizer_override);
-  if (dt == DT_BF16 && ld % 8 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0)
-    launch_overlapped(ce_bf16_kernel, M, 256, 0, st, (bf16*)logits, ld, labels, V, row_loss, n_valid);
+  if (dt == DT_BF16 && ld % 8 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0) {
+    // 256 threads per row, eight rows per SM; twice the threads (half the rows in flight) where eight rows per SM would
+    // crowd each other out of L2 before their second read, or where there are not eight rows per SM.  us, 256 threads
+    // without the cache hints -> this: 16384 rows of 50257 770 -> 650, 32768 1600 -> 1500, 8192 rows of 32000 250 -> 243,
+    // 512 of 50257 34 -> 31 (512 threads on the 32000-wide rows: 265; the row held in shared memory, two blocks per SM:
+    // 680-730, 1500-1800 and 320).
+    const int64_t sms = num_sms(), rows = M < 8 * sms ? M : 8 * sms;
+    if (rows * ld * 2 > 96000000 || M <= 4 * sms)
+      launch_overlapped(ce_bf16_kernel<512>, M, 512, 0, st, (bf16*)logits, ld, labels, V, row_loss, n_valid);
+    else
+      launch_overlapped(ce_bf16_kernel<256>, M, 256, 0, st, (bf16*)logits, ld, labels, V, row_loss, n_valid);
+  }
   else if (dt == DT_BF16) launch_overlapped(ce_kernel<bf16>, M, 256, 0, st, (bf16*)logits, ld, labels, V, row_loss, n_valid);
   else launch_overlapped(ce_kernel<float>, M, 256, 0, st, (float*)logits, ld, labels, V, row_loss, n_valid);
   launch_overlapped(loss_reduce_kernel, 1, 1024, 0, st, row_loss, M, n_valid, loss);
