@@ -284,7 +284,8 @@ int splitlora_profile_report(splitlora_ctx* ctx, char (*names)[48], int64_t* lau
 /* Grouped LoRA linear forward (Sec. II-C applied to G adapters over one shared frozen W):
  *   y[m,:] = x[m,:] W^T + bias + (alpha/r) (x[m,:] A_g^T) B_g^T,  g = m / (M/G)
  * x [M, in], W [out, in], bias [out] or NULL, y [M, out] in `dtype`; A [G, r, in], B [G, out, r] fp32.
- * M % G == 0; in bf16 mode M/G % 128 == 0, in % 64 == 0, out % 8 == 0. */
+ * M % G == 0, M/G % 128 == 0 when G > 1; in and out multiples of 8.  Every such shape runs on the tensor cores
+ * in bf16 mode. */
 int splitlora_lora_linear_workspace_bytes(int dtype, int M, int n_in, int n_out, int r, int G, size_t* bytes);
 int splitlora_lora_linear_fwd(int dtype, int use_tensor_cores, const void* x, const void* W, const void* bias,
                               const float* A, const float* B, float alpha, int M, int n_in, int n_out,
