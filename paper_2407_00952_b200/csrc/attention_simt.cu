@@ -61,10 +61,11 @@ __device__ __forceinline__ void dot4(const float* rows, int lr, const float* til
   }
 }
 
-// acc[r][c] += sum_j p[r][j] * tile[j][lane + 32 c]
-__device__ __forceinline__ void accumulate4(float (*acc)[DPL], const float* p, const float* tile, int lt, int lane, int nfeat) {
+// acc[r][c] += sum over j0 <= j < j1 (multiples of 4) of p[r][j] * tile[j][lane + 32 c]
+__device__ __forceinline__ void accumulate4(float (*acc)[DPL], const float* p, const float* tile, int lt, int lane, int nfeat,
+                                            int j0, int j1) {
 #pragma unroll 2
-  for (int j = 0; j < KT; j += 4) {
+  for (int j = j0; j < j1; j += 4) {
     float4 pv[RPW];
 #pragma unroll
     for (int r = 0; r < RPW; ++r) pv[r] = *reinterpret_cast<const float4*>(p + r * KT + j);
@@ -78,6 +79,40 @@ __device__ __forceinline__ void accumulate4(float (*acc)[DPL], const float* p, c
         acc[r][c] = fmaf(pv[r].w, v3, fmaf(pv[r].z, v2, fmaf(pv[r].y, v1, fmaf(pv[r].x, v0, acc[r][c]))));
     }
   }
+}
+
+// The 4 x 4 block of the diagonal tile in which the warp's four rows meet their own positions: row r takes the tile rows
+// up to the r-th (keys, UP_TO) or from the r-th on (queries).  The pairs that causality hides are left out of the sums
+// and not multiplied by a probability of 0, which would turn an inf or NaN of a later key (an earlier query) into NaN.
+template <bool UP_TO>
+__device__ __forceinline__ void accumulate_diagonal(float (*acc)[DPL], const float* p, const float* tile, int lt, int lane,
+                                                    int nfeat, int j) {
+#pragma unroll
+  for (int c = 0; c < DPL; ++c) {
+    if (c >= nfeat) break;
+#pragma unroll
+    for (int jj = 0; jj < RPW; ++jj) {
+      const float v = tile[(j + jj) * lt + lane + 32 * c];
+#pragma unroll
+      for (int r = 0; r < RPW; ++r)
+        if (UP_TO ? jj <= r : jj >= r) acc[r][c] = fmaf(p[r * KT + j + jj], v, acc[r][c]);
+    }
+  }
+}
+
+// What the warp's rows (the w-th four of the block) see of a tile: all of it, or on the diagonal the part up to / from
+// their own positions.  Both tile sizes are the same, so the diagonal tile starts where the block's rows do.
+static_assert(RT == KT && RPW == 4, "");
+template <bool UP_TO>
+__device__ __forceinline__ void accumulate_tile(float (*acc)[DPL], const float* p, const float* tile, int lt, int lane,
+                                                int nfeat, bool diagonal, int w) {
+  if (!diagonal) {
+    accumulate4(acc, p, tile, lt, lane, nfeat, 0, KT);
+    return;
+  }
+  if (UP_TO) accumulate4(acc, p, tile, lt, lane, nfeat, 0, w * RPW);
+  accumulate_diagonal<UP_TO>(acc, p, tile, lt, lane, nfeat, w * RPW);
+  if (!UP_TO) accumulate4(acc, p, tile, lt, lane, nfeat, (w + 1) * RPW, KT);
 }
 
 struct Where { int b, h, r0; };
@@ -114,7 +149,6 @@ __global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restric
     load_rows<T>(t.a, t.lt, t.lr, base + d, ld, j0, Tn, dh);
     load_rows<T>(t.b, t.lt, t.lr, base + 2 * (size_t)d, ld, j0, Tn, dh);
     __syncthreads();
-    if (j0 > row0 + RPW - 1) continue;                 // nothing of this tile is visible to the warp's rows
     float s[RPW];
     dot4(rows, t.lr, t.a + lane * t.lt, s);
 #pragma unroll
@@ -122,10 +156,8 @@ __global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restric
       const bool vis = j0 + lane <= row0 + r;
       const float sc = vis ? s[r] * scale : -INFINITY;
       const float nm = fmaxf(m[r], warp_max(sc));
-      // a row that has seen no key yet in this tile keeps its state (its maximum is still -inf)
-      const bool none = j0 > row0 + r;
       const float p = vis ? expf(sc - nm) : 0.f;
-      const float corr = (none || m[r] == -INFINITY) ? (none ? 1.f : 0.f) : expf(m[r] - nm);
+      const float corr = m[r] == -INFINITY ? 0.f : expf(m[r] - nm);
       l[r] = l[r] * corr + warp_sum(p);
 #pragma unroll
       for (int c = 0; c < DPL; ++c) acc[r][c] *= corr;
@@ -133,7 +165,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_fwd_kernel(const T* __restric
       p_s[r * KT + lane] = p;
     }
     __syncwarp();
-    accumulate4(acc, p_s, t.b, t.lt, lane, nfeat);
+    accumulate_tile<true>(acc, p_s, t.b, t.lt, lane, nfeat, j0 == at.r0, w);
     __syncwarp();
   }
 #pragma unroll
@@ -191,7 +223,6 @@ __global__ void __launch_bounds__(WARPS * 32) attn_bwd_dq_kernel(const T* __rest
     load_rows<T>(t.a, t.lt, t.lr, base + d, ld, j0, Tn, dh);
     load_rows<T>(t.b, t.lt, t.lr, base + 2 * (size_t)d, ld, j0, Tn, dh);
     __syncthreads();
-    if (j0 > row0 + RPW - 1) continue;
     float s[RPW], dp[RPW];
     dot4(qrows, t.lr, t.a + lane * t.lt, s);
     dot4(dorows, t.lr, t.b + lane * t.lt, dp);
@@ -202,7 +233,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_bwd_dq_kernel(const T* __rest
       ds_s[r * KT + lane] = vis ? p * (dp[r] - D[r]) * scale : 0.f;
     }
     __syncwarp();
-    accumulate4(acc, ds_s, t.a, t.lt, lane, nfeat);
+    accumulate_tile<true>(acc, ds_s, t.a, t.lt, lane, nfeat, j0 == at.r0, w);
     __syncwarp();
   }
 #pragma unroll
@@ -262,8 +293,8 @@ __global__ void __launch_bounds__(WARPS * 32) attn_bwd_dkv_kernel(const T* __res
       ds_s[r * KT + lane] = vis ? p * (dp[r] - D) * scale : 0.f;
     }
     __syncwarp();
-    accumulate4(dv, p_s, t.b, t.lt, lane, nfeat);
-    accumulate4(dk, ds_s, t.a, t.lt, lane, nfeat);
+    accumulate_tile<false>(dv, p_s, t.b, t.lt, lane, nfeat, i0 == at.r0, w);
+    accumulate_tile<false>(dk, ds_s, t.a, t.lt, lane, nfeat, i0 == at.r0, w);
     __syncwarp();
   }
 #pragma unroll
