@@ -350,7 +350,9 @@ int splitlora_transpose(int dtype, const void* in, int rows, int cols, void* out
 int splitlora_aggregate_buffers(float* params, int K, int64_t P, const double* weights, void* stream);
 
 /* Causal multi-head attention on a fused qkv buffer [nseq*T, 3d] -> o [nseq*T, d], lse [nseq, H, T] fp32
- * (natural-log sum of exp of the scaled scores), and its backward -> dqkv [nseq*T, 3d]. */
+ * (natural-log sum of exp of the scaled scores), and its backward -> dqkv [nseq*T, 3d].
+ * An inf or NaN reaches the positions that see it and no others, except on the bf16 tensor-core kernels for
+ * head widths 64 and 128 at T a multiple of 64: there it may also make NaN of the other rows of its 64- or 128-row tile. */
 int splitlora_attention_fwd(int dtype, int use_tensor_cores, const void* qkv, int nseq, int T, int n_head,
                             int d_model, void* o, float* lse, void* stream);
 int splitlora_attention_bwd(int dtype, int use_tensor_cores, const void* qkv, const void* o, const float* lse,

@@ -17,6 +17,7 @@
 //             kernel per key tile (loops over query tiles).  No atomics: results are bit-reproducible.
 // Products use mma.sync m16n8k16 with ldmatrix-fed fragments from XOR-swizzled shared tiles.
 
+#include "attention_rows.cuh"
 #include "common.cuh"
 #include "host_common.h"
 #include "kernels.h"
@@ -170,6 +171,35 @@ template <int N> __device__ __forceinline__ void zero_acc(float (*a)[4]) {
     for (int j = 0; j < 4; ++j) a[i][j] = 0.f;
 }
 
+// A product with a 64-row tile multiplies the zero probability of a hidden pair with whatever the tile holds (0 x inf =
+// NaN), and an inf with hi + lo where lo may be negative.  So in the RG forms a warp whose results are not all finite does its rows
+// again, one by one in plain FMA over the visible pairs, which is how these shapes see values that are not finite
+// everywhere else.  Finite rounds pay for a test of the results as they are stored.
+// non-zero where one of two bf16 values is an inf or NaN (all exponent bits set)
+__device__ __forceinline__ uint32_t not_finite(uint32_t two) { return ((two & 0x7f807f80u) + 0x00800080u) & 0x80008000u; }
+__device__ __forceinline__ void redo_forward(const bf16* qkv, bf16* o, float* lse, int b, int h, int row, int end, int T, int H, int d, float* s) {
+  const rows::Head<bf16> hd(qkv, b, h, T, H, d);
+  for (; row < end; ++row)
+    rows::forward_row<bf16>(hd, row, s, o + ((size_t)b * T + row) * d + (size_t)h * hd.dh, lse + ((size_t)b * H + h) * T + row);
+}
+__device__ __forceinline__ void redo_dq(const bf16* qkv, const bf16* d_o, const float* lse, const float* rowdot, bf16* dqkv, int b, int h, int row,
+                                     int end, int T, int H, int d, float* s) {
+  const rows::Head<bf16> hd(qkv, b, h, T, H, d);
+  for (; row < end; ++row) {
+    const size_t stat = ((size_t)b * H + h) * T + row;
+    rows::dq_row<bf16>(hd, d_o + ((size_t)b * T + row) * d + (size_t)h * hd.dh, lse[stat], rowdot[stat], row, s,
+                       dqkv + ((size_t)b * T + row) * hd.ld + (size_t)h * hd.dh);
+  }
+}
+__device__ __forceinline__ void redo_dkv(const bf16* qkv, const bf16* d_o, const float* lse, const float* rowdot, bf16* dqkv, int b, int h, int row,
+                                      int end, int T, int H, int d, float* s) {
+  const rows::Head<bf16> hd(qkv, b, h, T, H, d);
+  const size_t stat = ((size_t)b * H + h) * T;
+  for (; row < end; ++row)
+    rows::dkv_row<bf16>(hd, d_o + (size_t)b * T * d + (size_t)h * hd.dh, lse + stat, rowdot + stat, row, s,
+                        dqkv + ((size_t)b * T + row) * hd.ld + d + (size_t)h * hd.dh);
+}
+
 // ------------------------------------------------------------------------------------------
 // forward
 // ------------------------------------------------------------------------------------------
@@ -255,16 +285,23 @@ __global__ void __launch_bounds__(NT, DH > 64 ? 1 : 3) attn_fwd_tc_kernel(const 
   bf16* o0 = o + ((size_t)b * T + (size_t)qt * BT + r0) * d + (size_t)h * dh;
   bf16* o1 = o + ((size_t)b * T + (size_t)qt * BT + r1) * d + (size_t)h * dh;
   const bool v0 = !RG || qt * BT + r0 < T, v1 = !RG || qt * BT + r1 < T;
+  uint32_t bad = 0;
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) {
     if (RG && n * 8 >= dh) break;
-    if (v0) *reinterpret_cast<uint32_t*>(o0 + n * 8 + 2 * t) = pack2(oacc[n][0] * i0, oacc[n][1] * i0);
-    if (v1) *reinterpret_cast<uint32_t*>(o1 + n * 8 + 2 * t) = pack2(oacc[n][2] * i1, oacc[n][3] * i1);
+    const uint32_t w0 = pack2(oacc[n][0] * i0, oacc[n][1] * i0), w1 = pack2(oacc[n][2] * i1, oacc[n][3] * i1);
+    if (v0) *reinterpret_cast<uint32_t*>(o0 + n * 8 + 2 * t) = w0;
+    if (v1) *reinterpret_cast<uint32_t*>(o1 + n * 8 + 2 * t) = w1;
+    if (RG) bad |= not_finite(w0) | not_finite(w1);
   }
   if (t == 0) {
     float* lrow = lse + ((size_t)b * H + h) * T + (size_t)qt * BT;
     if (v0) lrow[r0] = RG ? fmaf(m0, scale, logf(l0)) : (m0 + log2f(l0)) * LN2;
     if (v1) lrow[r1] = RG ? fmaf(m1, scale, logf(l1)) : (m1 + log2f(l1)) * LN2;
+  }
+  if (RG && __any_sync(0xffffffffu, bad != 0)) {
+    const int row = qt * BT + warp * 16;
+    redo_forward(qkv, o, lse, b, h, row, min(row + 16, T), T, H, d, reinterpret_cast<float*>(smem) + warp * 2 * dh);
   }
 }
 
@@ -301,7 +338,7 @@ __global__ void attn_rowdot_tc_kernel(const bf16* __restrict__ o, const bf16* __
 // RG: the kernel also forms D[row] = sum(dO * O) of its own rows (two threads per row) and leaves it in
 // `rowdot` for the dK/dV kernel, which runs second; otherwise a small kernel has put it there beforehand.
 template <int DH, bool RG>
-__global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ o,
+__global__ void __launch_bounds__(NT, RG ? (DH > 64 ? 1 : 3) : 0) attn_bwd_dq_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ o,
                                                             const bf16* __restrict__ d_o, const float* __restrict__ lse,
                                                             float* __restrict__ rowdot, bf16* __restrict__ dqkv, int T,
                                                             int H, int d, int dh, float scale) {
@@ -389,11 +426,18 @@ __global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restri
   }
   bf16* q0 = dqkv + ((size_t)b * T + (size_t)qt * BT + r0) * ld + (size_t)h * dh;
   bf16* q1 = dqkv + ((size_t)b * T + (size_t)qt * BT + r1) * ld + (size_t)h * dh;
+  uint32_t bad = 0;
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) {
     if (RG && n * 8 >= dh) break;
-    if (v0) *reinterpret_cast<uint32_t*>(q0 + n * 8 + 2 * t) = pack2(dq[n][0] * scale, dq[n][1] * scale);
-    if (v1) *reinterpret_cast<uint32_t*>(q1 + n * 8 + 2 * t) = pack2(dq[n][2] * scale, dq[n][3] * scale);
+    const uint32_t w0 = pack2(dq[n][0] * scale, dq[n][1] * scale), w1 = pack2(dq[n][2] * scale, dq[n][3] * scale);
+    if (v0) *reinterpret_cast<uint32_t*>(q0 + n * 8 + 2 * t) = w0;
+    if (v1) *reinterpret_cast<uint32_t*>(q1 + n * 8 + 2 * t) = w1;
+    if (RG) bad |= not_finite(w0) | not_finite(w1);
+  }
+  if (RG && __any_sync(0xffffffffu, bad != 0)) {
+    const int row = qt * BT + warp * 16;
+    redo_dq(qkv, d_o, lse, rowdot, dqkv, b, h, row, min(row + 16, T), T, H, d, reinterpret_cast<float*>(smem) + warp * 2 * dh);
   }
 }
 
@@ -403,7 +447,7 @@ __global__ void __launch_bounds__(NT) attn_bwd_dq_tc_kernel(const bf16* __restri
 // the next product needs as its left operand.
 // ------------------------------------------------------------------------------------------
 template <int DH, bool RG>
-__global__ void __launch_bounds__(NT) attn_bwd_dkv_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ d_o,
+__global__ void __launch_bounds__(NT, RG ? (DH > 64 ? 1 : DH > 32 ? 2 : 3) : 0) attn_bwd_dkv_tc_kernel(const bf16* __restrict__ qkv, const bf16* __restrict__ d_o,
                                                              const float* __restrict__ lse, const float* __restrict__ rowdot,
                                                              bf16* __restrict__ dqkv, int T, int H, int d, int dh,
                                                              float scale) {
@@ -480,17 +524,25 @@ __global__ void __launch_bounds__(NT) attn_bwd_dkv_tc_kernel(const bf16* __restr
   bf16* k0 = dqkv + ((size_t)b * T + (size_t)kt * BT + r0) * ld + d + (size_t)h * dh;
   bf16* k1 = dqkv + ((size_t)b * T + (size_t)kt * BT + r1) * ld + d + (size_t)h * dh;
   const bool v0 = !RG || kt * BT + r0 < T, v1 = !RG || kt * BT + r1 < T;
+  uint32_t bad = 0;
 #pragma unroll
   for (int n = 0; n < DH / 8; ++n) {
     if (RG && n * 8 >= dh) break;
+    const uint32_t w0 = pack2(dk[n][0] * scale, dk[n][1] * scale), w1 = pack2(dk[n][2] * scale, dk[n][3] * scale);
+    const uint32_t x0 = pack2(dv[n][0], dv[n][1]), x1 = pack2(dv[n][2], dv[n][3]);
     if (v0) {
-      *reinterpret_cast<uint32_t*>(k0 + n * 8 + 2 * t) = pack2(dk[n][0] * scale, dk[n][1] * scale);
-      *reinterpret_cast<uint32_t*>(k0 + d + n * 8 + 2 * t) = pack2(dv[n][0], dv[n][1]);
+      *reinterpret_cast<uint32_t*>(k0 + n * 8 + 2 * t) = w0;
+      *reinterpret_cast<uint32_t*>(k0 + d + n * 8 + 2 * t) = x0;
     }
     if (v1) {
-      *reinterpret_cast<uint32_t*>(k1 + n * 8 + 2 * t) = pack2(dk[n][2] * scale, dk[n][3] * scale);
-      *reinterpret_cast<uint32_t*>(k1 + d + n * 8 + 2 * t) = pack2(dv[n][2], dv[n][3]);
+      *reinterpret_cast<uint32_t*>(k1 + n * 8 + 2 * t) = w1;
+      *reinterpret_cast<uint32_t*>(k1 + d + n * 8 + 2 * t) = x1;
     }
+    if (RG) bad |= not_finite(w0) | not_finite(w1) | not_finite(x0) | not_finite(x1);
+  }
+  if (RG && __any_sync(0xffffffffu, bad != 0)) {
+    const int row = kt * BT + warp * 16;
+    redo_dkv(qkv, d_o, lse, rowdot, dqkv, b, h, row, min(row + 16, T), T, H, d, reinterpret_cast<float*>(smem) + warp * 2 * dh);
   }
 }
 

@@ -47,8 +47,8 @@ def _same(got, ref, tol):
 
 @pytest.mark.parametrize("where", ["q", "k", "v", "do"])
 @pytest.mark.parametrize("value", [math.inf, -math.inf, math.nan])
-@pytest.mark.parametrize("T,dh", [(70, 24), (64, 64), (33, 5), (9, 128)])
-@pytest.mark.parametrize("dtype,use_tc", [(torch.float32, False), (torch.bfloat16, False)])
+@pytest.mark.parametrize("T,dh", [(70, 24), (64, 40), (33, 5), (9, 128), (100, 64)])
+@pytest.mark.parametrize("dtype,use_tc", [(torch.float32, False), (torch.bfloat16, False), (torch.bfloat16, True)])
 def test_non_finite_values_reach_what_sees_them_only(T, dh, dtype, use_tc, value, where):
     nseq, H = 2, 2
     d = H * dh
