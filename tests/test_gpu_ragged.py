@@ -40,10 +40,8 @@ def test_attention_any_length_and_width(T, dh):
         dqkv = B.attention_bwd(qkv, o, lse, do, nseq, T, H, use_tensor_cores=tc)
         errs.append([_norm_err(a, r) for a, r in zip((o, lse, dqkv), ref)])
     assert B.library_status() == 0
-    # lse is an fp32 result: half a unit in its last place, and as much again for every 16-deep step of a score's
-    # accumulation, which the tensor core rounds towards zero (at most one unit of the partial sum per step)
-    lse_bound = (1 + (dh + 15) // 16) * 2.0 ** -24
-    for got, plain, bound in zip(*errs, (2e-6, lse_bound, 2e-6)):
+    # lse is an fp32 result: no further off either, up to one rounding of the result (few values at the short lengths)
+    for got, plain, bound in zip(*errs, (2e-6, 2.0 ** -24, 2e-6)):
         assert got <= 1.02 * plain + bound, errs
     static = B.attention_bwd_static(qkv, o, lse, do, nseq, T, H)
     assert torch.equal(static, B.attention_bwd(qkv, o, lse, do, nseq, T, H))
