@@ -757,8 +757,8 @@ bool prepare(const GemmArgs& a, int* status, int w_box_rows, CUtensorMap* mX, CU
   p->w_group_rows = a.w_grouped ? a.N : 0;
   p->we_group_rows = a.we_grouped ? a.N : 0;
   p->epi = a.epi; p->gelu_tanh = a.gelu_tanh;
-  // Off the tile sizes these layers are otherwise computed with tanhf (gemm_simt.cu): they keep that accuracy here
-  // (two special-function instructions per element instead of one).
+  // Off the tile sizes these layers used to be computed with tanhf (gemm_simt.cu): they keep fp32 accuracy here (see
+  // gelu_sigmoid), for two special-function instructions per element instead of one.
   p->gelu_exact = a.gelu_tanh && (a.M % BM != 0 || a.K % BK != 0);
   p->bias = (const bf16*)a.bias; p->R = (const bf16*)a.R; p->ldr = a.ldr;
   p->Y = (bf16*)a.Y; p->ldy = a.ldy; p->Z = (bf16*)a.Z; p->ldz = a.ldz;

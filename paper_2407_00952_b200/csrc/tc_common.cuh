@@ -30,7 +30,7 @@ struct TcParams {
   int we_group_rows;              // rows between groups in We
   int tiles_m, tiles_n;
   int epi, gelu_tanh;
-  int gelu_exact;                 // tanh to fp32 accuracy instead of tanh.approx (see gemm_tc.cu, prepare)
+  int gelu_exact;                 // fp32 accuracy instead of tanh.approx (see gemm_tc.cu, prepare)
   const bf16* bias;
   const bf16* R; long long ldr;
   bf16* Y; long long ldy;
@@ -294,17 +294,27 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 __device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t w) {
   return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
-// tanh as 1 - 2 / (1 + e^2x): two special-function instructions, absolute error of a few 2^-24 (tanh.approx: 2^-11)
-__device__ __forceinline__ float tanh_exact(float x) { return 1.0f - __fdividef(2.0f, 1.0f + __expf(2.0f * x)); }
+// Tanh-form GELU without the 2^-11 of tanh.approx: 0.5 (1 + tanh u) = 1 / (1 + e^-2u) =: s, from e = e^-|2u| <= 1 as
+// q = 1 / (1 + e) or e q, and s (1 - s) = e q^2.  Nothing cancels and nothing overflows, so s is good to a few 2^-23 of
+// itself also where it is tiny (1 + tanhf(u) there has an error of 2^-25 of one).  Two special-function instructions.
+__device__ __forceinline__ void gelu_sigmoid(float z, float& s, float& ds) {
+  constexpr float C1 = (float)(2.0 * 0.7978845608028654 * 1.4426950408889634), C2 = (float)(2.0 * 0.7978845608028654 * 0.044715 * 1.4426950408889634);
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-fabsf(z * fmaf(C2, z * z, C1))));
+  const float q = __fdividef(1.0f, 1.0f + e), eq = e * q;
+  s = z < 0.f ? eq : q;
+  ds = eq * q;
+}
 __device__ __forceinline__ float gelu_tanh_exact(float z) {
-  const float hz = 0.5f * z;
-  return fmaf(hz, tanh_exact(z * fmaf(0.7978845608028654f * 0.044715f, z * z, 0.7978845608028654f)), hz);
+  float s, ds;
+  gelu_sigmoid(z, s, ds);
+  return z * s;
 }
 __device__ __forceinline__ float gelu_grad_tanh_exact(float z) {
-  const float z2 = z * z;
-  const float t = tanh_exact(z * fmaf(0.7978845608028654f * 0.044715f, z2, 0.7978845608028654f));
-  const float du = fmaf(0.7978845608028654f * 0.134145f, z2, 0.7978845608028654f);
-  return fmaf(0.5f * z * du, fmaf(-t, t, 1.0f), fmaf(0.5f, t, 0.5f));
+  constexpr float C1 = (float)(2.0 * 0.7978845608028654), C3 = (float)(2.0 * 0.7978845608028654 * 0.134145);   // d 2u / dz = C1 + C3 z^2
+  float s, ds;
+  gelu_sigmoid(z, s, ds);
+  return fmaf(z * ds, fmaf(C3, z * z, C1), s);
 }
 __device__ __forceinline__ void gelu_tanh_pair(float& a, float& b) {
   const uint64_t c1 = pack2(0.7978845608028654f, 0.7978845608028654f);

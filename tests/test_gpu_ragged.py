@@ -92,6 +92,46 @@ def test_linear_any_row_count_and_depth(M, K, N, epilogue):
         assert got <= 1.02 * plain + 2e-5, errs
 
 
+@pytest.mark.parametrize("epilogue", [B.EPI_BIAS_GELU, B.EPI_MUL_GELUGRAD])
+def test_gelu_off_the_tile_sizes_for_every_pre_activation(epilogue):
+    """All bf16 pre-activations up to 1e4 through a layer whose product is exact: the result is the 64-bit value rounded to
+    bf16, but for fp32 errors before that rounding.  They are relative to s = sigmoid(2u): three roundings of the exponent,
+    2^-24 of 2u each, 2^-22 of the exponential, eight roundings of the rest; the derivative is a sum of s and
+    z s (1 - s) d2u/dz, which cancels near z = -0.75.  No more values are misrounded than in plain FMA."""
+    bits = torch.arange(65536, dtype=torch.int32, device="cuda").to(torch.int16).view(torch.bfloat16)
+    z = bits[bits.isfinite() & (bits.abs() <= 1e4)]
+    M, K, N = z.numel(), 8, 8
+    x, W = (torch.zeros(n, K, device="cuda", dtype=torch.bfloat16) for n in (M, N))
+    W[:, 0] = 1
+    z64 = z.double().requires_grad_()
+    gelu = torch.nn.functional.gelu(z64, approximate="tanh")
+    # the exact product 0.5 z (1 + tanh u) = z / (1 + exp(-2u)); torch's own form cancels in 64 bits far out
+    u2 = 2 * (2 / np.pi) ** 0.5 * (z64 + 0.044715 * z64 ** 3)
+    s = torch.sigmoid(u2)
+    assert float((gelu - z64 * s).detach().abs().max()) < 1e-11
+    rel = (3 * u2.detach().abs() + 12) * 2.0 ** -24
+    if epilogue == B.EPI_BIAS_GELU:
+        ref = (z64 * s).detach()
+        slack = rel * ref.abs()
+        x[:, 0] = z
+    else:
+        ds = s * torch.sigmoid(-u2) * 2 * (2 / np.pi) ** 0.5 * (1 + 0.134145 * z64 ** 2)
+        ref = (s + z64 * ds).detach()
+        slack = rel * (s + 2 * (z64 * ds).abs()).detach()
+        x[:, 0] = 1
+    r = z[:, None].expand(M, N).contiguous()
+    wrong = []
+    for tc in (True, False):
+        out = B.linear(x, W, None, epilogue, r=r, use_tensor_cores=tc)
+        y = (out[0] if epilogue == B.EPI_BIAS_GELU else out)[:, 3].double()
+        wrong.append(int((y != ref.bfloat16().double()).sum()))
+        if tc:
+            slack = slack + (1 + z.double().abs()) ** 3 * 2.0 ** -126      # exponentials below 2^-126 count as 0
+            ok = ((y >= (ref - slack).bfloat16().double()) & (y <= (ref + slack).bfloat16().double()))
+            assert bool(ok.all()), (z[~ok], y[~ok], ref[~ok])
+    assert wrong[0] <= wrong[1], wrong
+
+
 @pytest.mark.parametrize("M,n_in,n_out,r,G", [(1, 64, 72, 4, 1), (77, 200, 136, 6, 1), (129, 768, 256, 1, 1), (300, 136, 768, 40, 1),
                                               (512, 200, 1000, 8, 2), (640, 72, 72, 64, 5),
                                               (512, 1024, 1024, 4, 2), (256, 4096, 512, 16, 1), (1024, 1024, 1024, 40, 4)])
