@@ -15,7 +15,7 @@
 //                         tile, the leader issues 256 x 256 x 16 products that read both CTAs'
 //                         shared memory and write both CTAs' tensor memory.  32 KB per CTA per
 //                         64-deep block (131 FLOP per byte from L2), 6 stages.
-//   gemm_tc_kernel<BN>    one CTA per tile of 128 x BN (BN 256 / 128 / 64): narrow outputs (the
+//   gemm_tc_kernel<BN, EXACT>    one CTA per tile of 128 x BN (BN 256 / 128 / 64): narrow outputs (the
 //                         rank-r down projections) and shapes the pair kernel does not take.
 //   gemm_tc_split_kernel  few tiles: one 128 x 64 or 128 x 128 tile per cluster of 1-8 CTAs that share the
 //                         contraction.
@@ -58,7 +58,7 @@ template <int BN> struct Cfg {
   static constexpr uint32_t IDESC = make_idesc(BM, BN);
 };
 
-template <int BN>
+template <int BN, bool EXACT>
 __global__ void __launch_bounds__(NUM_THREADS, Cfg<BN>::CTAS_PER_SM)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                const __grid_constant__ CUtensorMap mapXe, const __grid_constant__ CUtensorMap mapWe,
@@ -200,7 +200,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
       if (!mbar_wait(tfull_bar(as), aphase, abort_flag, p.status, 4)) { ok = false; break; }
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN);
-      epilogue_tile(p, t_row, m_warp0, lane, n0, c_begin, c_end, m_next, n_next, tanh_form, stage, est, &mapY, &mapZ);
+      if (m_warp0 < p.M) epilogue_tile<EXACT>(p, t_row, m_warp0, lane, n0, c_begin, c_end, m_next, n_next, tanh_form, stage, est, &mapY, &mapZ);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar(as));
@@ -226,6 +226,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
 // ------------------------------------------------------------------------------------------
 // CTA pairs
 // ------------------------------------------------------------------------------------------
+// One kernel per epilogue: with two in one kernel, what one gains from a change of the code the other loses (2-4 %).
 // NEED_R: the epilogue has a second operand R (residual, or the pre-activation for GELU').  Its
 // [128 x 256] block per CTA tile is brought into shared memory by the producer warp with TMA about
 // one tile ahead of its use, so the epilogue never waits on a global load; the room comes from a
@@ -242,12 +243,13 @@ template <bool NEED_R> struct PairCfg {
   static constexpr uint32_t IDESC = make_idesc(2 * BM, BN);
 };
 
-template <bool NEED_R>
+template <int EPI, bool EXACT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                     const __grid_constant__ CUtensorMap mapXe, const __grid_constant__ CUtensorMap mapWe,
                     const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapZ,
                     const __grid_constant__ CUtensorMap mapR, TcParams p) {
+  constexpr bool NEED_R = EPI == EPI_BIAS_RESID || EPI == EPI_MUL_GELUGRAD;
   using C = PairCfg<NEED_R>;
   constexpr int BN = C::BN;
   extern __shared__ uint8_t smem_raw[];
@@ -413,8 +415,9 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
       if (NEED_R && !mbar_wait(rfull_bar, (uint32_t)tcount & 1u, abort_flag, p.status, 16)) { ok = false; break; }
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN);
-      epilogue_tile_smem_r(p, t_row, m_warp0, lane, n0, c_begin, c_end, tanh_form, stage, buf, &mapY, &mapZ,
-                           NEED_R ? r_base : 0u, q * 32 + lane, bfirst);
+      if (m_warp0 < p.M)
+        epilogue_tile_smem_r<EXACT, EPI>(p, t_row, m_warp0, lane, n0, c_begin, c_end, tanh_form, stage, buf, &mapY, &mapZ,
+                                    NEED_R ? r_base : 0u, q * 32 + lane, bfirst);
       if (NEED_R) { __syncwarp(); if (lane == 0) mbar_arrive(rempty_bar); }   // 8 warps release the R buffer
       tc_fence_before();
       __syncwarp();
@@ -460,7 +463,7 @@ template <int BN, int S, int STAGES_> struct SplitCfg {
   static_assert(STAGES * STAGE_BYTES >= EPI_STAGE_BYTES && (8 * PIECES) % S == 0, "");
 };
 
-template <int BN, int S, int STAGES_>
+template <int BN, int S, int STAGES_, bool EXACT>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_split_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                      const __grid_constant__ CUtensorMap mapXe, const __grid_constant__ CUtensorMap mapWe,
@@ -612,7 +615,7 @@ gemm_tc_split_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
 #pragma unroll
       for (int j = 0; j < C::PIECES; ++j) {
         const int u = piece(j), n = n0 + column(j);
-        if ((S > 1 && u % S != rank) || n >= p.N) continue;
+        if ((S > 1 && u % S != rank) || n >= p.N || m_warp0 >= p.M) continue;
         float v[32];
         tc_ld32(t_row + (uint32_t)column(j), v);
         tc_wait_ld();
@@ -641,7 +644,7 @@ gemm_tc_split_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = acc[i];
         }
-        epilogue_chunk(p, v, bcur[j], rcur[j], n, tanh_form, stage, buf, &mapY, &mapZ, m_warp0, lane);
+        epilogue_chunk<EXACT, -1>(p, v, bcur[j], rcur[j], n, tanh_form, stage, buf, &mapY, &mapZ, m_warp0, lane);
       }
     }
     epilogue_drain(lane);
@@ -757,23 +760,26 @@ bool prepare(const GemmArgs& a, int* status, int w_box_rows, CUtensorMap* mX, CU
   p->w_group_rows = a.w_grouped ? a.N : 0;
   p->we_group_rows = a.we_grouped ? a.N : 0;
   p->epi = a.epi; p->gelu_tanh = a.gelu_tanh;
-  // Off the tile sizes these layers used to be computed with tanhf (gemm_simt.cu): they keep fp32 accuracy here (see
-  // gelu_sigmoid), for two special-function instructions per element instead of one.
-  p->gelu_exact = a.gelu_tanh && (a.M % BM != 0 || a.K % BK != 0);
   p->bias = (const bf16*)a.bias; p->R = (const bf16*)a.R; p->ldr = a.ldr;
   p->Y = (bf16*)a.Y; p->ldy = a.ldy; p->Z = (bf16*)a.Z; p->ldz = a.ldz;
   p->status = status;
   return true;
 }
 
-template <int BN>
+// Off the tile sizes the layers with a tanh-form GELU used to be computed with tanhf (gemm_simt.cu): they keep fp32
+// accuracy here (see gelu_sigmoid), for two special-function instructions per element instead of one.
+bool exact_gelu(const GemmArgs& a) {
+  return (a.epi == EPI_BIAS_GELU || a.epi == EPI_MUL_GELUGRAD) && a.gelu_tanh && (a.M % BM != 0 || a.K % BK != 0);
+}
+
+template <int BN, bool EXACT>
 cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
   using C = Cfg<BN>;
   const int sms = num_sms();
   static PerDeviceOnce once;                    // one per instantiation; attributes are per device
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
@@ -784,17 +790,17 @@ cudaError_t launch(const GemmArgs& a, int* status, cudaStream_t st) {
   const int tiles = p.tiles_m * p.tiles_n;
   const int slots = sms * C::CTAS_PER_SM;
   const int grid = tiles < slots ? tiles : slots;
-  launch_overlapped(gemm_tc_kernel<BN>, grid, NUM_THREADS, C::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, p);
+  launch_overlapped(gemm_tc_kernel<BN, EXACT>, grid, NUM_THREADS, C::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, p);
   return cudaGetLastError();
 }
 
-template <int BN, int S, int STAGES>
+template <int BN, int S, int STAGES, bool EXACT>
 cudaError_t launch_split(const GemmArgs& a, int* status, cudaStream_t st) {
   using C = SplitCfg<BN, S, STAGES>;
   static PerDeviceOnce once;
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_split_kernel<BN, S, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_split_kernel<BN, S, STAGES, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
@@ -809,26 +815,39 @@ cudaError_t launch_split(const GemmArgs& a, int* status, cudaStream_t st) {
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = chain_attribute(at, 1);
-  return cudaLaunchKernelEx(&cfg, gemm_tc_split_kernel<BN, S, STAGES>, mX, mW, mXe, mWe, mY, mZ, p);
+  return cudaLaunchKernelEx(&cfg, gemm_tc_split_kernel<BN, S, STAGES, EXACT>, mX, mW, mXe, mWe, mY, mZ, p);
 }
 
-cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
-  constexpr int BN = PairCfg<false>::BN;
+template <int EPI, bool EXACT>
+cudaError_t launch_pair_epi(const GemmArgs& a, int* status, cudaStream_t st) {
+  constexpr bool NEED_R = EPI == EPI_BIAS_RESID || EPI == EPI_MUL_GELUGRAD;
+  using C = PairCfg<NEED_R>;
+  static PerDeviceOnce once;
+  const int dev = current_device();
+  if (once.needed(dev)) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_pair_kernel<EPI, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    once.done(dev);
+  }
   CUtensorMap mX, mW, mXe, mWe, mY, mZ, mR;
   TcParams p;
-  if (!prepare(a, status, BN / 2, &mX, &mW, &mXe, &mWe, &mY, &mZ, &p)) return cudaErrorInvalidValue;
-  p.tiles_m = (a.M + 2 * BM - 1) / (2 * BM); p.tiles_n = (a.N + BN - 1) / BN;
+  if (!prepare(a, status, C::BN / 2, &mX, &mW, &mXe, &mWe, &mY, &mZ, &p)) return cudaErrorInvalidValue;
+  p.tiles_m = (a.M + 2 * BM - 1) / (2 * BM); p.tiles_n = (a.N + C::BN - 1) / C::BN;
   const int tiles = p.tiles_m * p.tiles_n;
   const int pairs = tiles < max_pairs() ? tiles : max_pairs();
-  const bool need_r = a.epi == EPI_BIAS_RESID || a.epi == EPI_MUL_GELUGRAD;
-  if (need_r) {
-    if (!make_map(&mR, a.R, a.M, a.N, a.ldr, BM)) return cudaErrorInvalidValue;
-    launch_overlapped(gemm_tc_pair_kernel<true>, 2 * pairs, NUM_THREADS, PairCfg<true>::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
-  } else {
-    mR = mY;
-    launch_overlapped(gemm_tc_pair_kernel<false>, 2 * pairs, NUM_THREADS, PairCfg<false>::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
-  }
+  mR = mY;
+  if (NEED_R && !make_map(&mR, a.R, a.M, a.N, a.ldr, BM)) return cudaErrorInvalidValue;
+  launch_overlapped(gemm_tc_pair_kernel<EPI, EXACT>, 2 * pairs, NUM_THREADS, C::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
   return cudaGetLastError();
+}
+template <bool EXACT>
+cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
+  switch (a.epi) {
+    case EPI_BIAS_GELU: return launch_pair_epi<EPI_BIAS_GELU, EXACT>(a, status, st);
+    case EPI_MUL_GELUGRAD: return launch_pair_epi<EPI_MUL_GELUGRAD, EXACT>(a, status, st);
+    case EPI_BIAS_RESID: return launch_pair_epi<EPI_BIAS_RESID, false>(a, status, st);
+    default: return launch_pair_epi<EPI_BIAS, false>(a, status, st);
+  }
 }
 
 }  // namespace
@@ -840,8 +859,7 @@ int gemm_tc_init() {
   if (!g_pair_once.needed(dev)) return 0;
   // how many CTA pairs fit on this device at once (the pair kernel is persistent: one wave)
   g_max_pairs[dev] = 0;
-  if (cudaFuncSetAttribute(gemm_tc_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<false>::SMEM_BYTES) == cudaSuccess &&
-      cudaFuncSetAttribute(gemm_tc_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<true>::SMEM_BYTES) == cudaSuccess) {
+  if (cudaFuncSetAttribute(gemm_tc_pair_kernel<EPI_BIAS_RESID, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<true>::SMEM_BYTES) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sms & ~1); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = PairCfg<true>::SMEM_BYTES;
     cudaLaunchAttribute at;
@@ -849,7 +867,7 @@ int gemm_tc_init() {
     at.val.clusterDim.x = 2; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
     cfg.attrs = &at; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<true>, &cfg) == cudaSuccess && n > 0)
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<EPI_BIAS_RESID, false>, &cfg) == cudaSuccess && n > 0)
       g_max_pairs[dev] = n < sms / 2 ? n : sms / 2;
     cudaGetLastError();
   }
@@ -879,24 +897,31 @@ bool gemm_tc_supported(const GemmArgs& a) {
   return true;
 }
 
+namespace {
+template <bool EXACT>
+cudaError_t launch_picked(const GemmArgs& a, int* status, cudaStream_t st) {
+  switch (pick_kernel(a)) {
+    case KERNEL_SPLIT64_1: return launch_split<64, 1, 8, EXACT>(a, status, st);
+    case KERNEL_SPLIT64_2: return launch_split<64, 2, 8, EXACT>(a, status, st);
+    case KERNEL_SPLIT64_4: return launch_split<64, 4, 8, EXACT>(a, status, st);
+    case KERNEL_SPLIT64_8: return launch_split<64, 8, 8, EXACT>(a, status, st);
+    case KERNEL_SPLIT128_1: return launch_split<128, 1, 6, EXACT>(a, status, st);
+    case KERNEL_PAIR: return launch_pair<EXACT>(a, status, st);
+    default: break;
+  }
+  switch (pick_bn(a)) {
+    case 256: return launch<256, EXACT>(a, status, st);
+    case 128: return launch<128, EXACT>(a, status, st);
+    default: return launch<64, EXACT>(a, status, st);
+  }
+}
+}  // namespace
+
 cudaError_t gemm_tc(const GemmArgs& args, int* status, cudaStream_t st) {
   if (!gemm_tc_supported(args)) return cudaErrorInvalidValue;
   GemmArgs a = args;
   if (a.rows_per_group >= a.M) a.rows_per_group = 0;      // one group
-  switch (pick_kernel(a)) {
-    case KERNEL_SPLIT64_1: return launch_split<64, 1, 8>(a, status, st);
-    case KERNEL_SPLIT64_2: return launch_split<64, 2, 8>(a, status, st);
-    case KERNEL_SPLIT64_4: return launch_split<64, 4, 8>(a, status, st);
-    case KERNEL_SPLIT64_8: return launch_split<64, 8, 8>(a, status, st);
-    case KERNEL_SPLIT128_1: return launch_split<128, 1, 6>(a, status, st);
-    case KERNEL_PAIR: return launch_pair(a, status, st);
-    default: break;
-  }
-  switch (pick_bn(a)) {
-    case 256: return launch<256>(a, status, st);
-    case 128: return launch<128>(a, status, st);
-    default: return launch<64>(a, status, st);
-  }
+  return exact_gelu(a) ? launch_picked<true>(a, status, st) : launch_picked<false>(a, status, st);
 }
 
 }  // namespace sl

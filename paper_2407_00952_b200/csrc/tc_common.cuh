@@ -30,7 +30,6 @@ struct TcParams {
   int we_group_rows;              // rows between groups in We
   int tiles_m, tiles_n;
   int epi, gelu_tanh;
-  int gelu_exact;                 // fp32 accuracy instead of tanh.approx (see gemm_tc.cu, prepare)
   const bf16* bias;
   const bf16* R; long long ldr;
   bf16* Y; long long ldy;
@@ -460,10 +459,16 @@ __device__ __forceinline__ void load_bias_chunk(const TcParams& p, int n, uint4*
 // instructions.
 __device__ __forceinline__ void epi_yield() { __syncwarp(); }
 
+// EXACT: tanh-form GELU without tanh.approx (a template parameter, because the mere presence of that branch costs the
+// layers that do not take it 3-5 %: 4096 x 768 -> 3072 with GELU 24.5 us against 23.6).
+// EPI: the epilogue where the kernel is made for one of them, -1 where p.epi says.
+// Warps whose 32 rows are all past row M do not come here.
+template <bool EXACT, int EPI>
 __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, const uint4* bcur, const uint4* rpre, int n,
                                                bool tanh_form, uint32_t stage, int& buf, const CUtensorMap* mapY,
                                                const CUtensorMap* mapZ, int m_warp0, int lane) {
-  if (p.bias != nullptr && p.epi != EPI_MUL_GELUGRAD) {      // warp-uniform; layers without a bias skip 64 instructions
+  const int epi = EPI >= 0 ? EPI : p.epi;
+  if (p.bias != nullptr && epi != EPI_MUL_GELUGRAD) {      // warp-uniform; layers without a bias skip 64 instructions
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const bf16* bp = reinterpret_cast<const bf16*>(&bcur[j]);
@@ -473,7 +478,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
     }
   }
   uint32_t packed[16];
-  if (p.epi == EPI_BIAS_GELU) {
+  if (epi == EPI_BIAS_GELU) {
     float zr[32];                       // the pre-activation as stored (rounded to bf16)
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -483,7 +488,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
       zr[2 * i + 1] = __high2float(z2);
     }
     epi_yield();
-    if (p.gelu_exact) {
+    if constexpr (EXACT) {
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = gelu_tanh_exact(zr[i]);
     } else if (tanh_form) {
@@ -496,9 +501,9 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = gelu_f(zr[i], false);
     }
-    if (m_warp0 < p.M) stage_and_store(stage + (uint32_t)buf * 2048u, mapZ, packed, lane, n, m_warp0);
+    stage_and_store(stage + (uint32_t)buf * 2048u, mapZ, packed, lane, n, m_warp0);
     buf ^= 1;
-  } else if (p.epi == EPI_BIAS_RESID) {
+  } else if (epi == EPI_BIAS_RESID) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const bf16* rp = reinterpret_cast<const bf16*>(&rpre[j]);
@@ -506,8 +511,8 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
       for (int i = 0; i < 8; ++i) v[8 * j + i] += __bfloat162float(rp[i]);
       if (j & 1) epi_yield();
     }
-  } else if (p.epi == EPI_MUL_GELUGRAD) {
-    if (p.gelu_exact) {
+  } else if (epi == EPI_MUL_GELUGRAD) {
+    if constexpr (EXACT) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const bf16* rp = reinterpret_cast<const bf16*>(&rpre[j]);
@@ -539,7 +544,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams& p, float* v, cons
     packed[i] = *reinterpret_cast<uint32_t*>(&y2);
   }
   epi_yield();
-  if (m_warp0 < p.M) stage_and_store(stage + (uint32_t)buf * 2048u, mapY, packed, lane, n, m_warp0);   // clipped at row M
+  stage_and_store(stage + (uint32_t)buf * 2048u, mapY, packed, lane, n, m_warp0);   // clipped at row M
   buf ^= 1;
 }
 
@@ -555,6 +560,7 @@ struct EpiState {
 // at m_warp0, accumulator lanes at tensor-memory address t_row.  (m_next, n_next) is the first chunk
 // this warp will process in its next tile (m_next < 0: none); its second operand is requested while
 // the last chunk of this tile is being worked on.
+template <bool EXACT>
 __device__ __forceinline__ void epilogue_tile(const TcParams& p, uint32_t t_row, int m_warp0, int lane, int n0,
                                               int c_begin, int c_end, int m_next, int n_next, bool tanh_form,
                                               uint32_t stage, EpiState& st, const CUtensorMap* mapY,
@@ -584,7 +590,7 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, uint32_t t_row,
     float v[32];
     tc_ld32(t_row + (uint32_t)c, v);
     tc_wait_ld();
-    epilogue_chunk(p, v, bcur, rcur, n, tanh_form, stage, st.buf, mapY, mapZ, m_warp0, lane);
+    epilogue_chunk<EXACT, -1>(p, v, bcur, rcur, n, tanh_form, stage, st.buf, mapY, mapZ, m_warp0, lane);
   }
 }
 
@@ -592,6 +598,7 @@ __device__ __forceinline__ void epilogue_tile(const TcParams& p, uint32_t t_row,
 // [128 rows x 256 columns] block of R as four [128 x 64] tiles in the 128-byte-swizzled layout a
 // TMA load produces (rtile == 0: the epilogue has no second operand).  row = this thread's row
 // inside the CTA tile.
+template <bool EXACT, int EPI>
 __device__ __forceinline__ void epilogue_tile_smem_r(const TcParams& p, uint32_t t_row, int m_warp0, int lane, int n0,
                                                      int c_begin, int c_end, bool tanh_form, uint32_t stage, int& buf,
                                                      const CUtensorMap* mapY, const CUtensorMap* mapZ, uint32_t rtile,
@@ -620,7 +627,7 @@ __device__ __forceinline__ void epilogue_tile_smem_r(const TcParams& p, uint32_t
     float v[32];
     tc_ld32(t_row + (uint32_t)c, v);
     tc_wait_ld();
-    epilogue_chunk(p, v, bcur, rcur, n, tanh_form, stage, buf, mapY, mapZ, m_warp0, lane);
+    epilogue_chunk<EXACT, EPI>(p, v, bcur, rcur, n, tanh_form, stage, buf, mapY, mapZ, m_warp0, lane);
   }
 }
 
