@@ -666,6 +666,7 @@ gemm_tc_split_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
 // ---- host side -----------------------------------------------------------------------------
 // CTA pairs that can be resident at once, per device (0: pair kernel unavailable there)
 int g_max_pairs[MAX_DEVICES] = {};
+int g_max_split_clusters[MAX_DEVICES][3] = {};      // of 2, 4 and 8 CTAs
 PerDeviceOnce g_pair_once;
 
 // 2-D bf16 tensor [rows, cols] with leading dimension ld (elements); box = 64 columns x box_rows rows.
@@ -682,6 +683,14 @@ bool make_out_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols,
 int max_pairs() {
   const int dev = current_device();
   return dev < 0 ? 0 : g_max_pairs[dev];
+}
+// Clusters of S CTAs of the split kernel that can be resident at once (0: unknown).  Fewer than SMs / S, because a cluster
+// stays within one group of SMs: 74, 33 and 15 of 2, 4 and 8 CTAs on 148 SMs.  One tile too many is a second round:
+// 36 tiles (384 x 768 -> 768) as clusters of four 10.6 us, as clusters of two 6.2; 16 (2048 x 4096 -> 64) of eight
+// 13.3 us, of four 8.4.
+int max_split_clusters(int S) {
+  const int dev = current_device();
+  return dev < 0 ? 0 : g_max_split_clusters[dev][S == 2 ? 0 : S == 4 ? 1 : 2];
 }
 
 int pick_bn(const GemmArgs& a) {
@@ -722,7 +731,8 @@ Kernel pick_kernel(const GemmArgs& a) {
     offer(KERNEL_SINGLE, 5500 + cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), bn == 64 ? 2 * sms : sms) * kb * (bn == 64 ? 200 : 300));
   }
   auto split = [&](Kernel k, int bn, int s, int64_t fixed) {
-    const int64_t rounds = cdiv(cdiv(a.M, BM) * cdiv(a.N, bn) * s, sms);
+    const int64_t slots = s == 1 ? sms : max_split_clusters(s) > 0 ? max_split_clusters(s) : sms / s;
+    const int64_t rounds = cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), slots);
     if (s == 1 || kb >= 2 * s) offer(k, fixed + rounds * cdiv(kb, s) * 190 + (rounds - 1) * 3000);
   };
   split(KERNEL_SPLIT64_1, 64, 1, 3600);
@@ -850,6 +860,21 @@ cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
   }
 }
 
+template <int S>
+int query_split_clusters() {
+  using C = SplitCfg<64, S, 8>;
+  const auto kernel = gemm_tc_split_kernel<64, S, 8, false>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(S); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = C::SMEM_BYTES;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = S; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess ? n : 0;
+}
+
 }  // namespace
 
 int gemm_tc_init() {
@@ -869,8 +894,11 @@ int gemm_tc_init() {
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<EPI_BIAS_RESID, false>, &cfg) == cudaSuccess && n > 0)
       g_max_pairs[dev] = n < sms / 2 ? n : sms / 2;
-    cudaGetLastError();
   }
+  g_max_split_clusters[dev][0] = query_split_clusters<2>();
+  g_max_split_clusters[dev][1] = query_split_clusters<4>();
+  g_max_split_clusters[dev][2] = query_split_clusters<8>();
+  cudaGetLastError();
   g_pair_once.done(dev);
   return 0;
 }
