@@ -702,9 +702,7 @@ int pick_bn(const GemmArgs& a) {
 
 bool pair_ok(const GemmArgs& a) {
   if (max_pairs() < 1 || a.k_gap_len > 0) return false;
-  if (a.M <= BM || a.N < 256) return false;
-  if (a.rows_per_group > 0 && a.rows_per_group % (2 * BM) != 0) return false;   // 0 when there is one group
-  return a.rows_per_group > 0 || a.M % (2 * BM) == 0 || a.M % BM != 0;
+  return a.M > BM && a.N >= 256 && a.rows_per_group % (2 * BM) == 0;     // rows_per_group 0: one group, any M
 }
 
 // Which kernel takes a layer: the one with the least estimated time, from the number of rounds its CTAs need on the
@@ -715,7 +713,9 @@ bool pair_ok(const GemmArgs& a) {
 // block takes a lone CTA pair 275 ns whatever the tile.  Measured at M 512 (pair kernel -> this choice): 1024 -> 1024
 // 10.9 -> 7.0 us, 1024 -> 3072 11.3 -> 8.4, 4096 -> 1024 24.4 -> 11.8, rank-r projections from 1024 8.6 -> 6.4 and
 // (8192 tokens) from 4096 21.5 -> 16.0; 4096 tokens and more of the wide layers stay with the pair kernel
-// (1024 -> 1024: 11.6 against 17.4).
+// (1024 -> 1024: 11.6 against 17.4).  Tiles of 128 rows win over pairs where 256-row tiles need a round more: 1152 x 4096
+// -> 4096 (144 tiles on 148 SMs, or 80 on 74 pairs) 27.1 us, as pairs 34.3; 2176 x 768 -> 3072 with a residual 19.6, as
+// pairs 15.0.
 enum Kernel { KERNEL_SINGLE, KERNEL_PAIR, KERNEL_SPLIT64_1, KERNEL_SPLIT64_2, KERNEL_SPLIT64_4, KERNEL_SPLIT64_8, KERNEL_SPLIT128_1 };
 Kernel pick_kernel(const GemmArgs& a) {
   const int64_t sms = num_sms();
@@ -724,12 +724,13 @@ Kernel pick_kernel(const GemmArgs& a) {
   Kernel best = KERNEL_SINGLE;
   int64_t best_ns = INT64_MAX;
   auto offer = [&](Kernel k, int64_t ns) { if (ns < best_ns) { best_ns = ns; best = k; } };
-  if (pair_ok(a)) {
-    offer(KERNEL_PAIR, 5500 + cdiv(cdiv(a.M, 2 * BM) * cdiv(a.N, 256), max_pairs()) * kb * 275);
-  } else {
-    const int bn = pick_bn(a);
-    offer(KERNEL_SINGLE, 5500 + cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), bn == 64 ? 2 * sms : sms) * kb * (bn == 64 ? 200 : 300));
-  }
+  if (pair_ok(a)) offer(KERNEL_PAIR, 5500 + cdiv(cdiv(a.M, 2 * BM) * cdiv(a.N, 256), max_pairs()) * kb * 275);
+  // (where both take about as many rounds, two CTAs by themselves are 10-20 % slower than a pair, and their epilogue waits
+  // for its second operand, 2 us a round, which the pair kernel brings ahead by TMA)
+  const int bn = pick_bn(a);
+  const int64_t block = bn == 256 ? 330 : bn == 64 ? 200 : 300;
+  const bool need_r = a.epi == EPI_BIAS_RESID || a.epi == EPI_MUL_GELUGRAD;
+  offer(KERNEL_SINGLE, 5500 + cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), bn == 64 ? 2 * sms : sms) * (kb * block + (need_r ? 2000 : 0)));
   auto split = [&](Kernel k, int bn, int s, int64_t fixed) {
     const int64_t slots = s == 1 ? sms : max_split_clusters(s) > 0 ? max_split_clusters(s) : sms / s;
     const int64_t rounds = cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), slots);

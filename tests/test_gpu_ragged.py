@@ -66,7 +66,11 @@ def test_attention_ragged_writes_inside_its_rows_only():
                                    (128, 4096, 64), (512, 1024, 64), (256, 512, 64), (512, 4096, 1024), (300, 584, 1000),
                                    (1024, 1024, 1024), (512, 1024, 3072), (2000, 1032, 1000),
                                    # as many tiles as clusters of four or eight would have SMs, and one more than fit
-                                   (384, 768, 768), (384, 584, 768), (1920, 4096, 64), (2048, 4096, 64)])
+                                   (384, 768, 768), (384, 584, 768), (1920, 4096, 64), (2048, 4096, 64),
+                                   # many tiles: CTA pairs (whole tiles, a ragged last one, one whose second CTA has no
+                                   # row, half a tile) and one CTA per tile (whole and ragged)
+                                   (2048, 768, 3072), (1665, 768, 3072), (4001, 1000, 4096), (2100, 264, 2048), (2176, 768, 3072),
+                                   (1152, 1024, 4096), (1100, 1000, 4096)])
 @pytest.mark.parametrize("epilogue", [B.EPI_BIAS, B.EPI_BIAS_GELU, B.EPI_BIAS_RESID, B.EPI_MUL_GELUGRAD])
 def test_linear_any_row_count_and_depth(M, K, N, epilogue):
     """Against 64 bits: no further off than the plain-FMA kernel (the products of bf16 values are exact in both and
