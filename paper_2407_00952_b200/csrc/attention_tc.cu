@@ -616,8 +616,17 @@ cudaError_t launch_bwd(const void* qkv, const void* o, const float* lse, const v
       return attention_bwd_t5_128(qkv, lse, d_o, rowdot, nseq, T, H, d, dqkv, status, st);
   }
   dim3 grid((T + BT - 1) / BT, H, nseq);
+  // Few blocks, but more than half as many as SMs: a kernel that starts early is placed where the one before it leaves
+  // room, some SMs with three blocks (as many as are resident at once at width 64) and some with none, and then takes as
+  // long as the fullest SM.  So these start in order.  Backward us, early -> in order: 8 x 192, 8 heads of 64 23.4 -> 19.6;
+  // 16 x 64 11.9 -> 9.7; 2 x 960 76.9 -> 61.9; outside the range 4 x 64 8.0 -> 8.6, 32 x 192 39.3 -> 40.3.  (The RG forms
+  // have no kernel in front of dQ that would upset its placement: 8 x 100 12.7 -> 13.3, so they start early.)
+  const int64_t blocks = (int64_t)grid.x * H * nseq, sms = num_sms();
+  const bool in_order = !RG && 2 * blocks > sms && blocks <= 3 * sms;
+  if (in_order) break_chain();
   launch_overlapped(attn_bwd_dq_tc_kernel<DH, RG>, grid, NT, Sizes<DH>::DQ, st, (const bf16*)qkv, (const bf16*)o, (const bf16*)d_o, lse, rowdot,
                                                                 (bf16*)dqkv, T, H, d, dh, scale);
+  if (in_order) break_chain();
   launch_overlapped(attn_bwd_dkv_tc_kernel<DH, RG>, grid, NT, Sizes<DH>::DKV, st, (const bf16*)qkv, (const bf16*)d_o, lse, rowdot, (bf16*)dqkv,
                                                                   T, H, d, dh, scale);
   return cudaGetLastError();
