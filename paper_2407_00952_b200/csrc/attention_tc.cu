@@ -233,10 +233,9 @@ __device__ __forceinline__ void redo_dkv(const bf16* qkv, const bf16* d_o, const
 // ------------------------------------------------------------------------------------------
 // forward
 // ------------------------------------------------------------------------------------------
-// dh: head width (RG only; DH otherwise).  Registers for one block per SM at widths above 64: 4 sequences of 500, 8 heads
-// of 128 33 -> 27.5 us against the compiler's own choice (at 64 three blocks, the same as its choice).
-template <int DH, bool RG>
-__global__ void __launch_bounds__(NT, DH > 64 ? 1 : 3) attn_fwd_tc_kernel(const bf16* __restrict__ qkv, bf16* __restrict__ o,
+// dh: head width (RG only; DH otherwise).  BLOCKS: registers for that many blocks per SM (launch_fwd chooses).
+template <int DH, bool RG, int BLOCKS>
+__global__ void __launch_bounds__(NT, BLOCKS) attn_fwd_tc_kernel(const bf16* __restrict__ qkv, bf16* __restrict__ o,
                                                          float* __restrict__ lse, int T, int H, int d, int dh,
                                                          float scale, float scale_log2) {
   overlap_sync();
@@ -578,20 +577,35 @@ __global__ void __launch_bounds__(NT, RG ? (DH > 64 ? 1 : DH > 32 ? 2 : 3) : 0) 
   }
 }
 
-template <int DH, bool RG>
-cudaError_t launch_fwd(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st) {
+template <int DH, bool RG, int BLOCKS>
+cudaError_t launch_fwd_blocks(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st) {
   static PerDeviceOnce once;                    // one per instantiation; attributes are per device
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(attn_fwd_tc_kernel<DH, RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::FWD);
+    cudaError_t e = cudaFuncSetAttribute(attn_fwd_tc_kernel<DH, RG, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sizes<DH>::FWD);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
   const int dh = d / H;
   dim3 grid((T + BT - 1) / BT, H, nseq);
-  launch_overlapped(attn_fwd_tc_kernel<DH, RG>, grid, NT, Sizes<DH>::FWD, st, (const bf16*)qkv, (bf16*)o, lse, T, H, d, dh,
+  launch_overlapped(attn_fwd_tc_kernel<DH, RG, BLOCKS>, grid, NT, Sizes<DH>::FWD, st, (const bf16*)qkv, (bf16*)o, lse, T, H, d, dh,
                                                               1.0f / sqrtf((float)dh), (float)(1.4426950408889634 / sqrt((double)dh)));
   return cudaGetLastError();
+}
+
+// Registers for one block per SM at widths above 64: 4 sequences of 500, 8 heads of 128 33 -> 27.5 us against the
+// compiler's own choice.  At width 64 for three, which beats four where a block walks several tiles (8 x 448, 8 heads 14.1
+// against 16.2 us) or all blocks are resident at once.  Blocks of one to three tiles mostly wait for their loads: more than
+// three per SM of them are better off with four at a time (64 x 64, 16 heads 10.5 -> 9.6 us; 24 x 192, 8 heads 10.7 -> 9.9).
+template <int DH, bool RG>
+cudaError_t launch_fwd(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st) {
+  if constexpr (DH > 64) return launch_fwd_blocks<DH, RG, 1>(qkv, nseq, T, H, d, o, lse, st);
+  else {
+    if constexpr (DH == 64 && !RG) {
+      if (T <= 3 * BT && (int64_t)(T / BT) * H * nseq > 3 * num_sms()) return launch_fwd_blocks<DH, RG, 4>(qkv, nseq, T, H, d, o, lse, st);
+    }
+    return launch_fwd_blocks<DH, RG, 3>(qkv, nseq, T, H, d, o, lse, st);
+  }
 }
 
 template <int DH, bool RG>

@@ -47,6 +47,20 @@ def test_attention_any_length_and_width(T, dh):
     assert torch.equal(static, B.attention_bwd(qkv, o, lse, do, nseq, T, H))
 
 
+@pytest.mark.parametrize("nseq,T,H", [(64, 64, 16), (26, 192, 8), (8, 64, 64), (2, 192, 8)])
+def test_attention_forward_of_short_whole_tiles(nseq, T, H):
+    """One to three tiles per sequence, more and fewer blocks than three per SM, width 64: within the rounding of the
+    probabilities and the output to bf16 (2^-8 each)."""
+    dh = 64
+    g = torch.Generator(device="cuda").manual_seed(nseq + T)
+    qkv = torch.randn(nseq * T, 3 * H * dh, device="cuda", generator=g).bfloat16()
+    do = torch.randn(nseq * T, H * dh, device="cuda", generator=g).bfloat16()
+    o, lse = B.attention_fwd(qkv, nseq, T, H)
+    dqkv = B.attention_bwd(qkv, o, lse, do, nseq, T, H)
+    ref = _attention64(qkv, do, nseq, T, H, dh)
+    assert [_norm_err(a, r) <= b for a, r, b in zip((o, lse, dqkv), ref, (2 * 2.0 ** -8, 1e-6, 3 * 2.0 ** -8))] == [True] * 3
+
+
 def test_attention_ragged_writes_inside_its_rows_only():
     nseq, T, H, dh = 2, 77, 2, 24
     d, guard = H * dh, 64
