@@ -1,12 +1,14 @@
 // Causal multi-head attention with plain FMA arithmetic (fp32 or bf16 storage, any shape, head width up to 128): the
 // arithmetic of the fp32 configuration and a second opinion for the tensor-core kernels.
-// A block of eight warps owns RT = 32 rows (queries, or keys in the dK/dV kernel) of one (sequence, head), four rows per
-// warp, and walks the other side in tiles of 32 rows that all its warps share through shared memory.  Scores are one
-// column of the tile per lane; the accumulations are one feature per lane, with the tile's probabilities read back as
-// broadcasts from shared memory.  A tile element read from shared memory serves four rows, a probability all features.
+// Short sequences take a warp per row (by_rows says which).  Otherwise a block of eight warps owns RT = 32 rows (queries,
+// or keys in the dK/dV kernel) of one (sequence, head), four rows per warp, and walks the other side in tiles of 32 rows
+// that all its warps share through shared memory.  Scores are one column of the tile per lane; the accumulations are one
+// feature per lane, with the tile's probabilities read back as broadcasts from shared memory.  A tile element read from
+// shared memory serves four rows, a probability all features.
 // What bounds it: shared-memory reads (about five per sixteen products).  Against one warp per row that reads the other side
 // from global memory: the fp32 round of 512 tokens (8 sequences of 64, 4 heads of 32) 514 -> 355 us together with the
 // sixteen-lane adapter gradients of lora_grad.cu; errors against 64 bits a little smaller.
+#include "attention_rows.cuh"
 #include "common.cuh"
 #include "host_common.h"
 #include "kernels.h"
@@ -16,7 +18,7 @@ namespace sl {
 namespace {
 
 constexpr int WARPS = 8, RPW = 4, RT = WARPS * RPW, KT = 32;
-constexpr int MAX_DH = 128;
+constexpr int MAX_DH = rows::MAX_DH;
 constexpr int DPL = MAX_DH / 32;   // features per lane
 
 // Shared memory, in floats: two tiles [32][width + 1], width = dh rounded up to 32 so that "one feature per lane" reads
@@ -312,6 +314,57 @@ __global__ void __launch_bounds__(WARPS * 32, BLOCKS) attn_bwd_dkv_kernel(const 
   }
 }
 
+// ---- short sequences: a warp per row (attention_rows.cuh) ----
+// A tile of 32 rows would be mostly padding, with loads and barriers for the whole of it.
+constexpr int ROW_WARPS = 4;
+
+template <typename T>
+__global__ void __launch_bounds__(ROW_WARPS * 32) attn_rows_fwd_kernel(const T* __restrict__ qkv, int nseq, int Tn, int H, int d,
+                                                                       T* __restrict__ o, float* __restrict__ lse) {
+  overlap_sync();
+  __shared__ float s[ROW_WARPS][MAX_DH];
+  const int64_t w = (int64_t)blockIdx.x * ROW_WARPS + (threadIdx.x >> 5);
+  if (w >= (int64_t)nseq * H * Tn) return;
+  const int i = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
+  const rows::Head<T> hd(qkv, b, h, Tn, H, d);
+  rows::forward_row<T>(hd, i, s[threadIdx.x >> 5], o + ((size_t)b * Tn + i) * d + (size_t)h * hd.dh, lse + ((size_t)b * H + h) * Tn + i);
+}
+
+// dQ, and D[row] = sum(dO * O) of its row, which the dK/dV kernel (second) reads from `rowdot`
+template <typename T>
+__global__ void __launch_bounds__(ROW_WARPS * 32) attn_rows_dq_kernel(const T* __restrict__ qkv, const T* __restrict__ o,
+                                                                      const float* __restrict__ lse, const T* __restrict__ d_o,
+                                                                      float* __restrict__ rowdot, int nseq, int Tn, int H, int d,
+                                                                      T* __restrict__ dqkv) {
+  overlap_sync();
+  __shared__ float s[ROW_WARPS][2 * MAX_DH];
+  const int64_t w = (int64_t)blockIdx.x * ROW_WARPS + (threadIdx.x >> 5);
+  if (w >= (int64_t)nseq * H * Tn) return;
+  const int lane = threadIdx.x & 31, i = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
+  const rows::Head<T> hd(qkv, b, h, Tn, H, d);
+  const size_t row = ((size_t)b * Tn + i) * d + (size_t)h * hd.dh, stat = ((size_t)b * H + h) * Tn + i;
+  float D = 0.f;
+  for (int c = lane; c < hd.dh; c += 32) D = fmaf(to_f<T>(o[row + c]), to_f<T>(d_o[row + c]), D);
+  D = warp_sum(D);
+  if (lane == 0) rowdot[stat] = D;
+  rows::dq_row<T>(hd, d_o + row, lse[stat], D, i, s[threadIdx.x >> 5], dqkv + ((size_t)b * Tn + i) * hd.ld + (size_t)h * hd.dh);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(ROW_WARPS * 32) attn_rows_dkv_kernel(const T* __restrict__ qkv, const float* __restrict__ lse,
+                                                                       const T* __restrict__ d_o, const float* __restrict__ rowdot,
+                                                                       int nseq, int Tn, int H, int d, T* __restrict__ dqkv) {
+  overlap_sync();
+  __shared__ float s[ROW_WARPS][2 * MAX_DH];
+  const int64_t w = (int64_t)blockIdx.x * ROW_WARPS + (threadIdx.x >> 5);
+  if (w >= (int64_t)nseq * H * Tn) return;
+  const int j = (int)(w % Tn), h = (int)((w / Tn) % H), b = (int)(w / ((int64_t)Tn * H));
+  const rows::Head<T> hd(qkv, b, h, Tn, H, d);
+  const size_t stat = ((size_t)b * H + h) * Tn;
+  rows::dkv_row<T>(hd, d_o + (size_t)b * Tn * d + (size_t)h * hd.dh, lse + stat, rowdot + stat, j, s[threadIdx.x >> 5],
+                   dqkv + ((size_t)b * Tn + j) * hd.ld + d + (size_t)h * hd.dh);
+}
+
 // room for the widest head, once per device and kernel
 template <typename K> cudaError_t allow_smem(K kernel, PerDeviceOnce& once) {
   const int dev = current_device();
@@ -352,11 +405,34 @@ cudaError_t bwd(const void* qkv, const void* o, const float* lse, const void* d_
                                           : bwd_blocks<T, 3>(qkv, o, lse, d_o, blocks, T_, H, d, dqkv, rowdot, st);
 }
 
-bool grid_of(int nseq, int T, int H, int d, unsigned* blocks) {
+// Whether a warp per row beats tiles of 32 rows: forward up to 10 rows, backward up to 9 (10 up to width 32), and up to 16
+// while all the rows are at work at once.  us, forward / backward, rows against tiles, fp32: 8192 heads of 1 x 128 12 / 39
+// against 277 / 803; 2048 of 8 x 64 29 / 101 against 45 / 133, of 10 x 64 39 / 142 against 46 / 133, of 12 x 64 51 / 189
+// against 47 / 134; 32 of 16 x 64 7.6 / 17 against 7.7 / 19, 128 of them 13 / 41 against 8 / 19.
+bool by_rows(int nseq, int T, int H, int d, bool forward) {
+  return T <= (forward || d / H <= 32 ? 10 : 9) || (T <= 16 && (int64_t)nseq * H * T <= 4 * num_sms());
+}
+
+bool grid_of(int nseq, int T, int H, int d, bool rows, unsigned* blocks) {
   if (d % H != 0 || d / H > MAX_DH) return false;
-  const int64_t n = (int64_t)nseq * H * ((T + RT - 1) / RT);
+  const int64_t items = (int64_t)nseq * H, n = rows ? (items * T + ROW_WARPS - 1) / ROW_WARPS : items * ((T + RT - 1) / RT);
   *blocks = (unsigned)n;
   return n <= 0x7fffffff;
+}
+
+template <typename T>
+cudaError_t fwd_rows(const void* qkv, unsigned blocks, int nseq, int T_, int H, int d, void* o, float* lse, cudaStream_t st) {
+  return launch_overlapped(attn_rows_fwd_kernel<T>, blocks, ROW_WARPS * 32, 0, st, (const T*)qkv, nseq, T_, H, d, (T*)o, lse);
+}
+
+template <typename T>
+cudaError_t bwd_rows(const void* qkv, const void* o, const float* lse, const void* d_o, unsigned blocks, int nseq, int T_, int H,
+                     int d, void* dqkv, float* rowdot, cudaStream_t st) {
+  cudaError_t e = launch_overlapped(attn_rows_dq_kernel<T>, blocks, ROW_WARPS * 32, 0, st, (const T*)qkv, (const T*)o, lse,
+                                    (const T*)d_o, rowdot, nseq, T_, H, d, (T*)dqkv);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(attn_rows_dkv_kernel<T>, blocks, ROW_WARPS * 32, 0, st, (const T*)qkv, lse, (const T*)d_o, rowdot, nseq,
+                           T_, H, d, (T*)dqkv);
 }
 
 }  // namespace
@@ -364,14 +440,20 @@ bool grid_of(int nseq, int T, int H, int d, unsigned* blocks) {
 cudaError_t attention_fwd_simt(int dt, const void* qkv, int nseq, int T, int H, int d, void* o, float* lse,
                                cudaStream_t st) {
   unsigned blocks;
-  if (!grid_of(nseq, T, H, d, &blocks)) return cudaErrorInvalidValue;
+  const bool rows = by_rows(nseq, T, H, d, true);
+  if (!grid_of(nseq, T, H, d, rows, &blocks)) return cudaErrorInvalidValue;
+  if (rows) return dt == DT_BF16 ? fwd_rows<bf16>(qkv, blocks, nseq, T, H, d, o, lse, st) : fwd_rows<float>(qkv, blocks, nseq, T, H, d, o, lse, st);
   return dt == DT_BF16 ? fwd<bf16>(qkv, blocks, T, H, d, o, lse, st) : fwd<float>(qkv, blocks, T, H, d, o, lse, st);
 }
 
 cudaError_t attention_bwd_simt(int dt, const void* qkv, const void* o, const float* lse, const void* d_o,
                                int nseq, int T, int H, int d, void* dqkv, float* rowdot, cudaStream_t st) {
   unsigned blocks;
-  if (!grid_of(nseq, T, H, d, &blocks)) return cudaErrorInvalidValue;
+  const bool rows = by_rows(nseq, T, H, d, false);
+  if (!grid_of(nseq, T, H, d, rows, &blocks)) return cudaErrorInvalidValue;
+  if (rows)
+    return dt == DT_BF16 ? bwd_rows<bf16>(qkv, o, lse, d_o, blocks, nseq, T, H, d, dqkv, rowdot, st)
+                         : bwd_rows<float>(qkv, o, lse, d_o, blocks, nseq, T, H, d, dqkv, rowdot, st);
   return dt == DT_BF16 ? bwd<bf16>(qkv, o, lse, d_o, blocks, T, H, d, dqkv, rowdot, st)
                        : bwd<float>(qkv, o, lse, d_o, blocks, T, H, d, dqkv, rowdot, st);
 }

@@ -671,13 +671,19 @@ cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, c
                      : launch_bwd<128, false>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
 }
 
-// The 16-byte copies need every head's first column of every row on a 16-byte boundary (d and the head width
+// The shapes these kernels take.  The 16-byte copies need every head's first column of every row on a 16-byte boundary (d and the head width
 // multiples of 8, aligned bases); sequences and heads are grid dimensions y and z.
 bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const void* qkv, const void* o, const void* d_o,
                                 const void* dqkv) {
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   if (dt != DT_BF16 || H < 1 || d % H != 0 || T < 1 || nseq < 1) return false;
   const int dh = d / H;
+  // Many heads of a few rows: the tiles of 64 are padding, and a warp per row (attention_simt.cu) is faster.  us, forward /
+  // backward, rows against tiles: 2048 heads of 1 x 64 4.8 / 11 against 19 / 53, of 5 x 64 15 / 47 against 19 / 53, of 6 x
+  // 64 20 / 63 against 19 / 53; 8192 of 6 x 64 59 / 211 against 67 / 195; 128 of 1 x 64 4.2 / 10 against 3.6 / 9, 512 4.3 /
+  // 10 against 7.1 / 18.
+  const int64_t heads = (int64_t)nseq * H, sms = num_sms();
+  if ((T <= 5 && heads > 2 * sms) || (T == 6 && !d_o && heads > 16 * sms)) return false;
   return dh % 8 == 0 && dh <= 128 && H <= 65535 && nseq <= 65535 && al16(qkv) && al16(o) && al16(d_o) && al16(dqkv);
 }
 

@@ -61,6 +61,25 @@ def test_attention_forward_of_short_whole_tiles(nseq, T, H):
     assert [_norm_err(a, r) <= b for a, r, b in zip((o, lse, dqkv), ref, (2 * 2.0 ** -8, 1e-6, 3 * 2.0 ** -8))] == [True] * 3
 
 
+@pytest.mark.parametrize("T", [1, 2, 5, 6, 8, 9, 10, 11, 16, 17])
+@pytest.mark.parametrize("dh", [5, 32, 64, 128])
+@pytest.mark.parametrize("nseq,H", [(2, 3), (150, 4)])
+def test_attention_of_short_sequences(T, dh, nseq, H):
+    """Both sides of the lengths and head counts at which short sequences change kernels (tiles, a warp per row, tensor
+    cores), fp32 and bf16.  fp32: about as many roundings of random sign as terms in a score and in a row's sum, taken four
+    times; bf16: the rounding of the output."""
+    g = torch.Generator(device="cuda").manual_seed(T * dh + nseq)
+    for dtype, bounds in ((torch.float32, [4 * (T + dh) ** 0.5 * 2.0 ** -24] * 3), (torch.bfloat16, (4e-3, 1e-6, 4e-3))):
+        qkv = torch.randn(nseq * T, 3 * H * dh, device="cuda", generator=g).to(dtype)
+        do = torch.randn(nseq * T, H * dh, device="cuda", generator=g).to(dtype)
+        o, lse = B.attention_fwd(qkv, nseq, T, H)
+        dqkv = B.attention_bwd(qkv, o, lse, do, nseq, T, H)
+        errs = [_norm_err(a, r) for a, r in zip((o, lse, dqkv), _attention64(qkv, do, nseq, T, H, dh))]
+        assert all(e <= b for e, b in zip(errs, bounds)), (dtype, errs)
+        assert torch.equal(dqkv, B.attention_bwd_static(qkv, o, lse, do, nseq, T, H))
+    assert B.library_status() == 0
+
+
 def test_attention_ragged_writes_inside_its_rows_only():
     nseq, T, H, dh = 2, 77, 2, 24
     d, guard = H * dh, 64
