@@ -379,8 +379,8 @@ def test_error_paths():
 
 @pytest.mark.parametrize("M,n_in,n_out", [(256, 128, 512), (1024, 1024, 1000), (512, 256, 64)])
 def test_linear_epilogues_bf16(M, n_in, n_out):
-    """Frozen linear with each fused epilogue (pair kernel, single-CTA kernel, ragged width)
-    against fp64: bias, bias + GELU (pre-activation saved), bias + residual, product with GELU'."""
+    """Frozen linear with each fused epilogue (few tiles, whole and ragged width: the split kernels; the shapes that
+    the pair and the single-CTA kernel take are in test_gpu_ragged.py) against fp64: bias, bias + GELU (pre-activation saved), bias + residual, product with GELU'."""
     rng = np.random.default_rng(M + n_out)
     bfv = lambda a: synth._to_bf16_values(a.astype(np.float32))
     x, W = bfv(rng.normal(size=(M, n_in))), bfv(rng.normal(size=(n_out, n_in)) / np.sqrt(n_in))

@@ -26,8 +26,9 @@ def _attention64(qkv, do, nseq, T, H, dh):
 @pytest.mark.parametrize("T,dh", [(1, 64), (2, 8), (31, 32), (63, 24), (64, 32), (65, 64), (128, 96), (129, 128), (200, 40),
                                   (333, 64), (257, 104), (191, 16)])
 def test_attention_any_length_and_width(T, dh):
-    """Against 64 bits: no further off than the plain-FMA kernels (fp32 probabilities), whose error is that of the
-    bf16 output; 2 % more is allowed for another order of the sums.  Rows around the tensors stay untouched."""
+    """Against 64 bits: both forms within the rounding of their bf16 outputs (half a unit, 2^-9 on average) and the
+    tensor-core form no further off than the plain-FMA kernels (fp32 probabilities); 2 % more is allowed for another order
+    of the sums."""
     nseq, H = 3, 2
     d = H * dh
     g = torch.Generator(device="cuda").manual_seed(100 * T + dh)
@@ -41,8 +42,8 @@ def test_attention_any_length_and_width(T, dh):
         errs.append([_norm_err(a, r) for a, r in zip((o, lse, dqkv), ref)])
     assert B.library_status() == 0
     # lse is an fp32 result: no further off either, up to one rounding of the result (few values at the short lengths)
-    for got, plain, bound in zip(*errs, (2e-6, 2.0 ** -24, 2e-6)):
-        assert got <= 1.02 * plain + bound, errs
+    for got, plain, bound, most in zip(*errs, (2e-6, 2.0 ** -24, 2e-6), (4e-3, 1e-6, 4e-3)):
+        assert got <= 1.02 * plain + bound and max(got, plain) <= most, errs
     static = B.attention_bwd_static(qkv, o, lse, do, nseq, T, H)
     assert torch.equal(static, B.attention_bwd(qkv, o, lse, do, nseq, T, H))
 
@@ -106,8 +107,10 @@ def test_attention_ragged_writes_inside_its_rows_only():
                                    (1152, 1024, 4096), (1100, 1000, 4096)])
 @pytest.mark.parametrize("epilogue", [B.EPI_BIAS, B.EPI_BIAS_GELU, B.EPI_BIAS_RESID, B.EPI_MUL_GELUGRAD])
 def test_linear_any_row_count_and_depth(M, K, N, epilogue):
-    """Against 64 bits: no further off than the plain-FMA kernel (the products of bf16 values are exact in both and
-    both round to bf16 once, so the errors agree to a few per mille); rows past M stay untouched."""
+    """Against 64 bits: both kernels within the rounding of a bf16 result (2^-8 at most; for GELU also that of the stored
+    pre-activation), and the tensor-core one no further off than plain FMA (the products of bf16 values are exact in both and
+    both round to bf16 once, so the errors agree to a few per mille); rows past M stay untouched.  With 3e5 results and
+    more, the two orders of the sums round a few of them differently: equal bits would mean one kernel ran twice."""
     g = torch.Generator(device="cuda").manual_seed(M + K + N)
     mk = lambda *s, sc=1.0: (torch.randn(*s, device="cuda", generator=g) * sc).bfloat16()  # noqa: E731
     x, W, bias, r = mk(M, K), mk(N, K, sc=K ** -0.5), mk(N), mk(M, N, sc=2.0)
@@ -120,15 +123,19 @@ def test_linear_any_row_count_and_depth(M, K, N, epilogue):
         ref = acc * t.grad
     else:
         ref = {B.EPI_BIAS: z, B.EPI_BIAS_GELU: gelu(z), B.EPI_BIAS_RESID: z + r.double()}[epilogue]
-    errs = []
+    errs, results = [], []
     for tc in (True, False):
         buf = torch.full((M + 160, N), 7.0, device="cuda", dtype=torch.bfloat16)
         zbuf = torch.full((M + 160, N), 7.0, device="cuda", dtype=torch.bfloat16)
         B.linear(x, W, None if epilogue == B.EPI_MUL_GELUGRAD else bias, epilogue, r=r, y=buf[:M], z=zbuf[:M], use_tensor_cores=tc)
         assert bool((buf[M:] == 7).all()) and bool((zbuf[M:] == 7).all())
         errs.append([_norm_err(buf[:M], ref)] + ([_norm_err(zbuf[:M], z)] if epilogue == B.EPI_BIAS_GELU else []))
+        results.append(buf)
+    most = 2.0 ** -8 * (2 if epilogue == B.EPI_BIAS_GELU else 1)
     for got, plain in zip(*errs):
-        assert got <= 1.02 * plain + 2e-5, errs
+        # tanh.approx of whole tiles: 2^-11 of the value, far below the rounding of the result
+        assert got <= 1.02 * plain + 2e-5 and max(got, plain) <= most, errs
+    assert M * N < 300_000 or K < 200 or not torch.equal(*results)
 
 
 @pytest.mark.parametrize("epilogue", [B.EPI_BIAS_GELU, B.EPI_MUL_GELUGRAD])
@@ -175,7 +182,8 @@ def test_gelu_off_the_tile_sizes_for_every_pre_activation(epilogue):
                                               (512, 200, 1000, 8, 2), (640, 72, 72, 64, 5),
                                               (512, 1024, 1024, 4, 2), (256, 4096, 512, 16, 1), (1024, 1024, 1024, 40, 4)])
 def test_lora_linear_any_size(M, n_in, n_out, r, G):
-    """Forward and backward against 64 bits, next to the plain-FMA kernels' errors."""
+    """Forward and backward against 64 bits: within two bf16 roundings (the rank-r projection and the result), and no
+    further off than the plain-FMA kernels."""
     g = torch.Generator(device="cuda").manual_seed(M + n_in)
     x = torch.randn(M, n_in, device="cuda", generator=g).bfloat16()
     W = (torch.randn(n_out, n_in, device="cuda", generator=g) * n_in ** -0.5).bfloat16()
@@ -194,7 +202,7 @@ def test_lora_linear_any_size(M, n_in, n_out, r, G):
         errs.append([_norm_err(a, b) for a, b in zip(got, ref)])
     assert B.library_status() == 0
     for got, plain in zip(*errs):
-        assert got <= 1.02 * plain + 2e-5, errs
+        assert got <= 1.02 * plain + 2e-5 and max(got, plain) <= 2 * 2.0 ** -8, errs
 
 
 @pytest.mark.parametrize("M,K,N", [(1, 8, 8), (33, 72, 40), (65, 136, 200), (512, 1024, 128), (31, 64, 1000), (700, 200, 1000),
