@@ -28,17 +28,13 @@
 // All mbarrier waits are bounded (tc_common.cuh); on expiry a code is left in `status`.
 #include "host_common.h"
 #include "launch.cuh"
-#include "tc_common.cuh"
+#include "attention_t5.cuh"
 
 namespace sl {
 namespace {
 
-using namespace tc;
+using namespace t5;
 
-constexpr int DH = 64;
-constexpr int BT = 128;                   // rows of a query tile and of a key tile
-constexpr int TILE = BT * DH * 2;         // 16 KB: one [128 x 64] bf16 tile
-constexpr int OUT_THREADS = 128;
 // Warp roles: warp 0 TMA, warp 1 score products, then the element-wise warps (EWQ per accumulator lane
 // quarter, each computing CW of a half's 64 columns), one warp for the accumulating products, and four
 // output warps that move finished accumulators to global memory.  Head width 64 takes four
@@ -70,20 +66,6 @@ template <int DHT> struct Roles {
 // 16-byte rows of columns 0..7 (128 bytes) and then those of columns 8..15.  Columns: 0, 1 = -lse/scale
 // (hi, lo), 2, 3 = -D (hi, lo), the rest zero; the constant tiles have ones in columns 0, 1 (for S) or 2, 3
 // (for dP).
-constexpr int AUG_TILE = 128 * 16 * 2;
-constexpr uint32_t DESC_HI_AUG = (uint32_t)(256 >> 4) | (1u << 14);           // 8-row groups 256 bytes apart, no swizzle
-__device__ __forceinline__ uint32_t desc_lo_aug(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | ((uint32_t)(128 >> 4) << 16); }
-__device__ __forceinline__ void tc_mma_aug(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 p, 1, 0;\n\t"
-      "mov.b64 da, {%1, %3};\n\t"
-      "mov.b64 db, {%2, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-      ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(DESC_HI_AUG), "r"(idesc) : "memory");
-}
-// byte offset of row r's columns 0..7 inside such a tile
-__device__ __forceinline__ uint32_t aug_row(int r) { return (uint32_t)(r >> 3) * 256u + (uint32_t)(r & 7) * 16u; }
 // -x as hi + lo, two bf16 values in one word (hi in the low half)
 __device__ __forceinline__ uint32_t neg_split(float x) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(-x);
@@ -101,55 +83,15 @@ __device__ __forceinline__ void aug_init(uint8_t* ones_s, uint8_t* ones_d, int r
     *reinterpret_cast<uint4*>(ones_d + off) = make_uint4(0u, (i & 1) ? 0u : one2, 0u, 0u);
   }
 }
-constexpr int TMEM_COLS = 512;
-constexpr uint32_t IDESC_64KK = make_idesc(BT, DH);                   // [128 x 64] products, both operands K-major
-constexpr uint32_t IDESC_64MN = make_idesc(BT, DH) | (1u << 16);      // [128 x 64] products, right operand MN-major
-constexpr float LOG2E = 1.4426950408889634f;
-
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-// 16 consecutive tensor-memory columns of this thread's lane
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr) : "memory");
-}
-// 8 packed words of this thread's lane to 8 consecutive tensor-memory columns
-__device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* w) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-      ::"r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-}
 template <int CW> __device__ __forceinline__ void tc_ld_cw(uint32_t taddr, float* v) {
   if constexpr (CW == 32) tc_ld32(taddr, v); else tc_ld16(taddr, v);
 }
 template <int CW> __device__ __forceinline__ void tc_st_cw(uint32_t taddr, const uint32_t* w) {   // CW / 2 packed words
   if constexpr (CW == 32) tc_st16(taddr, w); else tc_st8(taddr, w);
 }
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-               ::"l"(map), "r"(src), "r"(c0), "r"(c1) : "memory");
-}
-// one row (lane r) of a [128 x 64] bf16 tile in the 128-byte-swizzled layout: 16-byte chunk jj
-__device__ __forceinline__ void st_row_chunk(uint32_t tile, int r, uint32_t jj, const uint32_t* w) {
-  const uint32_t addr = tile + (uint32_t)r * 128u + ((jj ^ ((uint32_t)r & 7u)) << 4);
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
 }
 // Operand descriptors are passed as their address-carrying lower halves (desc_lo); the upper half
 // is the same constant for the K-major tiles and for the MN-major ones (128-byte rows, 128-byte
@@ -171,16 +113,6 @@ __device__ __forceinline__ void mma_acc_half(uint32_t d_tmem, uint32_t a_tmem, u
   tc_mma_ts_lo(d_tmem, a0 + HOP, b0 + 256, IDESC_64MN, 1u);
   tc_mma_ts_lo(d_tmem, a0 + HOP + 8, b0 + 384, IDESC_64MN, 1u);
 }
-// 4 products [128 x 64] = A[128 x 64] * (rows [64h, 64h + 64) of the K-major tile at blo)^T:
-// one half (64 columns) of a [128 x 128] score tile.  64 rows of 128 bytes = 512 descriptor units.
-__device__ __forceinline__ void mma_score_half(uint32_t d_tmem, uint32_t alo, uint32_t blo, int h, bool fresh = true) {
-  const uint32_t b0 = blo + (uint32_t)(512 * h);
-  tc_mma_lo(d_tmem, alo, b0, IDESC_64KK, fresh ? 0u : 1u);
-  tc_mma_lo_acc(d_tmem, alo + 2, b0 + 2, IDESC_64KK);
-  tc_mma_lo_acc(d_tmem, alo + 4, b0 + 4, IDESC_64KK);
-  tc_mma_lo_acc(d_tmem, alo + 6, b0 + 6, IDESC_64KK);
-}
-
 struct BwdParams {
   int T, H, d;
   float scale;             // 1/sqrt(dh)
@@ -228,11 +160,6 @@ struct BwdParams {
     tc_fence_after();                                                                                     \
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory"); \
   }
-
-// parity to wait on for "the n-th completion (0-based) of this barrier has happened"
-__device__ __forceinline__ uint32_t done(int n) { return (uint32_t)n & 1u; }
-// parity to wait on before the n-th use of a slot whose release is signalled once per use
-__device__ __forceinline__ uint32_t freed(int n) { return ((uint32_t)n & 1u) ^ 1u; }
 
 // ==========================================================================================
 // dK, dV

@@ -10,7 +10,8 @@
 //     lost (error of o / dqkv against 64 bits over odd T is that of the bf16 output alone, as before).  Measured,
 //     16 sequences of 777 tokens, 12 heads of 64, forward + backward: 466 us against 72.9 ms.  Bound by the
 //     tensor issue of mma.sync and by ldmatrix traffic (the hi and lo products share one fragment of the right
-//     operand).  Shapes that the aligned forms take stay with them.
+//     operand).  Shapes that the aligned forms take stay with them; the backward pass of most of those of width 64
+//     runs on tcgen05 (attention_t5_ragged.cu).
 //   forward : one CTA per (sequence, head, 64-row query tile), 4 warps x 16 rows, K/V tiles double
 //             buffered in shared memory with cp.async, online softmax in registers.
 //   backward: rowdot = sum(dO*O); a dQ kernel per query tile (loops over key tiles) and a dK/dV
@@ -698,7 +699,13 @@ cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d,
 }
 
 cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
-                                 int d, void* dqkv, float* rowdot, cudaStream_t st) {
+                                 int d, void* dqkv, float* rowdot, int* status, cudaStream_t st) {
+  // Tiles of 128 on tcgen05 against tiles of 64 here, backward us: 16 sequences of 777, 12 heads 339 -> 123; 32 x 288 134 -> 62;
+  // 5 x 333 44 -> 22; one of 150 with 4 heads 14.2 -> 14.1.  Up to 128 rows a head is one tile there, whose fixed part (set-up,
+  // first loads) shows until there are about as many heads as SMs: 64 x 70, 16 heads 80 -> 41; 16 x 100, 8 heads 16.8 -> 15.4;
+  // 8 x 100 12.3 -> 13.5; 2 x 96, 12 heads 11.8 -> 13.3.  Up to 64 rows half of that tile is padding: 64 x 50, 16 heads 33.6 -> 34.6.
+  if (attention_bwd_ragged_t5_supported(nseq, T, H, d) && (T > 128 || (T > 64 && (int64_t)nseq * H * 4 > 3 * (int64_t)num_sms())))
+    return attention_bwd_ragged_t5(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
   switch ((d / H + 31) / 32) {
     case 1: return launch_bwd<32, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);
     case 2: return launch_bwd<64, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);

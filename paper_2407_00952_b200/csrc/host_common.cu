@@ -21,7 +21,7 @@ int g_sms[MAX_DEVICES] = {};
 int* g_status_addr[MAX_DEVICES] = {};
 
 struct MapKey {
-  uint64_t ptr, rows, cols, ld;
+  uint64_t ptr, planes, rows, cols, ld, plane_ld;      // planes 0: two-dimensional
   uint32_t box_cols, box_rows, swizzle, promo;
   int32_t dev, pad;
   bool operator==(const MapKey& o) const { return std::memcmp(this, &o, sizeof(MapKey)) == 0; }
@@ -82,13 +82,14 @@ int* library_status_word() {
   return g_status_addr[dev];
 }
 
-bool cached_map_2d(CUtensorMap* out, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols,
-                   uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promo) {
+namespace {
+bool cached_map(CUtensorMap* out, const void* ptr, uint64_t planes, uint64_t rows, uint64_t cols, uint64_t ld, uint64_t plane_ld,
+                uint32_t box_cols, uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promo) {
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return false;
   MapKey k;
   std::memset(&k, 0, sizeof(k));
-  k.ptr = (uint64_t)(uintptr_t)ptr; k.rows = rows; k.cols = cols; k.ld = ld;
+  k.ptr = (uint64_t)(uintptr_t)ptr; k.planes = planes; k.rows = rows; k.cols = cols; k.ld = ld; k.plane_ld = plane_ld;
   k.box_cols = box_cols; k.box_rows = box_rows; k.swizzle = (uint32_t)swizzle; k.promo = (uint32_t)promo;
   k.dev = current_device();
   {
@@ -96,17 +97,28 @@ bool cached_map_2d(CUtensorMap* out, const void* ptr, uint64_t rows, uint64_t co
     auto it = g_maps.find(k);
     if (it != g_maps.end()) { *out = it->second; return true; }
   }
-  cuuint64_t dims[2] = {cols, rows};
-  cuuint64_t strides[1] = {ld * 2};
-  cuuint32_t box[2] = {box_cols, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  if (enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+  cuuint64_t dims[3] = {cols, rows, planes};
+  cuuint64_t strides[2] = {ld * 2, plane_ld * 2};
+  cuuint32_t box[3] = {box_cols, box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  if (enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, planes > 0 ? 3 : 2, const_cast<void*>(ptr), dims, strides, box, estr,
           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return false;
   std::lock_guard<std::mutex> lock(g_mutex);
   if (g_maps.size() >= MAP_CACHE_LIMIT) g_maps.clear();
   g_maps.emplace(k, *out);
   return true;
+}
+}  // namespace
+
+bool cached_map_2d(CUtensorMap* out, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols,
+                   uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promo) {
+  return cached_map(out, ptr, 0, rows, cols, ld, 0, box_cols, box_rows, swizzle, promo);
+}
+
+bool cached_map_3d(CUtensorMap* out, const void* ptr, uint64_t planes, uint64_t rows, uint64_t cols, uint64_t ld, uint64_t plane_ld,
+                   uint32_t box_cols, uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promo) {
+  return cached_map(out, ptr, planes, rows, cols, ld, plane_ld, box_cols, box_rows, swizzle, promo);
 }
 
 }  // namespace sl

@@ -39,5 +39,9 @@ struct PerDeviceOnce {
 // its maps here instead of encoding six or seven of them.
 bool cached_map_2d(CUtensorMap* out, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols,
                    uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promo);
+// The same for `planes` matrices [rows, cols] plane_ld elements apart; a box lies in one plane, and rows past the end of a
+// plane are filled with zeros (loads) or left out (stores).
+bool cached_map_3d(CUtensorMap* out, const void* ptr, uint64_t planes, uint64_t rows, uint64_t cols, uint64_t ld, uint64_t plane_ld,
+                   uint32_t box_cols, uint32_t box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion promo);
 
 }  // namespace sl

@@ -116,7 +116,11 @@ bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const voi
                                 const void* dqkv);
 cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st);
 cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
-                                 int d, void* dqkv, float* rowdot, cudaStream_t st);
+                                 int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
+// the backward pass of those of width 64 on tcgen05 (attention_t5_ragged.cu); status as above
+bool attention_bwd_ragged_t5_supported(int nseq, int T, int H, int d);
+cudaError_t attention_bwd_ragged_t5(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
+                                    int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
 
 // Adapter gradients: for nt targets of rank r (weight columns wcol0 + t*rp + jj of Wt),
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c],  c < C,

@@ -521,7 +521,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
     if (aligned_form)
       e = attention_bwd_tc(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->status, c->st);
     else if (ragged_form)
-      e = attention_bwd_ragged(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->st);
+      e = attention_bwd_ragged(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->status, c->st);
     else
       e = attention_bwd_simt(c->dt, qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->st);
     if (e) return e; }
