@@ -651,7 +651,7 @@ cudaError_t aggregate_broadcast(const float* sum, int K, int64_t P, float* param
 // adapter compute copies (only live entries are written; the padding was zeroed once)
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void adapter_copy_kernel(AdapterCopyArgs a) {
+__global__ void adapter_copy_kernel(const __grid_constant__ AdapterCopyArgs a) {
   overlap_sync();
   const int64_t nA = (int64_t)a.r * a.d_in, nB = (int64_t)a.r * a.d_out;
   const int64_t per_t = nA + nB;
@@ -662,10 +662,14 @@ __global__ void adapter_copy_kernel(AdapterCopyArgs a) {
   int64_t rem = idx % (a.n_targets * per_t);
   const int t = (int)(rem / per_t);
   rem = rem % per_t;
-  T* Acat = (T*)a.Acat; T* AcatT = (T*)a.AcatT; T* Bext = (T*)a.Bext; T* BextT = (T*)a.BextT;
+  const int64_t layer = blockIdx.y, la = layer * a.acat_ls, lb = layer * a.bext_ls;
+  const float* A = a.A + layer * a.layer_stride;
+  const float* B = a.B + layer * a.layer_stride;
+  T* Acat = a.Acat ? (T*)a.Acat + la : nullptr; T* AcatT = a.AcatT ? (T*)a.AcatT + la : nullptr;
+  T* Bext = a.Bext ? (T*)a.Bext + lb : nullptr; T* BextT = a.BextT ? (T*)a.BextT + lb : nullptr;
   if (rem < nA) {
     const int j = (int)(rem / a.d_in), c = (int)(rem % a.d_in);
-    const float av = a.A[(size_t)g * a.a_gs + (size_t)t * a.a_ts + (size_t)j * a.d_in + c];
+    const float av = A[(size_t)g * a.a_gs + (size_t)t * a.a_ts + (size_t)j * a.d_in + c];
     const int col = t * a.rp + j;
     const size_t base = (size_t)g * a.ext * a.d_in;
     if (Acat) Acat[base + (size_t)col * a.d_in + c] = from_f<T>(av);
@@ -673,7 +677,7 @@ __global__ void adapter_copy_kernel(AdapterCopyArgs a) {
   } else {
     rem -= nA;
     const int c = (int)(rem / a.r), j = (int)(rem % a.r);
-    const float bv = a.scale * a.B[(size_t)g * a.b_gs + (size_t)t * a.b_ts + (size_t)c * a.r + j];
+    const float bv = a.scale * B[(size_t)g * a.b_gs + (size_t)t * a.b_ts + (size_t)c * a.r + j];
     const int col = t * a.rp + j;
     const int row = a.slice_off[t] + c;
     const size_t base = (size_t)g * a.n_out * a.ext;
@@ -685,7 +689,7 @@ __global__ void adapter_copy_kernel(AdapterCopyArgs a) {
 cudaError_t refresh_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st) {
   int64_t total = (int64_t)a.G * a.n_targets * a.r * ((int64_t)a.d_in + a.d_out);
   if (total == 0) return cudaSuccess;
-  unsigned blocks = (unsigned)((total + 255) / 256);
+  const dim3 blocks((unsigned)((total + 255) / 256), (unsigned)a.layers);
   if (a.dtype == DT_BF16) launch_overlapped(adapter_copy_kernel<bf16>, blocks, 256, 0, st, a);
   else launch_overlapped(adapter_copy_kernel<float>, blocks, 256, 0, st, a);
   return cudaGetLastError();

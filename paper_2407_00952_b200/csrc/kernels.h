@@ -173,7 +173,7 @@ cudaError_t aggregate(float* params, int K, int64_t P, const float* w_host, cuda
 cudaError_t aggregate_local_sum(const float* params, int K, int64_t P, const float* w_host, float* sum, cudaStream_t st);
 cudaError_t aggregate_broadcast(const float* sum, int K, int64_t P, float* params, cudaStream_t st);
 
-// Compute copies of the adapters of one layer (G groups), built from fp32 masters.
+// Compute copies of the adapters of `layers` layers (G groups), built from fp32 masters.
 // Target t of group g has A_t [r, d_in] at A + g*a_gs + t*a_ts and B_t [d_out, r] at B + g*b_gs + t*b_ts.
 // With col = t*rp + j the copies are
 //   Acat  [G][ext, d_in]  : Acat[col, c]  = A_t[j, c]          AcatT [G][d_in, ext] : its transpose
@@ -188,9 +188,11 @@ struct AdapterCopyArgs {
   int slice_off[4];
   float scale;
   void *Acat, *AcatT, *Bext, *BextT;   // any of them may be null (skipped)
+  int layers = 1;                      // of layers further on: masters layer_stride, Acat / AcatT acat_ls, Bext / BextT bext_ls elements apart
+  int64_t layer_stride = 0, acat_ls = 0, bext_ls = 0;
   int* status = nullptr;               // write_adapter_copies: a word to clear
 };
-// The same for one target (n_targets 1, slice_off 0, n_out = d_out) into uninitialised copies: padding included.
+// The same for one layer and target (n_targets 1, slice_off 0, n_out = d_out) into uninitialised copies: padding included.
 cudaError_t write_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st);
 cudaError_t refresh_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st);
 
