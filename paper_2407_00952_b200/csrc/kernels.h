@@ -139,22 +139,25 @@ struct LoraGradJob {
   const void* Wt = nullptr; int64_t ldwt = 0; int wcol0 = 0, r = 0, rp = 0, nt = 1;
   float scale = 1.f; float* out = nullptr;
   int64_t out_group_stride = 0, out_target_stride = 0, out_sj = 0, out_sc = 0;
+  int64_t z_ls = 0, wt_ls = 0, out_ls = 0;     // lora_grad_layers: elements between two layers
 };
+// Up to LORA_GRAD_MAX_JOBS reductions of each of `layers` layers at once (the adapter gradients of a side of the model), all
+// with the same C: one launch, or two where the rows of a group are split.  Whether the shapes are taken:
+constexpr int LORA_GRAD_MAX_JOBS = 6;
+bool lora_grad_layers_supported(int dt, const LoraGradJob* jobs, int njobs, int layers, int M, int rows_per_group, bool use_tc);
+cudaError_t lora_grad_layers(int dt, const LoraGradJob* jobs, int njobs, int layers, int M, int rows_per_group, float* partial,
+                             size_t partial_floats, cudaStream_t st, int* status, bool use_tc);
+// its tcgen05 form: partials of chunks > 1 as [job][layer][chunk][R_j][C], results directly where a group is one chunk
+cudaError_t lora_grad_tc_layers(const LoraGradJob* jobs, int njobs, int layers, int M, int rows_per_group, float* partial,
+                                size_t partial_floats, int* status, int* chunks_per_group, size_t* offsets, cudaStream_t st);
 // partial: scratch of partial_floats floats.  Falls back to one lora_grad per job where the batched
 // tensor-core path does not apply.
 cudaError_t lora_grad_batch(int dt, const LoraGradJob* jobs, int njobs, int M, int rows_per_group, float* partial,
                             size_t partial_floats, cudaStream_t st, int* status, bool use_tc);
-cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M, int rows_per_group, float* partial,
-                                       size_t partial_floats, int* status, int* chunks_per_group, size_t* offsets,
-                                       cudaStream_t st);
-// The same reduction as a tcgen05 product with both operands MN-major (bf16, rp in {16, 32, 64},
-// ldwt a multiple of 64, the wanted weight columns inside one 64-column tile).  Writes per-chunk
-// partials [chunk][nt*r][C]; lora_grad adds them.  status: device word for an expired bounded wait.
+// The reduction as a tcgen05 product with both operands MN-major takes bf16, rp in {16, 32, 64}, ldwt a multiple of 64 and
+// the wanted weight columns inside one 64-column tile.  status: device word for an expired bounded wait.
 bool lora_grad_tc_supported(int dt, const void* Z, int64_t ldz, int zcol0, int C, const void* Wt, int64_t ldwt,
                             int wcol0, int r, int rp, int nt, int M, int rows_per_group);
-cudaError_t lora_grad_tc_partial(const void* Z, int64_t ldz, int zcol0, int C, const void* Wt, int64_t ldwt, int wcol0,
-                                 int r, int rp, int nt, int M, int rows_per_group, float* partial, int* status,
-                                 int* chunks_per_group, cudaStream_t st);
 
 struct OptArgs {
   int optimizer; float lr, beta1, beta2, eps, wd; float bc1, bc2;   // bc = 1 - beta^step

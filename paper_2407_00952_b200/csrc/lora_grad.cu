@@ -158,24 +158,114 @@ lora_grad_reduce_lanes_kernel(const float* __restrict__ partial, int r, int R, i
   }
 }
 
-// The second kernel for a batch of jobs (blockIdx.z): one output per thread, chunks added in order.
-struct RedJob { const float* partial; float* out; int r, R, C; float scale; int64_t ogs, ots, osj, osc; };
-struct RedBatch { RedJob j[4]; };
+// The second kernel for a batch of jobs and layers (blockIdx.z): one output per thread, chunks added in order.
+struct RedJob { const float* partial; float* out; int r, R, C; float scale; int64_t ols, ogs, ots, osj, osc; };
+struct RedBatch { RedJob j[LORA_GRAD_MAX_JOBS]; int njobs; };
 __global__ void __launch_bounds__(RED_THREADS)
 lora_grad_reduce_batch_kernel(RedBatch b, int chunks_per_group) {
   overlap_sync();
-  const RedJob& jb = b.j[blockIdx.z];
+  const int layer = (int)blockIdx.z / b.njobs;
+  const RedJob& jb = b.j[(int)blockIdx.z % b.njobs];
   const int idx = blockIdx.x * RED_THREADS + threadIdx.x;   // over R*C
   const int g = blockIdx.y;
   const int C = jb.C;
   if (idx >= jb.R * C) return;
   const size_t rc = (size_t)jb.R * C;
-  const float* p = jb.partial + (size_t)g * chunks_per_group * rc + idx;
+  const float* p = jb.partial + ((size_t)layer * gridDim.y + g) * chunks_per_group * rc + idx;
   float s = 0.f;
 #pragma unroll 4
   for (int k = 0; k < chunks_per_group; ++k) s += p[(size_t)k * rc];
   const int j = idx / C, c = idx % C;
-  jb.out[(size_t)g * jb.ogs + (size_t)(j / jb.r) * jb.ots + (size_t)(j % jb.r) * jb.osj + (size_t)c * jb.osc] = jb.scale * s;
+  jb.out[(size_t)layer * jb.ols + (size_t)g * jb.ogs + (size_t)(j / jb.r) * jb.ots + (size_t)(j % jb.r) * jb.osj + (size_t)c * jb.osc] = jb.scale * s;
+}
+cudaError_t launch_reduce_batch(const LoraGradJob* jobs, int njobs, int layers, int groups, int chunks, const float* partial,
+                                const size_t* offsets, cudaStream_t st) {
+  RedBatch rb;
+  int maxRC = 0;
+  for (int j = 0; j < LORA_GRAD_MAX_JOBS; ++j) {
+    const LoraGradJob& jb = jobs[j < njobs ? j : 0];
+    rb.j[j] = {partial + offsets[j < njobs ? j : 0], jb.out, jb.r, jb.nt * jb.r, jb.C, jb.scale, jb.out_ls, jb.out_group_stride,
+               jb.out_target_stride, jb.out_sj, jb.out_sc};
+    if (jb.nt * jb.r * jb.C > maxRC) maxRC = jb.nt * jb.r * jb.C;
+  }
+  rb.njobs = njobs;
+  launch_overlapped(lora_grad_reduce_batch_kernel, dim3((maxRC + RED_THREADS - 1) / RED_THREADS, groups, layers * njobs), RED_THREADS, 0, st, rb, chunks);
+  return cudaGetLastError();
+}
+
+// fp32, the jobs of all layers of a side in one launch.  A block: RJ weight columns x 128 feature columns (32 threads of
+// four) x one chunk of a group's rows, over 32 row lanes that are summed through shared memory in a fixed order; the result
+// goes to the gradient where the chunk is the whole group, else to scratch as [job][layer][chunk][R][C].  What bounds it is
+// the number of launches it replaces (two per job and layer, 4-5 us each): 512 tokens of width 128 are 16 loads per lane.
+constexpr int LL_CT = 32, LL_RL = 32, LL_ROWS = 512;
+struct LayersJob { const float *Z, *Wt; int64_t ldz, zls, ldwt, wls; int r, rp, R, C, jtile0; float* partial; float* out; int64_t ols, ogs, ots, osj, osc; float scale; };
+struct LayersBatch { LayersJob j[LORA_GRAD_MAX_JOBS]; int njobs, jtiles, rows_per_group, chunks, chunk_rows, M; };
+__global__ void __launch_bounds__(LL_CT * LL_RL) lora_grad_layers_kernel(const __grid_constant__ LayersBatch b) {
+  overlap_sync();
+  __shared__ float red[LL_RL / 2][RJ * 4][LL_CT];
+  const int layer = (int)blockIdx.z / b.jtiles, jt = (int)blockIdx.z % b.jtiles;
+  int job = 0;
+  while (job + 1 < b.njobs && jt >= b.j[job + 1].jtile0) ++job;
+  const LayersJob& jb = b.j[job];
+  const int j0 = (jt - jb.jtile0) * RJ;
+  const int tx = threadIdx.x, ty = threadIdx.y, c = (blockIdx.x * LL_CT + tx) * 4;
+  const int g = (int)blockIdx.y / b.chunks, chunk = (int)blockIdx.y % b.chunks;
+  const int m0 = g * b.rows_per_group + chunk * b.chunk_rows;
+  const int m1 = min(min(m0 + b.chunk_rows, (g + 1) * b.rows_per_group), b.M);
+  const bool active = c < jb.C;
+  const float* Z = jb.Z + layer * jb.zls + c;
+  const float* Wt = jb.Wt + layer * jb.wls;
+  int wc[RJ];
+#pragma unroll
+  for (int j = 0; j < RJ; ++j) wc[j] = j0 + j < jb.R ? (j0 + j) / jb.r * jb.rp + (j0 + j) % jb.r : -1;
+  float acc[RJ][4];
+#pragma unroll
+  for (int j = 0; j < RJ; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
+  if (active) {
+#pragma unroll 4
+    for (int m = m0 + ty; m < m1; m += LL_RL) {
+      const float4 z = *reinterpret_cast<const float4*>(Z + (size_t)m * jb.ldz);
+#pragma unroll
+      for (int j = 0; j < RJ; ++j) {
+        const float w = wc[j] >= 0 ? Wt[(size_t)m * jb.ldwt + wc[j]] : 0.f;
+        acc[j][0] = fmaf(w, z.x, acc[j][0]); acc[j][1] = fmaf(w, z.y, acc[j][1]);
+        acc[j][2] = fmaf(w, z.z, acc[j][2]); acc[j][3] = fmaf(w, z.w, acc[j][3]);
+      }
+    }
+  }
+#pragma unroll
+  for (int half = LL_RL / 2; half > 0; half >>= 1) {
+    if (ty >= half && ty < 2 * half) {
+#pragma unroll
+      for (int j = 0; j < RJ; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) red[ty - half][j * 4 + i][tx] = acc[j][i];
+    }
+    __syncthreads();
+    if (ty < half) {
+#pragma unroll
+      for (int j = 0; j < RJ; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[j][i] += red[ty][j * 4 + i][tx];
+    }
+    __syncthreads();
+  }
+  if (ty != 0 || !active) return;
+#pragma unroll
+  for (int j = 0; j < RJ; ++j) {
+    const int jj = j0 + j;
+    if (jj >= jb.R) break;
+    if (jb.partial) {
+      *reinterpret_cast<float4*>(jb.partial + (((size_t)layer * gridDim.y + blockIdx.y) * jb.R + jj) * jb.C + c) =
+          make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+    } else {
+      float* o = jb.out + (size_t)layer * jb.ols + (size_t)g * jb.ogs + (size_t)(jj / jb.r) * jb.ots + (size_t)(jj % jb.r) * jb.osj;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) o[(size_t)(c + i) * jb.osc] = jb.scale * acc[j][i];
+    }
+  }
 }
 
 // picks the second kernel by the number of outputs (both add in a fixed order)
@@ -232,10 +322,14 @@ cudaError_t lora_grad(int dt, const void* Z, int64_t ldz, int zcol0, int C, cons
       for (int t0 = 0; t0 < nt; t0 += tw) {
         const int ntw = min(tw, nt - t0), Rw = ntw * r;
         int cpg = 0;
-        cudaError_t e = lora_grad_tc_partial(Z, ldz, zcol0, C, Wt, ldwt, wcol0 + t0 * rp, r, rp, ntw, M, rows_per_group,
-                                             partial, status, &cpg, st);
+        LoraGradJob jb;
+        jb.Z = Z; jb.ldz = ldz; jb.zcol0 = zcol0; jb.C = C; jb.Wt = Wt; jb.ldwt = ldwt; jb.wcol0 = wcol0 + t0 * rp; jb.r = r; jb.rp = rp; jb.nt = ntw;
+        jb.scale = scale; jb.out = out + (size_t)t0 * out_target_stride; jb.out_group_stride = out_group_stride; jb.out_target_stride = out_target_stride;
+        jb.out_sj = out_sj; jb.out_sc = out_sc;
+        size_t off;
+        cudaError_t e = lora_grad_tc_layers(&jb, 1, 1, M, rows_per_group, partial, (size_t)-1, status, &cpg, &off, st);
         if (e != cudaSuccess) return e;
-        launch_reduce(partial, r, Rw, C, cpg, groups, scale, out + (size_t)t0 * out_target_stride, out_group_stride,
+        if (cpg > 1) launch_reduce(partial, r, Rw, C, cpg, groups, scale, out + (size_t)t0 * out_target_stride, out_group_stride,
                       out_target_stride, out_sj, out_sc, st);
       }
       return cudaGetLastError();
@@ -263,34 +357,64 @@ cudaError_t lora_grad(int dt, const void* Z, int64_t ldz, int zcol0, int C, cons
   return cudaGetLastError();
 }
 
+bool lora_grad_layers_supported(int dt, const LoraGradJob* jobs, int njobs, int layers, int M, int rows_per_group, bool use_tc) {
+  if (njobs < 1 || njobs > LORA_GRAD_MAX_JOBS || layers < 1) return false;
+  const int groups = rows_per_group > 0 && rows_per_group < M ? M / rows_per_group : 1;
+  int64_t rows = 0;
+  for (int j = 0; j < njobs; ++j) {
+    const LoraGradJob& jb = jobs[j];
+    rows += jb.nt * jb.r;
+    if (dt == DT_BF16) {
+      if (!use_tc || !lora_grad_tc_supported(dt, jb.Z, jb.ldz, jb.zcol0, jb.C, jb.Wt, jb.ldwt, jb.wcol0, jb.r, jb.rp, jb.nt, M, rows_per_group))
+        return false;
+    } else if (jb.C % 4 != 0 || jb.ldz % 4 != 0 || jb.zcol0 % 4 != 0 || jb.z_ls % 4 != 0 || jb.C != jobs[0].C || M % groups != 0) {
+      return false;
+    }
+  }
+  return (int64_t)layers * rows <= 65535;                   // the grid's third dimension
+}
+
+cudaError_t lora_grad_layers(int dt, const LoraGradJob* jobs, int njobs, int layers, int M, int rows_per_group, float* partial,
+                             size_t partial_floats, cudaStream_t st, int* status, bool use_tc) {
+  if (!lora_grad_layers_supported(dt, jobs, njobs, layers, M, rows_per_group, use_tc)) return cudaErrorInvalidValue;
+  const int groups = rows_per_group > 0 && rows_per_group < M ? M / rows_per_group : 1;
+  size_t offs[LORA_GRAD_MAX_JOBS];
+  int cpg = 0;
+  if (dt == DT_BF16) {
+    cudaError_t e = lora_grad_tc_layers(jobs, njobs, layers, M, rows_per_group, partial, partial_floats, status, &cpg, offs, st);
+    if (e != cudaSuccess || cpg == 1) return e;
+    return launch_reduce_batch(jobs, njobs, layers, groups, cpg, partial, offs, st);
+  }
+  LayersBatch b;
+  b.njobs = njobs; b.M = M; b.rows_per_group = M / groups;
+  size_t set_floats = 0;
+  b.jtiles = 0;
+  for (int j = 0; j < njobs; ++j) set_floats += (size_t)layers * groups * jobs[j].nt * jobs[j].r * jobs[j].C;
+  cpg = (b.rows_per_group + LL_ROWS - 1) / LL_ROWS;
+  if ((size_t)cpg > partial_floats / set_floats) cpg = partial_floats / set_floats > 1 ? (int)(partial_floats / set_floats) : 1;
+  b.chunk_rows = (b.rows_per_group + cpg - 1) / cpg;
+  b.chunks = cpg;
+  size_t off = 0;
+  for (int j = 0; j < LORA_GRAD_MAX_JOBS; ++j) {
+    const LoraGradJob& jb = jobs[j < njobs ? j : 0];
+    const int R = jb.nt * jb.r;
+    b.j[j] = {(const float*)jb.Z + jb.zcol0, (const float*)jb.Wt + jb.wcol0, jb.ldz, jb.z_ls, jb.ldwt, jb.wt_ls, jb.r, jb.rp, R, jb.C, b.jtiles,
+              cpg > 1 ? partial + off : nullptr, jb.out, jb.out_ls, jb.out_group_stride, jb.out_target_stride, jb.out_sj, jb.out_sc, jb.scale};
+    if (j >= njobs) continue;
+    offs[j] = off;
+    off += (size_t)layers * groups * cpg * R * jb.C;
+    b.jtiles += (R + RJ - 1) / RJ;
+  }
+  const dim3 grid((jobs[0].C / 4 + LL_CT - 1) / LL_CT, groups * cpg, layers * b.jtiles);
+  launch_overlapped(lora_grad_layers_kernel, grid, dim3(LL_CT, LL_RL), 0, st, b);
+  if (cpg == 1) return cudaGetLastError();
+  return launch_reduce_batch(jobs, njobs, layers, groups, cpg, partial, offs, st);
+}
+
 cudaError_t lora_grad_batch(int dt, const LoraGradJob* jobs, int njobs, int M, int rows_per_group, float* partial,
                             size_t partial_floats, cudaStream_t st, int* status, bool use_tc) {
-  bool batched = use_tc && status && dt == DT_BF16 && njobs >= 1 && njobs <= 4;
-  for (int j = 0; j < njobs && batched; ++j) {
-    const LoraGradJob& jb = jobs[j];
-    batched = (jb.rp == 16 || jb.rp == 32 || jb.rp == 64) &&
-              lora_grad_tc_supported(dt, jb.Z, jb.ldz, jb.zcol0, jb.C, jb.Wt, jb.ldwt, jb.wcol0, jb.r, jb.rp, jb.nt, M, rows_per_group);
-  }
-  if (batched) {
-    const int groups = rows_per_group > 0 && rows_per_group < M ? M / rows_per_group : 1;
-    int cpg = 0;
-    size_t offs[4];
-    cudaError_t e = lora_grad_tc_partial_batch(jobs, njobs, M, rows_per_group, partial, partial_floats, status, &cpg, offs, st);
-    if (e == cudaSuccess) {
-      RedBatch rb;
-      int maxRC = 0;
-      for (int j = 0; j < 4; ++j) {
-        const LoraGradJob& jb = jobs[j < njobs ? j : 0];
-        rb.j[j] = {partial + offs[j < njobs ? j : 0], jb.out, jb.r, jb.nt * jb.r, jb.C, jb.scale, jb.out_group_stride,
-                   jb.out_target_stride, jb.out_sj, jb.out_sc};
-        if (j < njobs && jb.nt * jb.r * jb.C > maxRC) maxRC = jb.nt * jb.r * jb.C;
-      }
-      dim3 g2((maxRC + RED_THREADS - 1) / RED_THREADS, groups, njobs);
-      launch_overlapped(lora_grad_reduce_batch_kernel, g2, RED_THREADS, 0, st, rb, cpg);
-      return cudaGetLastError();
-    }
-    if (e != cudaErrorInvalidValue) return e;      // invalid value: the scratch does not hold the batch, go one by one
-  }
+  if (dt == DT_BF16 && status && lora_grad_layers_supported(dt, jobs, njobs, 1, M, rows_per_group, use_tc))
+    return lora_grad_layers(dt, jobs, njobs, 1, M, rows_per_group, partial, partial_floats, st, status, use_tc);
   for (int j = 0; j < njobs; ++j) {
     const LoraGradJob& jb = jobs[j];
     cudaError_t e = lora_grad(dt, jb.Z, jb.ldz, jb.zcol0, jb.C, jb.Wt, jb.ldwt, jb.wcol0, jb.r, jb.rp, jb.nt, M, rows_per_group,

@@ -5,9 +5,9 @@
 //   D[c, j] (128 x 64, fp32 in tensor memory) += Z_tile^T (128 c x 64 tokens) * Wt_tile (64 tokens x 64 j)
 // One CTA owns 128 feature columns and one chunk of the token range; TMA streams 64-token blocks
 // through a 4-stage ring, one thread issues the products, four warps read the accumulator back and
-// write the wanted columns to scratch; a second kernel adds the chunks in a fixed order (no float
-// atomics).  HBM-bound: every Z element is read once, the 64-column weight tile is re-read per
-// column tile (from L2).
+// write the wanted columns to scratch, where a second kernel adds the chunks in a fixed order (no float
+// atomics), or straight to the gradient where a group's rows are one chunk.  HBM-bound: every Z element is
+// read once, the 64-column weight tile is re-read per column tile (from L2).
 #include <cuda.h>
 
 #include "common.cuh"
@@ -36,20 +36,23 @@ constexpr uint32_t LT_IDESC = make_idesc(LT_C, LT_N) | (1u << 15) | (1u << 16);
 
 struct LgParams {
   int C, rows_per_chunk, R, r, rp, wsel0;
-  float* partial;
+  float* partial;                                // [layer][chunk][R][C], or nullptr: a group is one chunk
+  float* out; int64_t out_ls, ogs, ots, osj, osc; float scale;
   int* status;
 };
-// Up to LT_MAX_JOBS reductions over the same token rows in one launch (blockIdx.z picks the job): the
-// adapter gradients of one layer, e.g. G_A of all targets from u and G_B of each target from its slice
-// of dy.  One launch instead of one per job: the jobs are short (tens of microseconds), so their start-up,
-// tail and launch gaps weigh as much as their traffic.
-constexpr int LT_MAX_JOBS = 4;
+// Up to LT_MAX_JOBS reductions over the same token rows, of several layers, in one launch (blockIdx.z picks layer and
+// job): the adapter gradients of a layer, e.g. G_A of all targets from u and G_B of each target from its slice of dy, or
+// those of all layers of a side.  One launch instead of one per job: the jobs are short (microseconds to tens of them), so
+// their start-up, tail and launch gaps weigh as much as their traffic.
+constexpr int LT_MAX_JOBS = LORA_GRAD_MAX_JOBS;
 struct LgBatch {
   CUtensorMap mapZ[LT_MAX_JOBS];
   CUtensorMap mapW[LT_MAX_JOBS];
   LgParams p[LT_MAX_JOBS];
   int wx0[LT_MAX_JOBS];
+  int njobs;
 };
+static_assert(sizeof(LgBatch) <= 4000, "kernel parameters");
 
 // MN-major operand stored as [k rows][64 elements] boxes (128-byte rows, 128-byte swizzle): groups
 // of 8 k-rows are 1024 bytes apart; `mn_stride` is the distance between consecutive 64-element
@@ -64,12 +67,15 @@ __device__ __forceinline__ uint64_t desc_mn(uint32_t addr, uint32_t mn_stride) {
   return d;
 }
 
+// LAYERS: the operands are planes of three-dimensional maps, one per layer (a single layer: two-dimensional ones).
+template <bool LAYERS>
 __global__ void __launch_bounds__(LT_THREADS, 2)
 lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
-  const CUtensorMap& mapZ = bt.mapZ[blockIdx.z];
-  const CUtensorMap& mapW = bt.mapW[blockIdx.z];
-  const LgParams& p = bt.p[blockIdx.z];
-  const int wx0 = bt.wx0[blockIdx.z];
+  const int layer = LAYERS ? (int)blockIdx.z / bt.njobs : 0, job = LAYERS ? (int)blockIdx.z % bt.njobs : (int)blockIdx.z;
+  const CUtensorMap& mapZ = bt.mapZ[job];
+  const CUtensorMap& mapW = bt.mapW[job];
+  const LgParams& p = bt.p[job];
+  const int wx0 = bt.wx0[job];
   if ((int)blockIdx.x * LT_C >= p.C) return;             // the grid is as wide as the widest job
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -113,9 +119,12 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
       const int row = row0 + kb * LT_K;
       if (leader) {
         mbar_expect_tx(FULL(s), LT_STAGE);
-        tma_load_2d(dst, &mapZ, FULL(s), c0, row);
-        tma_load_2d(dst + LT_ZBOX, &mapZ, FULL(s), c0 + 64, row);      // past the last column: zero fill
-        tma_load_2d(dst + 2 * LT_ZBOX, &mapW, FULL(s), wx0, row);
+        auto load = [&](uint32_t to, const CUtensorMap* map, int c) {
+          if constexpr (LAYERS) tma_load_3d(to, map, FULL(s), c, row, layer); else tma_load_2d(to, map, FULL(s), c, row);
+        };
+        load(dst, &mapZ, c0);
+        load(dst + LT_ZBOX, &mapZ, c0 + 64);       // past the last column: zero fill
+        load(dst + 2 * LT_ZBOX, &mapW, wx0);
       }
       __syncwarp();
     }
@@ -149,14 +158,16 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
       tc_wait_ld();
       const int c = c0 + q * 32 + lane;
       if (c < p.C) {
-        float* out = p.partial + (size_t)chunk * p.R * p.C + c;
         const int sh = p.rp == 16 ? 4 : (p.rp == 32 ? 5 : 6);
+        float* out = p.partial ? p.partial + ((size_t)layer * gridDim.y + chunk) * p.R * p.C + c
+                               : p.out + (size_t)layer * p.out_ls + (size_t)chunk * p.ogs + (size_t)c * p.osc;
+        const int64_t ots = p.partial ? (int64_t)p.r * p.C : p.ots, osj = p.partial ? p.C : p.osj;
+        const float scale = p.partial ? 1.f : p.scale;
 #pragma unroll
         for (int col = 0; col < LT_N; ++col) {
           const int rel = col - p.wsel0;
           const int t = rel >> sh, jj = rel & (p.rp - 1);
-          const int j = t * p.r + jj;
-          if (rel >= 0 && jj < p.r && j < p.R) out[(size_t)j * p.C] = v[col];
+          if (rel >= 0 && jj < p.r && t * p.r + jj < p.R) out[t * ots + jj * osj] = scale * v[col];
         }
       }
     }
@@ -176,18 +187,18 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
 
 PerDeviceOnce g_once;
 
-// bf16 [rows, cols] with leading dimension ld; box = 64 columns x 64 rows, 128-byte swizzle
-bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t ld) {
-  return cached_map_2d(m, ptr, rows, cols, ld, 64, (uint32_t)LT_K, CU_TENSOR_MAP_SWIZZLE_128B,
-                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+// `layers` bf16 matrices [rows, cols] with leading dimension ld, ls elements apart; box = 64 columns x 64 rows, 128-byte swizzle
+bool make_map(CUtensorMap* m, const void* ptr, uint64_t layers, uint64_t rows, uint64_t cols, uint64_t ld, uint64_t ls) {
+  if (layers == 1) return cached_map_2d(m, ptr, rows, cols, ld, 64, (uint32_t)LT_K, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+  return cached_map_3d(m, ptr, layers, rows, cols, ld, ls, 64, (uint32_t)LT_K, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
 bool init_device() {
   const int dev = current_device();
   if (dev < 0 || !tensor_map_encoder()) return false;
   if (!g_once.needed(dev)) return true;
-  if (cudaFuncSetAttribute(lora_grad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_SMEM) != cudaSuccess)
-    return false;
+  for (auto kernel : {lora_grad_tc_kernel<false>, lora_grad_tc_kernel<true>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_SMEM) != cudaSuccess) return false;
   g_once.done(dev);
   return true;
 }
@@ -208,26 +219,26 @@ bool lora_grad_tc_supported(int dt, const void* Z, int64_t ldz, int zcol0, int C
 }
 
 // Chunks per group (at most max_chunks) for a grid of `ctas_per_chunk_set` CTAs per chunk: the choice that minimises
-// (waves of 296 resident CTAs) x (rows per chunk), every chunk a whole number of 128-row blocks.
+// (waves of 296 resident CTAs) x (rows per chunk), every chunk a whole number of 128-row blocks.  One chunk needs no second
+// kernel, which is worth about 4 us: 1000 rows of a CTA that has an SM's loads to itself, 300 of one among two per SM.
 static int pick_chunks(int ctas_per_chunk_set, int rpg, int64_t max_chunks) {
+  const double second_kernel = ctas_per_chunk_set > 148 ? 300.0 : 1000.0;
   int best = 1;
   double best_cost = 1e300;
-  for (int s = 1; s <= rpg / 128 && s <= max_chunks; ++s) {
+  for (int s = 1; s <= rpg / 128 && s <= (max_chunks > 1 ? max_chunks : 1); ++s) {
     if (rpg % (s * 128) != 0) continue;
     const int ctas = ctas_per_chunk_set * s;
-    const double cost = (double)((ctas + 295) / 296) * ((double)rpg / s + 256.0);   // + a chunk's start-up, in rows
+    const double cost = (double)((ctas + 295) / 296) * ((double)rpg / s + 256.0) + (s > 1 ? second_kernel : 0.0);   // 256: a chunk's start-up
     if (cost < best_cost) { best_cost = cost; best = s; }
   }
   return best;
 }
 
-// Chunk partials of job j go to partial + offset_j as [chunk][R_j][C] (R_j = nt*r); *chunks_per_group
-// receives the number of chunks per group (the same for every job) so that the caller's second kernel
-// can add them, offsets[j] the start of job j's partials (floats).  All jobs share M and rows_per_group.
-cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M, int rows_per_group, float* partial,
-                                       size_t partial_floats, int* status, int* chunks_per_group, size_t* offsets,
-                                       cudaStream_t st) {
-  if (njobs < 1 || njobs > LT_MAX_JOBS) return cudaErrorInvalidValue;
+// All jobs share M and rows_per_group.  With more than one chunk per group (*chunks_per_group) the partials of job j go to
+// partial + offsets[j] as [layer][chunk][R_j][C] (R_j = nt*r) for the caller's second kernel to add.
+cudaError_t lora_grad_tc_layers(const LoraGradJob* jobs, int njobs, int layers, int M, int rows_per_group, float* partial,
+                                size_t partial_floats, int* status, int* chunks_per_group, size_t* offsets, cudaStream_t st) {
+  if (njobs < 1 || njobs > LT_MAX_JOBS || layers < 1) return cudaErrorInvalidValue;
   if (!init_device()) return cudaErrorNotSupported;
   if (!status) status = library_status_word();
   if (!status) return cudaErrorNotSupported;
@@ -235,43 +246,35 @@ cudaError_t lora_grad_tc_partial_batch(const LoraGradJob* jobs, int njobs, int M
   const int rpg = one ? (M + 127) / 128 * 128 : rows_per_group;
   const int groups = one ? 1 : M / rpg;
   int ctiles = 0, ctiles_sum = 0;
-  size_t set_floats = 0;                       // partials of one chunk per group, all jobs
+  size_t set_floats = 0;                       // partials of one chunk per group, all jobs and layers
   for (int j = 0; j < njobs; ++j) {
     const int t = (jobs[j].C + LT_C - 1) / LT_C;
     ctiles = t > ctiles ? t : ctiles;
     ctiles_sum += t;
-    set_floats += (size_t)groups * jobs[j].nt * jobs[j].r * jobs[j].C;
+    set_floats += (size_t)layers * groups * jobs[j].nt * jobs[j].r * jobs[j].C;
   }
-  if (set_floats > partial_floats) return cudaErrorInvalidValue;
-  // the scratch bounds the number of chunks (few tokens: it holds one chunk of every job, not two)
-  const int s = pick_chunks(ctiles_sum * groups, rpg, (int64_t)(partial_floats / set_floats));
+  const int s = pick_chunks(ctiles_sum * groups * layers, rpg, (int64_t)(partial_floats / set_floats));   // the scratch bounds the number of chunks
   LgBatch bt;
   size_t off = 0;
   for (int j = 0; j < njobs; ++j) {
     const LoraGradJob& jb = jobs[j];
-    if (!make_map(&bt.mapZ[j], (const bf16*)jb.Z + jb.zcol0, (uint64_t)M, (uint64_t)jb.C, (uint64_t)jb.ldz)) return cudaErrorInvalidValue;
-    if (!make_map(&bt.mapW[j], jb.Wt, (uint64_t)M, (uint64_t)jb.ldwt, (uint64_t)jb.ldwt)) return cudaErrorInvalidValue;
+    if (!make_map(&bt.mapZ[j], (const bf16*)jb.Z + jb.zcol0, (uint64_t)layers, (uint64_t)M, (uint64_t)jb.C, (uint64_t)jb.ldz, (uint64_t)jb.z_ls)) return cudaErrorInvalidValue;
+    if (!make_map(&bt.mapW[j], jb.Wt, (uint64_t)layers, (uint64_t)M, (uint64_t)jb.ldwt, (uint64_t)jb.ldwt, (uint64_t)jb.wt_ls)) return cudaErrorInvalidValue;
     LgParams& p = bt.p[j];
     p.C = jb.C; p.rows_per_chunk = rpg / s; p.R = jb.nt * jb.r; p.r = jb.r; p.rp = jb.rp; p.wsel0 = jb.wcol0 % LT_N;
-    p.partial = partial + off; p.status = status;
+    p.partial = s > 1 ? partial + off : nullptr; p.status = status;
+    p.out = jb.out; p.out_ls = jb.out_ls; p.ogs = jb.out_group_stride; p.ots = jb.out_target_stride; p.osj = jb.out_sj; p.osc = jb.out_sc;
+    p.scale = jb.scale;
     bt.wx0[j] = jb.wcol0 - p.wsel0;
     offsets[j] = off;
-    off += (size_t)groups * s * p.R * jb.C;
+    off += (size_t)layers * groups * s * p.R * jb.C;
   }
   for (int j = njobs; j < LT_MAX_JOBS; ++j) { bt.mapZ[j] = bt.mapZ[0]; bt.mapW[j] = bt.mapW[0]; bt.p[j] = bt.p[0]; bt.wx0[j] = bt.wx0[0]; }
-  dim3 grid(ctiles, groups * s, njobs);
-  launch_overlapped(lora_grad_tc_kernel, grid, LT_THREADS, LT_SMEM, st, bt);
+  bt.njobs = njobs;
+  dim3 grid(ctiles, groups * s, layers * njobs);
+  launch_overlapped(layers > 1 ? lora_grad_tc_kernel<true> : lora_grad_tc_kernel<false>, grid, LT_THREADS, LT_SMEM, st, bt);
   *chunks_per_group = s;
   return cudaGetLastError();
-}
-
-cudaError_t lora_grad_tc_partial(const void* Z, int64_t ldz, int zcol0, int C, const void* Wt, int64_t ldwt, int wcol0,
-                                 int r, int rp, int nt, int M, int rows_per_group, float* partial, int* status,
-                                 int* chunks_per_group, cudaStream_t st) {
-  LoraGradJob jb;
-  jb.Z = Z; jb.ldz = ldz; jb.zcol0 = zcol0; jb.C = C; jb.Wt = Wt; jb.ldwt = ldwt; jb.wcol0 = wcol0; jb.r = r; jb.rp = rp; jb.nt = nt;
-  size_t off;
-  return lora_grad_tc_partial_batch(&jb, 1, M, rows_per_group, partial, (size_t)-1, status, chunks_per_group, &off, st);
 }
 
 }  // namespace sl

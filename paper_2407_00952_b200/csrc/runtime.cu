@@ -34,6 +34,9 @@ struct LayerBuf {
   float *mean1 = nullptr, *rstd1 = nullptr, *mean2 = nullptr, *rstd2 = nullptr, *lse = nullptr;
   const void* x_in = nullptr;     // base (row 0) of the buffer the block read its input from
   void* hcat_o = nullptr;         // down-projected input of an adapter on the attention output projection
+  // gradients the adapter gradients are formed from: buffers of the layer's own where those wait for the end of the pass
+  // (splitlora_ctx::defer_grads), else the same for all layers
+  void *dqkv = nullptr, *dhcat = nullptr, *dxmid = nullptr, *dhcat_o = nullptr;
   // Adapter compute copies of this layer: `cl` holds one set per client, stacked (blocks the clients
   // run), `sv` the server's single set (blocks the server runs).  A block between the shallowest and the
   // deepest client cut is run by both sides and has both.
@@ -84,6 +87,7 @@ struct splitlora_ctx {
   uint32_t target_bit[4] = {0, 0, 0, 0};
   float scale = 1.f;
   bool tc = false;
+  bool defer_grads = false;   // adapter gradients of all layers of a side in one launch (see derive)
   // frozen
   const void *wte = nullptr, *wpe = nullptr, *lnfg = nullptr, *lnfb = nullptr, *headw = nullptr;
   void* wteT = nullptr;       // transposed head [d, Vpad]
@@ -103,8 +107,8 @@ struct splitlora_ctx {
         *grad_scratch = nullptr;
   size_t grad_scratch_floats = 0;
   int *n_valid = nullptr, *status = nullptr;
-  void *g_a = nullptr, *g_b = nullptr, *g_dz = nullptr, *g_du2 = nullptr, *g_dxmid = nullptr, *g_do = nullptr,
-       *g_dqkv = nullptr, *g_dhcat = nullptr, *g_du = nullptr, *g_dhcat_o = nullptr;
+  void *g_a = nullptr, *g_b = nullptr, *g_dz = nullptr, *g_du2 = nullptr, *g_do = nullptr,
+       *g_du = nullptr;
   void *S = nullptr, *dS = nullptr;
   int32_t *tok_dev = nullptr, *lab_dev = nullptr;
   // state
@@ -171,6 +175,40 @@ int validate(const splitlora_config* c, std::string* why) {
   return SPLITLORA_OK;
 }
 
+// Jobs of the adapter gradients of `layers` layers (G_A = dh^T u of every qkv target in one pass over u, G_B = (alpha/r)
+// dy^T h of each target, and the same for the output projection), the first layer's buffers and gradients given, each kind
+// of buffer at one stride (plan).
+int grad_jobs(const splitlora_ctx* c, const LayerBuf& b, float* out, int64_t group_stride, LoraGradJob* jobs) {
+  const int d = c->d;
+  const size_t es = c->es, M = c->M;
+  auto stride = [&](size_t cols) { return (int64_t)(align_up(M * cols * es, 256) / es); };
+  int n = 0;
+  auto job = [&](const void* Z, int64_t ldz, int zcol0, int64_t z_ls, const void* Wt, int ext, int wcol0, int nt, float scale, float* o) -> LoraGradJob& {
+    LoraGradJob& j = jobs[n++];
+    j.Z = Z; j.ldz = ldz; j.zcol0 = zcol0; j.C = d; j.Wt = Wt; j.ldwt = ext; j.wcol0 = wcol0; j.r = c->r; j.rp = c->rp; j.nt = nt;
+    j.scale = scale; j.out = o; j.out_group_stride = group_stride; j.out_target_stride = (int64_t)2 * c->r * d;
+    j.z_ls = z_ls; j.wt_ls = stride(ext); j.out_ls = c->per_layer;
+    return j;
+  };
+  auto gA = [&](LoraGradJob& j) { j.out_sj = d; j.out_sc = 1; };
+  auto gB = [&](LoraGradJob& j) { j.out_sj = 1; j.out_sc = c->r; };
+  gA(job(b.u, d, 0, stride(d), b.dhcat, c->ext, 0, c->nq, 1.0f, out));
+  for (int t = 0; t < c->nq; ++t)
+    gB(job(b.dqkv, 3 * d, c->slice_idx[t] * d, stride(3 * (size_t)d), b.hcat, c->ext, t * c->rp, 1, c->scale, out + (size_t)t * 2 * c->r * d + (size_t)c->r * d));
+  if (c->has_o) {
+    float* o = out + (size_t)c->nq * 2 * c->r * d;
+    gA(job(b.o, d, 0, stride(d), b.dhcat_o, c->ext_o, 0, 1, 1.0f, o));
+    gB(job(b.dxmid, d, 0, stride(d), b.hcat_o, c->ext_o, 0, 1, c->scale, o + (size_t)c->r * d));
+  }
+  return n;
+}
+
+// Up to this many token rows the adapter gradients of all layers of a side are formed together at the end of its backward
+// pass: at 512 rows a layer's pair of launches is 10 us of a chain, and nothing waits for its results but the optimizer.
+// Beyond, their cost is the traffic either way, and the layers' gradients (4 d values per row and layer) would have to be kept.
+constexpr int DEFER_ROWS = 4096;
+constexpr size_t DEFER_SCRATCH_FLOATS = 16u << 20;
+
 void derive(splitlora_ctx* c) {
   const splitlora_config& g = c->cfg;
   c->dt = g.dtype; c->es = dtype_size(g.dtype);
@@ -198,6 +236,9 @@ void derive(splitlora_ctx* c) {
   c->Pc = c->per_layer * c->cut;
   c->Ps = c->per_layer * (c->L - c->cmin);
   c->tc = (g.dtype == SPLITLORA_DTYPE_BF16) && g.use_tensor_cores != 0;
+  LoraGradJob jobs[LORA_GRAD_MAX_JOBS];
+  const int n = grad_jobs(c, LayerBuf(), nullptr, 0, jobs);       // (the workspace's buffers are aligned: no addresses needed)
+  c->defer_grads = c->M <= DEFER_ROWS && c->cmin == c->cut && lora_grad_layers_supported(c->dt, jobs, n, c->L, c->M, c->K > 1 ? c->rows_per_client : 0, c->tc);
 }
 
 // Lays out the workspace.  With ws == nullptr only the size is computed.
@@ -236,14 +277,21 @@ size_t plan(splitlora_ctx* c, char* ws) {
       take(&LayerBuf::Copies::BextO, G * d * ext_o); take(&LayerBuf::Copies::BextOT, G * ext_o * d);
     }
   }
+  auto take_layers = [&](void* LayerBuf::*kind, size_t cols, bool each = true) {      // each: one per layer, at one stride
+    const size_t stride = align_up(M * cols * es, 256);
+    char* p = (char*)a.take(stride * (size_t)(each ? c->L : 1));
+    for (int l = 0; l < c->L; ++l) c->lb[l].*kind = p + (each ? stride * (size_t)l : 0);
+  };
+  take_layers(&LayerBuf::u, d); take_layers(&LayerBuf::hcat, ext); take_layers(&LayerBuf::o, d);
+  take_layers(&LayerBuf::dqkv, 3 * d, c->defer_grads); take_layers(&LayerBuf::dhcat, ext, c->defer_grads);
+  take_layers(&LayerBuf::dxmid, d, c->defer_grads && c->has_o);
+  if (c->has_o) { take_layers(&LayerBuf::hcat_o, ext_o); take_layers(&LayerBuf::dhcat_o, ext_o, c->defer_grads); }
   for (int l = 0; l < c->L; ++l) {
     FrozenLayer& f = c->fl[l];
     f.qkvwT = a.take(3 * d * d * es); f.projwT = a.take(d * d * es);
     f.fc1wT = a.take(Fz * d * es); f.fc2wT = a.take(d * F * es);
     LayerBuf& b = c->lb[l];
-    if (c->has_o) b.hcat_o = a.take(M * ext_o * es);
-    b.u = a.take(M * d * es); b.hcat = a.take(M * ext * es); b.qkv = a.take(M * 3 * d * es);
-    b.o = a.take(M * d * es); b.x_mid = a.take(M * d * es); b.z = a.take(M * Fz * es);
+    b.qkv = a.take(M * 3 * d * es); b.x_mid = a.take(M * d * es); b.z = a.take(M * Fz * es);
     b.x_out = a.take(M * d * es);
     b.mean1 = (float*)a.take(M * 4); b.rstd1 = (float*)a.take(M * 4);
     b.mean2 = (float*)a.take(M * 4); b.rstd2 = (float*)a.take(M * 4);
@@ -255,11 +303,16 @@ size_t plan(splitlora_ctx* c, char* ws) {
   c->meanf = (float*)a.take(M * 4); c->rstdf = (float*)a.take(M * 4); c->row_loss = (float*)a.take(M * 4);
   c->rowdot = (float*)a.take((size_t)c->nseq * c->cfg.n_head * c->cfg.seq * 4);
   c->grad_scratch_floats = lora_grad_scratch_floats(c->M > 256 ? c->M : 256, c->nq * c->r, c->d);   // room for a layer's jobs as one batch
+  if (c->defer_grads) {                         // eight chunks per group of a side, at most 64 MiB
+    const size_t groups = (size_t)c->K * c->cut > (size_t)(c->L - c->cmin) ? (size_t)c->K * c->cut : (size_t)(c->L - c->cmin);
+    const size_t want = 8 * groups * (size_t)c->per_layer;
+    const size_t most = want < DEFER_SCRATCH_FLOATS ? want : DEFER_SCRATCH_FLOATS;
+    if (c->grad_scratch_floats < most) c->grad_scratch_floats = most;
+  }
   c->grad_scratch = (float*)a.take(c->grad_scratch_floats * 4);
-  if (c->has_o) c->g_dhcat_o = a.take(M * ext_o * es);
   c->g_a = a.take(M * d * es); c->g_b = a.take(M * d * es); c->g_dz = a.take(M * Fz * es);
-  c->g_du2 = a.take(M * d * es); c->g_dxmid = a.take(M * d * es); c->g_do = a.take(M * d * es);
-  c->g_dqkv = a.take(M * 3 * d * es); c->g_dhcat = a.take(M * ext * es); c->g_du = a.take(M * d * es);
+  c->g_du2 = a.take(M * d * es); c->g_do = a.take(M * d * es);
+  c->g_du = a.take(M * d * es);
   c->S = a.take(M * d * es); c->dS = a.take(M * d * es);
   c->tok_dev = (int32_t*)a.take(M * 4); c->lab_dev = (int32_t*)a.take(M * 4);
   return align_up(a.off, 256);
@@ -492,6 +545,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   void* dx = dx_base ? at(dx_base, d) : nullptr;
   const void* u = at(b.u, d); const void* hcat = at(b.hcat, ext); const void* qkv = at(b.qkv, 3 * d);
   const void* o = at(b.o, d); const void* x_mid = at(b.x_mid, d); const void* z = at(b.z, c->Fz);
+  void *g_dqkv = b.dqkv, *g_dhcat = b.dhcat, *g_dxmid = b.dxmid, *g_dhcat_o = b.dhcat_o;
   cudaError_t e;
   const int Fz = c->Fz;
   float* gbase = client ? c->cg + (size_t)sp.client0 * c->Pc + (size_t)l * c->per_layer
@@ -509,44 +563,46 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   }
   { GemmArgs a = base_args(c, c->g_dz, Fz, f.fc1wT, Fz, c->g_du2, d, M, d, Fz);
     if ((e = linear(c, "linear_bwd", a))) return e; }
-  if ((e = norm_backward(c, M, c->g_du2, x_mid, f.ln2g, atf(b.mean2), atf(b.rstd2), dy, c->g_dxmid))) return e;
+  if ((e = norm_backward(c, M, c->g_du2, x_mid, f.ln2g, atf(b.mean2), atf(b.rstd2), dy, g_dxmid))) return e;
   if (c->has_o) {
     // dh_o = (alpha/r) dx_mid B_o,g ;  G_A = dh_o^T o ;  G_B = (alpha/r) dx_mid^T h_o   (Eq. 4-7)
     const void* hcat_o = at(b.hcat_o, c->ext_o);
-    { GemmArgs a = base_args(c, c->g_dxmid, d, grp(k.BextOT, (size_t)c->ext_o * d), d, c->g_dhcat_o, c->ext_o, M, c->ext_o, d);
+    { GemmArgs a = base_args(c, g_dxmid, d, grp(k.BextOT, (size_t)c->ext_o * d), d, g_dhcat_o, c->ext_o, M, c->ext_o, d);
       a.rows_per_group = rpg; a.w_grouped = grouped;
       if ((e = linear(c, "lora_down_bwd", a))) return e; }
     float* gA = gbase + (size_t)c->nq * 2 * c->r * d;
+    if (!c->defer_grads) {
     { Scope s(c, "lora_grad", 2);
-      if ((e = lora_grad(c->dt, o, d, 0, d, c->g_dhcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, 1.0f, gA, gstride, 0, d,
+      if ((e = lora_grad(c->dt, o, d, 0, d, g_dhcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, 1.0f, gA, gstride, 0, d,
                          1, c->grad_scratch, c->st, c->status, c->tc))) return e; }
     { Scope s(c, "lora_grad", 2);
-      if ((e = lora_grad(c->dt, c->g_dxmid, d, 0, d, hcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, c->scale,
+      if ((e = lora_grad(c->dt, g_dxmid, d, 0, d, hcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, c->scale,
                          gA + (size_t)c->r * d, gstride, 0, 1, c->r, c->grad_scratch, c->st, c->status, c->tc))) return e; }
+    }
   }
-  { GemmArgs a = base_args(c, c->g_dxmid, d, f.projwT, d, c->g_do, d, M, d, d);
+  { GemmArgs a = base_args(c, g_dxmid, d, f.projwT, d, c->g_do, d, M, d, d);
     if (c->has_o) {
       a.rows_per_group = rpg;
-      a.Xe = c->g_dhcat_o; a.ldxe = c->ext_o; a.We = grp(k.AcatOT, (size_t)d * c->ext_o); a.ldwe = c->ext_o; a.Ke = c->rp;
+      a.Xe = g_dhcat_o; a.ldxe = c->ext_o; a.We = grp(k.AcatOT, (size_t)d * c->ext_o); a.ldwe = c->ext_o; a.Ke = c->rp;
       a.we_grouped = grouped;
     }
     if ((e = linear(c, c->has_o ? "lora_linear_bwd" : "linear_bwd", a))) return e; }
   { const bool aligned_form = c->tc && attention_tc_supported(c->dt, T, H, d);
-    const bool ragged_form = !aligned_form && c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, c->g_do, c->g_dqkv);
+    const bool ragged_form = !aligned_form && c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, c->g_do, g_dqkv);
     Scope s(c, "attention_bwd", aligned_form && !attention_t5_supported(c->dt, T, H, d) ? 3 : 2);
     if (aligned_form)
-      e = attention_bwd_tc(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->status, c->st);
+      e = attention_bwd_tc(qkv, o, lse, c->g_do, M / T, T, H, d, g_dqkv, c->rowdot, c->status, c->st);
     else if (ragged_form)
-      e = attention_bwd_ragged(qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->status, c->st);
+      e = attention_bwd_ragged(qkv, o, lse, c->g_do, M / T, T, H, d, g_dqkv, c->rowdot, c->status, c->st);
     else
-      e = attention_bwd_simt(c->dt, qkv, o, lse, c->g_do, M / T, T, H, d, c->g_dqkv, c->rowdot, c->st);
+      e = attention_bwd_simt(c->dt, qkv, o, lse, c->g_do, M / T, T, H, d, g_dqkv, c->rowdot, c->st);
     if (e) return e; }
   if (c->llama) {  // the gradient of a rotation is the inverse rotation
     Scope s(c, "rope", 1);
-    if ((e = rope_inplace(c->dt, c->g_dqkv, c->rope_table, M, T, H, d, -1.0f, c->st))) return e;
+    if ((e = rope_inplace(c->dt, g_dqkv, c->rope_table, M, T, H, d, -1.0f, c->st))) return e;
   }
   {  // dh = (alpha/r) dqkv B_g for every target (the scale lives in the compute copy)
-    GemmArgs a = base_args(c, c->g_dqkv, 3 * d, grp(k.BextT, (size_t)ext * 3 * d), 3 * d, c->g_dhcat, ext, M, ext, 3 * d);
+    GemmArgs a = base_args(c, g_dqkv, 3 * d, grp(k.BextT, (size_t)ext * 3 * d), 3 * d, g_dhcat, ext, M, ext, 3 * d);
     a.rows_per_group = rpg; a.w_grouped = grouped;
     if (c->tc && c->nq < 3) {
       // only the adapted slices of dqkv contribute (the other rows of the compute copy are zero):
@@ -563,28 +619,39 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   }
   // G_A = dh^T u (every qkv target in one pass over u) and G_B = (alpha/r) dy^T h of each target, per
   // group (Eq. 4-7): one batch, i.e. one pair of launches where the tensor-core path applies
-  { LoraGradJob jobs[4];
+  if (!c->defer_grads) {
+    LoraGradJob jobs[4];
     int nj = 0;
     LoraGradJob& ja = jobs[nj++];
-    ja.Z = u; ja.ldz = d; ja.zcol0 = 0; ja.C = d; ja.Wt = c->g_dhcat; ja.ldwt = ext; ja.wcol0 = 0; ja.r = c->r; ja.rp = c->rp;
+    ja.Z = u; ja.ldz = d; ja.zcol0 = 0; ja.C = d; ja.Wt = g_dhcat; ja.ldwt = ext; ja.wcol0 = 0; ja.r = c->r; ja.rp = c->rp;
     ja.nt = c->nq; ja.scale = 1.0f; ja.out = gbase; ja.out_group_stride = gstride; ja.out_target_stride = (int64_t)2 * c->r * d;
     ja.out_sj = d; ja.out_sc = 1;
     for (int t = 0; t < c->nq; ++t) {
       LoraGradJob& jb = jobs[nj++];
-      jb.Z = c->g_dqkv; jb.ldz = 3 * d; jb.zcol0 = c->slice_idx[t] * d; jb.C = d; jb.Wt = hcat; jb.ldwt = ext; jb.wcol0 = t * c->rp;
+      jb.Z = g_dqkv; jb.ldz = 3 * d; jb.zcol0 = c->slice_idx[t] * d; jb.C = d; jb.Wt = hcat; jb.ldwt = ext; jb.wcol0 = t * c->rp;
       jb.r = c->r; jb.rp = c->rp; jb.nt = 1; jb.scale = c->scale; jb.out = gbase + (size_t)t * 2 * c->r * d + (size_t)c->r * d;
       jb.out_group_stride = gstride; jb.out_target_stride = 0; jb.out_sj = 1; jb.out_sc = c->r;
     }
     Scope s(c, "lora_grad", 2);
     if ((e = lora_grad_batch(c->dt, jobs, nj, M, rpg, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc))) return e; }
   if (dx) {
-    GemmArgs a = base_args(c, c->g_dqkv, 3 * d, f.qkvwT, 3 * d, c->g_du, d, M, d, 3 * d);
+    GemmArgs a = base_args(c, g_dqkv, 3 * d, f.qkvwT, 3 * d, c->g_du, d, M, d, 3 * d);
     a.rows_per_group = rpg;
-    a.Xe = c->g_dhcat; a.ldxe = ext; a.We = grp(k.AcatT, (size_t)d * ext); a.ldwe = ext; a.Ke = c->ke; a.we_grouped = grouped;
+    a.Xe = g_dhcat; a.ldxe = ext; a.We = grp(k.AcatT, (size_t)d * ext); a.ldwe = ext; a.Ke = c->ke; a.we_grouped = grouped;
     if ((e = linear(c, "lora_linear_bwd", a))) return e;
-    if ((e = norm_backward(c, M, c->g_du, at(b.x_in, d), f.ln1g, atf(b.mean1), atf(b.rstd1), c->g_dxmid, dx))) return e;
+    if ((e = norm_backward(c, M, c->g_du, at(b.x_in, d), f.ln1g, atf(b.mean1), atf(b.rstd1), g_dxmid, dx))) return e;
   }
   return cudaSuccess;
+}
+
+// the adapter gradients of all layers of a side, where the layers' own passes have left them out
+cudaError_t deferred_gradients(splitlora_ctx* c, bool client) {
+  const int l0 = client ? 0 : c->cmin, l1 = client ? c->cut : c->L;
+  if (!c->defer_grads || l1 <= l0) return cudaSuccess;
+  LoraGradJob jobs[LORA_GRAD_MAX_JOBS];
+  const int n = grad_jobs(c, c->lb[l0], client ? c->cg : c->sg, client ? c->Pc : 0, jobs);
+  Scope s(c, "lora_grad", 1);
+  return lora_grad_layers(c->dt, jobs, n, l1 - l0, c->M, client ? c->rows_per_client : 0, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc);
 }
 
 cudaError_t run_optimizer(splitlora_ctx* c, bool client) {
@@ -915,6 +982,7 @@ int splitlora_server_step(splitlora_ctx* c, const void* act_in, const int32_t* l
     other = cur; cur = dst;
   }
   if (!uni) CK(c, copy_client_rows(c, cur, act_grad_out, 0, first_client_above(c, c->cmin)));
+  CK(c, deferred_gradients(c, false));
   // Eq. 4-5: server update
   if (!c->defer_server_update) {
     CK(c, run_optimizer(c, false));
@@ -950,6 +1018,7 @@ int splitlora_client_bwd(splitlora_ctx* c, const void* act_grad_in) {
     CK(c, block_backward(c, l, sp, cur, dst));
     cur = dst; which ^= 1;
   }
+  CK(c, deferred_gradients(c, true));
   CK(c, run_optimizer(c, true));   // Eq. 6-7, all K clients in one launch
   c->client_copies_dirty = true;
   c->have_client_fwd = false;
