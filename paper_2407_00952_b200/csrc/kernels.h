@@ -122,6 +122,49 @@ bool attention_bwd_ragged_t5_supported(int nseq, int T, int H, int d);
 cudaError_t attention_bwd_ragged_t5(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                                     int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
 
+// Compute copies of the adapters of `layers` layers (G groups), built from fp32 masters.
+// Target t of group g has A_t [r, d_in] at A + g*a_gs + t*a_ts and B_t [d_out, r] at B + g*b_gs + t*b_ts.
+// With col = t*rp + j the copies are
+//   Acat  [G][ext, d_in]  : Acat[col, c]  = A_t[j, c]          AcatT [G][d_in, ext] : its transpose
+//   Bext  [G][n_out, ext] : Bext[slice_off[t] + c, col] = scale * B_t[c, j]
+//   BextT [G][ext, n_out] : its transpose
+// Only live entries are written; the padding must have been zeroed once.
+struct AdapterCopyArgs {
+  int dtype = 0;
+  const float* A = nullptr; int64_t a_gs = 0, a_ts = 0;
+  const float* B = nullptr; int64_t b_gs = 0, b_ts = 0;
+  int G = 0, n_targets = 0, r = 0, rp = 0, d_in = 0, d_out = 0, n_out = 0, ext = 0;
+  int slice_off[4] = {0, 0, 0, 0};
+  float scale = 0.f;
+  void *Acat = nullptr, *AcatT = nullptr, *Bext = nullptr, *BextT = nullptr;   // any of them may be null (skipped)
+  int layers = 1;                      // of layers further on: masters layer_stride, Acat / AcatT acat_ls, Bext / BextT bext_ls elements apart
+  int64_t layer_stride = 0, acat_ls = 0, bext_ls = 0;
+  int* status = nullptr;               // write_adapter_copies: a word to clear
+};
+// Rank-r projection of the LoRA path, bf16 (lora_proj.cu): Y[M, ext] = X[M, K] W_g[ext, K]^T where only columns
+// t*rp + j, j < r, t < nt of W and Y are used (the others of Y become zero).  W of group g = row / rows_per_group at
+// W + g*w_group_stride.  k_slice > 0 and nt > 1: target t's rows of W are zero outside columns [slice_col[t], + k_slice), and
+// K is not used.  status: as for the linear layers (nullptr: the library's own word).
+struct ProjArgs {
+  const void* X = nullptr; int64_t ldx = 0;
+  const void* W = nullptr; int64_t ldw = 0, w_group_stride = 0;
+  void* Y = nullptr;
+  int M = 0, K = 0, rows_per_group = 0, ext = 0, nt = 1, r = 0, rp = 0, k_slice = 0, slice_col[4] = {0, 0, 0, 0};
+  int* status = nullptr;
+};
+bool lora_proj_supported(const ProjArgs& a);
+// Rows up to which these kernels beat the linear layers' narrow tiles: (512, 2048 -> 2 x 4 of 32) 8.8 -> 5.5 us from cold
+// caches; 12 of 1665 x 1536 149 -> 104, of 16384 x 1536 225 -> 252, 24 of 32768 x 2048 910 -> 966.  With the norm in front
+// they save a launch and a read of its rows: 25 norms and 12 projections of 16384 x 768 520 -> 500 us, of 1665 x 768 308 ->
+// 226; 49 and 24 of 32768 x 1024 2.12 -> 2.23 ms.
+constexpr int LORA_PROJ_ROWS = 4096, NORM_PROJ_ROWS = 16384;
+cudaError_t lora_proj(const ProjArgs& a, cudaStream_t st);
+// The same for one target whose W is the fp32 A [r, K] itself, with the compute copies of write_adapter_copies in the same launch.
+cudaError_t lora_proj_copies(const ProjArgs& a, const AdapterCopyArgs& copies, cudaStream_t st);
+// The norm in front of it in the same launch: a.X [M, K] receives LayerNorm(x) (RMSNorm: b and mean unused), Y its projection.
+bool norm_proj_supported(const ProjArgs& a);
+cudaError_t norm_proj(bool rms, const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st);
+
 // Adapter gradients: for nt targets of rank r (weight columns wcol0 + t*rp + jj of Wt),
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c],  c < C,
 // stored at out + g*out_group_stride + t*out_target_stride + jj*out_sj + c*out_sc.
@@ -176,25 +219,6 @@ cudaError_t aggregate(float* params, int K, int64_t P, const float* w_host, cuda
 cudaError_t aggregate_local_sum(const float* params, int K, int64_t P, const float* w_host, float* sum, cudaStream_t st);
 cudaError_t aggregate_broadcast(const float* sum, int K, int64_t P, float* params, cudaStream_t st);
 
-// Compute copies of the adapters of `layers` layers (G groups), built from fp32 masters.
-// Target t of group g has A_t [r, d_in] at A + g*a_gs + t*a_ts and B_t [d_out, r] at B + g*b_gs + t*b_ts.
-// With col = t*rp + j the copies are
-//   Acat  [G][ext, d_in]  : Acat[col, c]  = A_t[j, c]          AcatT [G][d_in, ext] : its transpose
-//   Bext  [G][n_out, ext] : Bext[slice_off[t] + c, col] = scale * B_t[c, j]
-//   BextT [G][ext, n_out] : its transpose
-// Only live entries are written; the padding must have been zeroed once.
-struct AdapterCopyArgs {
-  int dtype;
-  const float* A; int64_t a_gs, a_ts;
-  const float* B; int64_t b_gs, b_ts;
-  int G, n_targets, r, rp, d_in, d_out, n_out, ext;
-  int slice_off[4];
-  float scale;
-  void *Acat, *AcatT, *Bext, *BextT;   // any of them may be null (skipped)
-  int layers = 1;                      // of layers further on: masters layer_stride, Acat / AcatT acat_ls, Bext / BextT bext_ls elements apart
-  int64_t layer_stride = 0, acat_ls = 0, bext_ls = 0;
-  int* status = nullptr;               // write_adapter_copies: a word to clear
-};
 // The same for one layer and target (n_targets 1, slice_off 0, n_out = d_out) into uninitialised copies: padding included.
 cudaError_t write_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st);
 cudaError_t refresh_adapter_copies(const AdapterCopyArgs& a, cudaStream_t st);

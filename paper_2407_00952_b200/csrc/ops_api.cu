@@ -53,6 +53,23 @@ cudaError_t run_gemm(int use_tc, const GemmArgs& a, int* status, cudaStream_t st
   if (use_tc && a.dtype == DT_BF16 && gemm_tc_supported(a)) return gemm_tc(a, status, st);
   return gemm_simt(a, st);
 }
+ProjArgs proj_args(const LinearPlan& p, const void* X, int K, const void* W, void* Y, int M, int r, int G, int* status) {
+  ProjArgs a;
+  a.X = X; a.ldx = K; a.W = W; a.ldw = K; a.w_group_stride = G > 1 ? (int64_t)p.ext * K : 0; a.Y = Y;
+  a.M = M; a.K = K; a.rows_per_group = G > 1 ? M / G : 0; a.ext = p.ext; a.r = r; a.rp = p.rp;
+  a.status = status;
+  return a;
+}
+// Y[M, ext] = X[M, K] W_g[ext, K]^T of the LoRA layer with plan p
+cudaError_t run_proj(int use_tc, int dtype, const LinearPlan& p, const void* X, int K, const void* W, void* Y, int M, int r, int G,
+                     int* status, cudaStream_t st) {
+  const ProjArgs a = proj_args(p, X, K, W, Y, M, r, G, status);
+  if (use_tc && dtype == DT_BF16 && M <= LORA_PROJ_ROWS && lora_proj_supported(a)) return lora_proj(a, st);
+  GemmArgs h;
+  h.dtype = dtype; h.X = X; h.ldx = K; h.W = W; h.ldw = K; h.Y = Y; h.ldy = p.ext;
+  h.M = M; h.N = p.ext; h.K = K; h.rows_per_group = a.rows_per_group; h.w_grouped = G > 1;
+  return run_gemm(use_tc, h, status, st);
+}
 }  // namespace
 
 extern "C" {
@@ -65,20 +82,33 @@ int splitlora_lora_linear_workspace_bytes(int dtype, int M, int n_in, int n_out,
   return SPLITLORA_OK;
 }
 
-static int make_copies(int dtype, const LinearPlan& p, const float* A, const float* B, float alpha, int n_in,
-                       int n_out, int r, int G, char* ws, bool fwd, cudaStream_t st) {
-  const size_t es = dtype_size(dtype);
+// The compute copies of one direction: Acat and Bext (forward), Acat, AcatT and BextT (backward).
+static AdapterCopyArgs copy_args(int dtype, const LinearPlan& p, const float* A, const float* B, float alpha, int n_in,
+                                 int n_out, int r, int G, char* ws, bool fwd) {
   AdapterCopyArgs a;
   a.dtype = dtype;
   a.A = A; a.a_gs = (int64_t)r * n_in; a.a_ts = 0;
   a.B = B; a.b_gs = (int64_t)n_out * r; a.b_ts = 0;
   a.G = G; a.n_targets = 1; a.r = r; a.rp = p.rp; a.d_in = n_in; a.d_out = n_out; a.n_out = n_out; a.ext = p.ext;
-  for (int t = 0; t < 4; ++t) a.slice_off[t] = 0;
   a.scale = alpha / (float)r;
   a.Acat = ws + p.off_acat; a.AcatT = fwd ? nullptr : ws + p.off_acatT;
   a.Bext = fwd ? ws + p.off_bext : nullptr; a.BextT = fwd ? nullptr : ws + p.off_bextT;
   a.status = (int*)(ws + p.off_status);
-  return write_adapter_copies(a, st) == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;
+  return a;
+}
+// The copies, and h = x A_g^T where `project`: one launch where the projection can take A as it is, else two.
+static cudaError_t copies_and_h(int use_tc, AdapterCopyArgs a, bool project, const LinearPlan& p, const void* x, int M, char* ws, cudaStream_t st) {
+  if (project && use_tc && a.dtype == DT_BF16 && (reinterpret_cast<uintptr_t>(a.A) & 15u) == 0) {
+    ProjArgs h = proj_args(p, x, a.d_in, a.A, ws + p.off_h, M, a.r, a.G, a.status);
+    if (a.G > 1) h.w_group_stride = a.a_gs;
+    if (lora_proj_supported(h)) {
+      a.Acat = nullptr;                        // nothing else reads it
+      return lora_proj_copies(h, a, st);
+    }
+  }
+  cudaError_t e = write_adapter_copies(a, st);
+  if (e != cudaSuccess || !project) return e;
+  return run_proj(use_tc, a.dtype, p, x, a.d_in, ws + p.off_acat, ws + p.off_h, M, a.r, a.G, a.status, st);
 }
 
 int splitlora_lora_linear_fwd(int dtype, int use_tc, const void* x, const void* W, const void* bias, const float* A,
@@ -106,11 +136,7 @@ int splitlora_lora_linear_fwd_parts(int dtype, int use_tc, const void* x, const 
   const int rpg = G > 1 ? M / G : 0;
   int* status = (int*)(ws + p.off_status);
   if (parts & 1) {
-    if ((rc = make_copies(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, true, st))) return rc;
-    GemmArgs h;
-    h.dtype = dtype; h.X = x; h.ldx = n_in; h.W = ws + p.off_acat; h.ldw = n_in; h.Y = ws + p.off_h; h.ldy = p.ext;
-    h.M = M; h.N = p.ext; h.K = n_in; h.rows_per_group = rpg; h.w_grouped = G > 1;
-    if (run_gemm(use_tc, h, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
+    if (copies_and_h(use_tc, copy_args(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, true), true, p, x, M, ws, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   }
   if (!(parts & 2)) return SPLITLORA_OK;
   GemmArgs a;
@@ -144,21 +170,14 @@ int splitlora_lora_linear_bwd_parts(int dtype, int use_tc, const void* x, const 
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
   if (gemm_tc_init() != 0) return SPLITLORA_ERR_CUDA;
-  if ((rc = make_copies(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, false, st))) return rc;
+  // h = x A_g^T is recomputed here; the training runtime keeps it from the forward pass
+  if (copies_and_h(use_tc, copy_args(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, false), parts & 1, p, x, M, ws, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   const int rpg = G > 1 ? M / G : 0;
   int* status = (int*)(ws + p.off_status);
   const float s = alpha / (float)r;
   if (parts & 1) {
-    // h = x A_g^T (recomputed here; the training runtime keeps it from the forward pass)
-    GemmArgs h;
-    h.dtype = dtype; h.X = x; h.ldx = n_in; h.W = ws + p.off_acat; h.ldw = n_in; h.Y = ws + p.off_h; h.ldy = p.ext;
-    h.M = M; h.N = p.ext; h.K = n_in; h.rows_per_group = rpg; h.w_grouped = G > 1;
-    if (run_gemm(use_tc, h, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
     // dh = s dy B_g
-    GemmArgs g;
-    g.dtype = dtype; g.X = dy; g.ldx = n_out; g.W = ws + p.off_bextT; g.ldw = n_out; g.Y = ws + p.off_dh; g.ldy = p.ext;
-    g.M = M; g.N = p.ext; g.K = n_out; g.rows_per_group = rpg; g.w_grouped = G > 1;
-    if (run_gemm(use_tc, g, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
+    if (run_proj(use_tc, dtype, p, dy, n_out, ws + p.off_bextT, ws + p.off_dh, M, r, G, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   }
   if (parts & 2) {
     // dx = dy W + dh A_g

@@ -352,6 +352,20 @@ cudaError_t linear(splitlora_ctx* c, const char* name, const GemmArgs& a) {
   return gemm_simt(a, c->st);
 }
 
+// Y[M, ext] = X W_g^T for the adapters of one LoRA layer (nt targets of rp columns each); a: as for `linear`
+ProjArgs proj_args(const splitlora_ctx* c, const GemmArgs& a, int nt) {
+  ProjArgs p;
+  p.X = a.X; p.ldx = a.ldx; p.W = a.W; p.ldw = a.ldw; p.w_group_stride = a.w_grouped ? (int64_t)a.N * a.ldw : 0;
+  p.Y = a.Y; p.M = a.M; p.K = a.K;
+  p.rows_per_group = a.rows_per_group; p.ext = a.N; p.nt = nt; p.r = c->r; p.rp = c->rp; p.status = c->status;
+  return p;
+}
+cudaError_t rank_proj(splitlora_ctx* c, const char* name, const GemmArgs& a, const ProjArgs& p) {
+  if (!c->tc || a.M > LORA_PROJ_ROWS || !lora_proj_supported(p)) return linear(c, name, a);
+  Scope s(c, name, 1);
+  return lora_proj(p, c->st);
+}
+
 GemmArgs base_args(splitlora_ctx* c, const void* X, int64_t ldx, const void* W, int64_t ldw, void* Y, int64_t ldy,
                    int M, int N, int K) {
   GemmArgs a;
@@ -469,11 +483,17 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
   void* u = at(b.u, d); void* hcat = at(b.hcat, ext); void* qkv = at(b.qkv, 3 * d); void* o = at(b.o, d);
   void* x_mid = at(b.x_mid, d); void* z = at(b.z, c->Fz); void* xout = at(x_out, d);
   cudaError_t e;
-  if ((e = norm_forward(c, M, xin, f.ln1g, f.ln1b, u, atf(b.mean1), atf(b.rstd1)))) return e;
-  {  // h = u A_g^T for every target of the layer, one padded block of `ext` columns
+  {  // u = norm(x) and h = u A_g^T for every target of the layer, one padded block of `ext` columns
     GemmArgs a = base_args(c, u, d, grp(k.Acat, (size_t)ext * d), d, hcat, ext, M, ext, d);
     a.rows_per_group = rpg; a.w_grouped = grouped;
-    if ((e = linear(c, "lora_down_fwd", a))) return e;
+    const ProjArgs p = proj_args(c, a, c->nq);
+    if (c->tc && M <= NORM_PROJ_ROWS && norm_proj_supported(p)) {
+      Scope s(c, "layernorm_fwd", 1);
+      if ((e = norm_proj(c->llama, xin, f.ln1g, f.ln1b, atf(b.mean1), atf(b.rstd1), c->cfg.norm_eps, p, c->st))) return e;
+    } else {
+      if ((e = norm_forward(c, M, xin, f.ln1g, f.ln1b, u, atf(b.mean1), atf(b.rstd1)))) return e;
+      if ((e = rank_proj(c, "lora_down_fwd", a, p))) return e;
+    }
   }
   {  // qkv = u Wqkv^T + b + hcat Bext_g^T   (the LoRA linear of Sec. II-C, grouped by client)
     GemmArgs a = base_args(c, u, d, f.qkvw, d, qkv, 3 * d, M, 3 * d, d);
@@ -497,7 +517,7 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
   if (c->has_o) {  // h_o = o A_o,g^T
     GemmArgs a = base_args(c, o, d, grp(k.AcatO, (size_t)c->ext_o * d), d, hcat_o, c->ext_o, M, c->ext_o, d);
     a.rows_per_group = rpg; a.w_grouped = grouped;
-    if ((e = linear(c, "lora_down_fwd", a))) return e;
+    if ((e = rank_proj(c, "lora_down_fwd", a, proj_args(c, a, 1)))) return e;
   }
   { GemmArgs a = base_args(c, o, d, f.projw, d, x_mid, d, M, d, d);
     a.bias = f.projb; a.epi = EPI_BIAS_RESID; a.R = xin; a.ldr = d;
@@ -569,7 +589,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
     const void* hcat_o = at(b.hcat_o, c->ext_o);
     { GemmArgs a = base_args(c, g_dxmid, d, grp(k.BextOT, (size_t)c->ext_o * d), d, g_dhcat_o, c->ext_o, M, c->ext_o, d);
       a.rows_per_group = rpg; a.w_grouped = grouped;
-      if ((e = linear(c, "lora_down_bwd", a))) return e; }
+      if ((e = rank_proj(c, "lora_down_bwd", a, proj_args(c, a, 1)))) return e; }
     float* gA = gbase + (size_t)c->nq * 2 * c->r * d;
     if (!c->defer_grads) {
     { Scope s(c, "lora_grad", 2);
@@ -604,7 +624,11 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   {  // dh = (alpha/r) dqkv B_g for every target (the scale lives in the compute copy)
     GemmArgs a = base_args(c, g_dqkv, 3 * d, grp(k.BextT, (size_t)ext * 3 * d), 3 * d, g_dhcat, ext, M, ext, 3 * d);
     a.rows_per_group = rpg; a.w_grouped = grouped;
-    if (c->tc && c->nq < 3) {
+    ProjArgs p = proj_args(c, a, c->nq);
+    p.k_slice = d;                                     // a target's columns of the copy are zero outside its slice of dqkv
+    for (int t = 0; t < c->nq; ++t) p.slice_col[t] = c->slice_idx[t] * d;
+    if (c->nq == 1) { p.X = (const char*)p.X + (size_t)p.slice_col[0] * es; p.W = (const char*)p.W + (size_t)p.slice_col[0] * es; p.K = d; }
+    if (c->tc && c->nq < 3 && (M > LORA_PROJ_ROWS || !lora_proj_supported(p))) {
       // only the adapted slices of dqkv contribute (the other rows of the compute copy are zero):
       // contract over those columns alone, which is one third less to read for q and v
       GemmArgs g = a;
@@ -615,7 +639,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
       if (hi - lo + 1 > c->nq) { g.k_gap_begin = d; g.k_gap_len = d; }     // q and v: skip the k slice
       if (gemm_tc_supported(g)) a = g;
     }
-    if ((e = linear(c, "lora_down_bwd", a))) return e;
+    if ((e = rank_proj(c, "lora_down_bwd", a, p))) return e;
   }
   // G_A = dh^T u (every qkv target in one pass over u) and G_B = (alpha/r) dy^T h of each target, per
   // group (Eq. 4-7): one batch, i.e. one pair of launches where the tensor-core path applies
