@@ -9,6 +9,7 @@
 namespace sl {
 
 thread_local bool t_in_chain = false;
+thread_local int64_t t_launches = 0;
 
 namespace {
 

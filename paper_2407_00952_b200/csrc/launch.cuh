@@ -2,6 +2,7 @@
 // (programmatic dependent launch), and the device-side half every kernel of the library executes.
 #pragma once
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 #include <utility>
 
@@ -23,6 +24,7 @@ __device__ __forceinline__ void overlap_sync() {
 // not by copies, memsets or other work of the caller.  Every entry point that launches starts a chain of its own, and
 // a copy or memset between two kernels breaks it.
 extern thread_local bool t_in_chain;
+extern thread_local int64_t t_launches;      // kernels launched by this thread
 inline void break_chain() { t_in_chain = false; }
 struct LaunchChain {
   LaunchChain() { t_in_chain = false; }
@@ -30,6 +32,7 @@ struct LaunchChain {
 };
 // Attributes of the next launch, `at` with room for one more after `n`; returns their number.
 inline unsigned chain_attribute(cudaLaunchAttribute* at, unsigned n) {
+  ++t_launches;
   if (!t_in_chain) { t_in_chain = true; return n; }
   at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[n].val.programmaticStreamSerializationAllowed = 1;

@@ -321,8 +321,8 @@ size_t plan(splitlora_ctx* c, char* ws) {
 // ---- profiling -----------------------------------------------------------------------------
 struct Scope {
   splitlora_ctx* c; int cls = -1; cudaEvent_t a = nullptr, b = nullptr;
-  Scope(splitlora_ctx* ctx, const char* name, int kernels) : c(ctx) {
-    c->launches += kernels;
+  int64_t launches0 = t_launches;
+  Scope(splitlora_ctx* ctx, const char* name) : c(ctx) {
     if (!c->prof_on) return;
     if (c->prof_on == 2 && !std::strstr(name, "linear_") && std::strncmp(name, "head_", 5) != 0) return;
     auto it = c->prof_ids.find(name);
@@ -340,6 +340,7 @@ struct Scope {
     cudaEventRecord(a, c->st);
   }
   ~Scope() {
+    c->launches += t_launches - launches0;
     if (cls < 0) return;
     cudaEventRecord(b, c->st);
     c->prof_recs.push_back({cls, a, b});
@@ -347,7 +348,7 @@ struct Scope {
 };
 
 cudaError_t linear(splitlora_ctx* c, const char* name, const GemmArgs& a) {
-  Scope s(c, name, 1);
+  Scope s(c, name);
   if (c->tc && gemm_tc_supported(a)) return gemm_tc(a, c->status, c->st);
   return gemm_simt(a, c->st);
 }
@@ -362,7 +363,7 @@ ProjArgs proj_args(const splitlora_ctx* c, const GemmArgs& a, int nt) {
 }
 cudaError_t rank_proj(splitlora_ctx* c, const char* name, const GemmArgs& a, const ProjArgs& p) {
   if (!c->tc || a.M > LORA_PROJ_ROWS || !lora_proj_supported(p)) return linear(c, name, a);
-  Scope s(c, name, 1);
+  Scope s(c, name);
   return lora_proj(p, c->st);
 }
 
@@ -401,7 +402,7 @@ cudaError_t refresh_side(splitlora_ctx* c, bool client) {
     for (int t = 0; t < 4; ++t) a.slice_off[t] = c->slice_idx[t] * c->d;
     a.Acat = k.Acat; a.AcatT = k.AcatT; a.Bext = k.Bext; a.BextT = k.BextT;
     copy_stride(a.n_out, a.ext, &a.acat_ls, &a.bext_ls);
-    Scope s(c, "adapter_copies", 1);
+    Scope s(c, "adapter_copies");
     cudaError_t e = refresh_adapter_copies(a, c->st);
     if (e != cudaSuccess) return e;
   }
@@ -411,7 +412,7 @@ cudaError_t refresh_side(splitlora_ctx* c, bool client) {
     for (int t = 0; t < 4; ++t) a.slice_off[t] = 0;
     a.Acat = k.AcatO; a.AcatT = k.AcatOT; a.Bext = k.BextO; a.BextT = k.BextOT;
     copy_stride(a.n_out, a.ext, &a.acat_ls, &a.bext_ls);
-    Scope s(c, "adapter_copies", 1);
+    Scope s(c, "adapter_copies");
     cudaError_t e = refresh_adapter_copies(a, c->st);
     if (e != cudaSuccess) return e;
   }
@@ -421,13 +422,13 @@ cudaError_t refresh_side(splitlora_ctx* c, bool client) {
 // LayerNorm or RMSNorm over M rows, by architecture (mean is unused by RMSNorm)
 cudaError_t norm_forward(splitlora_ctx* c, int M, const void* x, const void* g, const void* b, void* y, float* mean,
                          float* rstd) {
-  Scope s(c, "layernorm_fwd", 1);
+  Scope s(c, "layernorm_fwd");
   if (c->llama) return rmsnorm_fwd(c->dt, x, g, y, rstd, M, c->d, c->cfg.norm_eps, c->st);
   return layernorm_fwd(c->dt, x, g, b, y, mean, rstd, M, c->d, c->cfg.norm_eps, c->st);
 }
 cudaError_t norm_backward(splitlora_ctx* c, int M, const void* dy, const void* x, const void* g, const float* mean,
                           const float* rstd, const void* resid, void* dx) {
-  Scope s(c, "layernorm_bwd", 1);
+  Scope s(c, "layernorm_bwd");
   if (c->llama) return rmsnorm_bwd(c->dt, dy, x, g, rstd, resid, dx, M, c->d, c->st);
   return layernorm_bwd(c->dt, dy, x, g, mean, rstd, resid, dx, M, c->d, c->st);
 }
@@ -488,7 +489,7 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
     a.rows_per_group = rpg; a.w_grouped = grouped;
     const ProjArgs p = proj_args(c, a, c->nq);
     if (c->tc && M <= NORM_PROJ_ROWS && norm_proj_supported(p)) {
-      Scope s(c, "layernorm_fwd", 1);
+      Scope s(c, "layernorm_fwd");
       if ((e = norm_proj(c->llama, xin, f.ln1g, f.ln1b, atf(b.mean1), atf(b.rstd1), c->cfg.norm_eps, p, c->st))) return e;
     } else {
       if ((e = norm_forward(c, M, xin, f.ln1g, f.ln1b, u, atf(b.mean1), atf(b.rstd1)))) return e;
@@ -502,10 +503,10 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
     if ((e = linear(c, "lora_linear_fwd", a))) return e;
   }
   if (c->llama) {
-    Scope s(c, "rope", 1);
+    Scope s(c, "rope");
     if ((e = rope_inplace(c->dt, qkv, c->rope_table, M, T, H, d, 1.0f, c->st))) return e;
   }
-  { Scope s(c, "attention_fwd", 1);
+  { Scope s(c, "attention_fwd");
     if (c->tc && attention_tc_supported(c->dt, T, H, d))
       e = attention_fwd_tc(qkv, M / T, T, H, d, o, lse, c->status, c->st);
     else if (c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, nullptr, nullptr))
@@ -531,7 +532,7 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
   if (c->llama) {
     { GemmArgs a = base_args(c, c->u2, d, f.fc1w, d, z, 2 * F, M, 2 * F, d);     // (gate | up)
       if ((e = linear(c, "linear_fwd", a))) return e; }
-    { Scope s(c, "swiglu_fwd", 1);
+    { Scope s(c, "swiglu_fwd");
       if ((e = swiglu_fwd(c->dt, z, c->act, M, F, c->st))) return e; }
   } else {
     GemmArgs a = base_args(c, c->u2, d, f.fc1w, d, c->act, F, M, F, d);
@@ -574,7 +575,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   if (c->llama) {
     { GemmArgs a = base_args(c, dy, d, f.fc2wT, d, c->act, F, M, F, d);               // d act
       if ((e = linear(c, "linear_bwd", a))) return e; }
-    { Scope s(c, "swiglu_bwd", 1);
+    { Scope s(c, "swiglu_bwd");
       if ((e = swiglu_bwd(c->dt, c->act, z, c->g_dz, M, F, c->st))) return e; }
   } else {
     GemmArgs a = base_args(c, dy, d, f.fc2wT, d, c->g_dz, F, M, F, d);
@@ -592,10 +593,10 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
       if ((e = rank_proj(c, "lora_down_bwd", a, proj_args(c, a, 1)))) return e; }
     float* gA = gbase + (size_t)c->nq * 2 * c->r * d;
     if (!c->defer_grads) {
-    { Scope s(c, "lora_grad", 2);
+    { Scope s(c, "lora_grad");
       if ((e = lora_grad(c->dt, o, d, 0, d, g_dhcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, 1.0f, gA, gstride, 0, d,
                          1, c->grad_scratch, c->st, c->status, c->tc))) return e; }
-    { Scope s(c, "lora_grad", 2);
+    { Scope s(c, "lora_grad");
       if ((e = lora_grad(c->dt, g_dxmid, d, 0, d, hcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, c->scale,
                          gA + (size_t)c->r * d, gstride, 0, 1, c->r, c->grad_scratch, c->st, c->status, c->tc))) return e; }
     }
@@ -609,7 +610,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
     if ((e = linear(c, c->has_o ? "lora_linear_bwd" : "linear_bwd", a))) return e; }
   { const bool aligned_form = c->tc && attention_tc_supported(c->dt, T, H, d);
     const bool ragged_form = !aligned_form && c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, c->g_do, g_dqkv);
-    Scope s(c, "attention_bwd", aligned_form && !attention_t5_supported(c->dt, T, H, d) ? 3 : 2);
+    Scope s(c, "attention_bwd");
     if (aligned_form)
       e = attention_bwd_tc(qkv, o, lse, c->g_do, M / T, T, H, d, g_dqkv, c->rowdot, c->status, c->st);
     else if (ragged_form)
@@ -618,7 +619,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
       e = attention_bwd_simt(c->dt, qkv, o, lse, c->g_do, M / T, T, H, d, g_dqkv, c->rowdot, c->st);
     if (e) return e; }
   if (c->llama) {  // the gradient of a rotation is the inverse rotation
-    Scope s(c, "rope", 1);
+    Scope s(c, "rope");
     if ((e = rope_inplace(c->dt, g_dqkv, c->rope_table, M, T, H, d, -1.0f, c->st))) return e;
   }
   {  // dh = (alpha/r) dqkv B_g for every target (the scale lives in the compute copy)
@@ -656,7 +657,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
       jb.r = c->r; jb.rp = c->rp; jb.nt = 1; jb.scale = c->scale; jb.out = gbase + (size_t)t * 2 * c->r * d + (size_t)c->r * d;
       jb.out_group_stride = gstride; jb.out_target_stride = 0; jb.out_sj = 1; jb.out_sc = c->r;
     }
-    Scope s(c, "lora_grad", 2);
+    Scope s(c, "lora_grad");
     if ((e = lora_grad_batch(c->dt, jobs, nj, M, rpg, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc))) return e; }
   if (dx) {
     GemmArgs a = base_args(c, g_dqkv, 3 * d, f.qkvwT, 3 * d, c->g_du, d, M, d, 3 * d);
@@ -674,7 +675,7 @@ cudaError_t deferred_gradients(splitlora_ctx* c, bool client) {
   if (!c->defer_grads || l1 <= l0) return cudaSuccess;
   LoraGradJob jobs[LORA_GRAD_MAX_JOBS];
   const int n = grad_jobs(c, c->lb[l0], client ? c->cg : c->sg, client ? c->Pc : 0, jobs);
-  Scope s(c, "lora_grad", 1);
+  Scope s(c, "lora_grad");
   return lora_grad_layers(c->dt, jobs, n, l1 - l0, c->M, client ? c->rows_per_client : 0, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc);
 }
 
@@ -685,7 +686,7 @@ cudaError_t run_optimizer(splitlora_ctx* c, bool client) {
   int64_t step = client ? ++c->client_steps : ++c->server_steps;
   o.bc1 = (float)(1.0 - std::pow((double)c->cfg.beta1, (double)step));
   o.bc2 = (float)(1.0 - std::pow((double)c->cfg.beta2, (double)step));
-  Scope s(c, "optimizer", 1);
+  Scope s(c, "optimizer");
   if (client) return optimizer_step(c->cp, c->cg, c->cm, c->cv, (int64_t)c->K * c->Pc, o, c->st);
   return optimizer_step(c->sp, c->sg, c->sm, c->sv, c->Ps, o, c->st);
 }
@@ -823,7 +824,7 @@ int splitlora_bind_frozen(splitlora_ctx* c, const char* name, const void* dev, s
     if (n == "wte") set(&c->wte);
     if (n == "head.w" || !c->llama) {      // the head: tied to wte unless the architecture has its own
       if (c->llama) set(&c->headw); else c->headw = dev;
-      Scope s(c, "transpose", 1);
+      Scope s(c, "transpose");
       CK(c, transpose(c->dt, dev, c->V, c->d, c->wteT, c->Vpad, c->st));
     }
     return SPLITLORA_OK;
@@ -854,7 +855,7 @@ int splitlora_bind_frozen(splitlora_ctx* c, const char* name, const void* dev, s
       if (!expect(e.elems)) return bad_size();
       set(e.slot);
       if (e.tr) {
-        Scope s(c, "transpose", 1);
+        Scope s(c, "transpose");
         CK(c, transpose(c->dt, dev, e.rows, e.cols, e.tr, e.rows, c->st));
       }
       return SPLITLORA_OK;
@@ -941,7 +942,7 @@ int splitlora_client_fwd(splitlora_ctx* c, const int32_t* tokens, void* act_out)
   if (!tokens || !act_out) return fail(c, SPLITLORA_ERR_ARG, "null pointer");
   if (!aligned16(tokens) || !aligned16(act_out)) return fail(c, SPLITLORA_ERR_ALIGN, "tokens / act_out not 16-byte aligned");
   if (c->client_copies_dirty) { CK(c, refresh_side(c, true)); c->client_copies_dirty = false; }
-  { Scope s(c, "embed", 1);
+  { Scope s(c, "embed");
     CK(c, embed(c->dt, tokens, c->wte, c->wpe, c->emb, c->M, c->cfg.seq, c->d, c->V, c->st)); }
   const void* x = c->emb;
   for (int l = 0; l < c->cut; ++l) {
@@ -989,7 +990,7 @@ int splitlora_server_step(splitlora_ctx* c, const void* act_in, const int32_t* l
   { GemmArgs a = base_args(c, c->xf, d, c->headw, d, c->logits, c->Vpad, M, c->Vpad, d);
     a.w_rows = c->V;
     CK(c, linear(c, "head_fwd", a)); }
-  { Scope s(c, "cross_entropy", 3);
+  { Scope s(c, "cross_entropy");
     CK(c, cross_entropy(c->dt, c->logits, c->Vpad, labels, M, c->V, c->row_loss, c->n_valid, c->loss_dev,
                         (int)c->loss_normalizer, c->st)); }
   // backward: head, final norm, blocks L-1 .. first
@@ -1091,7 +1092,7 @@ int splitlora_aggregate(splitlora_ctx* c, const int64_t* counts) {
   int rc = aggregation_weights(c, counts, 0.0, w);
   if (rc) return rc;
   if (uniform_cut(c)) {
-    Scope s(c, "aggregate", 1);
+    Scope s(c, "aggregate");
     CK(c, aggregate(c->cp, c->K, c->Pc, w, c->st));
   } else {
     // Eq. 8-9 per block over the clients that hold it (a suffix of the clients), weights renormalised
@@ -1104,13 +1105,13 @@ int splitlora_aggregate(splitlora_ctx* c, const int64_t* counts) {
       if (!(tot > 0.0)) return fail(c, SPLITLORA_ERR_COUNTS, "all sample counts of a block's holders are zero");
       float wl[AGG_MAX_CLIENTS];
       for (int i = 0; i < nh; ++i) wl[i] = (float)((double)counts[h0 + i] / tot);
-      Scope s(c, "aggregate", 1);
+      Scope s(c, "aggregate");
       CK(c, aggregate(c->cp + (size_t)h0 * c->Pc + (size_t)l * c->per_layer, nh, c->per_layer, wl, c->st, c->Pc));
     }
   }
   // clients of lower rank keep only their own components of the (zero-padded) average
   if (!c->client_rank.empty()) {
-    Scope s(c, "aggregate", 1);
+    Scope s(c, "aggregate");
     CK(c, rank_mask(c->cp, c->K, c->Pc, c->r, c->d, c->client_rank.data(), c->st));
   }
   c->client_copies_dirty = true;
@@ -1143,7 +1144,7 @@ int splitlora_aggregate_local_sum(splitlora_ctx* c, const int64_t* counts, int64
   float w[AGG_MAX_CLIENTS];
   int rc = aggregation_weights(c, counts, (double)total_count, w);
   if (rc) return rc;
-  { Scope s(c, "aggregate", 1);
+  { Scope s(c, "aggregate");
     CK(c, aggregate_local_sum(c->cp, c->K, c->Pc, w, c->agg_sum, c->st)); }
   *sum_dev = c->agg_sum; *count = c->Pc;
   return SPLITLORA_OK;
@@ -1153,7 +1154,7 @@ int splitlora_aggregate_broadcast(splitlora_ctx* c) {
   LaunchChain chain;
   if (!c) return SPLITLORA_ERR_ARG;
   if (!c->ws) return fail(c, SPLITLORA_ERR_WORKSPACE, "no workspace bound");
-  { Scope s(c, "aggregate", c->client_rank.empty() ? 1 : 2);
+  { Scope s(c, "aggregate");
     CK(c, aggregate_broadcast(c->agg_sum, c->K, c->Pc, c->cp, c->st));
     // the mask comes after the sum over devices: the sum holds every client's components
     if (!c->client_rank.empty()) CK(c, rank_mask(c->cp, c->K, c->Pc, c->r, c->d, c->client_rank.data(), c->st)); }
@@ -1235,7 +1236,7 @@ int splitlora_round_compressed(splitlora_ctx* c, const int32_t* tokens, const in
   const size_t Md = (size_t)c->M * (size_t)c->d;
   // what crosses the cut is codes + scales; the receiving side restores into the buffer it reads
   auto cross = [&](void* buf, uint8_t* q, float* sc) -> int {
-    Scope s(c, "handoff_codec", 2);
+    Scope s(c, "handoff_codec");
     CK(c, handoff_quantize(c->dt, buf, c->M, c->d, q, sc, c->st));
     CK(c, handoff_dequantize(c->dt, q, sc, c->M, c->d, buf, c->st));
     return SPLITLORA_OK;
