@@ -250,7 +250,12 @@ cudaError_t gemm_simt(const GemmArgs& a, cudaStream_t st) {
   if (f32_vector_ok(a)) {
     // 64 x 64 tiles once they fill the chip, else a quarter of the tile and four thread groups along the contraction
     const int64_t tiles = (int64_t)((a.M + 63) / 64) * ((a.N + 63) / 64);
-    return tiles >= num_sms() ? launch_f32<F32Cfg<64, 64, 1, 32>>(a, st) : launch_f32<F32Cfg<32, 32, 4, 64>>(a, st);
+    if (tiles >= num_sms()) return launch_f32<F32Cfg<64, 64, 1, 32>>(a, st);
+    // still fewer: halves and quarters of that tile, as long as a block has an SM to itself
+    const int64_t small = (int64_t)((a.M + 31) / 32) * ((a.N + 31) / 32);
+    if (4 * small <= num_sms()) return launch_f32<F32Cfg<16, 16, 16, 64>>(a, st);
+    if (2 * small <= num_sms()) return launch_f32<F32Cfg<32, 16, 8, 64>>(a, st);
+    return launch_f32<F32Cfg<32, 32, 4, 64>>(a, st);
   }
   dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM);
   if (a.dtype == DT_BF16) launch_overlapped(gemm_simt_kernel<bf16>, grid, 256, 0, st, a);

@@ -238,3 +238,23 @@ def test_linear_fp32_any_size(M, K, N):
         buf = torch.full((M + 64, N), 7.0, device="cuda", dtype=torch.float32)
         B.linear(xin, W, bias, B.EPI_BIAS_RESID, r=r, y=buf[:M])
         assert bool((buf[M:] == 7).all()) and bool(((buf[:M].double() - ref).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("M,n_in,n_out,r,G", [(15, 1024, 1032, 8, 1), (17, 1000, 2304, 9, 1), (33, 3080, 40, 7, 1), (100, 4104, 64, 8, 1),
+                                              (2048, 2048, 2056, 12, 2), (4096, 256, 4096, 16, 1), (4097, 1024, 256, 8, 1), (256, 1024, 1024, 33, 1)])
+def test_rank_projections_of_every_shape(M, n_in, n_out, r, G):
+    """Rows and columns around the tiles and slabs of the rank-r projections, one to four slabs and more than they take, ranks
+    around their column tiles, and the row counts at which they hand over to the linear layers' kernels."""
+    test_lora_linear_any_size(M, n_in, n_out, r, G)
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (512, 128, 64), (512, 512, 128), (100, 520, 128), (77, 1000, 40), (512, 128, 384), (1200, 72, 1000)])
+def test_linear_fp32_tiles(M, K, N):
+    """Few to many tiles, with the contraction over one, four, eight and sixteen thread groups: roundings of random sign, one
+    per term of the longest sum, taken four times."""
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    x, W = (torch.randn(n, K, device="cuda", generator=g, dtype=torch.float32) for n in (M, N))
+    buf = torch.full((M + 16, N), 7.0, device="cuda", dtype=torch.float32)
+    B.linear(x, W, None, y=buf[:M])
+    assert bool((buf[M:] == 7).all())
+    assert _norm_err(buf[:M], x.double() @ W.double().T) <= 4 * K ** 0.5 * 2.0 ** -24
