@@ -167,6 +167,9 @@ cudaError_t norm_proj(bool rms, const void* x, const void* g, const void* b, flo
 
 // Adapter gradients: for nt targets of rank r (weight columns wcol0 + t*rp + jj of Wt),
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c],  c < C,
+// the same in fp32, LayerNorm only
+bool norm_proj_f32_supported(const ProjArgs& a);
+cudaError_t norm_proj_f32(const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st);
 // stored at out + g*out_group_stride + t*out_target_stride + jj*out_sj + c*out_sc.
 // rows_per_group must be a multiple of 128 unless there is one group (0, or >= M).  partial: scratch of at least
 // lora_grad_scratch_floats(M, nt*r, C) floats.

@@ -309,6 +309,64 @@ __global__ void __launch_bounds__(THREADS) norm_proj_kernel(const __grid_constan
   store_rows<NT>(p, red, row0);
 }
 
+// fp32: LayerNorm and the projection of a row by one warp, the row in registers (at most NV vectors of 4 per lane); one dot
+// product with a row of W after another.  Over few rows the two launches it replaces were 8 us of a layer's 65.
+template <int NV>
+__global__ void __launch_bounds__(THREADS) norm_proj_f32_kernel(const float* __restrict__ x, const float* __restrict__ gain, const float* __restrict__ shift,
+                                                                float* __restrict__ u, float* __restrict__ mean, float* __restrict__ rstd, float eps,
+                                                                const float* __restrict__ W, int64_t w_gs, int rows_per_group, float* __restrict__ Y,
+                                                                int M, int d, int ext, int nt, int r, int rp) {
+  overlap_sync();
+  const int row = (int)blockIdx.x * WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= M) return;
+  if (w_gs) W += (int64_t)(row / rows_per_group) * w_gs;
+  float4 v[NV];
+  float s = 0.f, q = 0.f;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const int c = (k * 32 + lane) * 4;
+    v[k] = c < d ? *reinterpret_cast<const float4*>(x + (int64_t)row * d + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    s += v[k].x; s += v[k].y; s += v[k].z; s += v[k].w;
+  }
+  const float mu = warp_sum(s) / d;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    if ((k * 32 + lane) * 4 >= d) break;
+    float t;
+    t = v[k].x - mu; q += t * t; t = v[k].y - mu; q += t * t; t = v[k].z - mu; q += t * t; t = v[k].w - mu; q += t * t;
+  }
+  const float rs = rsqrtf(warp_sum(q) / d + eps);
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const int c = (k * 32 + lane) * 4;
+    if (c >= d) break;
+    const float4 gv = *reinterpret_cast<const float4*>(gain + c), bv = *reinterpret_cast<const float4*>(shift + c);
+    v[k] = make_float4((v[k].x - mu) * rs * gv.x + bv.x, (v[k].y - mu) * rs * gv.y + bv.y, (v[k].z - mu) * rs * gv.z + bv.z, (v[k].w - mu) * rs * gv.w + bv.w);
+    *reinterpret_cast<float4*>(u + (int64_t)row * d + c) = v[k];
+  }
+  if (lane == 0) { mean[row] = mu; rstd[row] = rs; }
+  float mine = 0.f;                              // lane i: component i of nt * r
+  for (int i = 0; i < nt * r; ++i) {
+    const float* w = W + (int64_t)(i / r * rp + i % r) * d;
+    float dot = 0.f;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int c = (k * 32 + lane) * 4;
+      if (c >= d) break;
+      const float4 a = *reinterpret_cast<const float4*>(w + c);
+      dot = fmaf(v[k].w, a.w, fmaf(v[k].z, a.z, fmaf(v[k].y, a.y, fmaf(v[k].x, a.x, dot))));
+    }
+    dot = warp_sum(dot);
+    if (lane == i) mine = dot;
+  }
+  for (int c0 = 0; c0 < ext; c0 += 32) {
+    const int c = c0 + lane, t = c / rp, j = c % rp;
+    const bool used = t < nt && j < r;
+    const float h = __shfl_sync(0xffffffffu, mine, used ? t * r + j : 0);
+    if (c < ext) Y[(int64_t)row * ext + c] = used ? h : 0.f;
+  }
+}
+
 template <int SLABS, int N, bool SEPARATE, bool COPIES>
 cudaError_t launch(Proj p, const AdapterCopyArgs& copies, cudaStream_t st) {
   const auto kernel = proj_kernel<SLABS, N, SEPARATE, COPIES>;
@@ -468,6 +526,21 @@ cudaError_t norm_proj(bool rms, const void* x, const void* g, const void* b, flo
   fill(a, s, p);
   const NormIn in = {(const bf16*)x, (const bf16*)g, (const bf16*)b, (bf16*)const_cast<void*>(a.X), mean, rstd, a.K, eps};
   return rms ? launch_norm_tiles<true>(s.n, p, in, st) : launch_norm_tiles<false>(s.n, p, in, st);
+}
+
+bool norm_proj_f32_supported(const ProjArgs& a) {
+  auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
+  return a.K % 4 == 0 && a.K <= 1024 && a.ldx == a.K && a.ldw == a.K && a.nt * a.r <= 32 && al16(a.X) && al16(a.W) &&
+         (a.rows_per_group <= 0 || a.w_group_stride % 4 == 0);
+}
+cudaError_t norm_proj_f32(const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st) {
+  if (!norm_proj_f32_supported(a)) return cudaErrorInvalidValue;
+  const int64_t w_gs = a.rows_per_group > 0 && a.rows_per_group < a.M ? a.w_group_stride : 0;
+  auto go = [&](auto kernel) {
+    return launch_overlapped(kernel, (a.M + WARPS - 1) / WARPS, THREADS, 0, st, (const float*)x, (const float*)g, (const float*)b, (float*)const_cast<void*>(a.X),
+                             mean, rstd, eps, (const float*)a.W, w_gs, a.rows_per_group, (float*)a.Y, a.M, a.K, a.ext, a.nt, a.r, a.rp);
+  };
+  return a.K <= 256 ? go(norm_proj_f32_kernel<2>) : a.K <= 512 ? go(norm_proj_f32_kernel<4>) : go(norm_proj_f32_kernel<8>);
 }
 
 }  // namespace sl

@@ -491,6 +491,9 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
     if (c->tc && M <= NORM_PROJ_ROWS && norm_proj_supported(p)) {
       Scope s(c, "layernorm_fwd");
       if ((e = norm_proj(c->llama, xin, f.ln1g, f.ln1b, atf(b.mean1), atf(b.rstd1), c->cfg.norm_eps, p, c->st))) return e;
+    } else if (c->dt == DT_F32 && !c->llama && M <= LORA_PROJ_ROWS && norm_proj_f32_supported(p)) {
+      Scope s(c, "layernorm_fwd");
+      if ((e = norm_proj_f32(xin, f.ln1g, f.ln1b, atf(b.mean1), atf(b.rstd1), c->cfg.norm_eps, p, c->st))) return e;
     } else {
       if ((e = norm_forward(c, M, xin, f.ln1g, f.ln1b, u, atf(b.mean1), atf(b.rstd1)))) return e;
       if ((e = rank_proj(c, "lora_down_fwd", a, p))) return e;
