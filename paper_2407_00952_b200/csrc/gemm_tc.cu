@@ -10,7 +10,7 @@
 // tile, so K clients with their own adapters share one pass over the frozen W.
 //
 // Three kernels (pick_kernel chooses):
-//   gemm_tc_pair_kernel   CTA pairs (cluster of 2, tcgen05 cta_group::2): a pair owns a 256 x 256
+//   gemm_tc_pair_kernel   CTA pairs (cluster of 2, tcgen05 cta_group::2): a pair owns a 256 x 256 (or 256 x 128)
 //                         tile; each CTA stages its 128 rows of X and one half (128 rows) of the W
 //                         tile, the leader issues 256 x 256 x 16 products that read both CTAs'
 //                         shared memory and write both CTAs' tensor memory.  32 KB per CTA per
@@ -231,27 +231,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__
 // [128 x 256] block per CTA tile is brought into shared memory by the producer warp with TMA about
 // one tile ahead of its use, so the epilogue never waits on a global load; the room comes from a
 // shorter operand ring (4 stages instead of 6).
-template <bool NEED_R> struct PairCfg {
-  static constexpr int BN = 256;                       // tile columns of the pair
+// BN_: tile columns of the pair.  256, or 128 where tiles of 256 would leave SMs idle.
+template <bool NEED_R, int BN_> struct PairCfg {
+  static constexpr int BN = BN_;
   static constexpr int A_BYTES = BM * BK * 2;          // this CTA's 128 rows of X
   static constexpr int B_BYTES = (BN / 2) * BK * 2;    // this CTA's half of the W tile
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = NEED_R ? 4 : 6;
+  static constexpr int STAGES = BN == 256 ? (NEED_R ? 4 : 6) : (NEED_R ? 6 : 8);
   static constexpr int R_BYTES = NEED_R ? BM * BN * 2 : 0;
-  static constexpr int TMEM_COLS = 512;
+  static constexpr int TMEM_COLS = 2 * BN;
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + R_BYTES + EPI_STAGE_BYTES + 1024 + 256;
   static constexpr uint32_t IDESC = make_idesc(2 * BM, BN);
 };
 
-template <int EPI, bool EXACT>
+template <int EPI, bool EXACT, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                     const __grid_constant__ CUtensorMap mapXe, const __grid_constant__ CUtensorMap mapWe,
                     const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapZ,
                     const __grid_constant__ CUtensorMap mapR, TcParams p) {
   constexpr bool NEED_R = EPI == EPI_BIAS_RESID || EPI == EPI_MUL_GELUGRAD;
-  using C = PairCfg<NEED_R>;
-  constexpr int BN = C::BN;
+  using C = PairCfg<NEED_R, BN>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -293,7 +293,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_const
   const uint32_t tmem_base = *tmem_slot;
   overlap_sync();
 
-  const int num_tiles = p.tiles_m * p.tiles_n;       // tiles of 256 x 256
+  const int num_tiles = p.tiles_m * p.tiles_n;       // tiles of 256 x BN
   const int kb_total = p.num_kb + p.ext_blocks;
 
   if (warp == 0) {
@@ -716,7 +716,8 @@ bool pair_ok(const GemmArgs& a) {
 // (1024 -> 1024: 11.6 against 17.4).  Tiles of 128 rows win over pairs where 256-row tiles need a round more: 1152 x 4096
 // -> 4096 (144 tiles on 148 SMs, or 80 on 74 pairs) 27.1 us, as pairs 34.3; 2176 x 768 -> 3072 with a residual 19.6, as
 // pairs 15.0.
-enum Kernel { KERNEL_SINGLE, KERNEL_PAIR, KERNEL_SPLIT64_1, KERNEL_SPLIT64_2, KERNEL_SPLIT64_4, KERNEL_SPLIT64_8, KERNEL_SPLIT128_1 };
+enum Kernel { KERNEL_SINGLE, KERNEL_PAIR, KERNEL_PAIR128, KERNEL_SPLIT64_1, KERNEL_SPLIT64_2, KERNEL_SPLIT64_4, KERNEL_SPLIT64_8, KERNEL_SPLIT128_1,
+              KERNEL_SPLIT128_2 };
 Kernel pick_kernel(const GemmArgs& a) {
   const int64_t sms = num_sms();
   const int64_t kb = (a.K + BK - 1) / BK + (a.Ke + BK - 1) / BK;
@@ -725,22 +726,27 @@ Kernel pick_kernel(const GemmArgs& a) {
   int64_t best_ns = INT64_MAX;
   auto offer = [&](Kernel k, int64_t ns) { if (ns < best_ns) { best_ns = ns; best = k; } };
   if (pair_ok(a)) offer(KERNEL_PAIR, 5500 + cdiv(cdiv(a.M, 2 * BM) * cdiv(a.N, 256), max_pairs()) * kb * 275);
+  // tiles of half the width where those of 256 fill their last round badly: 1665 x 768 -> 3072 with GELU (84 tiles on 74 pairs, or
+  // 168) 19.3 -> 16.6 us, its backward 20.2 -> 18.5, 1665 x 1024 -> 3072 16.7 -> 15.7; 2560 x 1024 -> 4096 27.2 as 256, 28.2 as 128
+  if (pair_ok(a)) offer(KERNEL_PAIR128, 4500 + cdiv(cdiv(a.M, 2 * BM) * cdiv(a.N, 128), max_pairs()) * kb * 200);
   // (where both take about as many rounds, two CTAs by themselves are 10-20 % slower than a pair, and their epilogue waits
   // for its second operand, 2 us a round, which the pair kernel brings ahead by TMA)
   const int bn = pick_bn(a);
   const int64_t block = bn == 256 ? 330 : bn == 64 ? 200 : 300;
   const bool need_r = a.epi == EPI_BIAS_RESID || a.epi == EPI_MUL_GELUGRAD;
   offer(KERNEL_SINGLE, 5500 + cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), bn == 64 ? 2 * sms : sms) * (kb * block + (need_r ? 2000 : 0)));
-  auto split = [&](Kernel k, int bn, int s, int64_t fixed) {
+  auto split = [&](Kernel k, int bn, int s, int64_t fixed, int64_t block_ns = 190) {
     const int64_t slots = s == 1 ? sms : max_split_clusters(s) > 0 ? max_split_clusters(s) : sms / s;
     const int64_t rounds = cdiv(cdiv(a.M, BM) * cdiv(a.N, bn), slots);
-    if (s == 1 || kb >= 2 * s) offer(k, fixed + rounds * cdiv(kb, s) * 190 + (rounds - 1) * 3000);
+    if (s == 1 || kb >= 2 * s) offer(k, fixed + rounds * cdiv(kb, s) * block_ns + (rounds - 1) * 3000);
   };
   split(KERNEL_SPLIT64_1, 64, 1, 3600);
   split(KERNEL_SPLIT64_2, 64, 2, 4700);
   split(KERNEL_SPLIT64_4, 64, 4, 5000);
   split(KERNEL_SPLIT64_8, 64, 8, 5500);
   split(KERNEL_SPLIT128_1, 128, 1, 4400);
+  // 1000 x 4096 -> 1024 17.4 -> 14.2 us (128 tiles of 64 columns, or 64 of 128 in clusters of two), x 2304 -> 768 11.3 -> 10.3
+  split(KERNEL_SPLIT128_2, 128, 2, 5350, 230);
   return best;
 }
 
@@ -829,14 +835,14 @@ cudaError_t launch_split(const GemmArgs& a, int* status, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, gemm_tc_split_kernel<BN, S, STAGES, EXACT>, mX, mW, mXe, mWe, mY, mZ, p);
 }
 
-template <int EPI, bool EXACT>
+template <int EPI, bool EXACT, int BN>
 cudaError_t launch_pair_epi(const GemmArgs& a, int* status, cudaStream_t st) {
   constexpr bool NEED_R = EPI == EPI_BIAS_RESID || EPI == EPI_MUL_GELUGRAD;
-  using C = PairCfg<NEED_R>;
+  using C = PairCfg<NEED_R, BN>;
   static PerDeviceOnce once;
   const int dev = current_device();
   if (once.needed(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_pair_kernel<EPI, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_pair_kernel<EPI, EXACT, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
@@ -848,16 +854,16 @@ cudaError_t launch_pair_epi(const GemmArgs& a, int* status, cudaStream_t st) {
   const int pairs = tiles < max_pairs() ? tiles : max_pairs();
   mR = mY;
   if (NEED_R && !make_map(&mR, a.R, a.M, a.N, a.ldr, BM)) return cudaErrorInvalidValue;
-  launch_overlapped(gemm_tc_pair_kernel<EPI, EXACT>, 2 * pairs, NUM_THREADS, C::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
+  launch_overlapped(gemm_tc_pair_kernel<EPI, EXACT, BN>, 2 * pairs, NUM_THREADS, C::SMEM_BYTES, st, mX, mW, mXe, mWe, mY, mZ, mR, p);
   return cudaGetLastError();
 }
-template <bool EXACT>
+template <bool EXACT, int BN>
 cudaError_t launch_pair(const GemmArgs& a, int* status, cudaStream_t st) {
   switch (a.epi) {
-    case EPI_BIAS_GELU: return launch_pair_epi<EPI_BIAS_GELU, EXACT>(a, status, st);
-    case EPI_MUL_GELUGRAD: return launch_pair_epi<EPI_MUL_GELUGRAD, EXACT>(a, status, st);
-    case EPI_BIAS_RESID: return launch_pair_epi<EPI_BIAS_RESID, false>(a, status, st);
-    default: return launch_pair_epi<EPI_BIAS, false>(a, status, st);
+    case EPI_BIAS_GELU: return launch_pair_epi<EPI_BIAS_GELU, EXACT, BN>(a, status, st);
+    case EPI_MUL_GELUGRAD: return launch_pair_epi<EPI_MUL_GELUGRAD, EXACT, BN>(a, status, st);
+    case EPI_BIAS_RESID: return launch_pair_epi<EPI_BIAS_RESID, false, BN>(a, status, st);
+    default: return launch_pair_epi<EPI_BIAS, false, BN>(a, status, st);
   }
 }
 
@@ -885,15 +891,15 @@ int gemm_tc_init() {
   if (!g_pair_once.needed(dev)) return 0;
   // how many CTA pairs fit on this device at once (the pair kernel is persistent: one wave)
   g_max_pairs[dev] = 0;
-  if (cudaFuncSetAttribute(gemm_tc_pair_kernel<EPI_BIAS_RESID, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<true>::SMEM_BYTES) == cudaSuccess) {
+  if (cudaFuncSetAttribute(gemm_tc_pair_kernel<EPI_BIAS_RESID, false, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<true, 256>::SMEM_BYTES) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(sms & ~1); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = PairCfg<true>::SMEM_BYTES;
+    cfg.gridDim = dim3(sms & ~1); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = PairCfg<true, 256>::SMEM_BYTES;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = 2; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
     cfg.attrs = &at; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<EPI_BIAS_RESID, false>, &cfg) == cudaSuccess && n > 0)
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<EPI_BIAS_RESID, false, 256>, &cfg) == cudaSuccess && n > 0)
       g_max_pairs[dev] = n < sms / 2 ? n : sms / 2;
   }
   g_max_split_clusters[dev][0] = query_split_clusters<2>();
@@ -935,7 +941,9 @@ cudaError_t launch_picked(const GemmArgs& a, int* status, cudaStream_t st) {
     case KERNEL_SPLIT64_4: return launch_split<64, 4, 8, EXACT>(a, status, st);
     case KERNEL_SPLIT64_8: return launch_split<64, 8, 8, EXACT>(a, status, st);
     case KERNEL_SPLIT128_1: return launch_split<128, 1, 6, EXACT>(a, status, st);
-    case KERNEL_PAIR: return launch_pair<EXACT>(a, status, st);
+    case KERNEL_SPLIT128_2: return launch_split<128, 2, 6, EXACT>(a, status, st);
+    case KERNEL_PAIR: return launch_pair<EXACT, 256>(a, status, st);
+    case KERNEL_PAIR128: return launch_pair<EXACT, 128>(a, status, st);
     default: break;
   }
   switch (pick_bn(a)) {

@@ -258,3 +258,10 @@ def test_linear_fp32_tiles(M, K, N):
     B.linear(x, W, None, y=buf[:M])
     assert bool((buf[M:] == 7).all())
     assert _norm_err(buf[:M], x.double() @ W.double().T) <= 4 * K ** 0.5 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("M,K,N", [(1000, 2304, 768), (999, 4096, 1000), (1700, 1032, 2952), (1665, 768, 2304)])
+@pytest.mark.parametrize("epilogue", [B.EPI_BIAS, B.EPI_BIAS_GELU, B.EPI_BIAS_RESID, B.EPI_MUL_GELUGRAD])
+def test_linear_tiles_of_128_columns(M, K, N, epilogue):
+    """Clusters of two and CTA pairs on tiles of 128 columns, whole and ragged, one and several tiles per pair."""
+    test_linear_any_row_count_and_depth(M, K, N, epilogue)
