@@ -36,7 +36,7 @@ constexpr uint32_t LT_IDESC = make_idesc(LT_C, LT_N) | (1u << 15) | (1u << 16);
 
 struct LgParams {
   int C, rows_per_chunk, R, r, rp, wsel0;
-  float* partial;                                // [layer][chunk][R][C], or nullptr: a group is one chunk
+  float* partial;                                // [layer][chunk][R][C]
   float* out; int64_t out_ls, ogs, ots, osj, osc; float scale;
   int* status;
 };
@@ -67,8 +67,9 @@ __device__ __forceinline__ uint64_t desc_mn(uint32_t addr, uint32_t mn_stride) {
   return d;
 }
 
-// LAYERS: the operands are planes of three-dimensional maps, one per layer (a single layer: two-dimensional ones).
-template <bool LAYERS>
+// LAYERS: the operands are planes of three-dimensional maps, one per layer (a single layer: two-dimensional ones).  DIRECT:
+// one chunk per group, the result goes to the gradient.
+template <bool LAYERS, bool DIRECT>
 __global__ void __launch_bounds__(LT_THREADS, 2)
 lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
   const int layer = LAYERS ? (int)blockIdx.z / bt.njobs : 0, job = LAYERS ? (int)blockIdx.z % bt.njobs : (int)blockIdx.z;
@@ -159,15 +160,18 @@ lora_grad_tc_kernel(const __grid_constant__ LgBatch bt) {
       const int c = c0 + q * 32 + lane;
       if (c < p.C) {
         const int sh = p.rp == 16 ? 4 : (p.rp == 32 ? 5 : 6);
-        float* out = p.partial ? p.partial + ((size_t)layer * gridDim.y + chunk) * p.R * p.C + c
-                               : p.out + (size_t)layer * p.out_ls + (size_t)chunk * p.ogs + (size_t)c * p.osc;
-        const int64_t ots = p.partial ? (int64_t)p.r * p.C : p.ots, osj = p.partial ? p.C : p.osj;
-        const float scale = p.partial ? 1.f : p.scale;
+        float* out = DIRECT ? p.out + (size_t)layer * p.out_ls + (size_t)chunk * p.ogs + (size_t)c * p.osc
+                            : p.partial + ((size_t)layer * gridDim.y + chunk) * p.R * p.C + c;
+        const int ots = DIRECT ? (int)p.ots : 0, osj = DIRECT ? (int)p.osj : 0;       // within one adapter pair of one layer
 #pragma unroll
         for (int col = 0; col < LT_N; ++col) {
           const int rel = col - p.wsel0;
           const int t = rel >> sh, jj = rel & (p.rp - 1);
-          if (rel >= 0 && jj < p.r && t * p.r + jj < p.R) out[t * ots + jj * osj] = scale * v[col];
+          const int j = t * p.r + jj;
+          if (rel >= 0 && jj < p.r && j < p.R) {
+            if constexpr (DIRECT) out[t * ots + jj * osj] = p.scale * v[col];
+            else out[(size_t)j * p.C] = v[col];
+          }
         }
       }
     }
@@ -197,7 +201,7 @@ bool init_device() {
   const int dev = current_device();
   if (dev < 0 || !tensor_map_encoder()) return false;
   if (!g_once.needed(dev)) return true;
-  for (auto kernel : {lora_grad_tc_kernel<false>, lora_grad_tc_kernel<true>})
+  for (auto kernel : {lora_grad_tc_kernel<false, false>, lora_grad_tc_kernel<false, true>, lora_grad_tc_kernel<true, false>, lora_grad_tc_kernel<true, true>})
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LT_SMEM) != cudaSuccess) return false;
   g_once.done(dev);
   return true;
@@ -262,7 +266,7 @@ cudaError_t lora_grad_tc_layers(const LoraGradJob* jobs, int njobs, int layers, 
     if (!make_map(&bt.mapW[j], jb.Wt, (uint64_t)layers, (uint64_t)M, (uint64_t)jb.ldwt, (uint64_t)jb.ldwt, (uint64_t)jb.wt_ls)) return cudaErrorInvalidValue;
     LgParams& p = bt.p[j];
     p.C = jb.C; p.rows_per_chunk = rpg / s; p.R = jb.nt * jb.r; p.r = jb.r; p.rp = jb.rp; p.wsel0 = jb.wcol0 % LT_N;
-    p.partial = s > 1 ? partial + off : nullptr; p.status = status;
+    p.partial = partial + off; p.status = status;
     p.out = jb.out; p.out_ls = jb.out_ls; p.ogs = jb.out_group_stride; p.ots = jb.out_target_stride; p.osj = jb.out_sj; p.osc = jb.out_sc;
     p.scale = jb.scale;
     bt.wx0[j] = jb.wcol0 - p.wsel0;
@@ -272,7 +276,9 @@ cudaError_t lora_grad_tc_layers(const LoraGradJob* jobs, int njobs, int layers, 
   for (int j = njobs; j < LT_MAX_JOBS; ++j) { bt.mapZ[j] = bt.mapZ[0]; bt.mapW[j] = bt.mapW[0]; bt.p[j] = bt.p[0]; bt.wx0[j] = bt.wx0[0]; }
   bt.njobs = njobs;
   dim3 grid(ctiles, groups * s, layers * njobs);
-  launch_overlapped(layers > 1 ? lora_grad_tc_kernel<true> : lora_grad_tc_kernel<false>, grid, LT_THREADS, LT_SMEM, st, bt);
+  const auto kernel = layers > 1 ? (s > 1 ? lora_grad_tc_kernel<true, false> : lora_grad_tc_kernel<true, true>)
+                                 : (s > 1 ? lora_grad_tc_kernel<false, false> : lora_grad_tc_kernel<false, true>);
+  launch_overlapped(kernel, grid, LT_THREADS, LT_SMEM, st, bt);
   *chunks_per_group = s;
   return cudaGetLastError();
 }
