@@ -663,9 +663,28 @@ cudaError_t attention_fwd_tc(const void* qkv, int nseq, int T, int H, int d, voi
                      : launch_fwd<128, false>(qkv, nseq, T, H, d, o, lse, st);
 }
 
+// The two tcgen05 forms of the backward pass at lengths that are multiples of 128.  attention_t5_bwd.cu needs about 0.83 of the
+// time per pair of tiles, but shares out whole items: a CTA takes one tile of an item per round, of lengths that rotate.
+// attention_t5_ragged.cu shares out single tiles, longest first, and runs both gradients at once where the tiles are few.
+// Backward us, whole items -> single tiles: 2 sequences of 256, 16 heads 15.0 -> 9.5; 4 x 128 13.3 -> 8.1; 1 x 2048, 12 heads 70 -> 48;
+// 8 x 1024, 8 heads 66 -> 53; 5 x 384, 12 heads 23.3 -> 20.3; 16 x 256, 12 heads 25.4 -> 24.4; 64 x 512, 16 heads 200 -> 233;
+// 32 x 512, 12 heads 87 -> 99; 64 x 128, 16 heads 43.5 -> 46.5.
+static bool w64_beats_whole_items(int nseq, int T, int H) {
+  const int64_t sms = num_sms(), nq = T / 128, items = (int64_t)nseq * H, units = items * nq;
+  if (2 * units <= sms) return true;
+  if (nq > 64 || sms < nq) return true;                       // (not taken there)
+  const int64_t per_round = (units < sms ? units : sms) / nq, rounds = (items + per_round - 1) / per_round;
+  int64_t longest = rounds / nq * (nq * (nq + 1) / 2);        // steps of the CTA with the most: whole turns, then the longest tiles
+  for (int64_t k = 0; k < rounds % nq; ++k) longest += nq - k;
+  const int64_t steps = items * (nq * (nq + 1) / 2), even = (steps + sms - 1) / sms;
+  return 12 * (even > nq ? even : nq) < 10 * longest;
+}
+
 cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                              int d, void* dqkv, float* rowdot, int* status, cudaStream_t st) {
   if (!attention_tc_supported(DT_BF16, T, H, d)) return cudaErrorInvalidValue;
+  if (d / H == 64 && T >= 128 && (T % 128 != 0 || w64_beats_whole_items(nseq, T, H)))
+    return attention_bwd_t5_w64(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
   if (attention_t5_supported(DT_BF16, T, H, d))
     return attention_bwd_t5(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
   return d / H == 64 ? launch_bwd<64, false>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st)
@@ -688,7 +707,12 @@ bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const voi
   return dh % 8 == 0 && dh <= 128 && H <= 65535 && nseq <= 65535 && al16(qkv) && al16(o) && al16(d_o) && al16(dqkv);
 }
 
-cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st) {
+cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, int* status, cudaStream_t st) {
+  // Tiles of 128 on tcgen05 against tiles of 64 here, us: 16 sequences of 777, 12 heads 115 -> 83; 32 x 288 44.7 -> 37.5; 5 x 333
+  // 17.6 -> 13.5; 4 x 1000, 8 heads 41.5 -> 29.9; 64 x 70, 16 heads 27 -> 17.3; with fewer tiles than SMs the longer steps of one CTA
+  // show: 1 x 1000, 8 heads 20.7 -> 27.7, 1 x 333 9.4 -> 13.1; up to 64 rows half a tile is padding: 64 x 50 11.3 -> 14.7.
+  if (attention_ragged_t5_supported(nseq, T, H, d) && T > 64 && (int64_t)nseq * H * ((T + 127) / 128) > num_sms())
+    return attention_fwd_ragged_t5(qkv, nseq, T, H, d, o, lse, status, st);
   switch ((d / H + 31) / 32) {
     case 1: return launch_fwd<32, true>(qkv, nseq, T, H, d, o, lse, st);
     case 2: return launch_fwd<64, true>(qkv, nseq, T, H, d, o, lse, st);
@@ -704,7 +728,7 @@ cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* ls
   // 5 x 333 44 -> 22; one of 150 with 4 heads 14.2 -> 14.1.  Up to 128 rows a head is one tile there, whose fixed part (set-up,
   // first loads) shows until there are about as many heads as SMs: 64 x 70, 16 heads 80 -> 41; 16 x 100, 8 heads 16.8 -> 15.4;
   // 8 x 100 12.3 -> 13.5; 2 x 96, 12 heads 11.8 -> 13.3.  Up to 64 rows half of that tile is padding: 64 x 50, 16 heads 33.6 -> 34.6.
-  if (attention_bwd_ragged_t5_supported(nseq, T, H, d) && (T > 128 || (T > 64 && (int64_t)nseq * H * 4 > 3 * (int64_t)num_sms())))
+  if (attention_ragged_t5_supported(nseq, T, H, d) && (T > 128 || (T > 64 && (int64_t)nseq * H * 4 > 3 * (int64_t)num_sms())))
     return attention_bwd_ragged_t5(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
   switch ((d / H + 31) / 32) {
     case 1: return launch_bwd<32, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, nullptr, st);

@@ -114,11 +114,15 @@ cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, c
 // 16 mantissa bits (attention_tc.cu).  Pointers that a direction does not use may be null.
 bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const void* qkv, const void* o, const void* d_o,
                                 const void* dqkv);
-cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, cudaStream_t st);
+cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, int* status, cudaStream_t st);
 cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                                  int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
-// the backward pass of those of width 64 on tcgen05 (attention_t5_ragged.cu); status as above
-bool attention_bwd_ragged_t5_supported(int nseq, int T, int H, int d);
+// Width 64 on tcgen05 (attention_t5_ragged.cu), any length; status as above.  attention_bwd_t5_w64: P and dS as bf16, for the
+// lengths that always held them so.
+bool attention_ragged_t5_supported(int nseq, int T, int H, int d);
+cudaError_t attention_fwd_ragged_t5(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, int* status, cudaStream_t st);
+cudaError_t attention_bwd_t5_w64(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
+                                 int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
 cudaError_t attention_bwd_ragged_t5(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                                     int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
 
@@ -163,13 +167,13 @@ cudaError_t lora_proj(const ProjArgs& a, cudaStream_t st);
 cudaError_t lora_proj_copies(const ProjArgs& a, const AdapterCopyArgs& copies, cudaStream_t st);
 // The norm in front of it in the same launch: a.X [M, K] receives LayerNorm(x) (RMSNorm: b and mean unused), Y its projection.
 bool norm_proj_supported(const ProjArgs& a);
+// the same in fp32, LayerNorm only
+bool norm_proj_f32_supported(const ProjArgs& a);
+cudaError_t norm_proj_f32(const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st);
 cudaError_t norm_proj(bool rms, const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st);
 
 // Adapter gradients: for nt targets of rank r (weight columns wcol0 + t*rp + jj of Wt),
 //   out[g][t][jj][c] = scale * sum_{m in group g} Wt[m, wcol0 + t*rp + jj] * Z[m, zcol0 + c],  c < C,
-// the same in fp32, LayerNorm only
-bool norm_proj_f32_supported(const ProjArgs& a);
-cudaError_t norm_proj_f32(const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st);
 // stored at out + g*out_group_stride + t*out_target_stride + jj*out_sj + c*out_sc.
 // rows_per_group must be a multiple of 128 unless there is one group (0, or >= M).  partial: scratch of at least
 // lora_grad_scratch_floats(M, nt*r, C) floats.

@@ -253,7 +253,7 @@ int splitlora_attention_fwd(int dtype, int use_tc, const void* qkv, int nseq, in
   if (use_tc && attention_tc_supported(dtype, T, n_head, d_model))
     e = attention_fwd_tc(qkv, nseq, T, n_head, d_model, o, lse, nullptr, (cudaStream_t)stream);
   else if (use_tc && attention_ragged_supported(dtype, nseq, T, n_head, d_model, qkv, o, nullptr, nullptr))
-    e = attention_fwd_ragged(qkv, nseq, T, n_head, d_model, o, lse, (cudaStream_t)stream);
+    e = attention_fwd_ragged(qkv, nseq, T, n_head, d_model, o, lse, nullptr, (cudaStream_t)stream);
   else
     e = attention_fwd_simt(dtype, qkv, nseq, T, n_head, d_model, o, lse, (cudaStream_t)stream);
   return e == cudaSuccess ? SPLITLORA_OK : SPLITLORA_ERR_CUDA;

@@ -513,7 +513,7 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
     if (c->tc && attention_tc_supported(c->dt, T, H, d))
       e = attention_fwd_tc(qkv, M / T, T, H, d, o, lse, c->status, c->st);
     else if (c->tc && attention_ragged_supported(c->dt, M / T, T, H, d, qkv, o, nullptr, nullptr))
-      e = attention_fwd_ragged(qkv, M / T, T, H, d, o, lse, c->st);
+      e = attention_fwd_ragged(qkv, M / T, T, H, d, o, lse, c->status, c->st);
     else
       e = attention_fwd_simt(c->dt, qkv, M / T, T, H, d, o, lse, c->st);
     if (e) return e; }

@@ -49,21 +49,23 @@ def test_attention_any_length_and_width(T, dh):
 
 
 @pytest.mark.parametrize("nseq,T,H", [(1, 129, 1), (40, 65, 4), (150, 70, 1), (2, 127, 70), (3, 191, 2), (2, 193, 3), (1, 257, 5), (5, 333, 12),
-                                      (3, 321, 60), (1, 1025, 2)])
-def test_attention_backward_of_any_length_in_tiles_of_128(nseq, T, H):
-    """Edges of the 128-row tiles and of their 64-row halves, one and several units of work per CTA, width 64: the bounds of
-    test_attention_any_length_and_width, and the same bits from run to run."""
+                                      (3, 321, 60), (1, 1025, 2), (30, 161, 12)])
+def test_attention_of_any_length_in_tiles_of_128(nseq, T, H):
+    """Edges of the 128-row tiles, of their 64-row halves and 32-key steps, one and several units of work per CTA, width 64:
+    the bounds of test_attention_any_length_and_width, and the same bits from run to run."""
     dh = 64
     g = torch.Generator(device="cuda").manual_seed(nseq * T + H)
     qkv = (1.5 * torch.randn(nseq * T, 3 * H * dh, device="cuda", generator=g)).bfloat16()
     do = torch.randn(nseq * T, H * dh, device="cuda", generator=g).bfloat16()
     o, lse = B.attention_fwd(qkv, nseq, T, H)
-    ref = _attention64(qkv, do, nseq, T, H, dh)[2]
-    got = B.attention_bwd(qkv, o, lse, do, nseq, T, H)
-    plain = B.attention_bwd(qkv, o, lse, do, nseq, T, H, use_tensor_cores=False)
+    out = (o, lse, B.attention_bwd(qkv, o, lse, do, nseq, T, H))
+    plain_o, plain_lse = B.attention_fwd(qkv, nseq, T, H, use_tensor_cores=False)
+    plain = (plain_o, plain_lse, B.attention_bwd(qkv, plain_o, plain_lse, do, nseq, T, H, use_tensor_cores=False))
     assert B.library_status() == 0
-    assert _norm_err(got, ref) <= min(1.02 * _norm_err(plain, ref) + 2e-6, 4e-3)
-    assert torch.equal(got, B.attention_bwd(qkv, o, lse, do, nseq, T, H))
+    for got, other, ref, bound, most in zip(out, plain, _attention64(qkv, do, nseq, T, H, dh), (2e-6, 2.0 ** -24, 2e-6), (4e-3, 1e-6, 4e-3)):
+        assert _norm_err(got, ref) <= min(1.02 * _norm_err(other, ref) + bound, most)
+    again = B.attention_fwd(qkv, nseq, T, H)
+    assert torch.equal(o, again[0]) and torch.equal(lse, again[1]) and torch.equal(out[2], B.attention_bwd(qkv, o, lse, do, nseq, T, H))
 
 
 @pytest.mark.parametrize("nseq,T,H", [(64, 64, 16), (26, 192, 8), (8, 64, 64), (2, 192, 8)])
