@@ -8,10 +8,10 @@
 //     hold P and dS in fp32, so here each of them enters its product as a sum of two bf16 values (hi + lo, 16
 //     mantissa bits) against the exact bf16 operand: twice the products of that operand, none of the precision
 //     lost (error of o / dqkv against 64 bits over odd T is that of the bf16 output alone, as before).  Measured,
-//     16 sequences of 777 tokens, 12 heads of 64, forward + backward: 466 us against 72.9 ms.  Bound by the
-//     tensor issue of mma.sync and by ldmatrix traffic (the hi and lo products share one fragment of the right
-//     operand).  Shapes that the aligned forms take stay with them; the backward pass of most of those of width 64
-//     runs on tcgen05 (attention_t5_ragged.cu).
+//     16 sequences of 777 tokens, 12 heads of 64, forward + backward: 466 us against 72.9 ms; width 64 now runs on
+//     tcgen05 from the lengths and tile counts on that the two dispatches below give (200 us, attention_t5_ragged.cu).
+//     Bound by the tensor issue of mma.sync and by ldmatrix traffic (the hi and lo products share one fragment of the
+//     right operand).  Shapes that the aligned forms take stay with them.
 //   forward : one CTA per (sequence, head, 64-row query tile), 4 warps x 16 rows, K/V tiles double
 //             buffered in shared memory with cp.async, online softmax in registers.
 //   backward: rowdot = sum(dO*O); a dQ kernel per query tile (loops over key tiles) and a dK/dV

@@ -110,8 +110,8 @@ cudaError_t attention_fwd_tc(const void* qkv, int nseq, int T, int H, int d, voi
 cudaError_t attention_bwd_tc(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq,
                              int T, int H, int d, void* dqkv, float* rowdot, int* status, cudaStream_t st);
 
-// mma.sync attention for the remaining bf16 shapes: any T, head widths that are multiples of 8; P and dS kept to
-// 16 mantissa bits (attention_tc.cu).  Pointers that a direction does not use may be null.
+// Attention for the remaining bf16 shapes: any T, head widths that are multiples of 8; P and dS kept to 16 mantissa
+// bits (mma.sync in attention_tc.cu, or the tcgen05 form below by the rules there).  Pointers that a direction does not use may be null.
 bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const void* qkv, const void* o, const void* d_o,
                                 const void* dqkv);
 cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, int* status, cudaStream_t st);
