@@ -41,7 +41,7 @@ inline unsigned chain_attribute(cudaLaunchAttribute* at, unsigned n) {
 
 // kernel<<<grid, block, smem, st>>>(args...), starting early where the chain allows.  Most of a round over few
 // tokens is launches of 3-6 us each, of which the gap to the kernel before and the set-up were 1.5-2 us: a
-// GPT-2-medium-shaped round of 512 tokens 4.88 -> 3.81 ms (586 launches then, 490 now).
+// GPT-2-medium-shaped round of 512 tokens 4.88 -> 3.81 ms (586 launches then).
 template <typename... Params, typename... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
