@@ -257,9 +257,8 @@ int splitlora_aggregate_broadcast(splitlora_ctx* ctx);
 int splitlora_loss_device(splitlora_ctx* ctx, const float** loss_dev);
 
 const char* splitlora_last_error(const splitlora_ctx* ctx);
-/* The stand-alone operators below that take no status word (attention, adapter gradients inside
- * lora_linear_bwd without a workspace word) record an expired bounded wait in a word the library keeps
- * per device.  This call synchronises the current device, copies that word to *code (HOST) and
+/* The stand-alone operators below that take no status word (attention, the LoRA linear layer) record an
+ * expired bounded wait in a word the library keeps per device.  This call synchronises the current device, copies that word to *code (HOST) and
  * returns SPLITLORA_ERR_TIMEOUT when it is non-zero, else SPLITLORA_OK.  The kernels of a context
  * report through splitlora_device_status instead. */
 int splitlora_library_status(int32_t* code);

@@ -19,7 +19,6 @@ inline int64_t adapter_copy_vectors(const AdapterCopyArgs& a) {
 template <typename T>
 __device__ __forceinline__ void write_copy_vector(const AdapterCopyArgs& a, int64_t idx, int64_t total) {
   constexpr int N = Vec16<T>::N;
-  if (idx == 0 && a.status) *a.status = 0;
   if (idx >= total) return;
   const int64_t nA = (int64_t)a.ext * a.d_in / N, nB = (int64_t)a.ext * a.d_out / N;
   const int64_t per_g = (a.Acat ? nA : 0) + (a.AcatT ? nA : 0) + (a.Bext ? nB : 0) + (a.BextT ? nB : 0);

@@ -143,7 +143,6 @@ struct AdapterCopyArgs {
   void *Acat = nullptr, *AcatT = nullptr, *Bext = nullptr, *BextT = nullptr;   // any of them may be null (skipped)
   int layers = 1;                      // of layers further on: masters layer_stride, Acat / AcatT acat_ls, Bext / BextT bext_ls elements apart
   int64_t layer_stride = 0, acat_ls = 0, bext_ls = 0;
-  int* status = nullptr;               // write_adapter_copies: a word to clear
 };
 // Rank-r projection of the LoRA path, bf16 (lora_proj.cu): Y[M, ext] = X[M, K] W_g[ext, K]^T where only columns
 // t*rp + j, j < r, t < nt of W and Y are used (the others of Y become zero).  W of group g = row / rows_per_group at

@@ -16,7 +16,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 struct LinearPlan {
   int rp, ext;
-  size_t off_acat, off_acatT, off_bext, off_bextT, off_h, off_dh, off_scratch, off_status, total, scratch_floats;
+  size_t off_acat, off_acatT, off_bext, off_bextT, off_h, off_dh, off_scratch, total, scratch_floats;
 };
 
 LinearPlan plan_linear(int dtype, int M, int n_in, int n_out, int r, int G) {
@@ -26,7 +26,6 @@ LinearPlan plan_linear(int dtype, int M, int n_in, int n_out, int r, int G) {
   p.ext = (int)align_up((size_t)p.rp, EXT_BLOCK);
   size_t off = 0;
   auto take = [&](size_t bytes) { off = align_up(off, 256); size_t o = off; off += bytes; return o; };
-  p.off_status = take(256);
   p.off_acat = take((size_t)G * p.ext * n_in * es);
   p.off_acatT = take((size_t)G * n_in * p.ext * es);
   p.off_bext = take((size_t)G * n_out * p.ext * es);
@@ -82,6 +81,9 @@ int splitlora_lora_linear_workspace_bytes(int dtype, int M, int n_in, int n_out,
   return SPLITLORA_OK;
 }
 
+// The layer's kernels report an expired wait to the library's word, which no launch clears: a word of the workspace would
+// have to be cleared first, and the first launch of a call (copies and projection) already has workers that may report to it.
+
 // The compute copies of one direction: Acat and Bext (forward), Acat, AcatT and BextT (backward).
 static AdapterCopyArgs copy_args(int dtype, const LinearPlan& p, const float* A, const float* B, float alpha, int n_in,
                                  int n_out, int r, int G, char* ws, bool fwd) {
@@ -93,14 +95,13 @@ static AdapterCopyArgs copy_args(int dtype, const LinearPlan& p, const float* A,
   a.scale = alpha / (float)r;
   a.Acat = ws + p.off_acat; a.AcatT = fwd ? nullptr : ws + p.off_acatT;
   a.Bext = fwd ? ws + p.off_bext : nullptr; a.BextT = fwd ? nullptr : ws + p.off_bextT;
-  a.status = (int*)(ws + p.off_status);
   return a;
 }
 // The copies, and h = x A_g^T where `project`: one launch where the projection can take A as it is, else two.
-static cudaError_t copies_and_h(int use_tc, AdapterCopyArgs a, bool project, const LinearPlan& p, const void* x, int M, char* ws, cudaStream_t st) {
+static cudaError_t copies_and_h(int use_tc, AdapterCopyArgs a, bool project, const LinearPlan& p, const void* x, int M, char* ws, int* status, cudaStream_t st) {
   // (16384 rows: 16.5 us as one launch, 10.6 + 4.8 as two)
   if (project && use_tc && M <= LORA_PROJ_ROWS && a.dtype == DT_BF16 && (reinterpret_cast<uintptr_t>(a.A) & 15u) == 0) {
-    ProjArgs h = proj_args(p, x, a.d_in, a.A, ws + p.off_h, M, a.r, a.G, a.status);
+    ProjArgs h = proj_args(p, x, a.d_in, a.A, ws + p.off_h, M, a.r, a.G, status);
     if (a.G > 1) h.w_group_stride = a.a_gs;
     if (lora_proj_supported(h)) {
       a.Acat = nullptr;                        // nothing else reads it
@@ -109,7 +110,7 @@ static cudaError_t copies_and_h(int use_tc, AdapterCopyArgs a, bool project, con
   }
   cudaError_t e = write_adapter_copies(a, st);
   if (e != cudaSuccess || !project) return e;
-  return run_proj(use_tc, a.dtype, p, x, a.d_in, ws + p.off_acat, ws + p.off_h, M, a.r, a.G, a.status, st);
+  return run_proj(use_tc, a.dtype, p, x, a.d_in, ws + p.off_acat, ws + p.off_h, M, a.r, a.G, status, st);
 }
 
 int splitlora_lora_linear_fwd(int dtype, int use_tc, const void* x, const void* W, const void* bias, const float* A,
@@ -133,11 +134,11 @@ int splitlora_lora_linear_fwd_parts(int dtype, int use_tc, const void* x, const 
   if (workspace_bytes < p.total) return SPLITLORA_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  if (gemm_tc_init() != 0) return SPLITLORA_ERR_CUDA;
+  int* status = library_status_word();
+  if (gemm_tc_init() != 0 || !status) return SPLITLORA_ERR_CUDA;
   const int rpg = G > 1 ? M / G : 0;
-  int* status = (int*)(ws + p.off_status);
   if (parts & 1) {
-    if (copies_and_h(use_tc, copy_args(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, true), true, p, x, M, ws, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
+    if (copies_and_h(use_tc, copy_args(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, true), true, p, x, M, ws, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   }
   if (!(parts & 2)) return SPLITLORA_OK;
   GemmArgs a;
@@ -170,11 +171,11 @@ int splitlora_lora_linear_bwd_parts(int dtype, int use_tc, const void* x, const 
   if (workspace_bytes < p.total) return SPLITLORA_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  if (gemm_tc_init() != 0) return SPLITLORA_ERR_CUDA;
+  int* status = library_status_word();
+  if (gemm_tc_init() != 0 || !status) return SPLITLORA_ERR_CUDA;
   // h = x A_g^T is recomputed here; the training runtime keeps it from the forward pass
-  if (copies_and_h(use_tc, copy_args(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, false), parts & 1, p, x, M, ws, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
+  if (copies_and_h(use_tc, copy_args(dtype, p, A, B, alpha, n_in, n_out, r, G, ws, false), parts & 1, p, x, M, ws, status, st) != cudaSuccess) return SPLITLORA_ERR_CUDA;
   const int rpg = G > 1 ? M / G : 0;
-  int* status = (int*)(ws + p.off_status);
   const float s = alpha / (float)r;
   if (parts & 1) {
     // dh = s dy B_g

@@ -5,6 +5,7 @@ import os
 import re
 
 import numpy as np
+import pytest
 
 from paper_2407_00952_b200 import binding as B
 from paper_2407_00952_b200 import build, synth
@@ -69,6 +70,20 @@ def test_workspace_plan_scales_with_the_configuration():
     bad = B.config_from_workload(synth.WORKLOADS[1])
     bad.lora_r = 65
     assert lib.splitlora_workspace_bytes(ctypes.byref(bad), ctypes.byref(ctypes.c_size_t(0))) == -1
+
+
+@pytest.mark.parametrize("dtype,es", [(B.DTYPE_FP32, 4), (B.DTYPE_BF16, 2)])
+def test_lora_linear_workspace_holds_operands_only(dtype, es):
+    """The workspace of the stand-alone layer is uninitialised memory, so a status word in it would have to be cleared by
+    a launch before the first one that may report to it; the layer reports to the library's own word, which nothing clears."""
+    M, n_in, n_out, r, G = 1024, 768, 2304, 6, 2
+    ext = 64                                                    # 6 padded to 16, to one contraction block
+    copies = 2 * G * ext * (n_in + n_out) * es                  # A and B and their transposes
+    projections = 2 * M * ext * es                              # h and dh
+    partial = M // 128 * r * n_out * 4                          # a chunk of 128 rows each, of the wider gradient
+    n = ctypes.c_size_t(0)
+    assert B.load().splitlora_lora_linear_workspace_bytes(dtype, M, n_in, n_out, r, G, ctypes.byref(n)) == 0
+    assert n.value == copies + projections + partial
 
 
 def test_generators_are_seeded_and_shaped():
