@@ -301,6 +301,28 @@ __device__ __forceinline__ void dq_block(const T* __restrict__ qkv, const T* __r
   }
 }
 
+// sum of a[c] * b[c], added up as dq_block's warp adds its D: 32 strided sums of NF products, then halves upon halves (D of
+// both gradients is the same number, and that of the form with a kernel for each; one chain is up to 1.6 % more error in dK)
+template <int NF> __device__ __forceinline__ float row_product(const float* a, const float* b, int dh) {
+  float half[16];
+#pragma unroll
+  for (int l = 0; l < 16; ++l) {
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int c = 0; c < NF; ++c) {
+      const int c0 = l + 32 * c, c1 = c0 + 16;
+      if (c0 < dh) s0 = fmaf(a[c0], b[c0], s0);
+      if (c1 < dh) s1 = fmaf(a[c1], b[c1], s1);
+    }
+    half[l] = s0 + s1;
+  }
+#pragma unroll
+  for (int n = 8; n > 0; n >>= 1)
+#pragma unroll
+    for (int l = 0; l < n; ++l) half[l] += half[l + n];
+  return half[0];
+}
+
 // dK, dV: rows are keys, tiles are queries.  OWN_D: D = sum(dO * O) of a tile's queries is formed here, one query per lane,
 // from the staged dO and one more tile, of O (behind the others in shared memory).
 template <typename T, int NF, bool OWN_D>
@@ -354,10 +376,7 @@ __device__ __forceinline__ void dkv_block(const T* __restrict__ qkv, const T* __
     float Di = D;
     __syncthreads();
     if (AHEAD<NF> && i0 + KT < Tn) ask(i0 + KT);
-    if (OWN_D) {
-      Di = 0.f;
-      for (int c = 0; c < dh; ++c) Di = fmaf(o_s[lane * t.lt + c], t.b[lane * t.lt + c], Di);
-    }
+    if (OWN_D) Di = row_product<NF>(o_s + lane * t.lt, t.b + lane * t.lt, dh);
     const int i = i0 + lane;
     float s[RPW], dp[RPW];
     dot4(krows, t.lr, t.a + lane * t.lt, s);

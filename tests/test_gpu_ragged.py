@@ -250,6 +250,20 @@ def test_rank_projections_of_every_shape(M, n_in, n_out, r, G):
     test_lora_linear_any_size(M, n_in, n_out, r, G)
 
 
+@pytest.mark.parametrize("T,H,dh", [(64, 4, 32), (100, 4, 64), (37, 3, 40), (200, 2, 128), (65, 2, 96), (50, 2, 5)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_plain_attention_backward_does_not_depend_on_the_batch(T, H, dh, dtype):
+    """Few blocks take both gradients in one launch, many a kernel for each: a sequence's gradients are the same bits."""
+    few, many = 1, 200
+    g = torch.Generator(device="cuda").manual_seed(T + dh)
+    qkv = torch.randn(many * T, 3 * H * dh, device="cuda", generator=g).to(dtype)
+    do = torch.randn(many * T, H * dh, device="cuda", generator=g).to(dtype)
+    o, lse = B.attention_fwd(qkv, many, T, H, use_tensor_cores=False)
+    n = few * T
+    part = B.attention_bwd(qkv[:n], o[:n].contiguous(), lse[:few].contiguous(), do[:n], few, T, H, use_tensor_cores=False)
+    assert torch.equal(part, B.attention_bwd(qkv, o, lse, do, many, T, H, use_tensor_cores=False)[:n])
+
+
 @pytest.mark.parametrize("M,K,N", [(1, 8, 8), (512, 128, 64), (512, 512, 128), (100, 520, 128), (77, 1000, 40), (512, 128, 384), (1200, 72, 1000)])
 def test_linear_fp32_tiles(M, K, N):
     """Few to many tiles, with the contraction over one, four, eight and sixteen thread groups: roundings of random sign, one
