@@ -34,8 +34,8 @@ struct LayerBuf {
   float *mean1 = nullptr, *rstd1 = nullptr, *mean2 = nullptr, *rstd2 = nullptr, *lse = nullptr;
   const void* x_in = nullptr;     // base (row 0) of the buffer the block read its input from
   void* hcat_o = nullptr;         // down-projected input of an adapter on the attention output projection
-  // gradients the adapter gradients are formed from: buffers of the layer's own where those wait for the end of the pass
-  // (splitlora_ctx::defer_grads), else the same for all layers
+  // gradients the adapter gradients are formed from: the same buffers for all layers, or, where the adapter gradients wait
+  // for the end of the pass (splitlora_ctx::defer_grads), the layer's own, in place of activations that are dead by then
   void *dqkv = nullptr, *dhcat = nullptr, *dxmid = nullptr, *dhcat_o = nullptr;
   // Adapter compute copies of this layer: `cl` holds one set per client, stacked (blocks the clients
   // run), `sv` the server's single set (blocks the server runs).  A block between the shallowest and the
@@ -88,6 +88,7 @@ struct splitlora_ctx {
   float scale = 1.f;
   bool tc = false;
   bool defer_grads = false;   // adapter gradients of all layers of a side in one launch (see derive)
+  size_t act_stride = 0;      // bytes from a layer's z, x_out and x_mid, in this order, to the next layer's
   // frozen
   const void *wte = nullptr, *wpe = nullptr, *lnfg = nullptr, *lnfb = nullptr, *headw = nullptr;
   void* wteT = nullptr;       // transposed head [d, Vpad]
@@ -106,6 +107,8 @@ struct splitlora_ctx {
   float *meanf = nullptr, *rstdf = nullptr, *row_loss = nullptr, *rowdot = nullptr, *loss_dev = nullptr,
         *grad_scratch = nullptr;
   size_t grad_scratch_floats = 0;
+  float* defer_scratch = nullptr;   // scratch of the adapter gradients of a side: temporaries that no later step reads
+  size_t defer_scratch_floats = 0;
   int *n_valid = nullptr, *status = nullptr;
   void *g_a = nullptr, *g_b = nullptr, *g_dz = nullptr, *g_du2 = nullptr, *g_do = nullptr,
        *g_du = nullptr;
@@ -182,30 +185,33 @@ int grad_jobs(const splitlora_ctx* c, const LayerBuf& b, float* out, int64_t gro
   const int d = c->d;
   const size_t es = c->es, M = c->M;
   auto stride = [&](size_t cols) { return (int64_t)(align_up(M * cols * es, 256) / es); };
+  const int64_t g_ls = (int64_t)(c->act_stride / es);            // of dqkv, dh, dx_mid and dh_o
   int n = 0;
-  auto job = [&](const void* Z, int64_t ldz, int zcol0, int64_t z_ls, const void* Wt, int ext, int wcol0, int nt, float scale, float* o) -> LoraGradJob& {
+  auto job = [&](const void* Z, int64_t ldz, int zcol0, int64_t z_ls, const void* Wt, int64_t wt_ls, int ext, int wcol0, int nt, float scale, float* o) -> LoraGradJob& {
     LoraGradJob& j = jobs[n++];
     j.Z = Z; j.ldz = ldz; j.zcol0 = zcol0; j.C = d; j.Wt = Wt; j.ldwt = ext; j.wcol0 = wcol0; j.r = c->r; j.rp = c->rp; j.nt = nt;
     j.scale = scale; j.out = o; j.out_group_stride = group_stride; j.out_target_stride = (int64_t)2 * c->r * d;
-    j.z_ls = z_ls; j.wt_ls = stride(ext); j.out_ls = c->per_layer;
+    j.z_ls = z_ls; j.wt_ls = wt_ls; j.out_ls = c->per_layer;
     return j;
   };
   auto gA = [&](LoraGradJob& j) { j.out_sj = d; j.out_sc = 1; };
   auto gB = [&](LoraGradJob& j) { j.out_sj = 1; j.out_sc = c->r; };
-  gA(job(b.u, d, 0, stride(d), b.dhcat, c->ext, 0, c->nq, 1.0f, out));
+  gA(job(b.u, d, 0, stride(d), b.dhcat, g_ls, c->ext, 0, c->nq, 1.0f, out));
   for (int t = 0; t < c->nq; ++t)
-    gB(job(b.dqkv, 3 * d, c->slice_idx[t] * d, stride(3 * (size_t)d), b.hcat, c->ext, t * c->rp, 1, c->scale, out + (size_t)t * 2 * c->r * d + (size_t)c->r * d));
+    gB(job(b.dqkv, 3 * d, c->slice_idx[t] * d, g_ls, b.hcat, stride(c->ext), c->ext, t * c->rp, 1, c->scale, out + (size_t)t * 2 * c->r * d + (size_t)c->r * d));
   if (c->has_o) {
     float* o = out + (size_t)c->nq * 2 * c->r * d;
-    gA(job(b.o, d, 0, stride(d), b.dhcat_o, c->ext_o, 0, 1, 1.0f, o));
-    gB(job(b.dxmid, d, 0, stride(d), b.hcat_o, c->ext_o, 0, 1, c->scale, o + (size_t)c->r * d));
+    gA(job(b.o, d, 0, stride(d), b.dhcat_o, g_ls, c->ext_o, 0, 1, 1.0f, o));
+    gB(job(b.dxmid, d, 0, g_ls, b.hcat_o, stride(c->ext_o), c->ext_o, 0, 1, c->scale, o + (size_t)c->r * d));
   }
   return n;
 }
 
 // Up to this many token rows the adapter gradients of all layers of a side are formed together at the end of its backward
 // pass: at 512 rows a layer's pair of launches is 10 us of a chain, and nothing waits for its results but the optimizer.
-// Beyond, their cost is the traffic either way, and the layers' gradients (4 d values per row and layer) would have to be kept.
+// Beyond, their cost is the traffic either way.  The layers' gradients (3-4 d values per row and layer) take the place of the
+// layer's own z, x_out and x_mid, which its backward pass has read by the time they are written, and the partial sums that
+// of the logits and the MLP's temporaries: the workspace is no larger than with a pair of launches per layer.
 constexpr int DEFER_ROWS = 4096;
 constexpr size_t DEFER_SCRATCH_FLOATS = 16u << 20;
 
@@ -236,9 +242,12 @@ void derive(splitlora_ctx* c) {
   c->Pc = c->per_layer * c->cut;
   c->Ps = c->per_layer * (c->L - c->cmin);
   c->tc = (g.dtype == SPLITLORA_DTYPE_BF16) && g.use_tensor_cores != 0;
+  auto rows = [&](size_t cols) { return align_up((size_t)c->M * cols * c->es, 256); };
+  c->act_stride = rows(c->Fz) + 2 * rows(c->d);
+  const size_t kept = rows(3 * (size_t)c->d) + rows(c->ext) + (c->has_o ? rows(c->d) + rows(c->ext_o) : 0);     // plan
   LoraGradJob jobs[LORA_GRAD_MAX_JOBS];
   const int n = grad_jobs(c, LayerBuf(), nullptr, 0, jobs);       // (the workspace's buffers are aligned: no addresses needed)
-  c->defer_grads = c->M <= DEFER_ROWS && c->cmin == c->cut && lora_grad_layers_supported(c->dt, jobs, n, c->L, c->M, c->K > 1 ? c->rows_per_client : 0, c->tc);
+  c->defer_grads = c->M <= DEFER_ROWS && c->cmin == c->cut && kept <= c->act_stride && lora_grad_layers_supported(c->dt, jobs, n, c->L, c->M, c->K > 1 ? c->rows_per_client : 0, c->tc);
 }
 
 // Lays out the workspace.  With ws == nullptr only the size is computed.
@@ -277,22 +286,41 @@ size_t plan(splitlora_ctx* c, char* ws) {
       take(&LayerBuf::Copies::BextO, G * d * ext_o); take(&LayerBuf::Copies::BextOT, G * ext_o * d);
     }
   }
-  auto take_layers = [&](void* LayerBuf::*kind, size_t cols, bool each = true) {      // each: one per layer, at one stride
-    const size_t stride = align_up(M * cols * es, 256);
-    char* p = (char*)a.take(stride * (size_t)(each ? c->L : 1));
-    for (int l = 0; l < c->L; ++l) c->lb[l].*kind = p + (each ? stride * (size_t)l : 0);
+  auto rows = [&](size_t cols) { return align_up(M * cols * es, 256); };
+  auto take_layers = [&](void* LayerBuf::*kind, size_t cols) {      // one per layer, at one stride
+    char* p = (char*)a.take(rows(cols) * (size_t)c->L);
+    for (int l = 0; l < c->L; ++l) c->lb[l].*kind = p + rows(cols) * (size_t)l;
   };
   take_layers(&LayerBuf::u, d); take_layers(&LayerBuf::hcat, ext); take_layers(&LayerBuf::o, d);
-  take_layers(&LayerBuf::dqkv, 3 * d, c->defer_grads); take_layers(&LayerBuf::dhcat, ext, c->defer_grads);
-  take_layers(&LayerBuf::dxmid, d, c->defer_grads && c->has_o);
-  if (c->has_o) { take_layers(&LayerBuf::hcat_o, ext_o); take_layers(&LayerBuf::dhcat_o, ext_o, c->defer_grads); }
+  if (c->has_o) take_layers(&LayerBuf::hcat_o, ext_o);
+  char* acts = (char*)a.take(c->act_stride * (size_t)c->L);
+  for (int l = 0; l < c->L; ++l) {
+    LayerBuf& b = c->lb[l];
+    char* z = acts + c->act_stride * (size_t)l;
+    b.z = z; b.x_out = z + rows(Fz); b.x_mid = z + rows(Fz) + rows(d);
+    if (!c->defer_grads) continue;
+    // dx_mid comes first, within z and x_out, because the launch that writes it reads x_mid; all others are written later
+    char* g = z;
+    if (c->has_o) { b.dxmid = g; g += rows(d); }
+    b.dqkv = g; g += rows(3 * d);
+    b.dhcat = g; g += rows(ext);
+    if (c->has_o) b.dhcat_o = g;
+  }
+  auto take_shared = [&](void* LayerBuf::*kind, size_t cols) {
+    void* p = a.take(M * cols * es);
+    for (LayerBuf& b : c->lb) b.*kind = p;
+  };
+  if (!c->defer_grads || !c->has_o) take_shared(&LayerBuf::dxmid, d);
+  if (!c->defer_grads) {
+    take_shared(&LayerBuf::dqkv, 3 * d); take_shared(&LayerBuf::dhcat, ext);
+    if (c->has_o) take_shared(&LayerBuf::dhcat_o, ext_o);
+  }
   for (int l = 0; l < c->L; ++l) {
     FrozenLayer& f = c->fl[l];
     f.qkvwT = a.take(3 * d * d * es); f.projwT = a.take(d * d * es);
     f.fc1wT = a.take(Fz * d * es); f.fc2wT = a.take(d * F * es);
     LayerBuf& b = c->lb[l];
-    b.qkv = a.take(M * 3 * d * es); b.x_mid = a.take(M * d * es); b.z = a.take(M * Fz * es);
-    b.x_out = a.take(M * d * es);
+    b.qkv = a.take(M * 3 * d * es);
     b.mean1 = (float*)a.take(M * 4); b.rstd1 = (float*)a.take(M * 4);
     b.mean2 = (float*)a.take(M * 4); b.rstd2 = (float*)a.take(M * 4);
     b.lse = (float*)a.take((size_t)c->nseq * c->cfg.n_head * c->cfg.seq * 4);
@@ -303,13 +331,16 @@ size_t plan(splitlora_ctx* c, char* ws) {
   c->meanf = (float*)a.take(M * 4); c->rstdf = (float*)a.take(M * 4); c->row_loss = (float*)a.take(M * 4);
   c->rowdot = (float*)a.take((size_t)c->nseq * c->cfg.n_head * c->cfg.seq * 4);
   c->grad_scratch_floats = lora_grad_scratch_floats(c->M > 256 ? c->M : 256, c->nq * c->r, c->d);   // room for a layer's jobs as one batch
-  if (c->defer_grads) {                         // eight chunks per group of a side, at most 64 MiB
-    const size_t groups = (size_t)c->K * c->cut > (size_t)(c->L - c->cmin) ? (size_t)c->K * c->cut : (size_t)(c->L - c->cmin);
-    const size_t want = 8 * groups * (size_t)c->per_layer;
-    const size_t most = want < DEFER_SCRATCH_FLOATS ? want : DEFER_SCRATCH_FLOATS;
-    if (c->grad_scratch_floats < most) c->grad_scratch_floats = most;
-  }
   c->grad_scratch = (float*)a.take(c->grad_scratch_floats * 4);
+  c->defer_scratch = c->grad_scratch; c->defer_scratch_floats = c->grad_scratch_floats;
+  if (c->defer_grads) {                         // eight chunks per group of a side, at most 64 MiB, as far as there is room
+    const size_t groups = (size_t)c->K * c->cut > (size_t)(c->L - c->cmin) ? (size_t)c->K * c->cut : (size_t)(c->L - c->cmin);
+    size_t want = 8 * groups * (size_t)c->per_layer;
+    want = want < DEFER_SCRATCH_FLOATS ? want : DEFER_SCRATCH_FLOATS;
+    const size_t room = (size_t)((char*)c->logits - (char*)c->u2) / 4 + M * (size_t)c->Vpad * es / 4;   // u2, act, xf, logits
+    want = want < room ? want : room;
+    if (c->defer_scratch_floats < want) { c->defer_scratch = (float*)c->u2; c->defer_scratch_floats = want; }
+  }
   c->g_a = a.take(M * d * es); c->g_b = a.take(M * d * es); c->g_dz = a.take(M * Fz * es);
   c->g_du2 = a.take(M * d * es); c->g_do = a.take(M * d * es);
   c->g_du = a.take(M * d * es);
@@ -679,7 +710,7 @@ cudaError_t deferred_gradients(splitlora_ctx* c, bool client) {
   LoraGradJob jobs[LORA_GRAD_MAX_JOBS];
   const int n = grad_jobs(c, c->lb[l0], client ? c->cg : c->sg, client ? c->Pc : 0, jobs);
   Scope s(c, "lora_grad");
-  return lora_grad_layers(c->dt, jobs, n, l1 - l0, c->M, client ? c->rows_per_client : 0, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc);
+  return lora_grad_layers(c->dt, jobs, n, l1 - l0, c->M, client ? c->rows_per_client : 0, c->defer_scratch, c->defer_scratch_floats, c->st, c->status, c->tc);
 }
 
 cudaError_t run_optimizer(splitlora_ctx* c, bool client) {

@@ -86,6 +86,20 @@ def test_lora_linear_workspace_holds_operands_only(dtype, es):
     assert n.value == copies + projections + partial
 
 
+@pytest.mark.parametrize("idx,targets", [(3, "qv"), (3, "qvo"), (5, "qkvo"), (1, "qv")])
+def test_workspace_grows_with_the_rows(idx, targets):
+    """No row count takes more memory than a larger one: the adapter gradients that wait for the end of a pass (up to 4096
+    rows) keep what they need in place of activations that have been read."""
+    lib, sizes = B.load(), []
+    for T in (512, 4088, 4096, 4104, 8192):
+        w = synth.scaled(synth.WORKLOADS[idx], n_clients=1, batch_per_client=1, seq=T, max_seq=T, targets=tuple(targets))
+        cfg = B.config_from_workload(w)
+        n = ctypes.c_size_t(0)
+        assert lib.splitlora_workspace_bytes(ctypes.byref(cfg), ctypes.byref(n)) == 0
+        sizes.append(n.value)
+    assert sizes == sorted(sizes)
+
+
 def test_generators_are_seeded_and_shaped():
     w = synth.WORKLOADS[1]
     a, b = synth.make_frozen(w), synth.make_frozen(w)
