@@ -11,7 +11,10 @@
 // half-steps are in flight next to dK and dV: the score products of one, the element-wise work of another, the
 // accumulating products of the third.
 // A row whose results are not all finite is done again in plain FMA over its visible pairs (attention_rows.cuh), because a
-// product multiplies the zero probability of a hidden pair with whatever the tile holds.
+// product multiplies the zero probability of a hidden pair with whatever the tile holds.  (Template KEEP; not backward at
+// multiples of 128, where the other form spoils its tiles of 128 rows too.  Odd multiples of 64 used to run in tiles of 64 rows
+// and spoil those: keeping the values apart costs 128 sequences of 192, 12 heads 122 -> 129 us, 16 of 960
+// 146 -> 147, 8 of 192 with 8 heads 15.0 -> 15.6; in tiles of 64 on mma.sync that one took 23.)
 // What bounds them: neither unit by itself.  A half-step is 10 + 16 (dQ: 10 + 8) products [128 x 64 x 16] of 45-48 cycles
 // (operand reads from shared memory) next to 512 cycles of exponentials; 16 sequences of 777 tokens, 12 heads, have 80 us of
 // products and take 123 us (mma.sync, attention_tc.cu: 339), the tensor pipe active for 36 % (dQ) and 43 % of the cycles.  With P
@@ -243,7 +246,7 @@ static_assert(SMEM <= 232448, "");
 
 // OWN_D: D is not in `rowdot` yet; the output warps, idle until the accumulators are complete, compute it for every step from
 // the staged dO rows and the rows of O in global memory, and write the operand rows in the statistics warp's place.
-template <bool HILO, bool OWN_D>
+template <bool HILO, bool KEEP, bool OWN_D>
 __device__ __forceinline__ void dkv_tiles(const CUtensorMap& mapQKV, const CUtensorMap& mapDO, const CUtensorMap& mapDQKV, const Params& p, int cta, int grid) {
   using namespace dkv;
   RG_SETUP(N_BARS, count<OWN_D>, TMEM_COLS)
@@ -477,8 +480,8 @@ __device__ __forceinline__ void dkv_tiles(const CUtensorMap& mapQKV, const CUten
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       }
-      bool redo = false;                         // only the lengths off the tile sizes keep such values to the pairs that see them
-      if constexpr (HILO) redo = out_warps_any(bad); else out_warps_sync();
+      bool redo = false;
+      if constexpr (KEEP) redo = out_warps_any(bad); else out_warps_sync();
       if (redo) {
         if (storer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         out_warps_sync();
@@ -527,7 +530,7 @@ constexpr int SMEM = OFF_BAR + 8 * N_BARS + 16 + 1024;
 static_assert(SMEM <= 232448, "");
 }  // namespace dq
 
-template <bool HILO>
+template <bool HILO, bool KEEP>
 __device__ __forceinline__ void dq_tiles(const CUtensorMap& mapQKV, const CUtensorMap& mapDO, const CUtensorMap& mapO, const CUtensorMap& mapDQKV,
                                          const Params& p, int cta, int grid) {
   using namespace dq;
@@ -740,8 +743,8 @@ __device__ __forceinline__ void dq_tiles(const CUtensorMap& mapQKV, const CUtens
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       }
-      bool redo = false;                         // only the lengths off the tile sizes keep such values to the pairs that see them
-      if constexpr (HILO) redo = out_warps_any(bad); else out_warps_sync();
+      bool redo = false;
+      if constexpr (KEEP) redo = out_warps_any(bad); else out_warps_sync();
       if (redo) {
         if (storer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         out_warps_sync();
@@ -761,26 +764,26 @@ __device__ __forceinline__ void dq_tiles(const CUtensorMap& mapQKV, const CUtens
   RG_TEARDOWN(TMEM_COLS)
 }
 
-template <bool HILO>
+template <bool HILO, bool KEEP>
 __global__ void __launch_bounds__(THREADS_DKV, 1)
 attn64_dkv_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_constant__ CUtensorMap mapDO,
                       const __grid_constant__ CUtensorMap mapDQKV, const __grid_constant__ Params p) {
-  dkv_tiles<HILO, false>(mapQKV, mapDO, mapDQKV, p, (int)blockIdx.x, (int)gridDim.x);
+  dkv_tiles<HILO, KEEP, false>(mapQKV, mapDO, mapDQKV, p, (int)blockIdx.x, (int)gridDim.x);
 }
-template <bool HILO>
+template <bool HILO, bool KEEP>
 __global__ void __launch_bounds__(THREADS_DQ, 1)
 attn64_dq_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_constant__ CUtensorMap mapDO,
                      const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapDQKV, const __grid_constant__ Params p) {
-  dq_tiles<HILO>(mapQKV, mapDO, mapO, mapDQKV, p, (int)blockIdx.x, (int)gridDim.x);
+  dq_tiles<HILO, KEEP>(mapQKV, mapDO, mapO, mapDQKV, p, (int)blockIdx.x, (int)gridDim.x);
 }
 // Few tiles: both at once on their own CTAs.  Each kernel by itself is set-up, first loads and a few steps one after another.
-template <bool HILO>
+template <bool HILO, bool KEEP>
 __global__ void __launch_bounds__(THREADS_DKV, 1)
 attn64_bwd_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_constant__ CUtensorMap mapDO,
                       const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapDQKV, const __grid_constant__ Params p) {
   const int units = p.nitems * p.nq;
-  if ((int)blockIdx.x < units) dkv_tiles<HILO, true>(mapQKV, mapDO, mapDQKV, p, (int)blockIdx.x, units);
-  else dq_tiles<HILO>(mapQKV, mapDO, mapO, mapDQKV, p, (int)blockIdx.x - units, units);
+  if ((int)blockIdx.x < units) dkv_tiles<HILO, KEEP, true>(mapQKV, mapDO, mapDQKV, p, (int)blockIdx.x, units);
+  else dq_tiles<HILO, KEEP>(mapQKV, mapDO, mapO, mapDQKV, p, (int)blockIdx.x - units, units);
 }
 
 // ==========================================================================================
@@ -1074,8 +1077,9 @@ bool init_device() {
   if (!g_once.needed(dev)) return true;
   auto allow = [](const void* kernel, int bytes) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess; };
   if (!allow((const void*)attn_rg_fwd_t5_kernel, fwd::SMEM)) return false;
-  if (!allow((const void*)attn64_bwd_t5_kernel<true>, BWD_SMEM) || !allow((const void*)attn64_dkv_t5_kernel<true>, dkv::SMEM) || !allow((const void*)attn64_dq_t5_kernel<true>, dq::SMEM)) return false;
-  if (!allow((const void*)attn64_bwd_t5_kernel<false>, BWD_SMEM) || !allow((const void*)attn64_dkv_t5_kernel<false>, dkv::SMEM) || !allow((const void*)attn64_dq_t5_kernel<false>, dq::SMEM)) return false;
+  if (!allow((const void*)attn64_bwd_t5_kernel<true, true>, BWD_SMEM) || !allow((const void*)attn64_dkv_t5_kernel<true, true>, dkv::SMEM) || !allow((const void*)attn64_dq_t5_kernel<true, true>, dq::SMEM)) return false;
+  if (!allow((const void*)attn64_bwd_t5_kernel<false, true>, BWD_SMEM) || !allow((const void*)attn64_dkv_t5_kernel<false, true>, dkv::SMEM) || !allow((const void*)attn64_dq_t5_kernel<false, true>, dq::SMEM)) return false;
+  if (!allow((const void*)attn64_bwd_t5_kernel<false, false>, BWD_SMEM) || !allow((const void*)attn64_dkv_t5_kernel<false, false>, dkv::SMEM) || !allow((const void*)attn64_dq_t5_kernel<false, false>, dq::SMEM)) return false;
   g_once.done(dev);
   return true;
 }
@@ -1105,7 +1109,7 @@ bool attention_ragged_t5_supported(int nseq, int T, int H, int d) {
 }
 
 namespace {
-template <bool HILO>
+template <bool HILO, bool KEEP>
 cudaError_t launch_bwd(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H, int d, void* dqkv,
                        float* rowdot, int* status, cudaStream_t st) {
   if (!attention_ragged_t5_supported(nseq, T, H, d)) return cudaErrorInvalidValue;
@@ -1121,24 +1125,24 @@ cudaError_t launch_bwd(const void* qkv, const void* o, const float* lse, const v
   p.lse = lse; p.rowdot = rowdot; p.d_o = (const bf16*)d_o; p.dqkv = (bf16*)dqkv; p.o = (bf16*)const_cast<void*>(o);
   const int units = p.nitems * p.nq;
   if (2 * units <= sms) {
-    launch_overlapped(attn64_bwd_t5_kernel<HILO>, 2 * units, THREADS_DKV, BWD_SMEM, st, mQKV, mDO, mO, mDQKV, p);
+    launch_overlapped(attn64_bwd_t5_kernel<HILO, KEEP>, 2 * units, THREADS_DKV, BWD_SMEM, st, mQKV, mDO, mO, mDQKV, p);
     return cudaGetLastError();
   }
   const int grid = units < sms ? units : sms;
-  launch_overlapped(attn64_dq_t5_kernel<HILO>, grid, THREADS_DQ, dq::SMEM, st, mQKV, mDO, mO, mDQKV, p);
-  launch_overlapped(attn64_dkv_t5_kernel<HILO>, grid, THREADS_DKV, dkv::SMEM, st, mQKV, mDO, mDQKV, p);
+  launch_overlapped(attn64_dq_t5_kernel<HILO, KEEP>, grid, THREADS_DQ, dq::SMEM, st, mQKV, mDO, mO, mDQKV, p);
+  launch_overlapped(attn64_dkv_t5_kernel<HILO, KEEP>, grid, THREADS_DKV, dkv::SMEM, st, mQKV, mDO, mDQKV, p);
   return cudaGetLastError();
 }
 }  // namespace
 
-
 cudaError_t attention_bwd_ragged_t5(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                                     int d, void* dqkv, float* rowdot, int* status, cudaStream_t st) {
-  return launch_bwd<true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
+  return launch_bwd<true, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
 }
 cudaError_t attention_bwd_t5_w64(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                                  int d, void* dqkv, float* rowdot, int* status, cudaStream_t st) {
-  return launch_bwd<false>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
+  return T % BT != 0 ? launch_bwd<false, true>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st)
+                     : launch_bwd<false, false>(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
 }
 
 cudaError_t attention_fwd_ragged_t5(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, int* status, cudaStream_t st) {

@@ -69,3 +69,34 @@ def test_non_finite_values_reach_what_sees_them_only(T, dh, dtype, use_tc, value
             _same(got, want, tol)
     _same(B.attention_bwd(qkv, o, lse, do, nseq, T, H, use_tc), ref[2], tol)
     assert B.library_status() == 0
+
+
+@pytest.mark.parametrize("where", ["q", "k", "v", "do"])
+@pytest.mark.parametrize("value", [math.inf, math.nan])
+@pytest.mark.parametrize("nseq,T,H", [(2, 192, 2), (40, 320, 2)])
+def test_non_finite_values_at_odd_multiples_of_64(nseq, T, H, value, where):
+    """Width 64, backward, both launch forms: lengths whose last tile of 128 rows is half a tile."""
+    _check_backward_in_tiles_of_128(nseq, T, H, value, where)
+
+
+def _check_backward_in_tiles_of_128(nseq, T, H, value, where):
+    """Bad values in the first and the last tile of the first sequence's first head; the sequences behind it as they were."""
+    dh = 64
+    d = H * dh
+    g = torch.Generator(device="cuda").manual_seed(nseq + T + H)
+    qkv = torch.randn(nseq * T, 3 * d, device="cuda", generator=g).bfloat16()
+    do = torch.randn(nseq * T, d, device="cuda", generator=g).bfloat16()
+    o, lse = B.attention_fwd(qkv, nseq, T, H)
+    before = B.attention_bwd(qkv, o, lse, do, nseq, T, H)
+    for pos in (T // 3, T - 1):
+        if where == "do":
+            do[pos, 1] = value
+        else:
+            qkv[pos, "qkv".index(where) * d + 1] = value
+    n = 2                                                      # the reference takes dh times the pairs in memory
+    ref = _reference(qkv[:n * T], o[:n * T], lse[:n], do[:n * T], n, T, H, dh)
+    got = B.attention_bwd(qkv, o, lse, do, nseq, T, H)
+    _same(got[:n * T], ref[2], 1e-2)
+    assert torch.equal(got[T:], before[T:])
+    assert B.library_status() == 0
+    return qkv, ref
