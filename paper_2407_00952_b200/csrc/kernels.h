@@ -158,9 +158,10 @@ struct ProjArgs {
 bool lora_proj_supported(const ProjArgs& a);
 // Rows up to which these kernels beat the linear layers' narrow tiles: (512, 2048 -> 2 x 4 of 32) 8.8 -> 5.5 us from cold
 // caches; 12 of 1665 x 1536 149 -> 104, of 16384 x 1536 225 -> 252, 24 of 32768 x 2048 910 -> 966.  With the norm in front
-// they save a launch and a read of its rows: 25 norms and 12 projections of 16384 x 768 520 -> 500 us, of 1665 x 768 308 ->
-// 226; 49 and 24 of 32768 x 1024 2.12 -> 2.23 ms.
-constexpr int LORA_PROJ_ROWS = 4096, NORM_PROJ_ROWS = 16384;
+// (fused, norm_proj) they save a launch and a read of its rows, which shows in rounds of few rows and costs in those of many,
+// where the two launches overlap: norm and projection apart -> one launch, 8 to 24 blocks, 512 rows of 1024 3068 -> 3058 us, 1665 of 768
+// 2285 -> 2264, 2048 of 768 1653 -> 1643, 4096 and 8192 equal, 12288 of 768 6148 -> 6197, 16384 of 768 8289 -> 8366, of 1024 11795 -> 11873.
+constexpr int LORA_PROJ_ROWS = 4096;
 cudaError_t lora_proj(const ProjArgs& a, cudaStream_t st);
 // The same for one target whose W is the fp32 A [r, K] itself, with the compute copies of write_adapter_copies in the same launch.
 cudaError_t lora_proj_copies(const ProjArgs& a, const AdapterCopyArgs& copies, cudaStream_t st);

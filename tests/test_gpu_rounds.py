@@ -176,3 +176,18 @@ def test_adamw_kernel_on_identical_inputs(step):
             else:
                 sel = np.ones_like(p_ref, dtype=bool)
             assert np.abs(p[part] - p_ref)[sel].max() <= 1e-6 * np.abs(p_ref).max(), (key, part)
+
+
+def _forward_classes(batch):
+    w = synth.scaled(synth.WORKLOADS[2], n_layer=3, cut=1, n_clients=1, counts=(7,), batch_per_client=batch, d_model=256, n_head=4, d_ff=512, vocab=512)
+    frozen, cads, sads, tokens, labels = H.build_case(w)
+    eng = runner.make_engine(w, frozen, cads, sads)
+    eng.profile_enable(True)
+    eng.round(torch.from_numpy(tokens).cuda(), torch.from_numpy(labels).cuda(), [7])
+    return {k: v[0] for k, v in eng.profile_report().items()}
+
+
+def test_many_rows_project_in_launches_of_their_own():
+    """The norm overlaps with the rank-r projection behind it; one launch for both is slower from some 8192 rows on."""
+    n = _forward_classes(batch=17)                                # 8704 rows
+    assert n["layernorm_fwd"] == 2 * 3 + 1 and n["lora_down_fwd"] == 3
