@@ -191,3 +191,8 @@ def test_many_rows_project_in_launches_of_their_own():
     """The norm overlaps with the rank-r projection behind it; one launch for both is slower from some 8192 rows on."""
     n = _forward_classes(batch=17)                                # 8704 rows
     assert n["layernorm_fwd"] == 2 * 3 + 1 and n["lora_down_fwd"] == 3
+
+
+def test_few_rows_name_the_launch_that_does_both():
+    n = _forward_classes(batch=3)
+    assert n["layernorm_fwd"] == 3 + 1 and n["layernorm_lora_down_fwd"] == 3 and "lora_down_fwd" not in n
