@@ -79,6 +79,20 @@ def test_non_finite_values_at_odd_multiples_of_64(nseq, T, H, value, where):
     _check_backward_in_tiles_of_128(nseq, T, H, value, where)
 
 
+@pytest.mark.parametrize("where", ["q", "k", "v", "do"])
+@pytest.mark.parametrize("value", [math.inf, -math.inf, math.nan])
+@pytest.mark.parametrize("nseq,T,H", [(2, 200, 2), (80, 200, 2), (80, 70, 2)])
+def test_non_finite_values_in_tiles_of_128(nseq, T, H, value, where):
+    """Width 64 off the tile sizes, as the kernels with tiles of 128 rows take it: both gradients in one launch (with the
+    forward pass in tiles of 64), a launch for each, sequences of one tile."""
+    qkv, ref = _check_backward_in_tiles_of_128(nseq, T, H, value, where)
+    if where != "do":
+        o, lse = B.attention_fwd(qkv, nseq, T, H)
+        _same(o[:2 * T], ref[0], 1e-2)
+        _same(lse[:2], ref[1], 1e-2)
+        assert B.library_status() == 0
+
+
 def _check_backward_in_tiles_of_128(nseq, T, H, value, where):
     """Bad values in the first and the last tile of the first sequence's first head; the sequences behind it as they were."""
     dh = 64
