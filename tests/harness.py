@@ -102,7 +102,21 @@ def qk_case(name):
     if name == "ranks_medium":
         return (synth.scaled(synth.WORKLOADS[3], n_layer=3, cut=2, n_clients=3, batch_per_client=2, seq=128,
                              max_seq=128), (2, 4, 1), None)
+    if name in RAGGED_ROUNDS:
+        return (synth.scaled(n_clients=1, counts=(7,), vocab=4096, **RAGGED_ROUNDS[name]), None, None)
     raise KeyError(name)
+
+
+# one client, row counts that are multiples of nothing (231 and 1665 rows)
+RAGGED_ROUNDS = {
+    "gpt_3x77": dict(w=synth.WORKLOADS[2], n_layer=4, cut=2, batch_per_client=3, seq=77, max_seq=77),
+    "gpt_5x333_qvo": dict(w=synth.WORKLOADS[2], n_layer=3, cut=1, batch_per_client=5, seq=333, max_seq=333, targets=("q", "v", "o"),
+                          d_model=512, n_head=8, d_ff=2048),
+    "llama_3x77": dict(w=synth.WORKLOADS[5], n_layer=4, cut=2, batch_per_client=3, seq=77, max_seq=77, d_model=512, n_head=4,
+                       d_ff=1280, lora_r=8),
+    "llama_5x333": dict(w=synth.WORKLOADS[5], n_layer=3, cut=1, batch_per_client=5, seq=333, max_seq=333, d_model=512, n_head=8,
+                        d_ff=1280, lora_r=8),
+}
 
 
 def cut_to_rank(ad, r):

@@ -4,7 +4,10 @@ import numpy as np
 import pytest
 import torch
 
+import harness
 from paper_2407_00952_b200 import binding as B
+from paper_2407_00952_b200 import synth
+from test_gpu_parity import TOL_FP32, check_three_calls
 
 pytestmark = pytest.mark.gpu
 
@@ -281,3 +284,18 @@ def test_linear_fp32_tiles(M, K, N):
 def test_linear_tiles_of_128_columns(M, K, N, epilogue):
     """Clusters of two and CTA pairs on tiles of 128 columns, whole and ragged, one and several tiles per pair."""
     test_linear_any_row_count_and_depth(M, K, N, epilogue)
+
+
+@pytest.mark.parametrize("name", sorted(harness.RAGGED_ROUNDS))
+def test_bf16_rounds_off_the_tile_sizes(name):
+    """Whole passes whose rows end inside a tile of every kernel: norm and projection in one launch, adapter gradients of all
+    layers of a side from planes whose last block is partial, attention, linear layers; the general bounds, which
+    test_storage_noise.py shows to hold for these cases."""
+    w, _, bound = harness.qk_case(name)
+    assert bound is None
+    eng = check_three_calls(w, harness.TOL_BF16)
+    assert eng.device_status() == 0
+
+
+def test_fp32_round_off_the_tile_sizes():
+    check_three_calls(synth.scaled(synth.WORKLOADS[1], n_layer=4, cut=2, n_clients=1, counts=(7,), batch_per_client=3, seq=37, max_seq=37), TOL_FP32)

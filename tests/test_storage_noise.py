@@ -77,7 +77,7 @@ def test_exact_storage_model_with_client_cuts_is_the_oracle():
             assert all(H.rel_err(a, b) <= 1e-9 for a, b in zip(cg[i][key], cg_ref[i][key])), (i, key)
 
 
-@pytest.mark.parametrize("name", ["federated_small", "llama_full_width", "ranks_medium", "cuts_medium"])
+@pytest.mark.parametrize("name", ["federated_small", "llama_full_width", "ranks_medium", "cuts_medium", *H.RAGGED_ROUNDS])
 def test_storage_noise_fixes_the_qk_bound(name):
     w, ranks, bound = H.qk_case(name)
     cuts = list(H.CUTS_MEDIUM) if name == "cuts_medium" else None
