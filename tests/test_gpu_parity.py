@@ -251,13 +251,15 @@ def test_lora_linear_fp32():
                                                 (3, 128, 2, 128, True), (2, 384, 4, 256, True),
                                                 (40, 128, 8, 512, True), (37, 256, 5, 320, True),
                                                 (3, 128, 2, 256, True), (2, 384, 3, 384, True),
-                                                (20, 256, 8, 1024, True)])
+                                                (20, 256, 8, 1024, True),
+                                                (16, 512, 16, 1024, True), (40, 384, 8, 512, True)])
 def test_attention_bf16(nseq, T, Hh, d, use_tc):
     """Causal attention forward/backward: tensor-core kernels (head width 64 and 128) and the plain kernels
-    (any head width, ragged length) against the oracle.  Cases 7-10 exercise the persistent tcgen05
-    kernels at head width 64: a single query tile, an odd number of tiles (ring and double-buffer
-    parities), and more (sequence, head) items than resident CTAs, so that a CTA walks several items
-    (320 and 185); the last three do the same at head width 128 (160 items in the last)."""
+    (any head width, ragged length) against the oracle.  Head width 64: a single query tile, an odd number
+    of tiles (ring and double-buffer parities), and more (sequence, head) items than resident CTAs, so that
+    a CTA walks several; the backward pass takes both gradients in one launch, or single tiles (37 x 256),
+    or whole items (40 x 128 of one tile, and the last two of several tiles whose lengths rotate).  Three
+    cases do the same at head width 128 (160 items in the last)."""
     torch.manual_seed(T + d)
     qkv = torch.randn(nseq * T, 3 * d, device="cuda").bfloat16()
     do = torch.randn(nseq * T, d, device="cuda").bfloat16()
