@@ -29,7 +29,8 @@ constexpr int ROWS = 16;                       // of a tile
 constexpr int SLAB = 1024;                     // columns of a slab at most: four chunks of 32 per warp
 constexpr int CHUNKS = SLAB / (32 * WARPS);
 constexpr int MAX_STAGES = 4;                  // of the ring; as many as leave room for two CTAs per SM (launch)
-constexpr int MAX_TILES = 8;                   // column tiles of 8 of Y
+constexpr int MAX_TILES = 4;                   // column tiles of 8 of Y: slabs * tiles bounds the fragments of W in registers, for two CTAs per SM
+constexpr int MAX_EXT = 512;                   // columns of Y, padding included
 
 struct Proj {
   const bf16* X; int64_t ldx;
@@ -41,7 +42,7 @@ struct Proj {
   int stages;
   int pitch;                                   // bytes of a row in the ring: an odd number of 64-byte pieces (no bank conflicts)
   int tile_col[MAX_TILES];                     // first output column of each column tile
-  int8_t tile_of[MAX_TILES * 8];               // ext / 8 entries: the tile that holds columns [8 i, 8 i + 8), or -1
+  int8_t tile_of[MAX_EXT / 8];                  // ext / 8 entries: the tile that holds columns [8 i, 8 i + 8), or -1
   int* status;
 };
 
@@ -108,9 +109,10 @@ __device__ __forceinline__ void put_partial(float (*mine)[8 * TILES], const floa
 // COPIES: W comes in fp32 (rounded to bf16 on the way, as the compute copies are), and the CTAs past `workers` write the
 // layer's compute copies, which the launches after this one need: one launch less in a layer of six.
 template <int SLABS, int N, bool SEPARATE, bool COPIES>
-__global__ void __launch_bounds__(THREADS, SLABS * N <= 4 ? 2 : 1)
+__global__ void __launch_bounds__(THREADS, 2)
 proj_kernel(const __grid_constant__ Proj p, int workers, const __grid_constant__ AdapterCopyArgs copies, int64_t copy_vectors) {
   constexpr int TILES = SEPARATE ? SLABS * N : N, COLS = 8 * TILES;
+  static_assert(SLABS * N <= MAX_TILES, "registers for two CTAs per SM");
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES];
   __shared__ __align__(16) float red[2][WARPS][ROWS][COLS];
@@ -370,9 +372,9 @@ __global__ void __launch_bounds__(THREADS) norm_proj_f32_kernel(const float* __r
 template <int SLABS, int N, bool SEPARATE, bool COPIES>
 cudaError_t launch(Proj p, const AdapterCopyArgs& copies, cudaStream_t st) {
   const auto kernel = proj_kernel<SLABS, N, SEPARATE, COPIES>;
-  // two CTAs per SM where registers allow (228 KB, of which each takes 1 KB and its static part), else one
-  constexpr int PER_SM = SLABS * N <= 4 ? 2 : 1, STATIC = 2 * WARPS * ROWS * 8 * (SEPARATE ? SLABS * N : N) * 4 + 1024;
-  constexpr int ROOM = (228 * 1024) / PER_SM - 1024 - STATIC;
+  // two CTAs per SM (228 KB, of which each takes 1 KB and its static part)
+  constexpr int STATIC = 2 * WARPS * ROWS * 8 * (SEPARATE ? SLABS * N : N) * 4 + 1024;
+  constexpr int ROOM = (228 * 1024) / 2 - 1024 - STATIC;
   p.stages = ROOM / (ROWS * p.pitch);
   p.stages = p.stages > MAX_STAGES ? MAX_STAGES : p.stages;
   const int smem = p.stages * ROWS * p.pitch;
@@ -384,7 +386,7 @@ cudaError_t launch(Proj p, const AdapterCopyArgs& copies, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     once.done(dev);
   }
-  const int tiles = (p.M + ROWS - 1) / ROWS, slots = PER_SM * num_sms();
+  const int tiles = (p.M + ROWS - 1) / ROWS, slots = 2 * num_sms();
   const int workers = tiles < slots ? tiles : slots;
   const int64_t vectors = COPIES ? adapter_copy_vectors(copies) : 0;
   return launch_overlapped(kernel, (unsigned)(workers + (vectors + THREADS - 1) / THREADS), THREADS, smem, st, p, workers, copies, vectors);
@@ -399,7 +401,7 @@ Shape shape_of(const ProjArgs& a) {
   s.separate = a.nt > 1 && a.k_slice > 0;
   s.slabs = s.separate ? a.nt : (a.K + SLAB - 1) / SLAB;
   s.n = s.separate ? per_target : a.nt * per_target;
-  const bool fits = s.separate ? a.k_slice <= SLAB && s.slabs <= 3 && s.slabs * s.n <= 4 : (s.slabs == 1 && s.n <= 4) || (s.slabs == 2 && s.n <= 2) || (s.slabs <= 4 && s.n == 1);
+  const bool fits = s.separate ? a.k_slice <= SLAB && s.slabs <= 3 && s.slabs * s.n <= MAX_TILES : (s.slabs == 1 && s.n <= 4) || (s.slabs == 2 && s.n <= 2) || (s.slabs <= 4 && s.n == 1);
   if (!fits) s.slabs = 0;
   return s;
 }
@@ -414,7 +416,7 @@ void fill(const ProjArgs& a, const Shape& s, Proj& p) {
   for (int i = 0; i < 4; ++i) p.slab_col[i] = i >= s.slabs ? 0 : s.separate ? a.slice_col[i] : i * p.slab_len;
   p.pitch = (2 * p.slab_len + 127) / 128 * 128 + 64;
   int n = 0;
-  for (int i = 0; i < MAX_TILES * 8; ++i) p.tile_of[i] = -1;
+  for (int i = 0; i < MAX_EXT / 8; ++i) p.tile_of[i] = -1;
   for (int t = 0; t < a.nt; ++t)
     for (int j = 0; j < a.r; j += 8) {
       p.tile_col[n] = t * a.rp + j;
@@ -493,7 +495,7 @@ bool with_status(Proj& p) {
 bool lora_proj_supported(const ProjArgs& a) {
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   if (a.M < 1 || a.K < 8 || a.K % 8 || a.ldx % 8 || a.ldw % 8 || a.w_group_stride % 8 || a.k_slice % 8) return false;
-  if (a.r < 1 || a.nt < 1 || a.ext % 8 || a.ext > 8 * MAX_TILES * 8 || a.rp % 8 || a.r > a.rp || a.nt * a.rp > a.ext) return false;
+  if (a.r < 1 || a.nt < 1 || a.ext % 8 || a.ext > MAX_EXT || a.rp % 8 || a.r > a.rp || a.nt * a.rp > a.ext) return false;
   if (a.rows_per_group > 0 && a.rows_per_group < a.M && (a.rows_per_group % ROWS || a.M % a.rows_per_group)) return false;
   return al16(a.X) && al16(a.W) && al16(a.Y) && shape_of(a).slabs > 0;
 }
