@@ -223,16 +223,17 @@ bool lora_grad_tc_supported(int dt, const void* Z, int64_t ldz, int zcol0, int C
 }
 
 // Chunks per group (at most max_chunks) for a grid of `ctas_per_chunk_set` CTAs per chunk: the choice that minimises
-// (waves of 296 resident CTAs) x (rows per chunk), every chunk a whole number of 128-row blocks.  One chunk needs no second
+// (waves of resident CTAs, two per SM) x (rows per chunk), every chunk a whole number of 128-row blocks.  One chunk needs no second
 // kernel, which is worth about 4 us: 1000 rows of a CTA that has an SM's loads to itself, 300 of one among two per SM.
 static int pick_chunks(int ctas_per_chunk_set, int rpg, int64_t max_chunks) {
-  const double second_kernel = ctas_per_chunk_set > 148 ? 300.0 : 1000.0;
+  const int sms = num_sms() > 0 ? num_sms() : 1, resident = 2 * sms;
+  const double second_kernel = ctas_per_chunk_set > sms ? 300.0 : 1000.0;
   int best = 1;
   double best_cost = 1e300;
   for (int s = 1; s <= rpg / 128 && s <= (max_chunks > 1 ? max_chunks : 1); ++s) {
     if (rpg % (s * 128) != 0) continue;
     const int ctas = ctas_per_chunk_set * s;
-    const double cost = (double)((ctas + 295) / 296) * ((double)rpg / s + 256.0) + (s > 1 ? second_kernel : 0.0);   // 256: a chunk's start-up
+    const double cost = (double)((ctas + resident - 1) / resident) * ((double)rpg / s + 256.0) + (s > 1 ? second_kernel : 0.0);   // 256: a chunk's start-up
     if (cost < best_cost) { best_cost = cost; best = s; }
   }
   return best;
