@@ -178,9 +178,9 @@ int validate(const splitlora_config* c, std::string* why) {
   return SPLITLORA_OK;
 }
 
-// Jobs of the adapter gradients of `layers` layers (G_A = dh^T u of every qkv target in one pass over u, G_B = (alpha/r)
-// dy^T h of each target, and the same for the output projection), the first layer's buffers and gradients given, each kind
-// of buffer at one stride (plan).
+// Jobs of the adapter gradients of a layer, or of several (the first one's buffers and gradients given, each kind of buffer
+// at one stride, see plan): G_A = dh^T u of every qkv target in one pass over u, G_B = (alpha/r) dy^T h of each target (nq + 1
+// jobs), and the same for the output projection (two more).
 int grad_jobs(const splitlora_ctx* c, const LayerBuf& b, float* out, int64_t group_stride, LoraGradJob* jobs) {
   const int d = c->d;
   const size_t es = c->es, M = c->M;
@@ -598,7 +598,7 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   const float* lse = b.lse + (size_t)(sp.row0 / T) * H * T;
   const void* dy = at(dy_base, d);
   void* dx = dx_base ? at(dx_base, d) : nullptr;
-  const void* u = at(b.u, d); const void* hcat = at(b.hcat, ext); const void* qkv = at(b.qkv, 3 * d);
+  const void* qkv = at(b.qkv, 3 * d);
   const void* o = at(b.o, d); const void* x_mid = at(b.x_mid, d); const void* z = at(b.z, c->Fz);
   void *g_dqkv = b.dqkv, *g_dhcat = b.dhcat, *g_dxmid = b.dxmid, *g_dhcat_o = b.dhcat_o;
   cudaError_t e;
@@ -606,6 +606,13 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   float* gbase = client ? c->cg + (size_t)sp.client0 * c->Pc + (size_t)l * c->per_layer
                         : c->sg + (size_t)(l - c->cmin) * c->per_layer;
   const int64_t gstride = client ? c->Pc : 0;
+  LoraGradJob jobs[LORA_GRAD_MAX_JOBS];
+  int njobs = 0;
+  if (!c->defer_grads) {
+    LayerBuf rows = b;                             // from the span's first row on (the gradients' buffers hold the span only)
+    rows.u = at(b.u, d); rows.hcat = at(b.hcat, ext); rows.o = at(b.o, d); rows.hcat_o = c->has_o ? at(b.hcat_o, c->ext_o) : nullptr;
+    njobs = grad_jobs(c, rows, gbase, gstride, jobs);
+  }
   if (c->llama) {
     { GemmArgs a = base_args(c, dy, d, f.fc2wT, d, c->act, F, M, F, d);               // d act
       if ((e = linear(c, "linear_bwd", a))) return e; }
@@ -621,18 +628,14 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   if ((e = norm_backward(c, M, c->g_du2, x_mid, f.ln2g, atf(b.mean2), atf(b.rstd2), dy, g_dxmid))) return e;
   if (c->has_o) {
     // dh_o = (alpha/r) dx_mid B_o,g ;  G_A = dh_o^T o ;  G_B = (alpha/r) dx_mid^T h_o   (Eq. 4-7)
-    const void* hcat_o = at(b.hcat_o, c->ext_o);
     { GemmArgs a = base_args(c, g_dxmid, d, grp(k.BextOT, (size_t)c->ext_o * d), d, g_dhcat_o, c->ext_o, M, c->ext_o, d);
       a.rows_per_group = rpg; a.w_grouped = grouped;
       if ((e = rank_proj(c, "lora_down_bwd", a, proj_args(c, a, 1)))) return e; }
-    float* gA = gbase + (size_t)c->nq * 2 * c->r * d;
-    if (!c->defer_grads) {
-    { Scope s(c, "lora_grad");
-      if ((e = lora_grad(c->dt, o, d, 0, d, g_dhcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, 1.0f, gA, gstride, 0, d,
-                         1, c->grad_scratch, c->st, c->status, c->tc))) return e; }
-    { Scope s(c, "lora_grad");
-      if ((e = lora_grad(c->dt, g_dxmid, d, 0, d, hcat_o, c->ext_o, 0, c->r, c->rp, 1, M, rpg, c->scale,
-                         gA + (size_t)c->r * d, gstride, 0, 1, c->r, c->grad_scratch, c->st, c->status, c->tc))) return e; }
+    for (int j = c->nq + 1; j < njobs; ++j) {
+      Scope s(c, "lora_grad");
+      const LoraGradJob& jb = jobs[j];
+      if ((e = lora_grad(c->dt, jb.Z, jb.ldz, jb.zcol0, jb.C, jb.Wt, jb.ldwt, jb.wcol0, jb.r, jb.rp, jb.nt, M, rpg, jb.scale, jb.out, jb.out_group_stride,
+                         jb.out_target_stride, jb.out_sj, jb.out_sc, c->grad_scratch, c->st, c->status, c->tc))) return e;
     }
   }
   { GemmArgs a = base_args(c, g_dxmid, d, f.projwT, d, c->g_do, d, M, d, d);
@@ -678,21 +681,9 @@ cudaError_t block_backward(splitlora_ctx* c, int l, const Span& sp, const void* 
   }
   // G_A = dh^T u (every qkv target in one pass over u) and G_B = (alpha/r) dy^T h of each target, per
   // group (Eq. 4-7): one batch, i.e. one pair of launches where the tensor-core path applies
-  if (!c->defer_grads) {
-    LoraGradJob jobs[4];
-    int nj = 0;
-    LoraGradJob& ja = jobs[nj++];
-    ja.Z = u; ja.ldz = d; ja.zcol0 = 0; ja.C = d; ja.Wt = g_dhcat; ja.ldwt = ext; ja.wcol0 = 0; ja.r = c->r; ja.rp = c->rp;
-    ja.nt = c->nq; ja.scale = 1.0f; ja.out = gbase; ja.out_group_stride = gstride; ja.out_target_stride = (int64_t)2 * c->r * d;
-    ja.out_sj = d; ja.out_sc = 1;
-    for (int t = 0; t < c->nq; ++t) {
-      LoraGradJob& jb = jobs[nj++];
-      jb.Z = g_dqkv; jb.ldz = 3 * d; jb.zcol0 = c->slice_idx[t] * d; jb.C = d; jb.Wt = hcat; jb.ldwt = ext; jb.wcol0 = t * c->rp;
-      jb.r = c->r; jb.rp = c->rp; jb.nt = 1; jb.scale = c->scale; jb.out = gbase + (size_t)t * 2 * c->r * d + (size_t)c->r * d;
-      jb.out_group_stride = gstride; jb.out_target_stride = 0; jb.out_sj = 1; jb.out_sc = c->r;
-    }
+  if (njobs > 0) {
     Scope s(c, "lora_grad");
-    if ((e = lora_grad_batch(c->dt, jobs, nj, M, rpg, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc))) return e; }
+    if ((e = lora_grad_batch(c->dt, jobs, c->nq + 1, M, rpg, c->grad_scratch, c->grad_scratch_floats, c->st, c->status, c->tc))) return e; }
   if (dx) {
     GemmArgs a = base_args(c, g_dqkv, 3 * d, f.qkvwT, 3 * d, c->g_du, d, M, d, 3 * d);
     a.rows_per_group = rpg;
