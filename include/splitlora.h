@@ -270,8 +270,8 @@ int splitlora_launch_count(const splitlora_ctx* ctx, int64_t* launches);
 /* Per-kernel-class device time: when enabled, each launch is bracketed by CUDA events on the
  * context stream; splitlora_profile_report copies up to `cap` entries of {name, launches,
  * milliseconds} into HOST arrays and returns the number of classes in *n.
- * A norm and the rank-r projection behind it are "layernorm_fwd" and "lora_down_fwd", or, up to 4096 rows where one launch
- * does both, "layernorm_lora_down_fwd".
+ * A norm and the rank-r projection behind it are "layernorm_fwd" and "lora_down_fwd", or, where one launch does both (few or
+ * narrow rows), "layernorm_lora_down_fwd".
  * on: 0 off; 1 every launch class; 2 only the tensor-bound linear layers (classes "lora_linear_*",
  * "linear_*", "head_*"), which leaves two thirds of a round's launches without events between them. */
 int splitlora_profile_enable(splitlora_ctx* ctx, int on);

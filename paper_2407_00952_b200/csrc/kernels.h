@@ -157,16 +157,19 @@ struct ProjArgs {
 };
 bool lora_proj_supported(const ProjArgs& a);
 // Rows up to which these kernels beat the linear layers' narrow tiles: (512, 2048 -> 2 x 4 of 32) 8.8 -> 5.5 us from cold
-// caches; 12 of 1665 x 1536 149 -> 104, of 16384 x 1536 225 -> 252, 24 of 32768 x 2048 910 -> 966.  With the norm in front
-// (fused, norm_proj) they save a launch and a read of its rows, which shows in rounds of few rows and costs in those of many,
-// where the two launches overlap: norm and projection apart -> one launch, 8 to 24 blocks, 512 rows of 1024 3068 -> 3058 us, 1665 of 768
-// 2285 -> 2264, 2048 of 768 1653 -> 1643, 4096 and 8192 equal, 12288 of 768 6148 -> 6197, 16384 of 768 8289 -> 8366, of 1024 11795 -> 11873.
+// caches; 12 of 1665 x 1536 149 -> 104, of 16384 x 1536 225 -> 252, 24 of 32768 x 2048 910 -> 966.
 constexpr int LORA_PROJ_ROWS = 4096;
 cudaError_t lora_proj(const ProjArgs& a, cudaStream_t st);
 // The same for one target whose W is the fp32 A [r, K] itself, with the compute copies of write_adapter_copies in the same launch.
 cudaError_t lora_proj_copies(const ProjArgs& a, const AdapterCopyArgs& copies, cudaStream_t st);
 // The norm in front of it in the same launch: a.X [M, K] receives LayerNorm(x) (RMSNorm: b and mean unused), Y its projection.
 bool norm_proj_supported(const ProjArgs& a);
+// Whether that pays: it saves a launch and a read of the rows, but two launches overlap, which weighs more where the rows are many
+// and wide.  Rounds of 4 blocks, apart -> together, us: width 256, 5120 rows 599 -> 587, 16384 1012 -> 996; 512, 5120 891 -> 874,
+// 12288 1475 -> 1463, 16384 1814 -> 1818; 768, 5120 1119 -> 1115, 8192 equal, 12288 2211 -> 2219, 16384 2945 -> 2962; 1024, 8192 equal,
+// 12288 3372 -> 3385, 16384 4397 -> 4417; 24 blocks of 512 x 1024 3068 -> 3058, 12 of 1665 x 768 2285 -> 2264.
+constexpr int NORM_PROJ_ROWS = 16384;
+inline bool norm_proj_pays(int M, int d) { return M <= NORM_PROJ_ROWS && (int64_t)M * d <= 8 << 20; }
 // the same in fp32, LayerNorm only
 bool norm_proj_f32_supported(const ProjArgs& a);
 cudaError_t norm_proj_f32(const void* x, const void* g, const void* b, float* mean, float* rstd, float eps, const ProjArgs& a, cudaStream_t st);

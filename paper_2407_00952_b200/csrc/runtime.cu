@@ -519,7 +519,7 @@ cudaError_t block_forward(splitlora_ctx* c, int l, const Span& sp, const void* x
     GemmArgs a = base_args(c, u, d, grp(k.Acat, (size_t)ext * d), d, hcat, ext, M, ext, d);
     a.rows_per_group = rpg; a.w_grouped = grouped;
     const ProjArgs p = proj_args(c, a, c->nq);
-    if (c->tc && M <= LORA_PROJ_ROWS && norm_proj_supported(p)) {
+    if (c->tc && norm_proj_pays(M, d) && norm_proj_supported(p)) {
       Scope s(c, "layernorm_lora_down_fwd");
       if ((e = norm_proj(c->llama, xin, f.ln1g, f.ln1b, atf(b.mean1), atf(b.rstd1), c->cfg.norm_eps, p, c->st))) return e;
     } else if (c->dt == DT_F32 && !c->llama && M <= LORA_PROJ_ROWS && norm_proj_f32_supported(p)) {

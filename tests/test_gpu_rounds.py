@@ -178,8 +178,8 @@ def test_adamw_kernel_on_identical_inputs(step):
             assert np.abs(p[part] - p_ref)[sel].max() <= 1e-6 * np.abs(p_ref).max(), (key, part)
 
 
-def _forward_classes(batch):
-    w = synth.scaled(synth.WORKLOADS[2], n_layer=3, cut=1, n_clients=1, counts=(7,), batch_per_client=batch, d_model=256, n_head=4, d_ff=512, vocab=512)
+def _forward_classes(batch, d):
+    w = synth.scaled(synth.WORKLOADS[2], n_layer=3, cut=1, n_clients=1, counts=(7,), batch_per_client=batch, d_model=d, n_head=d // 64, d_ff=512, vocab=512)
     frozen, cads, sads, tokens, labels = H.build_case(w)
     eng = runner.make_engine(w, frozen, cads, sads)
     eng.profile_enable(True)
@@ -187,12 +187,14 @@ def _forward_classes(batch):
     return {k: v[0] for k, v in eng.profile_report().items()}
 
 
-def test_many_rows_project_in_launches_of_their_own():
-    """The norm overlaps with the rank-r projection behind it; one launch for both is slower from some 8192 rows on."""
-    n = _forward_classes(batch=17)                                # 8704 rows
-    assert n["layernorm_fwd"] == 2 * 3 + 1 and n["lora_down_fwd"] == 3
+@pytest.mark.parametrize("batch,d", [(17, 1024), (33, 256)])
+def test_many_rows_project_in_launches_of_their_own(batch, d):
+    """8704 rows of 1024, 16896 of 256: the norm overlaps with the rank-r projection behind it, one launch for both is slower."""
+    n = _forward_classes(batch, d)
+    assert n["layernorm_fwd"] == 2 * 3 + 1 and n["lora_down_fwd"] == 3 and "layernorm_lora_down_fwd" not in n
 
 
-def test_few_rows_name_the_launch_that_does_both():
-    n = _forward_classes(batch=3)
+@pytest.mark.parametrize("batch,d", [(3, 1024), (32, 256)])
+def test_few_rows_name_the_launch_that_does_both(batch, d):
+    n = _forward_classes(batch, d)
     assert n["layernorm_fwd"] == 3 + 1 and n["layernorm_lora_down_fwd"] == 3 and "lora_down_fwd" not in n
