@@ -17,11 +17,11 @@
 // 146 -> 147, 8 of 192 with 8 heads 15.0 -> 15.6; in tiles of 64 on mma.sync that one took 23.)
 // What bounds them: neither unit by itself.  A half-step is 10 + 16 (dQ: 10 + 8) products [128 x 64 x 16] of 45-48 cycles
 // (operand reads from shared memory) next to 512 cycles of exponentials; 16 sequences of 777 tokens, 12 heads, have 80 us of
-// products and take 123 us (mma.sync, attention_tc.cu: 339), the tensor pipe active for 36 % (dQ) and 43 % of the cycles.  With P
-// and dS as single bf16 values (template HILO = false, for lengths that always had that precision) the time is the same, and so
-// it is with the element-wise warps in two groups on alternate half-steps: the chain of barriers, tensor-memory loads and
-// stores from a score to its release is what three half-steps in flight do not cover.  Errors against 64 bits agree with the
-// mma.sync form's to four digits.
+// products and take 120 us (mma.sync, attention_tc.cu: 336), the tensor pipe active for 36 % (dQ) and 43 % of the cycles.  P and dS
+// as single bf16 values (template HILO = false, for lengths that always had that precision) save 15 % (16 x 960, 12 heads 174 -> 148 us);
+// with the element-wise warps in two groups on alternate half-steps the time is the same: the chain of barriers, tensor-memory
+// loads and stores from a score to its release is what three half-steps in flight do not cover.  Errors against 64 bits agree with
+// the mma.sync form's to four digits.
 // Few tiles: both kernels run as one launch on their own CTAs (attn64_bwd_t5_kernel), the dK/dV tiles forming D themselves:
 // 2 sequences of 256, 16 heads 15.0 -> 9.5 us against the two kernels of attention_t5_bwd.cu.
 #include "attention_rows.cuh"
@@ -797,7 +797,7 @@ attn64_bwd_t5_kernel(const __grid_constant__ CUtensorMap mapQKV, const __grid_co
 // P as hi + lo pairs in two buffers; O stays in tensor memory and is rescaled only when a row's maximum has moved by more
 // than 2^2 since the one its exponentials are taken against (2^8 left lse 2 % further off: the exponents' rounding); the row
 // sum is compensated.  Bound by the chain of a step (scores, tensor-memory loads, softmax, store, product) of two CTAs per SM:
-// 16 sequences of 777 tokens, 12 heads 77 us (mma.sync 115) with the tensor pipe active for 18 % of the cycles.
+// 16 sequences of 777 tokens, 12 heads 76 us (mma.sync 114) with the tensor pipe active for 18 % of the cycles.
 namespace fwd {
 constexpr int HK = 32;                                     // keys per step
 constexpr int THREADS = 192;

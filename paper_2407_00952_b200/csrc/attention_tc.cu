@@ -9,7 +9,7 @@
 //     mantissa bits) against the exact bf16 operand: twice the products of that operand, none of the precision
 //     lost (error of o / dqkv against 64 bits over odd T is that of the bf16 output alone, as before).  Measured,
 //     16 sequences of 777 tokens, 12 heads of 64, forward + backward: 466 us against 72.9 ms; width 64 now runs on
-//     tcgen05 from the lengths and tile counts on that the two dispatches below give (200 us, attention_t5_ragged.cu).
+//     tcgen05 from the lengths and tile counts on that the two dispatches below give (196 us, attention_t5_ragged.cu).
 //     Bound by the tensor issue of mma.sync and by ldmatrix traffic (the hi and lo products share one fragment of the
 //     right operand).  Shapes that the aligned forms take stay with them.
 //   forward : one CTA per (sequence, head, 64-row query tile), 4 warps x 16 rows, K/V tiles double
@@ -633,9 +633,10 @@ cudaError_t launch_bwd(const void* qkv, const void* o, const float* lse, const v
   dim3 grid((T + BT - 1) / BT, H, nseq);
   // Few blocks, but more than half as many as SMs: a kernel that starts early is placed where the one before it leaves
   // room, some SMs with three blocks (as many as are resident at once at width 64) and some with none, and then takes as
-  // long as the fullest SM.  So these start in order.  Backward us, early -> in order: 8 x 192, 8 heads of 64 23.4 -> 19.6;
-  // 16 x 64 11.9 -> 9.7; 2 x 960 76.9 -> 61.9; outside the range 4 x 64 8.0 -> 8.6, 32 x 192 39.3 -> 40.3.  (The RG forms
-  // have no kernel in front of dQ that would upset its placement: 8 x 100 12.7 -> 13.3, so they start early.)
+  // long as the fullest SM.  So these start in order.  Backward us, early -> in order, 64-row sequences of width 64: 16 with
+  // 8 heads 11.7 -> 9.7, 24 13.6 -> 11.9, 10 10.1 -> 9.5, but 32 with 12 heads, the end of the range, 14.7 -> 15.7; width 128: 16 x 64, 8 heads
+  // 16.8 -> 13.3, 2 x 960, 4 heads 95.8 -> 68.5, 8 x 192, 4 heads 23.7 -> 20.8, 8 heads 29.8 -> 30.6.  (Width 64 comes here at 64 rows
+  // only.  The RG forms have no kernel in front of dQ that would upset its placement: 8 x 100 12.7 -> 13.3, so they start early.)
   const int64_t blocks = (int64_t)grid.x * H * nseq, sms = num_sms();
   const bool in_order = !RG && 2 * blocks > sms && blocks <= 3 * sms;
   if (in_order) break_chain();
@@ -708,9 +709,9 @@ bool attention_ragged_supported(int dt, int nseq, int T, int H, int d, const voi
 }
 
 cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d, void* o, float* lse, int* status, cudaStream_t st) {
-  // Tiles of 128 on tcgen05 against tiles of 64 here, us: 16 sequences of 777, 12 heads 115 -> 83; 32 x 288 44.7 -> 37.5; 5 x 333
-  // 17.6 -> 13.5; 4 x 1000, 8 heads 41.5 -> 29.9; 64 x 70, 16 heads 27 -> 17.3; with fewer tiles than SMs the longer steps of one CTA
-  // show: 1 x 1000, 8 heads 20.7 -> 27.7, 1 x 333 9.4 -> 13.1; up to 64 rows half a tile is padding: 64 x 50 11.3 -> 14.7.
+  // Tiles of 128 on tcgen05 against tiles of 64 here, us: 16 sequences of 777, 12 heads 114 -> 76; 32 x 288 44 -> 35.5; 5 x 333
+  // 17.4 -> 13.8; 4 x 1000, 8 heads 41.5 -> 30.6; 64 x 70, 16 heads 26.8 -> 17.6; with fewer tiles than SMs the longer steps of one CTA
+  // show: 1 x 1000, 8 heads 20.5 -> 28.2, 1 x 333 9.1 -> 12.9; up to 64 rows half a tile is padding: 64 x 50, 16 heads 11.1 -> 14.8.
   if (attention_ragged_t5_supported(nseq, T, H, d) && T > 64 && (int64_t)nseq * H * ((T + 127) / 128) > num_sms())
     return attention_fwd_ragged_t5(qkv, nseq, T, H, d, o, lse, status, st);
   switch ((d / H + 31) / 32) {
@@ -724,10 +725,11 @@ cudaError_t attention_fwd_ragged(const void* qkv, int nseq, int T, int H, int d,
 
 cudaError_t attention_bwd_ragged(const void* qkv, const void* o, const float* lse, const void* d_o, int nseq, int T, int H,
                                  int d, void* dqkv, float* rowdot, int* status, cudaStream_t st) {
-  // Tiles of 128 on tcgen05 against tiles of 64 here, backward us: 16 sequences of 777, 12 heads 339 -> 123; 32 x 288 134 -> 62;
-  // 5 x 333 44 -> 22; one of 150 with 4 heads 14.2 -> 14.1.  Up to 128 rows a head is one tile there, whose fixed part (set-up,
-  // first loads) shows until there are about as many heads as SMs: 64 x 70, 16 heads 80 -> 41; 16 x 100, 8 heads 16.8 -> 15.4;
-  // 8 x 100 12.3 -> 13.5; 2 x 96, 12 heads 11.8 -> 13.3.  Up to 64 rows half of that tile is padding: 64 x 50, 16 heads 33.6 -> 34.6.
+  // Tiles of 128 on tcgen05 against tiles of 64 here, backward us: 16 sequences of 777, 12 heads 336 -> 120; 32 x 288 133 -> 62;
+  // 5 x 333 44 -> 22; one of 150 with 4 heads 14.2 -> 10.1.  Up to 128 rows a head is one tile there, whose fixed part (set-up,
+  // first loads) shows until there are about as many heads as SMs, unless both gradients fit one launch: 64 x 70, 16 heads 79 -> 42;
+  // 16 x 100, 8 heads 16.2 -> 15.4; as two kernels 8 x 100 12.3 -> 13.5, 2 x 96, 12 heads 11.8 -> 13.3, which is where the line lies (in
+  // one launch, as they would run there now, 9.1 and 8.8).  Up to 64 rows half of that tile is padding: 64 x 50, 16 heads 32.8 -> 37.3.
   if (attention_ragged_t5_supported(nseq, T, H, d) && (T > 128 || (T > 64 && (int64_t)nseq * H * 4 > 3 * (int64_t)num_sms())))
     return attention_bwd_ragged_t5(qkv, o, lse, d_o, nseq, T, H, d, dqkv, rowdot, status, st);
   switch ((d / H + 31) / 32) {

@@ -226,7 +226,7 @@ bool lora_grad_tc_supported(int dt, const void* Z, int64_t ldz, int zcol0, int C
 // (waves of resident CTAs, two per SM) x (rows per chunk), every chunk a whole number of 128-row blocks.  One chunk needs no second
 // kernel, which is worth about 4 us: 1000 rows of a CTA that has an SM's loads to itself, 300 of one among two per SM.
 static int pick_chunks(int ctas_per_chunk_set, int rpg, int64_t max_chunks) {
-  const int sms = num_sms() > 0 ? num_sms() : 1, resident = 2 * sms;
+  const int n = num_sms(), sms = n > 0 ? n : 1, resident = 2 * sms;
   const double second_kernel = ctas_per_chunk_set > sms ? 300.0 : 1000.0;
   int best = 1;
   double best_cost = 1e300;

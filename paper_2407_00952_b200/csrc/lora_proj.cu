@@ -10,7 +10,7 @@
 // steps.  Only the column tiles of 8 that hold adapters are computed, of a slab that is one target's slice only that
 // target's; the padding is written as zeros.
 // What bounds it: over few rows the latency of one pass; over many rows the read of X, at which the linear-layer kernels'
-// narrow tiles are as good or better (lora_proj_preferred).
+// narrow tiles are as good or better (LORA_PROJ_ROWS).
 // norm_proj_kernel is the forward projection with the norm in front of it: u = LayerNorm(x) (or RMSNorm), h = u A^T.
 #include "adapter_copies.cuh"
 #include "common.cuh"

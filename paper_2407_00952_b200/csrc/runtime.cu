@@ -209,7 +209,8 @@ int grad_jobs(const splitlora_ctx* c, const LayerBuf& b, float* out, int64_t gro
 
 // Up to this many token rows the adapter gradients of all layers of a side are formed together at the end of its backward
 // pass: at 512 rows a layer's pair of launches is 10 us of a chain, and nothing waits for its results but the optimizer.
-// Beyond, their cost is the traffic either way.  The layers' gradients (3-4 d values per row and layer) take the place of the
+// Beyond, their cost is the traffic either way: whole rounds of 8 blocks, a pair of launches per layer -> deferred, 2048 x 768 rows 1669 ->
+// 1643 us, 4096 2495 -> 2477, 8192 4649 -> 4651; 2048 x 1024 1999 -> 1985, 8192 6137 -> 6105 (runs differ by 1 %).  The layers' gradients (3-4 d values per row and layer) take the place of the
 // layer's own z, x_out and x_mid, which its backward pass has read by the time they are written, and the partial sums that
 // of the logits and the MLP's temporaries: the workspace is no larger than with a pair of launches per layer.
 constexpr int DEFER_ROWS = 4096;
